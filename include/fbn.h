@@ -82,8 +82,8 @@ typedef struct fbn_options {
     int32_t statistic;   /* FBN_STAT_G2 (default) or FBN_STAT_X2: the statistic of every CI test */
     int32_t df_mode;     /* FBN_DF_FIXED (default) or FBN_DF_ADJUSTED: degrees of freedom of every CI test */
     int32_t loop;        /* FBN_LOOP_DEVICE (default) or FBN_LOOP_HOST: who drives the depth loop */
-    int32_t count;       /* FBN_COUNT_*: how contingency tables are counted (pool form and explicit tests; the
-                            plain form always uses byte histograms) */
+    int32_t count;       /* FBN_COUNT_*: how contingency tables are counted (pool form; the plain form and the
+                            explicit tests always use byte histograms) */
     int32_t tune;        /* FBN_TUNE_OFF (default) or FBN_TUNE_AUTO */
     int32_t reserved[4]; /* must be zero */
 } fbn_options;

@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/fbn.h"
+#include "fbn_ci.cuh"
 #include "fbn_gram.h"
 #include "fbn_nbr.h"
 #include "fbn_sepsets.h"
@@ -240,18 +241,21 @@ struct fbn_handle {
     int32_t* d_deg = nullptr;
     int32_t* d_sep_len = nullptr;
     int64_t* d_sep_off = nullptr;
-    ProblemDev* d_prob = nullptr;
-    // single-test scratch
-    CiTestDesc* d_ci = nullptr;
-    double* d_ci_out = nullptr;
-    unsigned* d_status = nullptr;
+    // explicit tests: the kernel writes its results and small tables straight
+    // into pinned host memory; larger tables and global tables on the device
+    double* h_ci_out = nullptr;   // pinned: statistic, df, p
+    unsigned* h_status = nullptr; // pinned
+    double* ci_out_dev = nullptr; // the two as the device addresses them
+    unsigned* status_dev = nullptr;
+    int ci_cluster_max = 0;       // 0: the kernel's limits are not set yet
+    int32_t* h_table = nullptr;   // pinned
+    long long h_table_cap = 0;
     int32_t* d_table = nullptr;
     long long table_cap = 0;
     int* d_gscratch = nullptr;
     long long gscratch_ints = 0;
-    CiTestDesc* h_ci = nullptr;   // pinned
-    double* h_ci_out = nullptr;   // pinned
-    unsigned* h_status = nullptr; // pinned
+    unsigned long long* d_bad = nullptr;   // first out-of-range value of an upload
+    unsigned* d_status = nullptr;
     // one-hot Gram (depth 0 on tensor cores)
     int M = 0;                          // sum of arities
     int Mp = 0;                         // M padded to the tile
@@ -411,13 +415,6 @@ int ensure_gscratch(fbn_handle* h, Workspace& ws, long long total_ints)
     return FBN_OK;
 }
 
-// Whether a table of C cells (plus its marginals, at most 1.25 C entries as
-// r_x, r_y >= 2) fits a shared-memory budget without a global table.
-bool fits_smem(long long C, size_t bytes = kSmemBytes)
-{
-    return C + (C * 5) / 4 + 8 <= (long long)(bytes / 4);
-}
-
 // Largest table a warp group takes: its eighth of the CTA's shared memory.
 long long warp_cells_cap()
 {
@@ -442,14 +439,6 @@ int bits_cells(const fbn_handle* h)
 {
     if (h->opt.form == FBN_FORM_PLAIN || h->opt.count == FBN_COUNT_HIST) return 0;
     return h->opt.count == FBN_COUNT_BITS ? (int)kMaxCells : kBitsCellsAuto;
-}
-
-// Whether the explicit test of (x, y | z) is counted from the bit planes.
-bool test_uses_bits(const fbn_handle* h, int32_t x, int32_t y, const int32_t* z, int32_t nz, long long cells)
-{
-    int mx = std::max(h->h_ar[x], h->h_ar[y]);
-    for (int k = 0; k < nz; ++k) mx = std::max<int>(mx, h->h_ar[z[k]]);
-    return bits_shape_ok(nz, mx, h->N) && cells <= bits_cells(h);
 }
 
 int launch_planes(fbn_handle* h, cudaStream_t st)
@@ -1317,24 +1306,60 @@ int check_test_args(fbn_handle* h, int32_t x, int32_t y, const int32_t* z, int32
     return FBN_OK;
 }
 
+constexpr long long kCiHostTable = 1 << 16;   // cells of a table the kernel writes into pinned host memory
+
+// One explicit test: its statistic, df and p into h->h_ci_out, or its table
+// (want_table) into *table: pinned host memory, or h->d_table for large ones.
+// One launch and one synchronisation: the descriptor goes by value and the
+// results are written straight to the host (with copies each way a test of
+// 5,000 samples took 48 us, of which the kernel was a quarter).
 int run_ci(fbn_handle* h, int32_t x, int32_t y, const int32_t* z, int32_t nz, long long cells, bool want_table)
 {
     CK(cudaSetDevice(h->device));
     cudaStream_t st = h->stream;
-    CiTestDesc& q = *h->h_ci;
-    std::memset(&q, 0, sizeof q);
-    q.x = x; q.y = y; q.d = nz;
-    for (int k = 0; k < nz; ++k) q.z[k] = z[k];
-    if (want_table && cells > h->table_cap) {
-        dfree(h->d_table);
-        h->d_table = nullptr;
-        h->table_cap = 0;
-        CK(dalloc(&h->d_table, cells));
-        h->table_cap = cells;
+    if (!h->ci_cluster_max) CK(prepare_ci(kSmemBytes, &h->ci_cluster_max));
+    CiArgs q{};
+    for (int k = 0; k < nz + 2; ++k) {
+        const int v = k < nz ? z[k] : k == nz ? x : y;
+        q.rows[k] = h->d_data + (long long)v * h->ld;
+        q.rad[k] = h->h_ar[v];
     }
-    long long gints = 0;
-    if (!fits_smem(cells)) {
-        gints = 3 * cells + 64;
+    q.nrows = nz + 2;
+    q.rx = h->h_ar[x];
+    q.ry = h->h_ar[y];
+    q.N = (int)h->N;
+    q.cells = cells;
+    q.smem_ints = (int)(kSmemBytes / 4);
+    q.stat = h->opt.statistic;
+    q.df_mode = h->opt.df_mode;
+    const int k = ci_cluster(h->N, cells, h->ci_cluster_max);
+    if (want_table) {
+        if (cells <= kCiHostTable) {
+            if (cells > h->h_table_cap) {
+                if (h->h_table) cudaFreeHost(h->h_table);
+                h->h_table = nullptr;
+                h->h_table_cap = 0;
+                CK(cudaMallocHost((void**)&h->h_table, cells * sizeof(int32_t)));
+                h->h_table_cap = cells;
+            }
+            CK(cudaHostGetDevicePointer((void**)&q.table_out, h->h_table, 0));
+        } else {
+            if (cells > h->table_cap) {
+                dfree(h->d_table);
+                h->d_table = nullptr;
+                h->table_cap = 0;
+                CK(dalloc(&h->d_table, cells));
+                h->table_cap = cells;
+            }
+            q.table_out = h->d_table;
+        }
+    } else {
+        q.out = h->ci_out_dev;
+        q.status = h->status_dev;
+        q.lgamma_a = ci_lgamma(q.rx, q.ry, cells);
+    }
+    if (!ci_fits_smem(cells, q.rx, q.ry, k, q.smem_ints)) {
+        const long long gints = 3 * cells + 64;
         if (gints > h->gscratch_ints) {
             dfree(h->d_gscratch);
             h->d_gscratch = nullptr;
@@ -1342,16 +1367,10 @@ int run_ci(fbn_handle* h, int32_t x, int32_t y, const int32_t* z, int32_t nz, lo
             CK(dalloc(&h->d_gscratch, gints));
             h->gscratch_ints = gints;
         }
+        q.gtab = h->d_gscratch;
     }
-    CK(set_kernel_smem(kSmemBytes));
-    CK(cudaMemcpyAsync(h->d_ci, h->h_ci, sizeof(CiTestDesc), cudaMemcpyHostToDevice, st));
-    CK(cudaMemsetAsync(h->d_status, 0, sizeof(unsigned), st));
-    launch_ci_tests(h->d_prob, h->d_ci, 1, h->d_ci_out, want_table ? h->d_table : nullptr,
-                    gints ? h->d_gscratch : nullptr, gints, h->d_status, kSmemBytes, h->opt.statistic, h->opt.df_mode,
-                    test_uses_bits(h, x, y, z, nz, cells), st);
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(h->h_ci_out, h->d_ci_out, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(h->h_status, h->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+    *h->h_status = 0;
+    CK(launch_ci(q, k, kSmemBytes, st));
     CK(cudaStreamSynchronize(st));
     return check_status(h, *h->h_status);
 }
@@ -1542,11 +1561,11 @@ void free_handle(fbn_handle* h)
     set_snapshot(h, nullptr);
     h->ws.release();
     dfree(h->d_data); dfree(h->d_planes); dfree(h->d_ar); dfree(h->d_adj); dfree(h->d_nbr); dfree(h->d_eid); dfree(h->d_npos); dfree(h->d_deg);
-    dfree(h->d_sep_len); dfree(h->d_sep_off); dfree(h->d_prob);
+    dfree(h->d_sep_len); dfree(h->d_sep_off);
     dfree(h->d_sep_cnt);
-    dfree(h->d_ci); dfree(h->d_ci_out); dfree(h->d_status); dfree(h->d_table); dfree(h->d_gscratch);
+    dfree(h->d_bad); dfree(h->d_status); dfree(h->d_table); dfree(h->d_gscratch);
     dfree(h->d_off);
-    if (h->h_ci) cudaFreeHost(h->h_ci);
+    if (h->h_table) cudaFreeHost(h->h_table);
     if (h->h_ci_out) cudaFreeHost(h->h_ci_out);
     if (h->h_status) cudaFreeHost(h->h_status);
     if (h->own_stream) cudaStreamDestroy(h->own_stream);
@@ -1653,20 +1672,19 @@ int fbn_create(const uint8_t* data, int32_t n_vars, int64_t n_samples, const uin
     CKC(dalloc(&h->d_deg, n_vars));
     CKC(dalloc(&h->d_sep_len, nn));
     CKC(dalloc(&h->d_sep_off, nn));
-    CKC(dalloc(&h->d_prob, 1));
-    CKC(dalloc(&h->d_ci, 1));
-    CKC(dalloc(&h->d_ci_out, 3));
+    CKC(dalloc(&h->d_bad, 1));
     CKC(dalloc(&h->d_status, 1));
-    CKC(cudaMallocHost((void**)&h->h_ci, sizeof(CiTestDesc)));
     CKC(cudaMallocHost((void**)&h->h_ci_out, 3 * sizeof(double)));
     CKC(cudaMallocHost((void**)&h->h_status, sizeof(unsigned long long)));
+    CKC(cudaHostGetDevicePointer((void**)&h->ci_out_dev, h->h_ci_out, 0));
+    CKC(cudaHostGetDevicePointer((void**)&h->status_dev, h->h_status, 0));
     cudaStream_t st = h->stream;
     CKC(cudaMemsetAsync(h->d_data, 0, (size_t)n_vars * h->ld, st));
     CKC(cudaMemsetAsync(h->d_eid, 0, nn * sizeof(int32_t), st));
     CKC(cudaMemcpy2DAsync(h->d_data, h->ld, data, n_samples, n_samples, n_vars, cudaMemcpyDefault, st));
     CKC(cudaMemcpyAsync(h->d_ar, arities, n_vars, cudaMemcpyHostToDevice, st));
     // values must lie below their arity: checked on the device
-    unsigned long long* bad = (unsigned long long*)h->d_ci_out;   // scratch, 8 bytes
+    unsigned long long* bad = h->d_bad;
     CKC(cudaMemsetAsync(bad, 0xff, sizeof(unsigned long long), st));
     {
         dim3 grid((unsigned)std::min<long long>((n_samples + 255) / 256, 64), n_vars);
@@ -1697,13 +1715,6 @@ int fbn_create(const uint8_t* data, int32_t n_vars, int64_t n_samples, const uin
         CKC(dalloc(&h->d_off, n_vars));
         CKC(cudaMemcpy(h->d_off, off.data(), n_vars * sizeof(int32_t), cudaMemcpyHostToDevice));
     }
-    ProblemDev P{};
-    P.data = h->d_data; P.ar = h->d_ar; P.adj = h->d_adj; P.nbr = h->d_nbr; P.eid = h->d_eid; P.npos = h->d_npos; P.deg = h->d_deg;
-    P.sep_len = h->d_sep_len; P.sep_off = h->d_sep_off; P.ld = h->ld; P.n = n_vars; P.N = (int32_t)n_samples;
-    P.max_arity = max_ar;
-    P.planes = h->d_planes; P.plane_ld = h->plane_ld;
-    CKC(cudaMemcpyAsync(h->d_prob, &P, sizeof P, cudaMemcpyHostToDevice, st));
-    CKC(cudaStreamSynchronize(st));
 #undef CKC
     *out = h;
     return FBN_OK;
@@ -1718,7 +1729,7 @@ int fbn_update_data(fbn_handle* h, const uint8_t* data)
     h->learnt = false;
     h->sep_pending = false;
     CK(cudaMemcpy2DAsync(h->d_data, h->ld, data, h->N, h->N, h->n, cudaMemcpyDefault, st));
-    unsigned long long* bad = (unsigned long long*)h->d_ci_out;   // 8 bytes of scratch
+    unsigned long long* bad = h->d_bad;
     CK(cudaMemsetAsync(bad, 0xff, sizeof(unsigned long long), st));
     dim3 grid((unsigned)std::min<long long>((h->N + 255) / 256, 64), h->n);
     k_validate<<<grid, 256, 0, st>>>(h->d_data, h->ld, h->n, h->N, h->d_ar, bad);
@@ -1754,7 +1765,7 @@ int fbn_update_data_batch(fbn_handle* const* hs, int32_t k, const uint8_t* const
         q->learnt = false;
         q->sep_pending = false;
         CK(cudaMemcpy2DAsync(q->d_data, q->ld, data[p], q->N, q->N, q->n, cudaMemcpyDefault, st));
-        unsigned long long* bad = (unsigned long long*)q->d_ci_out;   // 8 bytes of scratch
+        unsigned long long* bad = q->d_bad;
         CK(cudaMemsetAsync(bad, 0xff, sizeof(unsigned long long), st));
         dim3 grid((unsigned)std::min<long long>((q->N + 255) / 256, 64), q->n);
         k_validate<<<grid, 256, 0, st>>>(q->d_data, q->ld, q->n, q->N, q->d_ar, bad);
@@ -1811,7 +1822,8 @@ int fbn_ci_table(fbn_handle* h, int32_t x, int32_t y, const int32_t* z, int32_t 
     if (cap < cells) return fail(h, FBN_EINVAL, "cap %lld < %lld cells", (long long)cap, cells);
     rc = run_ci(h, x, y, z, nz, cells, true);
     if (rc) return rc;
-    CK(cudaMemcpy(counts, h->d_table, cells * sizeof(int32_t), cudaMemcpyDeviceToHost));
+    if (cells <= kCiHostTable) std::memcpy(counts, h->h_table, cells * sizeof(int32_t));
+    else CK(cudaMemcpy(counts, h->d_table, cells * sizeof(int32_t), cudaMemcpyDeviceToHost));
     return FBN_OK;
 }
 

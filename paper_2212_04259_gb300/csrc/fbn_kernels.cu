@@ -680,7 +680,7 @@ cudaError_t set_kernel_smem(size_t max_smem)
     if ((e = cudaFuncSetAttribute(k_pool_big, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
     if ((e = cudaFuncSetAttribute(k_pool_bits, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
     if ((e = cudaFuncSetAttribute(k_plain, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
-    return set_ci_smem(b);
+    return cudaSuccess;
 }
 
 int pool_blocks_per_sm(int cls, size_t smem_bytes)

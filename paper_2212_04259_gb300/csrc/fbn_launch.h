@@ -9,11 +9,7 @@
 
 namespace fbn {
 
-// One explicit CI test (fbn_ci_test / fbn_ci_table).
-struct CiTestDesc {
-    int32_t x, y, d, pad;
-    int32_t z[kMaxD];
-};
+struct CiArgs;   // one explicit CI test (fbn_ci.cuh)
 
 void launch_snapshot(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first,
                      int total_vertices, DepthCounters* ctr, cudaStream_t st);
@@ -47,12 +43,10 @@ void launch_depth_end(DepthCounters* ctr, DepthRecord* rec, int max_depth, unsig
 void launch_gate(DepthCounters* ctr, cudaGraphConditionalHandle loop, cudaStream_t st);
 // Programmatic dependent launch for the depth kernels (on by default).
 void set_pdl(bool on);
-void launch_ci_tests(const ProblemDev* prob, const CiTestDesc* tests, int ntests, double* out,
-                     int32_t* table_out, int* gscratch, long long gscratch_ints, unsigned* status,
-                     size_t smem_bytes, int stat, int df_mode, bool bits, cudaStream_t st);
+// Explicit tests: the kernel's limits and its largest cluster, then one test.
+cudaError_t prepare_ci(size_t smem_bytes, int* max_cluster);
+cudaError_t launch_ci(const CiArgs& q, int cluster, size_t smem_bytes, cudaStream_t st);
 cudaError_t set_kernel_smem(size_t max_smem);
-// The dynamic shared-memory limit of the explicit-test kernels (fbn_ci.cu).
-cudaError_t set_ci_smem(int max_smem);
 // Sets the message fbn_last_error(NULL) returns.
 void fbn_internal_set_error(const char* msg);
 int pool_blocks_per_sm(int cls, size_t smem_bytes);

@@ -6,8 +6,8 @@
 // exceed it), or a latency-critical loop where cudaMalloc/cudaFree stall the
 // device.  This entry point runs the same test as fbn_ci_test on buffers the
 // caller already owns and keeps its only scratch -- the global contingency
-// table for tables too big for shared memory, its marginals and a status
-// word -- in a fixed array compiled into the library.
+// table for tables too big for shared memory and its marginals -- in a fixed
+// array compiled into the library.
 #include <cstdarg>
 #include <cmath>
 #include <cstdio>
@@ -16,7 +16,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/fbn.h"
-#include "fbn_device.cuh"
+#include "fbn_ci.cuh"
 #include "fbn_launch.h"
 
 using namespace fbn;
@@ -30,65 +30,19 @@ constexpr int kNoAllocMaxDevices = 64;
 
 // 3 MiB per device that loads the library, held until the process exits.
 // Every call on a device shares it; the last call's contents stay in it.
-static __device__ __align__(256) int g_noalloc_scratch[kNoAllocTableInts + 64];
+static __device__ __align__(256) int g_noalloc_scratch[kNoAllocTableInts];
 
 std::mutex g_mu;
 bool g_ready[kNoAllocMaxDevices];
+int g_cluster[kNoAllocMaxDevices];    // largest cluster of the kernel on each device
 int* g_scratch[kNoAllocMaxDevices];   // device address of g_noalloc_scratch on each device
 
-// Whether some sample value of the test's rows is not below its variable's
-// arity (block-wide, every thread gets the answer).  The other entry points
-// validate data when it enters a handle; this one reads caller-owned rows
-// directly, and an out-of-range value would index past the table (in shared
-// memory or in the scratch array), so the rows are checked before counting:
-// 16 samples per 16-byte load, four byte comparisons per 32-bit word.
-__device__ bool rows_out_of_range(const TestSpec& s)
+__global__ void __launch_bounds__(kTestThreads, 2) k_ci_noalloc(const __grid_constant__ CiArgs q)
 {
-    bool bad = false;
-    const int nvec = s.N >> 4;
-    for (int k = 0; k < s.nrows; ++k) {
-        const unsigned rr = (unsigned)s.rad[k] * 0x01010101u;   // the arity in each byte
-        const uint4* row = reinterpret_cast<const uint4*>(s.rows[k]);
-        for (int v = threadIdx.x; v < nvec; v += blockDim.x) {
-            const uint4 w = __ldg(row + v);
-            bad |= (__vcmpgeu4(w.x, rr) | __vcmpgeu4(w.y, rr) | __vcmpgeu4(w.z, rr) | __vcmpgeu4(w.w, rr)) != 0u;
-        }
-        for (int t = (nvec << 4) + threadIdx.x; t < s.N; t += blockDim.x) bad |= s.rows[k][t] >= s.rad[k];
-    }
-    return __syncthreads_or(bad) != 0;
-}
-
-__global__ void __launch_bounds__(kTestThreads) k_ci_noalloc(TestSpec spec, int* scratch, double* out,
-                                                             int32_t* table_out, int smem_ints)
-{
-    extern __shared__ int smem[];
-    __shared__ TestSpec s;
-    __shared__ double red[32];
-    unsigned* status = reinterpret_cast<unsigned*>(scratch + kNoAllocTableInts);
-    if (threadIdx.x == 0) {
-        s = spec;
-        *status = 0;   // the previous call's status must not leak into this one
-    }
-    __syncthreads();
-    if (rows_out_of_range(s)) {   // a value >= its arity: no table, every output NaN
-        if (threadIdx.x == 0) out[0] = out[1] = out[2] = nan("");
-        return;
-    }
-    int* M = nullptr;
-    const int* T = grp_table<kTestThreads>(s, smem, smem_ints, scratch, kNoAllocTableInts, &M);
-    if (!T) {   // not reached: the host admits only tables that fit the scratch
-        if (threadIdx.x == 0) out[0] = out[1] = out[2] = nan("");
-        return;
-    }
-    grp_marginals<kTestThreads>(s, T, M);
-    const double g2 = grp_g2_exact<kTestThreads>(s, T, M, red, table_out);
-    if (threadIdx.x == 0) {
-        const double df = (double)(s.rx - 1) * (double)(s.ry - 1) * (double)(s.cells / (s.rx * s.ry));
-        const double p = chisq_q(df, g2, status);
-        out[0] = g2;
-        out[1] = df;
-        out[2] = *status ? nan("") : p;
-    }
+    // the other entry points validate data when it enters a handle; this one
+    // reads caller-owned rows, and an out-of-range value would index past the
+    // table, so the rows are checked before counting
+    ci_cluster_test<true>(q);
 }
 
 int nfail(int code, const char* fmt, ...)
@@ -115,7 +69,7 @@ extern "C" int fbn_ci_test_noalloc(const uint8_t* data, int64_t ld, int32_t n_va
         return nfail(FBN_EINVAL, "n_vars=%d or n_samples=%lld out of range", n_vars, (long long)n_samples);
     if (x < 0 || x >= n_vars || y < 0 || y >= n_vars || x == y) return nfail(FBN_EINVAL, "bad x=%d y=%d", x, y);
     if (nz < 0 || nz > kMaxD) return nfail(FBN_EINVAL, "conditioning set size %d outside [0, %d]", nz, kMaxD);
-    TestSpec spec{};
+    CiArgs spec{};
     long long cells = 1;
     for (int k = 0; k < nz; ++k) {
         if (z[k] < 0 || z[k] >= n_vars || z[k] == x || z[k] == y) return nfail(FBN_EINVAL, "bad conditioning variable %d", z[k]);
@@ -145,6 +99,7 @@ extern "C" int fbn_ci_test_noalloc(const uint8_t* data, int64_t ld, int32_t n_va
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kNoAllocMaxDevices)
         return nfail(FBN_ECUDA, "no usable current CUDA device");
     int* scratch = nullptr;
+    int cluster = 1;
     {
         // first call on this device: look up the device address of the scratch
         // array and raise the kernel's shared-memory limit
@@ -152,15 +107,21 @@ extern "C" int fbn_ci_test_noalloc(const uint8_t* data, int64_t ld, int32_t n_va
         if (!g_ready[dev]) {
             cudaError_t e = cudaGetSymbolAddress((void**)&g_scratch[dev], g_noalloc_scratch);
             if (e != cudaSuccess) return nfail(FBN_ECUDA, "cudaGetSymbolAddress: %s", cudaGetErrorString(e));
-            e = cudaFuncSetAttribute(k_ci_noalloc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNoAllocSmem);
-            if (e != cudaSuccess) return nfail(FBN_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+            e = ci_prepare(k_ci_noalloc, kNoAllocSmem, &g_cluster[dev]);
+            if (e != cudaSuccess) return nfail(FBN_ECUDA, "kernel limits: %s", cudaGetErrorString(e));
             g_ready[dev] = true;
         }
         scratch = g_scratch[dev];
+        cluster = g_cluster[dev];
     }
-    k_ci_noalloc<<<1, kTestThreads, kNoAllocSmem, (cudaStream_t)stream>>>(spec, scratch, out, table_out,
-                                                                         (int)(kNoAllocSmem / 4));
-    const cudaError_t e = cudaGetLastError();
+    spec.gtab = scratch;
+    spec.out = out;
+    spec.table_out = table_out;
+    spec.stat = kStatG2;
+    spec.lgamma_a = ci_lgamma(spec.rx, spec.ry, cells);
+    spec.smem_ints = (int)(kNoAllocSmem / 4);
+    const cudaError_t e =
+        ci_launch(k_ci_noalloc, spec, ci_cluster(n_samples, cells, cluster), kNoAllocSmem, (cudaStream_t)stream);
     if (e != cudaSuccess) return nfail(FBN_ECUDA, "launch: %s", cudaGetErrorString(e));
     return FBN_OK;
 }
