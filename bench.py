@@ -493,7 +493,7 @@ def main():
         fp8_peak, fp8_src = 2.0 * 1900.0, "of fallback (bf16 x 2)"
     roofline_hbm = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                     "peak_source": peak_src,
-                    "kernel": "k_pool_bits / k_pool_small / k_pool_big (depths %s)" % ",".join(str(d) for d in pool_depths)
+                    "kernel": "k_pool_marg / k_pool_small / k_pool_big (depths %s)" % ",".join(str(d) for d in pool_depths)
                     if args.form == "pool" else "k_plain", "kernel_ms_per_step": test_ms,
                     "algorithmic_bytes_per_step": alg_bytes,
                     "note": "sample bytes (d + 2) N of the oracle-equivalent tests over the pool's test windows; the "
@@ -514,7 +514,7 @@ def main():
         work = st["popc_work"][dstar] if bits else st["smem_updates"][dstar]
         peak_u = (rates["popc_per_s"] if bits else rates["smem_red_per_s"]) / 1e9
         ach = work / (per_ms[dstar] / 1e3) / 1e9
-        kname = ("k_pool_bits" if bits else "k_pool_small / k_pool_big") if args.form == "pool" else "k_plain"
+        kname = ("k_pool_marg" if bits else "k_pool_small / k_pool_big") if args.form == "pool" else "k_plain"
         traffic, traffic_launch = profiled_traffic(kname.split(" ")[0], name) if args.form == "pool" else (None, None)
         roofline = {"bound": "alu" if bits else "smem", "unit_op": "POPC" if bits else "red.shared.add",
                     "achieved": ach, "peak": peak_u, "unit": "Gop/s", "frac": ach / peak_u,

@@ -39,7 +39,7 @@ extern "C" {
 #define FBN_FORM_PLAIN 1   /* edge-level form: one CTA per edge, one launch per depth (Section IV-A) */
 
 #define FBN_DEPTH0_AUTO 0  /* tensor-core one-hot Gram when the problem is large enough, else histogram */
-#define FBN_DEPTH0_HIST 1  /* depth 0 through the shared-memory histogram path */
+#define FBN_DEPTH0_HIST 1  /* depth 0 without the Gram: one-hot bit planes, or byte histograms (count) */
 #define FBN_DEPTH0_GRAM 2  /* depth 0 through the tcgen05 one-hot Gram */
 
 #define FBN_DEPTH1_AUTO   0  /* the work pool (the faster of the two on the measured workloads) */
@@ -53,12 +53,12 @@ extern "C" {
 #define FBN_DF_ADJUSTED 1  /* df = sum over strata with N_++z > 0 of (values of X seen - 1)(values of Y seen - 1);
                               a test with df = 0 cannot reject (p = 1) */
 
-#define FBN_COUNT_AUTO 0   /* tables of small tests (every arity <= 4, at most 2 conditioning variables, few
-                              cells) counted from bit planes with popcounts, the others by byte histograms */
+#define FBN_COUNT_AUTO 0   /* depths 0 and 1 counted from one-hot bit planes with popcounts when every arity of the
+                              call is <= 5 (depth 0 by the Gram where that applies), the others by byte histograms */
 #define FBN_COUNT_HIST 1   /* every table by the byte histogram (shared-memory reductions, or a global table) */
-#define FBN_COUNT_BITS 2   /* bit planes for every test that qualifies and fits shared memory, whatever its size */
+#define FBN_COUNT_BITS 2   /* as FBN_COUNT_AUTO; the autotuner then tries no histogram at those depths */
 
-#define FBN_TUNE_OFF  0    /* fixed rules: bit planes where every small table qualifies, group size by a cost model,
+#define FBN_TUNE_OFF  0    /* fixed rules: one-hot planes at the depths they serve, group size by a cost model,
                               depth 0 on the Gram by problem size */
 #define FBN_TUNE_AUTO 1    /* the first skeleton call on a workload shape runs fbn_autotune (or reuses its result
                               for this device and shape from earlier in the process) and applies its choices */
@@ -105,8 +105,9 @@ typedef struct fbn_stats {
     int64_t gram_samples;                   /* padded samples of the Gram */
     int64_t test_samples[FBN_MAX_DEPTHS];   /* sum over the tests_oracle[d] tests of their data set's N
                                                (in a batch each test counts its own problem's samples) */
-    int64_t popc_work[FBN_MAX_DEPTHS];      /* counting work executed from bit planes: cells x 32-sample words
-                                               (one POPC each) over the tests so counted, redundant ones included */
+    int64_t popc_work[FBN_MAX_DEPTHS];      /* counting work executed from one-hot planes: counted cells (every value
+                                               >= 1) x 32-sample words, one POPC each, over the tests so counted,
+                                               redundant ones included */
     int64_t smem_updates[FBN_MAX_DEPTHS];   /* counting work executed by byte histograms: samples of the tests so
                                                counted (one shared-memory reduction each, or a global one for the
                                                largest tables), redundant ones included */
@@ -150,7 +151,7 @@ int fbn_update_data(fbn_handle* h, const uint8_t* data);
 
 /* fbn_update_data_batch -- fbn_update_data on k handles of one device at
  * once (data[p] for handle p, each in its handle's shape, host or device): the
- * copies, the arity checks and the bit-plane builds of every data set are
+ * copies, the arity checks and the plane builds of every data set are
  * queued on the first handle's stream and end with one synchronisation.
  * Errors: FBN_EINVAL, FBN_EDATA (the first offending data set is named; the
  * data of every handle of the call is then undefined until the next
@@ -254,7 +255,7 @@ int fbn_learn_skeleton_sharded(fbn_handle* h, double alpha, int32_t max_depth, f
  * paper's group-size study, Section V-D, is such a measured trade-off).  Runs
  * the skeleton (same results as fbn_learn_skeleton_batch) once per candidate
  * configuration -- byte histograms with 32, 64, 128 or 256 threads per test,
- * bit planes where every small table qualifies, and, where the one-hot Gram
+ * one-hot planes at the depths they serve, and, where the one-hot Gram
  * applies, depth 0 on the Gram or on the histogram -- timing every depth with
  * the device clock, and keeps per depth the fastest.  The choices are stored
  * in every handle (later skeleton calls use them) and in a process-wide cache

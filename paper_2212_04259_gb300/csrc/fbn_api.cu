@@ -30,11 +30,8 @@ thread_local std::string g_create_error;
 constexpr size_t kSmemBytes = 100 * 1024;     // dynamic shared memory of a CTA test group: 2 CTAs / SM with the ~9 KB static
 constexpr long long kSplitStride = 4096;        // cells of a split test's global table at most
 constexpr size_t kWarpSmemBytes = 56 * 1024;  // dynamic shared memory of a CTA of 8 warp groups (3 CTAs / SM)
-constexpr size_t kBitsSmemBytes = 36 * 1024;  // the bit-plane pool: 8 groups of 32 x 32 counter words, table and
-                                              // marginals (4 CTAs / SM)
 constexpr int kCritCap = 8192;                // critical-value cache slots (power of two)
 constexpr int kCritDense = 8192;              // critical values kept in a dense table: df < kCritDense
-constexpr int kBitsCellsAuto = 64;            // largest table counted from bit planes by default
 
 template <typename T>
 cudaError_t dalloc(T** p, size_t count)
@@ -50,39 +47,41 @@ void dfree(void* p)
 }
 
 // ---- small kernels of the host engine ------------------------------------
-__global__ void k_validate(const uint8_t* data, int64_t ld, int n, int64_t N, const uint8_t* ar,
-                           unsigned long long* first_bad)
+// One pass over new samples: the first value at or above its arity (row-major
+// index over n x N), and the one-hot planes (nplanes > 0).  One thread per
+// 32-sample word: two 16-byte loads, four comparisons per 32-bit word and
+// value; a multiply gathers a word's four comparison bits.  The rows' zero
+// padding covers the words past the samples.  (Checking and planes took two
+// passes before, the check one byte per thread and load.)
+__global__ void k_ingest(const uint8_t* __restrict__ data, int64_t ld, int64_t N, const uint8_t* __restrict__ ar,
+                         int nplanes, int64_t wp, uint32_t* __restrict__ planes, unsigned long long* first_bad)
 {
     const int v = blockIdx.y;
-    const uint8_t r = ar[v];
+    const int r = ar[v];
+    const unsigned rr = 0x01010101u * (unsigned)r;
     const uint8_t* row = data + (long long)v * ld;
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < N;
-         s += (long long)gridDim.x * blockDim.x) {
-        if (row[s] >= r) atomicMin(first_bad, (unsigned long long)v * (unsigned long long)N + s);
-    }
-}
-
-// Bit planes of the samples: word w of plane b of variable v holds bit b of
-// the values of samples 32 w .. 32 w + 31.  One thread per word reads its 32
-// bytes (two 16-byte loads; the zero padding of the rows covers the words
-// past the samples, which therefore stay zero).
-__global__ void k_planes(const uint8_t* __restrict__ data, int64_t ld, int64_t wp, uint32_t* __restrict__ planes)
-{
-    const int v = blockIdx.y;
-    const uint8_t* row = data + (long long)v * ld;
+    const int values = nplanes > 0 ? r - 1 : 0;
     for (long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x; w < wp; w += (long long)gridDim.x * blockDim.x) {
         const uint4* p = reinterpret_cast<const uint4*>(row + w * 32);
         const uint4 a = p[0], b = p[1];
         const unsigned q[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-        unsigned m0 = 0, m1 = 0;
+        unsigned bad = 0;
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            const unsigned val = (q[k >> 2] >> ((k & 3) * 8)) & 0xFFu;
-            m0 |= (val & 1u) << k;
-            m1 |= ((val >> 1) & 1u) << k;
+        for (int k = 0; k < 8; ++k) bad |= __vcmpgeu4(q[k], rr);
+        if (bad) {
+            for (int k = 0; k < 32; ++k)
+                if (((q[k >> 2] >> ((k & 3) * 8)) & 0xFFu) >= (unsigned)r && w * 32 + k < N) {
+                    atomicMin(first_bad, (unsigned long long)v * (unsigned long long)N + (unsigned long long)(w * 32 + k));
+                    break;
+                }
         }
-        planes[(2LL * v) * wp + w] = m0;
-        planes[(2LL * v + 1) * wp + w] = m1;
+        for (int x = 1; x <= values; ++x) {
+            unsigned m = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                m |= (((__vcmpeq4(q[k], 0x01010101u * (unsigned)x) & 0x08040201u) * 0x01010101u) >> 24) << (4 * k);
+            planes[((long long)v * nplanes + x - 1) * wp + w] = m;
+        }
     }
 }
 
@@ -158,7 +157,7 @@ struct Workspace {
     long long shard_cap = 0;
     unsigned long long* d_shard_count = nullptr;
     // launch geometry of the device, fixed once (kernel attributes set)
-    int dev_sms = 0, grid_small = 0, grid_big = 0, grid_bits = 0;
+    int dev_sms = 0, grid_small = 0, grid_big = 0, grid_marg = 0;
     // the problem descriptors and vertex maps as last uploaded (skipped when
     // unchanged), staged through pinned memory
     std::vector<uint8_t> up_last;
@@ -177,7 +176,7 @@ struct Workspace {
     // the graph of the generic depths (a device-driven while loop)
     cudaGraphExec_t loop = nullptr;
     std::vector<uint8_t> graph_key;
-    cudaEvent_t tev[2][2] = {};   // test-kernel windows of depths 0 and 1 when launched directly
+    cudaEvent_t tev[2] = {};   // window of the neighbourhood product
     bool events = false;
 
     void release()
@@ -194,8 +193,7 @@ struct Workspace {
         dfree(d_owned); dfree(d_shard); dfree(d_shard_count);
         if (events) {
             for (auto& e : kev) cudaEventDestroy(e);
-            for (auto& row : tev)
-                for (auto& e : row) cudaEventDestroy(e);
+            for (auto& e : tev) cudaEventDestroy(e);
         }
         if (loop) cudaGraphExecDestroy(loop);
         dfree(d_rec);
@@ -231,7 +229,8 @@ struct fbn_handle {
     int max_arity = 0;
     std::vector<uint8_t> h_ar;
     uint8_t* d_data = nullptr;
-    uint32_t* d_planes = nullptr;       // two bit planes per variable (see k_planes)
+    uint32_t* d_planes = nullptr;       // one-hot planes (see k_ingest), none above arity kMargMaxArity
+    int nplanes = 0;                    // planes per variable
     int64_t plane_ld = 0;               // words per plane, a multiple of 4
     uint8_t* d_ar = nullptr;
     uint8_t* d_adj = nullptr;
@@ -314,8 +313,7 @@ int grow_workspace(fbn_handle* h, Workspace& ws, long long edge_cap, int max_n, 
         CK(dalloc(&ws.d_ctr, 1));
         CK(cudaMallocHost((void**)&ws.h_ctr, sizeof(DepthCounters)));
         for (auto& e : ws.kev) CK(cudaEventCreate(&e));
-        for (auto& row : ws.tev)
-            for (auto& e : row) CK(cudaEventCreate(&e));
+        for (auto& e : ws.tev) CK(cudaEventCreate(&e));
         ws.events = true;
         CK(dalloc(&ws.d_rec, kMaxDepthRecords));
         CK(cudaMallocHost((void**)&ws.h_rec, kMaxDepthRecords * sizeof(DepthRecord)));
@@ -433,18 +431,13 @@ int check_status(fbn_handle* h, unsigned status)
     return FBN_OK;
 }
 
-// Largest table a test of h counts from the bit planes (0: none): the
-// option's choice; the plain edge-level form keeps the byte histogram.
-int bits_cells(const fbn_handle* h)
+// Check and planes of the samples now in d_data; h->d_bad receives the first
+// bad value (all ones: none).
+int launch_ingest(fbn_handle* h, cudaStream_t st)
 {
-    if (h->opt.form == FBN_FORM_PLAIN || h->opt.count == FBN_COUNT_HIST) return 0;
-    return h->opt.count == FBN_COUNT_BITS ? (int)kMaxCells : kBitsCellsAuto;
-}
-
-int launch_planes(fbn_handle* h, cudaStream_t st)
-{
+    CK(cudaMemsetAsync(h->d_bad, 0xff, sizeof(unsigned long long), st));
     dim3 grid((unsigned)std::min<long long>((h->plane_ld + 255) / 256, 64), h->n);
-    k_planes<<<grid, 256, 0, st>>>(h->d_data, h->ld, h->plane_ld, h->d_planes);
+    k_ingest<<<grid, 256, 0, st>>>(h->d_data, h->ld, h->N, h->d_ar, h->nplanes, h->plane_ld, h->d_planes, h->d_bad);
     CK(cudaGetLastError());
     return FBN_OK;
 }
@@ -478,6 +471,33 @@ bool use_nbr1(fbn_handle* const* hs, int k)
     return true;
 }
 
+// How the first depths of a skeleton call run.
+struct DepthPlan {
+    bool gram = false;    // depth 0 as the tensor-core Gram
+    bool popc0 = false;   // depth 0 from one-hot planes (k_pairs_popc)
+    bool marg1 = false;   // depth 1 from one-hot planes and depth 0's pair tables (k_pool_marg)
+    bool nbr1 = false;    // depth 1 as the neighbourhood product
+};
+
+// The planes take every problem of the call or none (one pool per depth), at
+// arities the planes hold; the caller may ask for histograms (count), and the
+// autotuner for histograms at a depth.  A sharded skeleton counts every pair
+// itself, without the Gram.
+DepthPlan depth_plan(fbn_handle* const* hs, int k, bool shard)
+{
+    const fbn_handle* h = hs[0];
+    DepthPlan p;
+    if (h->opt.form == FBN_FORM_PLAIN) return p;
+    p.gram = !shard && use_gram(hs, k);
+    p.nbr1 = !shard && use_nbr1(hs, k);
+    bool planes = h->opt.count != FBN_COUNT_HIST;
+    for (int q = 0; q < k; ++q) planes = planes && hs[q]->nplanes > 0;
+    auto hist_at = [&](int d) { return (size_t)d < h->tune.size() && (h->tune[d] & kTuneNoBits) != 0; };
+    p.popc0 = planes && !p.gram && !hist_at(0);
+    p.marg1 = planes && !p.nbr1 && (p.gram || p.popc0) && !hist_at(1);
+    return p;
+}
+
 // Room for every problem's samples at 4 bits each; sets the problems' pk rows.
 int prepare_pack(fbn_handle* const* hs, int k, Workspace& ws, ProblemDev* P)
 {
@@ -500,6 +520,30 @@ int prepare_pack(fbn_handle* const* hs, int k, Workspace& ws, ProblemDev* P)
     return FBN_OK;
 }
 
+// Room for every problem's pair tables (the Gram layout); sets the problems'
+// pointers.
+int prepare_pairs(fbn_handle* const* hs, int k, Workspace& ws, ProblemDev* P)
+{
+    fbn_handle* h = hs[0];
+    long long total = 0;
+    for (int p = 0; p < k; ++p) total += (long long)hs[p]->Mp * hs[p]->Mp;
+    if (total > ws.gram_G_cap) {
+        dfree(ws.gram_G);
+        ws.gram_G = nullptr;
+        ws.gram_G_cap = 0;
+        CK(dalloc(&ws.gram_G, total));
+        ws.gram_G_cap = total;
+    }
+    long long go = 0;
+    for (int p = 0; p < k; ++p) {
+        P[p].off = hs[p]->d_off;
+        P[p].gram = ws.gram_G + go;
+        P[p].gram_ld = hs[p]->Mp;
+        go += (long long)hs[p]->Mp * hs[p]->Mp;
+    }
+    return FBN_OK;
+}
+
 // Lay out the one-hot matrices and Grams of every problem in the workspace,
 // set the problems' pointers, and upload one tensor map per problem and the
 // work units (problem, tile pair, chunk), problem-major.
@@ -507,24 +551,16 @@ int prepare_gram(fbn_handle* const* hs, int k, Workspace& ws, ProblemDev* P)
 {
     fbn_handle* h = hs[0];
     cudaStream_t st = h->stream;
-    long long e_total = 0, g_total = 0;
-    for (int p = 0; p < k; ++p) {
-        e_total += (long long)hs[p]->Mp * hs[p]->K;
-        g_total += (long long)hs[p]->Mp * hs[p]->Mp;
-    }
+    const int prc = prepare_pairs(hs, k, ws, P);
+    if (prc) return prc;
+    long long e_total = 0;
+    for (int p = 0; p < k; ++p) e_total += (long long)hs[p]->Mp * hs[p]->K;
     if (e_total > ws.gram_E_cap) {
         dfree(ws.gram_E);
         ws.gram_E = nullptr;
         ws.gram_E_cap = 0;
         CK(dalloc(&ws.gram_E, e_total));
         ws.gram_E_cap = e_total;
-    }
-    if (g_total > ws.gram_G_cap) {
-        dfree(ws.gram_G);
-        ws.gram_G = nullptr;
-        ws.gram_G_cap = 0;
-        CK(dalloc(&ws.gram_G, g_total));
-        ws.gram_G_cap = g_total;
     }
     const size_t mb = tensor_map_bytes();
     if ((long long)(k * mb) > ws.gram_maps_cap) {
@@ -536,15 +572,12 @@ int prepare_gram(fbn_handle* const* hs, int k, Workspace& ws, ProblemDev* P)
     }
     ws.h_maps.assign(k * mb, 0);
     std::vector<int4> units;
-    long long eo = 0, go = 0;
+    long long eo = 0;
     ws.gram_layout.assign(1, (long long)(uintptr_t)ws.gram_E);
     for (int p = 0; p < k; ++p) {
         const fbn_handle* q = hs[p];
-        P[p].off = q->d_off;
         P[p].onehot = ws.gram_E + eo;
-        P[p].gram = ws.gram_G + go;
         P[p].onehot_ld = q->K;
-        P[p].gram_ld = q->Mp;
         CK(encode_onehot_map(ws.h_maps.data() + p * mb, P[p].onehot, q->Mp, q->K));
         // 128-row tiles a against 256-row tiles b that reach the upper triangle
         const int T = q->Mp / 128, T2 = (T + 1) / 2, C = gram_chunks(q->K);
@@ -556,7 +589,6 @@ int prepare_gram(fbn_handle* const* hs, int k, Workspace& ws, ProblemDev* P)
         ws.gram_layout.push_back(q->Mp);
         ws.gram_layout.push_back(q->K);
         eo += (long long)q->Mp * q->K;
-        go += (long long)q->Mp * q->Mp;
     }
     if ((long long)units.size() > ws.gram_units_cap) {
         dfree(ws.gram_units);
@@ -573,8 +605,8 @@ int prepare_gram(fbn_handle* const* hs, int k, Workspace& ws, ProblemDev* P)
 
 // One-hot matrices and their INT32 Grams (upper tile triangle) for the
 // problems already in ws.probs (prepared by prepare_gram).
-int run_gram(fbn_handle* h, Workspace& ws, int k, int total_vtx, unsigned* d_status, cudaEvent_t ev0 = nullptr,
-             cudaEvent_t ev1 = nullptr)
+int run_gram(fbn_handle* h, Workspace& ws, int k, int total_vtx, unsigned* d_status, const DepthCounters* ctr = nullptr,
+             cudaEvent_t ev0 = nullptr, cudaEvent_t ev1 = nullptr)
 {
     cudaStream_t st = h->stream;
     int sms = 0;
@@ -583,7 +615,7 @@ int run_gram(fbn_handle* h, Workspace& ws, int k, int total_vtx, unsigned* d_sta
         CK(launch_zero_pad(ws.probs, k, st));
         ws.gram_zeroed = ws.gram_layout;
     }
-    CK(launch_onehot(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx, st));
+    CK(launch_onehot(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx, ctr, st));
     CK(cudaMemsetAsync(ws.gram_G, 0, ws.gram_G_cap * sizeof(int32_t), st));
     if (ev0) CK(cudaEventRecord(ev0, st));
     CK(launch_gram(ws.gram_maps, ws.gram_units, ws.gram_n_units, ws.probs, sms, d_status, h->opt.wait_limit, st));
@@ -764,15 +796,16 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         ProblemDev& d = P[p];
         d.data = q->d_data; d.ar = q->d_ar; d.adj = q->d_adj; d.nbr = q->d_nbr; d.eid = q->d_eid; d.npos = q->d_npos; d.deg = q->d_deg;
         d.sep_len = q->d_sep_len; d.sep_off = q->d_sep_off; d.ld = q->ld; d.n = q->n; d.N = (int32_t)q->N;
-        d.max_arity = q->max_arity; d.pad = 0;
+        d.max_arity = q->max_arity; d.nplanes = q->nplanes;
         d.planes = q->d_planes; d.plane_ld = q->plane_ld;
     }
     int rc = grow_workspace(h, ws, edge_cap, max_n, k, total_vtx);
     if (rc) return rc;
     const bool plain = h->opt.form == FBN_FORM_PLAIN;
     if (shard && k != 1) return fail(h, FBN_EINVAL, "a sharded skeleton learns one problem");
-    const bool gram = !plain && !shard && use_gram(hs, k);
-    const bool nbr1 = !shard && use_nbr1(hs, k);
+    const DepthPlan plan = depth_plan(hs, k, shard != nullptr);
+    const bool gram = plan.gram, nbr1 = plan.nbr1, popc0 = plan.popc0;
+    const bool marg1 = plan.marg1 && max_depth != 0;
     if (shard) {   // this process's edges (n x n) and the depth's removal records (3 per edge at most)
         const long long nn = (long long)h->n * h->n;
         if (nn > ws.owned_cap) {
@@ -797,6 +830,9 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     }
     if (gram) {
         rc = prepare_gram(hs, k, ws, P.data());
+        if (rc) return rc;
+    } else if (popc0) {
+        rc = prepare_pairs(hs, k, ws, P.data());
         if (rc) return rc;
     }
     if (ws.sep_cap == 0) {
@@ -844,10 +880,10 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         // CTAs of the small-table pool (any group size) and of the big-table pool
         ws.grid_small = sms * std::max(1, pool_blocks_per_sm(kClassWarp, kWarpSmemBytes));
         ws.grid_big = sms * std::max(1, pool_blocks_per_sm(kClassCta, kSmemBytes));
-        ws.grid_bits = sms * std::max(1, pool_blocks_per_sm(kClassBits, kBitsSmemBytes));
+        ws.grid_marg = sms * std::max(1, pool_blocks_per_sm(kClassMarg, 0));
         ws.dev_sms = sms;
     }
-    const int dev_sms = ws.dev_sms, grid_small = ws.grid_small, grid_big = ws.grid_big, grid_bits = ws.grid_bits;
+    const int dev_sms = ws.dev_sms, grid_small = ws.grid_small, grid_big = ws.grid_big, grid_marg = ws.grid_marg;
     const long long groups[4] = {(long long)grid_small * 8, (long long)grid_small * 4, (long long)grid_small * 2,
                                  (long long)grid_small};
     const long long groups_big[4] = {(long long)grid_big * 8, (long long)grid_big * 4, (long long)grid_big * 2,
@@ -879,7 +915,6 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     }
     DepthCounters c0{};
     c0.active = 1;
-    c0.bits_ok = 1;
     c0.tune = h->tune.empty() ? nullptr : ws.d_tune;
     c0.rec = ws.d_rec;
     *ws.h_ctr = c0;
@@ -910,24 +945,21 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
 
     // The kernels of one depth after the edge list: ordering and the pool of
     // each class; then removal and the end of the depth.
+    auto enqueue_order = [&](bool marg) {   // both classes up front: their sorted orders do not overlap
+        ScanClass sc[2];
+        for (int cls = 0; cls < 2; ++cls) {
+            sc[cls].hist = ws.hist + cls * ws.ord_cap;
+            sc[cls].alive = ws.alive + cls * ws.ord_cap;
+            sc[cls].base = ws.base + cls * ws.ord_cap;
+            for (int k = 0; k < 4; ++k) sc[cls].groups[k] = cls == 0 ? groups[k] : groups_big[k];
+            sc[cls].smem_ints = (long long)((cls == 0 ? kWarpSmemBytes : kSmemBytes) / 4);
+        }
+        launch_order(ws.probs, ws.edges, ws.edge_cap, marg ? 1 : 2, ws.d_ctr, sc, ws.cursor, ws.cursor + ws.ord_cap,
+                     ws.sorted, mean_n, forced, kSplitStride, 1, marg, grid_aux, st);
+    };
     auto enqueue_tests = [&]() {
         const int nclass = 2;
-        if (!plain) {   // both classes ordered up front: their sorted orders do not overlap
-            ScanClass sc[2];
-            for (int cls = 0; cls < 2; ++cls) {
-                sc[cls].hist = ws.hist + cls * ws.ord_cap;
-                sc[cls].alive = ws.alive + cls * ws.ord_cap;
-                sc[cls].base = ws.base + cls * ws.ord_cap;
-                for (int k = 0; k < 4; ++k) {
-                    sc[cls].groups[k] = cls == 0 ? groups[k] : groups_big[k];
-                    sc[cls].groups_bits[k] = ((long long)grid_bits * 8) >> k;
-                }
-                sc[cls].smem_ints = (long long)((cls == 0 ? kWarpSmemBytes : kSmemBytes) / 4);
-                sc[cls].smem_ints_bits = (long long)(kBitsSmemBytes / 4);
-            }
-            launch_order(ws.edges, ws.edge_cap, nclass, ws.d_ctr, sc, ws.cursor, ws.cursor + ws.ord_cap, ws.sorted,
-                         mean_n, forced, kSplitStride, 1, grid_aux, st);
-        }
+        if (!plain) enqueue_order(false);
         for (int cls = 0; cls < nclass; ++cls) {
             PoolArgs a = base;
             a.cls = cls;
@@ -944,18 +976,27 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
             }
             a.base = ws.base + cls * ws.ord_cap;
             a.sorted = ws.sorted;
-            if (small) {   // the bit-plane pool first; exactly one of the two runs the class
-                PoolArgs b = a;
-                b.smem_ints = (int)(kBitsSmemBytes / 4);
-                launch_pool_bits(b, grid_bits, kBitsSmemBytes, st);
-            }
             launch_pool(a, cls, small ? grid_small : grid_big, smem, st);
         }
     };
-    auto enqueue_head = [&]() {
+    // depth 1 from one-hot planes: every edge is in the small-table class
+    auto enqueue_marg = [&]() {
+        enqueue_order(true);
+        PoolArgs a = base;
+        a.cls = kClassWarp;
+        a.base = ws.base;
+        a.sorted = ws.sorted;
+        launch_pool_marg(a, grid_marg, st);
+    };
+    auto enqueue_popc0 = [&]() {
+        const long long tasks = (long long)total_vtx * max_n;
+        launch_pairs_popc(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx, max_n, shard ? ws.d_owned : nullptr, base,
+                          (int)std::min<long long>((tasks + 7) / 8, dev_sms * 8), st);
+    };
+    auto enqueue_head = [&](bool marg = false) {
         launch_snapshot(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx, ws.d_ctr, st);
         launch_edges(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx, gs_forced, gs_edges, ws.binom, ws.brows, wcap,
-                     bits_cells(h), shard ? ws.d_owned : nullptr, ws.edges, ws.min_accept, ws.edge_cap, ws.d_ctr,
+                     marg ? (long long)(kMargThreads / 32) * grid_marg : 0, shard ? ws.d_owned : nullptr, ws.edges, ws.min_accept, ws.edge_cap, ws.d_ctr,
                      ws.hist, st);
     };
     auto enqueue_tail = [&]() {
@@ -963,7 +1004,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
                      grid_aux, st);
         launch_depth_end(ws.d_ctr, ws.d_rec, max_depth, ws.hist, ws.cursor, st);
     };
-    const int body_launches = plain ? 7 : 10;
+    const int body_launches = plain ? 7 : 9;
     auto capture_loop = [&]() -> cudaError_t {
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaGraphCreate(&g, 0);
@@ -1040,8 +1081,8 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
                               ws.split_ticket};
         put(ptrs, sizeof ptrs);
         const long long ints[] = {total_vtx, gs_forced, gs_edges, ws.brows, wcap, ws.edge_cap, ws.ord_cap, forced,
-                                  grid_aux, grid_small, grid_big, grid_bits, ws.gs_cells, ws.sep_cap, max_depth, plain,
-                                  h->opt.statistic, h->opt.df_mode, bits_cells(h),
+                                  grid_aux, grid_small, grid_big, ws.gs_cells, ws.sep_cap, max_depth, plain,
+                                  h->opt.statistic, h->opt.df_mode,
                                   groups[0], groups[1], groups[2], groups[3]};
         put(ints, sizeof ints);
         put(&mean_n, sizeof mean_n);
@@ -1065,39 +1106,48 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
 
     fbn_stats stats{};
     int d_loop = 0;   // first depth of the graph loop
-    bool direct[2] = {false, false};   // depths 0 and 1 launched directly (timed by events)
-    if (gram) {
+    bool direct1 = false;   // depth 1 as the neighbourhood product (timed by events)
+    if (shard) {
+        // depth by depth below
+    } else if (gram) {
         enqueue_head();
-        CK(cudaEventRecord(ws.tev[0][0], st));
-        rc = run_gram(h, ws, k, total_vtx, &ws.d_ctr->status, ws.kev[2 * FBN_MAX_DEPTHS],
+        rc = run_gram(h, ws, k, total_vtx, &ws.d_ctr->status, ws.d_ctr, ws.kev[2 * FBN_MAX_DEPTHS],
                       ws.kev[2 * FBN_MAX_DEPTHS + 1]);
         if (rc) return rc;
         CK(launch_pairs_decide(ws.edges, ws.edge_cap, ws.probs, ws.min_accept, ct, alpha, ws.d_ctr,
                                h->opt.statistic, h->opt.df_mode, grid_aux, st));
-        CK(cudaEventRecord(ws.tev[0][1], st));
         enqueue_tail();
         launches += 6;
-        direct[0] = true;
         d_loop = 1;
+    } else if (popc0) {
+        enqueue_head();
+        enqueue_popc0();
+        enqueue_tail();
+        launches += 5;
+        d_loop = 1;
+    }
+    if (marg1 && !shard) {
+        enqueue_head(true);
+        enqueue_marg();
+        enqueue_tail();
+        launches += 7;
+        d_loop = 2;
     }
     if (nbr1 && (max_depth < 0 || max_depth >= 1)) {
         if (d_loop == 0) {   // depth 0 on the pool, launched directly
             enqueue_head();
-            CK(cudaEventRecord(ws.tev[0][0], st));
             enqueue_tests();
-            CK(cudaEventRecord(ws.tev[0][1], st));
             enqueue_tail();
             launches += body_launches - 1;
-            direct[0] = true;
         }
         enqueue_head();
-        CK(cudaEventRecord(ws.tev[1][0], st));
+        CK(cudaEventRecord(ws.tev[0], st));
         CK(launch_nbr1(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx, ws.edges, ws.min_accept, ct, alpha, ws.d_ctr,
                        dev_sms, h->opt.wait_limit, st));
-        CK(cudaEventRecord(ws.tev[1][1], st));
+        CK(cudaEventRecord(ws.tev[1], st));
         enqueue_tail();
         launches += 5;
-        direct[1] = true;
+        direct1 = true;
         d_loop = 2;
     }
     const bool loop = max_depth < 0 || d_loop <= max_depth;
@@ -1131,8 +1181,10 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
                 return fail(h, FBN_EINVAL, "the own callback failed at depth %d", d);
             CK(cudaMemcpyAsync(ws.d_owned, own_h.data(), own_h.size(), cudaMemcpyHostToDevice, st));
             CK(cudaMemsetAsync(ws.d_shard_count, 0, sizeof(unsigned long long), st));
-            enqueue_head();
-            enqueue_tests();
+            enqueue_head(d == 1 && marg1);
+            if (d == 0 && popc0) enqueue_popc0();
+            else if (d == 1 && marg1) enqueue_marg();
+            else enqueue_tests();
             launch_shard_export(ws.probs, ws.edges, ws.min_accept, ws.edge_cap, ws.d_ctr, ws.d_shard, ws.d_shard_count,
                                 grid_aux, st);
             unsigned long long m = 0;
@@ -1201,12 +1253,11 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
                 CK(cudaMemcpyAsync(adj_out[p], hs[p]->d_adj, (size_t)hs[p]->n * hs[p]->n, cudaMemcpyDefault, st));
     CK(cudaStreamSynchronize(st));
     if (loop && !shard) launches += (long long)(body_launches - (host_loop ? 1 : 0)) * std::max(0, ws.h_ctr->d - d_loop);
-    for (int q = 0; q < 2; ++q)
-        if (direct[q]) {
-            float kms = 0.f;
-            CK(cudaEventElapsedTime(&kms, ws.tev[q][0], ws.tev[q][1]));
-            stats.test_ms[q] = kms;
-        }
+    if (direct1) {
+        float kms = 0.f;
+        CK(cudaEventElapsedTime(&kms, ws.tev[0], ws.tev[1]));
+        stats.test_ms[1] = kms;
+    }
     const DepthCounters& c = *ws.h_ctr;
     if (c.status == 0) ws.split_dirty = false;   // every split test's last part zeroed its table
     if (c.status & (kStatusSepPool | kStatusScratch)) {
@@ -1241,7 +1292,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         const unsigned long long next = d + 1 < kMaxDepthRecords ? ws.h_rec[d + 1].t_begin : 0;
         const unsigned long long end = next > r.t_begin ? next : r.t_end;
         stats.ms[d] = end > r.t_begin && r.t_begin ? (float)((end - r.t_begin) * 1e-6) : 0.f;
-        if (d >= d_loop && r.t_tests_end > r.t_tests && r.t_tests)
+        if (!(direct1 && d == 1) && r.t_tests_end > r.t_tests && r.t_tests)
             stats.test_ms[d] = (float)((r.t_tests_end - r.t_tests) * 1e-6);
     }
     if (gram) {
@@ -1450,7 +1501,7 @@ int autotune_impl(fbn_handle* const* hs, int k, double alpha, int32_t max_depth,
     const fbn_options& o = h->opt;
     const bool pool = o.form == FBN_FORM_POOL;
     // candidates for the pool depths: byte histograms at each group size, and
-    // bit planes where every small table qualifies (their pool runs warp groups)
+    // one-hot planes at the depths they serve (their pools run warp groups)
     std::vector<int> cands;
     if (pool && o.group_threads == 0) {
         for (int g : {32, 64, 128, kTestThreads}) cands.push_back(g | (o.count == FBN_COUNT_BITS ? 0 : kTuneNoBits));
@@ -1509,24 +1560,17 @@ int autotune_impl(fbn_handle* const* hs, int k, double alpha, int32_t max_depth,
     const bool gram_used = choice.depth0 ? choice.depth0 == FBN_DEPTH0_GRAM : gram_rule;
     rep.depths = depths;
     rep.depth0 = gram_used ? FBN_DEPTH0_GRAM : FBN_DEPTH0_HIST;
-    int max_ar = 0;
-    long long max_n = 0;
-    for (int p = 0; p < k; ++p) {
-        max_ar = std::max(max_ar, hs[p]->max_arity);
-        max_n = std::max<long long>(max_n, hs[p]->N);
-    }
+    apply_tuning(hs, k, choice.table, choice.depth0);
+    const DepthPlan plan = depth_plan(hs, k, false);
     for (int d = 0; d < depths && d < FBN_MAX_DEPTHS; ++d) {
         const int c = choice.table.empty() ? 0 : choice.table[d];
-        // bit planes only where the depth's tables can take them
-        const bool bits = !(c & kTuneNoBits) && bits_cells(h) > 0 && bits_shape_ok(d, max_ar, max_n) &&
-                          !(d == 0 && gram_used);
+        const bool bits = d == 0 ? plan.popc0 : d == 1 && plan.marg1;
         rep.count[d] = bits ? FBN_COUNT_BITS : FBN_COUNT_HIST;
         rep.group_threads[d] = bits ? 32 : o.group_threads ? o.group_threads : (c & kTuneGroupMask);   // 0: cost model
     }
     rep.ms_fixed = ms_fixed;
     rep.ms_tuned = ms_tuned;
     choice.report = rep;
-    apply_tuning(hs, k, choice.table, choice.depth0);
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         g_tune_cache[tune_key(hs, k, alpha, max_depth)] = choice;
@@ -1663,7 +1707,8 @@ int fbn_create(const uint8_t* data, int32_t n_vars, int64_t n_samples, const uin
     const size_t nn = (size_t)n_vars * n_vars;
     CKC(dalloc(&h->d_data, (size_t)n_vars * h->ld));
     h->plane_ld = ((n_samples + 31) / 32 + 3) / 4 * 4;   // 32-sample words, whole uint4 groups
-    CKC(dalloc(&h->d_planes, (size_t)n_vars * 2 * h->plane_ld));
+    h->nplanes = max_ar <= kMargMaxArity ? max_ar - 1 : 0;
+    CKC(dalloc(&h->d_planes, (size_t)n_vars * h->nplanes * h->plane_ld));
     CKC(dalloc(&h->d_ar, n_vars));
     CKC(dalloc(&h->d_adj, nn));
     CKC(dalloc(&h->d_nbr, nn));
@@ -1684,16 +1729,9 @@ int fbn_create(const uint8_t* data, int32_t n_vars, int64_t n_samples, const uin
     CKC(cudaMemcpy2DAsync(h->d_data, h->ld, data, n_samples, n_samples, n_vars, cudaMemcpyDefault, st));
     CKC(cudaMemcpyAsync(h->d_ar, arities, n_vars, cudaMemcpyHostToDevice, st));
     // values must lie below their arity: checked on the device
-    unsigned long long* bad = h->d_bad;
-    CKC(cudaMemsetAsync(bad, 0xff, sizeof(unsigned long long), st));
-    {
-        dim3 grid((unsigned)std::min<long long>((n_samples + 255) / 256, 64), n_vars);
-        k_validate<<<grid, 256, 0, st>>>(h->d_data, h->ld, n_vars, n_samples, h->d_ar, bad);
-    }
-    CKC(cudaGetLastError());
-    if (launch_planes(h, st)) return bail(FBN_ECUDA);
+    if (launch_ingest(h, st)) return bail(FBN_ECUDA);
     unsigned long long first_bad = 0;
-    CKC(cudaMemcpyAsync(h->h_status, bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+    CKC(cudaMemcpyAsync(h->h_status, h->d_bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
     CKC(cudaStreamSynchronize(st));
     std::memcpy(&first_bad, h->h_status, sizeof first_bad);
     if (first_bad != ~0ULL) {
@@ -1729,14 +1767,9 @@ int fbn_update_data(fbn_handle* h, const uint8_t* data)
     h->learnt = false;
     h->sep_pending = false;
     CK(cudaMemcpy2DAsync(h->d_data, h->ld, data, h->N, h->N, h->n, cudaMemcpyDefault, st));
-    unsigned long long* bad = h->d_bad;
-    CK(cudaMemsetAsync(bad, 0xff, sizeof(unsigned long long), st));
-    dim3 grid((unsigned)std::min<long long>((h->N + 255) / 256, 64), h->n);
-    k_validate<<<grid, 256, 0, st>>>(h->d_data, h->ld, h->n, h->N, h->d_ar, bad);
-    CK(cudaGetLastError());
-    const int prc = launch_planes(h, st);
+    const int prc = launch_ingest(h, st);
     if (prc) return prc;
-    CK(cudaMemcpyAsync(h->h_status, bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(h->h_status, h->d_bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     unsigned long long first_bad;
     std::memcpy(&first_bad, h->h_status, sizeof first_bad);
@@ -1765,14 +1798,9 @@ int fbn_update_data_batch(fbn_handle* const* hs, int32_t k, const uint8_t* const
         q->learnt = false;
         q->sep_pending = false;
         CK(cudaMemcpy2DAsync(q->d_data, q->ld, data[p], q->N, q->N, q->n, cudaMemcpyDefault, st));
-        unsigned long long* bad = q->d_bad;
-        CK(cudaMemsetAsync(bad, 0xff, sizeof(unsigned long long), st));
-        dim3 grid((unsigned)std::min<long long>((q->N + 255) / 256, 64), q->n);
-        k_validate<<<grid, 256, 0, st>>>(q->d_data, q->ld, q->n, q->N, q->d_ar, bad);
-        CK(cudaGetLastError());
-        const int prc = launch_planes(q, st);
+        const int prc = launch_ingest(q, st);
         if (prc) return fail(h, prc, "%s", q->err.c_str());
-        CK(cudaMemcpyAsync(q->h_status, bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(q->h_status, q->d_bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
     }
     CK(cudaStreamSynchronize(st));
     for (int p = 0; p < k; ++p) {

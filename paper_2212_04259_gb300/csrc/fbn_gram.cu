@@ -29,7 +29,7 @@
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
-#include "fbn_device.cuh"
+#include "fbn_depth.cuh"
 #include "fbn_gram.h"
 #include "fbn_tc.cuh"
 
@@ -241,11 +241,14 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram(GramArgs g)
 // One-hot matrix E of every problem: row off_v + x holds 0x38 (E4M3 1.0)
 // where V_v = x, else 0; samples at or beyond N (the padding of the store)
 // are 0 for every row.  One CTA per variable of the batch.
+// ctr: nullable; the depth whose tests start here.
 __global__ void k_onehot(const ProblemDev* __restrict__ probs, const int32_t* __restrict__ vtx_prob,
-                         const int32_t* __restrict__ vtx_first, int total_vertices)
+                         const int32_t* __restrict__ vtx_first, int total_vertices, const DepthCounters* ctr)
 {
     const int g = blockIdx.x;
     if (g >= total_vertices) return;
+    if (ctr && g == 0 && threadIdx.x == 0)
+        if (DepthRecord* r = depth_rec(ctr, ctr->d)) r->t_tests = gtime();
     const int p = vtx_prob[g];
     const ProblemDev& P = probs[p];
     const int v = g - vtx_first[p];
@@ -476,7 +479,11 @@ __global__ void k_pairs_decide(const EdgeWork* __restrict__ edges, long long edg
         pair_decide(edges, k < n0 ? k : edge_cap - n1 + (k - n0), probs, min_accept, crit, alpha, ctr, stat,
                     df_mode, local);
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&ctr->tests, (unsigned long long)(n0 + n1));   // one test per pair
+    __syncthreads();
+    if (threadIdx.x == 0)
+        if (DepthRecord* r = depth_rec(ctr, ctr->d)) atomicMax(&r->t_tests_end, gtime());
 }
+
 // Zero the pad rows M..Mp of every problem's one-hot matrix (one CTA per
 // problem); rows below M are rewritten by k_onehot on every call.
 __global__ void k_zero_pad(const ProblemDev* __restrict__ probs)
@@ -520,9 +527,9 @@ int gram_rows_padded(int M) { return (M + kTile - 1) / kTile * kTile; }
 long long gram_samples_padded(long long N) { return (N + kKSlice - 1) / kKSlice * kKSlice; }
 
 cudaError_t launch_onehot(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first,
-                          int total_vertices, cudaStream_t st)
+                          int total_vertices, const DepthCounters* ctr, cudaStream_t st)
 {
-    k_onehot<<<total_vertices, 256, 0, st>>>(probs, vtx_prob, vtx_first, total_vertices);
+    k_onehot<<<total_vertices, 256, 0, st>>>(probs, vtx_prob, vtx_first, total_vertices, ctr);
     return cudaGetLastError();
 }
 

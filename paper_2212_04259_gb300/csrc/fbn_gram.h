@@ -13,7 +13,7 @@ size_t gram_smem_bytes();
 int gram_rows_padded(int M);
 long long gram_samples_padded(long long N);
 cudaError_t launch_onehot(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first,
-                          int total_vertices, cudaStream_t st);
+                          int total_vertices, const DepthCounters* ctr, cudaStream_t st);
 cudaError_t launch_zero_pad(const ProblemDev* probs, int nprob, cudaStream_t st);
 cudaError_t encode_onehot_map(void* map, const uint8_t* E, int Mp, long long K);
 size_t tensor_map_bytes();

@@ -24,19 +24,10 @@ constexpr unsigned kStatusEdges = 8u;     // edge list overflow
 constexpr unsigned kStatusTimeout = 16u;  // a bounded device wait gave up
 constexpr unsigned kStatusScratch = 32u;  // a table needed more global scratch than allocated
 constexpr int kMaxArityPairs = 256;       // arity bound of the depth-0 pair epilogue
-// Bit-plane counting: every variable of a test has arity <= kBitsMaxArity (two
-// bit planes per variable) and at most kBitsMaxD conditioning variables.
-constexpr int kBitsMaxArity = 4;
-constexpr int kBitsMaxD = 1;
-constexpr long long kBitsMaxN = 2000000;   // samples within the 16-bit counters of the bit-plane count
-
-// Whether a test can be counted from the bit planes (all arities <= 4, d <= 1,
-// N within the 16-bit counters).  The same rule, applied to an edge's bound on
-// its tables, puts the edge into the bit-plane pool.
-__host__ __device__ __forceinline__ bool bits_shape_ok(int d, int max_arity, long long N)
-{
-    return d <= kBitsMaxD && max_arity <= kBitsMaxArity && N <= kBitsMaxN;
-}
+// Depths 0 and 1 from one-hot bit planes: largest arity (kMargMaxArity - 1
+// planes per variable; the x and y values of a test share one warp's lanes).
+constexpr int kMargMaxArity = 5;
+constexpr int kMargThreads = 256;          // threads of a k_pool_marg CTA
 
 // One learning problem (one data set).  Arrays are device pointers.
 struct ProblemDev {
@@ -51,7 +42,7 @@ struct ProblemDev {
     int32_t n;
     int32_t N;
     int32_t max_arity;
-    int32_t pad;
+    int32_t nplanes;       // one-hot planes per variable: max_arity - 1, or 0 without planes
     // one-hot Gram of depth 0 (unused when depth 0 runs on the histogram path)
     const int32_t* off;    // [n] first one-hot row of each variable
     uint8_t* onehot;       // [gram_ld][onehot_ld] E4M3 one-hot rows
@@ -62,10 +53,10 @@ struct ProblemDev {
     int32_t* npos;         // [n][n] npos[v][u] = index of u in nbr[v] (u adjacent to v in the snapshot)
     uint8_t* pk;           // [n][pk_ld] samples 4 bits each (depth-1 tensor-core path; arities <= 8)
     int64_t pk_ld;         // ld / 2
-    // bit planes: plane b of variable v, word w = bit b of the values of
-    // samples 32 w .. 32 w + 31 (bit i = sample 32 w + i); planes[(2 v + b) *
-    // plane_ld + w].  plane_ld is a multiple of 4 words; words past the samples
-    // are zero.  Meaningful for variables of arity <= kBitsMaxArity.
+    // one-hot planes (every arity of the problem <= kMargMaxArity): bit s of
+    // planes[(v * nplanes + a) * plane_ld + w] says that sample 32 w + s of
+    // variable v has value a + 1.  plane_ld is a multiple of 4 words; bits past
+    // the samples are zero; planes a >= r_v - 1 are not written.
     const uint32_t* planes;
     int64_t plane_ld;
 };
@@ -93,7 +84,7 @@ __host__ __device__ __forceinline__ int tune_code(const int* tune, int d)
 // workers, the others on CTA workers.
 constexpr int kClassWarp = 0;
 constexpr int kClassCta = 1;
-constexpr int kClassBits = 2;   // not an edge class: the small-table class run on the bit-plane pool
+constexpr int kClassMarg = 2;   // not an edge class: the pool of depth 1 counted from one-hot planes
 
 // Device-side state of the depth loop.  Per-depth fields are cleared by
 // k_depth_begin; d, active, status and sep_used persist across depths.
@@ -132,9 +123,8 @@ struct DepthCounters {
     unsigned long long nbr_claim;       // vertex claims of the depth-1 tensor-core kernel
     unsigned long long max_total[2];    // largest rank count of an edge per class
     int split[2];                       // sample parts per test per class (1 = whole tests)
-    int bits_ok;                        // 1 while every small-table edge of the depth can be counted from bit
-                                        // planes (k_edges clears it); 1 again for the next depth
-    int pad_bits;
+    int whole;                          // depth 1 from one-hot planes: an item is a whole edge (set by k_edges)
+    int pad_whole;
     DepthRecord* rec;                   // per-depth records (persists)
     const int* tune;                    // per-depth choices of the autotuner, or nullptr (persists):
                                         // kTuneGroupMask = threads per test of the small-table class (0: cost
@@ -165,6 +155,19 @@ __host__ __device__ __forceinline__ long long chunk_count(long long total, int g
     return (total + c - 1) / c;
 }
 
+// Order key of an edge that is one work item of k_pool_marg, 1 .. kMaxPasses,
+// descending: edges of one counting shape (the endpoints' arities) together, so
+// that the warps of an SM run the same loop and its instructions stay cached;
+// within a shape the longest (tests times samples, 8 steps per octave) first.
+__device__ __forceinline__ long long edge_item_key(long long total, int N, int ra, int rb)
+{
+    const int A = ra > rb ? ra : rb, B = ra > rb ? rb : ra;        // 2 <= B <= A <= kMargMaxArity
+    const int shape = (A - 2) * (A - 1) / 2 + (B - 2);             // 0 .. 9
+    int w = (__float_as_int((float)total * (float)N) >> 20) - (127 << 3);
+    w = w < 0 ? 0 : w > 399 ? 399 : w;
+    return (long long)shape * 400 + w + 1;
+}
+
 // Per-class arguments of the ordering scan.
 struct ScanClass {
     const unsigned long long* hist;   // chunk-count histogram of the class
@@ -172,8 +175,6 @@ struct ScanClass {
     unsigned long long* base;         // [maxc + 1] first item of pass k
     long long groups[4];              // groups of 32, 64, 128, 256 threads the class's pool runs
     long long smem_ints;              // shared ints of one pool CTA of the class
-    long long groups_bits[4];         // the same for the bit-plane pool (class 0 when every edge qualifies)
-    long long smem_ints_bits;
 };
 
 // Cache of critical values, see fbn_device.cuh.

@@ -1,7 +1,7 @@
 // fbn_kernels.cu -- per-depth kernels of the PC-stable skeleton (Algorithm 1)
 // and their host launchers, for sm_103a.  The work-pool kernels live in
-// fbn_pool_small.cu, fbn_pool_bits.cu, fbn_pool_big.cu and fbn_plain.cu (device
-// code in fbn_pool.cuh); the explicit-test kernel in fbn_ci.cu.
+// fbn_pool_small.cu, fbn_pool_big.cu, fbn_plain.cu (device code in
+// fbn_pool.cuh) and fbn_pool_marg.cu; the explicit-test kernel in fbn_ci.cu.
 //
 // Depth pipeline (every kernel runs over all problems of a batch at once):
 //   k_snapshot   a(v) for every vertex: adjacency row -> ascending neighbour list
@@ -42,7 +42,9 @@ static bool g_pdl = true;
 
 // The work-pool kernels, each defined in its own translation unit.
 __global__ void k_pool_small(PoolArgs a);
-__global__ void k_pool_bits(PoolArgs a);
+__global__ void k_pool_marg(PoolArgs a);
+__global__ void k_pairs_popc(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first,
+                             int total_vertices, int max_n, const uint8_t* owned, PoolArgs a);
 __global__ void k_pool_big(PoolArgs a);
 __global__ void k_plain(PoolArgs a);
 
@@ -87,9 +89,19 @@ __device__ __forceinline__ long long binom_sat(const long long* B, int brows, in
     return B[(long long)n * kBinomCols + k];
 }
 
+// Depth 1 from one-hot planes: edges per warp from which an item is a whole
+// edge (no test beyond the first accepting one, no claim per chunk), and the
+// ranks per item from one edge per warp on.  Below, single ranks: the depth is
+// then as long as its longest chain of tests.  Measured (depth 1, ms): 4.4 edges
+// per warp (1,000 variables) whole 3.70, chunks of 1 / 2 / 4 / 8 ranks 1.73 /
+// 1.62 / 1.63 / 1.75; 9 per warp (20 problems) whole 0.73, chunks 0.92 / 0.70 /
+// 0.62 / 0.61; 131 per warp (256 problems) whole 5.4.
+constexpr long long kWholeEdges = 16;
+constexpr int kMargChunk = 4;
+
 __global__ void k_edges(const ProblemDev* __restrict__ probs, const int32_t* __restrict__ vtx_prob,
                         const int32_t* __restrict__ vtx_first, int total_vertices, int gs_forced, long long gs_edges,
-                        const long long* __restrict__ binom, int brows, long long warp_cells_cap, int bits_cells,
+                        const long long* __restrict__ binom, int brows, long long warp_cells_cap, long long marg_warps,
                         const uint8_t* __restrict__ owned, EdgeWork* __restrict__ edges,
                         unsigned long long* __restrict__ min_accept, long long edge_cap, DepthCounters* ctr,
                         unsigned long long* __restrict__ hist)
@@ -101,8 +113,19 @@ __global__ void k_edges(const ProblemDev* __restrict__ probs, const int32_t* __r
     const int d = ctr->d;
     // ranks per chunk: 1 while the live edges are few against the groups
     // (latency of a single test dominates), 4 when there are many (fewer claims)
-    const int gs = gs_forced > 0 ? gs_forced : ((long long)(ctr->adj_ends / 2) >= gs_edges ? 4 : 1);
-    if (g == 0 && lane == 0) ctr->gs = gs;
+    const long long live = (long long)(ctr->adj_ends / 2);
+    int gs = gs_forced > 0 ? gs_forced : live >= gs_edges ? 4 : 1;
+    // depth 1 from one-hot planes (marg_warps > 0: the warps of its pool): a
+    // whole edge per item from kWholeEdges edges per warp
+    bool whole = false;
+    if (marg_warps > 0 && d == 1 && gs_forced == 0) {
+        whole = live >= kWholeEdges * marg_warps;
+        gs = live >= marg_warps ? kMargChunk : 1;
+    }
+    if (g == 0 && lane == 0) {
+        ctr->gs = gs;
+        ctr->whole = whole;
+    }
     const int p = vtx_prob[g];
     const ProblemDev P = probs[p];
     const int i = g - vtx_first[p];
@@ -135,14 +158,9 @@ __global__ void k_edges(const ProblemDev* __restrict__ probs, const int32_t* __r
                 cells *= (unsigned long long)P.max_arity;
         }
         const int cls = cells <= (unsigned long long)warp_cells_cap ? kClassWarp : kClassCta;
-        // the small-table class runs on the bit-plane pool only if every one
-        // of its edges qualifies there (all arities <= 4, d <= 1, table bound
-        // within bits_cells)
-        const bool bits = bits_cells > 0 && !(tune_code(ctr->tune, d) & kTuneNoBits) && bits_shape_ok(d, P.max_arity, P.N) &&
-                          cells <= (unsigned long long)bits_cells;
-        if (__any_sync(0xffffffffu, total > 0 && cls == kClassWarp && !bits) && lane == 0) ctr->bits_ok = 0;
-        {   // chunk-count histogram of each class: one atomic per distinct bin in the warp
-            const long long bin = total > 0 ? (long long)cls * (kMaxPasses + 1) + chunk_count(total, gs) : -1;
+        {   // histogram of each class's order key: one atomic per distinct bin in the warp
+            const long long key = whole ? edge_item_key(total, P.N, P.ar[i], P.ar[j]) : chunk_count(total, gs);
+            const long long bin = total > 0 ? (long long)cls * (kMaxPasses + 1) + key : -1;
             const unsigned same = __match_any_sync(0xffffffffu, bin);
             if (bin >= 0 && lane == __ffs(same) - 1) atomicAdd(&hist[bin], (unsigned long long)__popc(same));
         }
@@ -168,7 +186,7 @@ __global__ void k_edges(const ProblemDev* __restrict__ probs, const int32_t* __r
             min_accept[e] = (unsigned long long)total;
             P.eid[(long long)i * P.n + t] = (int32_t)e;
             P.eid[(long long)j * P.n + lo] = (int32_t)e;
-            const unsigned long long ch = (unsigned long long)chunk_count(total, gs);
+            const unsigned long long ch = (unsigned long long)(whole ? edge_item_key(total, P.N, P.ar[i], P.ar[j]) : chunk_count(total, gs));
             mc[c] = ch > mc[c] ? ch : mc[c];
             mcell[c] = cells > mcell[c] ? cells : mcell[c];
             mtot[c] = (unsigned long long)total > mtot[c] ? (unsigned long long)total : mtot[c];
@@ -233,10 +251,9 @@ __device__ __forceinline__ unsigned long long block_exclusive_scan(unsigned long
 // may force a size.
 constexpr double kTestOverhead = 10000.0;
 constexpr double kCyclesPerSample = 8.0;
-constexpr double kCyclesPerSampleBits = 3.0;   // the bit-plane pool
 
 __global__ void k_scan(ScanClass c0, ScanClass c1, DepthCounters* ctr, double mean_n, int forced_group,
-                       long long split_stride, int allow_split)
+                       long long split_stride, int allow_split, int marg)
 {
     pdl_enter();
     __shared__ unsigned long long sh[32];
@@ -248,10 +265,8 @@ __global__ void k_scan(ScanClass c0, ScanClass c1, DepthCounters* ctr, double me
     const unsigned long long* __restrict__ hist = sc.hist;
     unsigned long long* __restrict__ alive = sc.alive;
     unsigned long long* __restrict__ base = sc.base;
-    const bool bits = cls == kClassWarp && ctr->bits_ok;   // the class runs on the bit-plane pool
-    const long long* grp = bits ? sc.groups_bits : sc.groups;
-    const long long g32 = grp[0], g64 = grp[1], g128 = grp[2], g256 = grp[3];
-    const long long smem_ints = bits ? sc.smem_ints_bits : sc.smem_ints;
+    const long long g32 = sc.groups[0], g64 = sc.groups[1], g128 = sc.groups[2], g256 = sc.groups[3];
+    const long long smem_ints = sc.smem_ints;
     const long long maxc = (long long)ctr->maxc[cls];
     if (ctr->n_edges[cls] == 0) return;
     const int T = blockDim.x;
@@ -281,6 +296,11 @@ __global__ void k_scan(ScanClass c0, ScanClass c1, DepthCounters* ctr, double me
         run += alive[c];
     }
     if (fhi == len && flo < fhi) {
+        if (marg) {   // one warp per item; whole edges in the order of edge_item_key, else passes of chunks
+            ctr->total_items[cls] = ctr->whole ? ctr->n_edges[cls] : base[maxc];
+            ctr->next_item[cls] = 0;
+            return;
+        }
         const unsigned long long W = base[maxc];
         ctr->total_items[cls] = W;
         ctr->next_item[cls] = 0;
@@ -291,16 +311,15 @@ __global__ void k_scan(ScanClass c0, ScanClass c1, DepthCounters* ctr, double me
             for (int k = 0; k < 4; ++k) {
                 const int G = 32 << k;
                 const double rounds = (double)((W + groups[k] - 1) / groups[k]);
-                const double t = rounds * (kTestOverhead + (bits ? kCyclesPerSampleBits : kCyclesPerSample) * mean_n / G);
+                const double t = rounds * (kTestOverhead + kCyclesPerSample * mean_n / G);
                 if (t < best_t) {
                     best_t = t;
                     best = G;
                 }
             }
-            // the bit-plane pool: warp groups; else the caller's choice, the
-            // autotuner's for this depth, or the cost model's
+            // the caller's choice, the autotuner's for this depth, or the cost model's
             const int tuned = tune_code(ctr->tune, ctr->d) & kTuneGroupMask;
-            ctr->gsel = bits ? 32 : forced_group ? forced_group : tuned ? tuned : best;
+            ctr->gsel = forced_group ? forced_group : tuned ? tuned : best;
         }
         // sample split: few single-rank tests against the groups of the class
         const int G = cls == 0 ? ctr->gsel : kTestThreads;
@@ -324,7 +343,7 @@ __global__ void k_scan(ScanClass c0, ScanClass c1, DepthCounters* ctr, double me
 
 // Both classes at once: class c's order goes to sorted[class_base(c) ..], the
 // same region its edges occupy, so the two never overlap.
-__global__ void k_place(const EdgeWork* __restrict__ edges, long long edge_cap, int nclass,
+__global__ void k_place(const ProblemDev* __restrict__ probs, const EdgeWork* __restrict__ edges, long long edge_cap, int nclass,
                         const DepthCounters* ctr, const unsigned long long* __restrict__ alive0,
                         unsigned long long* __restrict__ cursor0, const unsigned long long* __restrict__ alive1,
                         unsigned long long* __restrict__ cursor1, int32_t* __restrict__ sorted)
@@ -332,6 +351,7 @@ __global__ void k_place(const EdgeWork* __restrict__ edges, long long edge_cap, 
     pdl_enter();
     if (!ctr->active) return;
     const int gs = ctr->gs;
+    const bool whole = ctr->whole != 0;
     const long long E0 = (long long)ctr->n_edges[0];
     const long long E = E0 + (nclass > 1 ? (long long)ctr->n_edges[1] : 0);
     const long long b1 = class_base(ctr, 1, edge_cap);
@@ -339,7 +359,8 @@ __global__ void k_place(const EdgeWork* __restrict__ edges, long long edge_cap, 
         const bool first = k < E0;
         const long long e = first ? k : k - E0;
         const long long cb = first ? 0 : b1;
-        const long long ch = chunk_count(edges[cb + e].total, gs);
+        const EdgeWork w = edges[cb + e];
+        const long long ch = whole ? edge_item_key(w.total, probs[w.prob].N, probs[w.prob].ar[w.i], probs[w.prob].ar[w.j]) : chunk_count(w.total, gs);
         const unsigned long long pos =
             first ? alive0[ch] + atomicAdd(&cursor0[ch], 1ULL) : alive1[ch] + atomicAdd(&cursor1[ch], 1ULL);
         sorted[cb + (long long)pos] = (int32_t)e;
@@ -537,7 +558,7 @@ __global__ void k_depth_end(DepthCounters* ctr, DepthRecord* rec, int max_depth,
         ctr->nbr_claim = 0;
         ctr->max_total[0] = ctr->max_total[1] = 0;
         ctr->split[0] = ctr->split[1] = 1;
-        ctr->bits_ok = 1;
+        ctr->whole = 0;
         ctr->d = next;
         __threadfence();
         ctr->active = stop ? 0 : 1;
@@ -594,23 +615,24 @@ void launch_snapshot(const ProblemDev* probs, const int32_t* vtx_prob, const int
 
 void launch_edges(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first,
                   int total_vertices, int gs_forced, long long gs_edges, const long long* binom, int brows,
-                  long long warp_cells_cap, int bits_cells, const uint8_t* owned,
+                  long long warp_cells_cap, long long marg_warps, const uint8_t* owned,
                   EdgeWork* edges, unsigned long long* min_accept, long long edge_cap, DepthCounters* ctr,
                   unsigned long long* hist, cudaStream_t st)
 {
     const int warps = 8;
     launch_pdl(k_edges, dim3((total_vertices + warps - 1) / warps), dim3(warps * 32), 0, st, probs, vtx_prob,
-               vtx_first, total_vertices, gs_forced, gs_edges, binom, brows, warp_cells_cap, bits_cells, owned, edges,
+               vtx_first, total_vertices, gs_forced, gs_edges, binom, brows, warp_cells_cap, marg_warps, owned, edges,
                min_accept, edge_cap, ctr, hist);
 }
 
-void launch_order(const EdgeWork* edges, long long edge_cap, int nclass, DepthCounters* ctr, const ScanClass* sc,
-                  unsigned long long* cursor0, unsigned long long* cursor1, int32_t* sorted, double mean_n,
-                  int forced_group, long long split_stride, int allow_split, int grid, cudaStream_t st)
+void launch_order(const ProblemDev* probs, const EdgeWork* edges, long long edge_cap, int nclass, DepthCounters* ctr,
+                  const ScanClass* sc, unsigned long long* cursor0, unsigned long long* cursor1, int32_t* sorted,
+                  double mean_n, int forced_group, long long split_stride, int allow_split, int marg, int grid,
+                  cudaStream_t st)
 {
     launch_pdl(k_scan, dim3(nclass), dim3(256), 0, st, sc[0], sc[nclass > 1 ? 1 : 0], ctr, mean_n, forced_group,
-               split_stride, allow_split);
-    launch_pdl(k_place, dim3(grid), dim3(256), 0, st, edges, edge_cap, nclass, ctr, (const unsigned long long*)sc[0].alive,
+               split_stride, allow_split, marg);
+    launch_pdl(k_place, dim3(grid), dim3(256), 0, st, probs, edges, edge_cap, nclass, ctr, (const unsigned long long*)sc[0].alive,
                cursor0, (const unsigned long long*)sc[nclass > 1 ? 1 : 0].alive, cursor1, sorted);
 }
 
@@ -620,9 +642,16 @@ void launch_pool(const PoolArgs& a, int cls, int grid, size_t smem_bytes, cudaSt
     else launch_pdl(k_pool_big, dim3(grid), dim3(kTestThreads), smem_bytes, st, a);
 }
 
-void launch_pool_bits(const PoolArgs& a, int grid, size_t smem_bytes, cudaStream_t st)
+void launch_pool_marg(const PoolArgs& a, int grid, cudaStream_t st)
 {
-    launch_pdl(k_pool_bits, dim3(grid), dim3(kTestThreads), smem_bytes, st, a);
+    launch_pdl(k_pool_marg, dim3(grid), dim3(kMargThreads), 0, st, a);
+}
+
+void launch_pairs_popc(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first, int total_vertices,
+                       int max_n, const uint8_t* owned, const PoolArgs& a, int grid, cudaStream_t st)
+{
+    launch_pdl(k_pairs_popc, dim3(grid), dim3(kTestThreads), 0, st, probs, vtx_prob, vtx_first, total_vertices, max_n,
+               owned, a);
 }
 
 void launch_plain(const PoolArgs& a, int grid, size_t smem_bytes, cudaStream_t st)
@@ -678,7 +707,6 @@ cudaError_t set_kernel_smem(size_t max_smem)
     const int b = (int)max_smem;
     if ((e = cudaFuncSetAttribute(k_pool_small, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
     if ((e = cudaFuncSetAttribute(k_pool_big, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
-    if ((e = cudaFuncSetAttribute(k_pool_bits, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
     if ((e = cudaFuncSetAttribute(k_plain, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
     return cudaSuccess;
 }
@@ -686,8 +714,8 @@ cudaError_t set_kernel_smem(size_t max_smem)
 int pool_blocks_per_sm(int cls, size_t smem_bytes)
 {
     int nb = 0;
-    if (cls == kClassBits)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pool_bits, kTestThreads, smem_bytes);
+    if (cls == kClassMarg)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pool_marg, kMargThreads, smem_bytes);
     else if (cls == kClassWarp)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pool_small, kTestThreads, smem_bytes);
     else

@@ -15,16 +15,20 @@ void launch_snapshot(const ProblemDev* probs, const int32_t* vtx_prob, const int
                      int total_vertices, DepthCounters* ctr, cudaStream_t st);
 void launch_edges(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first,
                   int total_vertices, int gs_forced, long long gs_edges, const long long* binom, int brows,
-                  long long warp_cells_cap, int bits_cells, const uint8_t* owned,
+                  long long warp_cells_cap, long long marg_warps, const uint8_t* owned,
                   EdgeWork* edges, unsigned long long* min_accept, long long edge_cap, DepthCounters* ctr,
                   unsigned long long* hist, cudaStream_t st);
 // Ordering of the depth's edges, one CTA per class (nclass = 1: the small-
 // table class only), then the placement of both classes.
-void launch_order(const EdgeWork* edges, long long edge_cap, int nclass, DepthCounters* ctr, const ScanClass* sc,
-                  unsigned long long* cursor0, unsigned long long* cursor1, int32_t* sorted, double mean_n,
-                  int forced_group, long long split_stride, int allow_split, int grid, cudaStream_t st);
+// marg: the depth's pool is k_pool_marg.
+void launch_order(const ProblemDev* probs, const EdgeWork* edges, long long edge_cap, int nclass, DepthCounters* ctr,
+                  const ScanClass* sc, unsigned long long* cursor0, unsigned long long* cursor1, int32_t* sorted,
+                  double mean_n, int forced_group, long long split_stride, int allow_split, int marg, int grid,
+                  cudaStream_t st);
 void launch_pool(const PoolArgs& a, int cls, int grid, size_t smem_bytes, cudaStream_t st);
-void launch_pool_bits(const PoolArgs& a, int grid, size_t smem_bytes, cudaStream_t st);
+void launch_pool_marg(const PoolArgs& a, int grid, cudaStream_t st);
+void launch_pairs_popc(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first, int total_vertices,
+                       int max_n, const uint8_t* owned, const PoolArgs& a, int grid, cudaStream_t st);
 void launch_plain(const PoolArgs& a, int grid, size_t smem_bytes, cudaStream_t st);
 void launch_apply(const ProblemDev* probs, const EdgeWork* edges, const unsigned long long* min_accept,
                   long long edge_cap, const long long* binom, int32_t* sep_pool, long long sep_cap,

@@ -18,12 +18,12 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_plain(PoolArgs a)
     const long long E = (long long)ctr->n_edges[a.cls];
     const long long cb = class_base(ctr, a.cls, a.edge_cap);
     int* gtab = a.gscratch ? a.gscratch + (long long)blockIdx.x * a.gscratch_ints : nullptr;
-    if (threadIdx.x == 0) S.tests = S.popc_work = S.smem_updates = 0;
+    if (threadIdx.x == 0) S.tests = S.smem_updates = 0;
     for (long long e = blockIdx.x; e < E; e += gridDim.x) {
         const EdgeWork w = a.edges[cb + e];
         const ProblemDev& P = a.probs[w.prob];
         for (long long rk = 0; rk < w.total; ++rk) {
-            const int res = run_rank<kTestThreads, false>(a, d, P, w, rk, rk == 0, S, spec, smem, a.smem_ints, gtab, red);
+            const int res = run_rank<kTestThreads>(a, d, P, w, rk, rk == 0, S, spec, smem, a.smem_ints, gtab, red);
             if (res == 1 && threadIdx.x == 0) a.min_accept[cb + e] = (unsigned long long)rk;
             if (res != 0) break;
         }

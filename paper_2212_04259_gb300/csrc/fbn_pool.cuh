@@ -2,8 +2,9 @@
 // IV-B) and of the edge-level form (Section IV-A): per-group state, the set-up
 // of one conditioning set (Section IV-C), counting, the bounded decision,
 // sample-split tests and the pool loop.  Each pool kernel is defined in its
-// own translation unit (fbn_pool_small.cu, fbn_pool_bits.cu, fbn_pool_big.cu,
-// fbn_plain.cu), so that they compile in parallel.
+// own translation unit (fbn_pool_small.cu, fbn_pool_big.cu, fbn_plain.cu;
+// depth 1 from one-hot planes in fbn_pool_marg.cu), so that they compile in
+// parallel.
 #pragma once
 
 #include <cstdint>
@@ -18,7 +19,7 @@ namespace fbn {
 struct GroupState {
     long long r0, r1;
     unsigned long long tests;
-    unsigned long long popc_work, smem_updates;   // counting work done, flushed with tests
+    unsigned long long smem_updates;   // counting work done, flushed with tests
     unsigned long long item;   // split tests: the test's item and this group's part
     int part;
     unsigned ticket;
@@ -34,7 +35,7 @@ struct GroupState {
 // successor of the previous rank of the same side); one thread per
 // conditioning variable then resolves its row.  Returns false (uniformly)
 // when the table is over the cell limit.
-template <int G, bool BITS>
+template <int G>
 __device__ __forceinline__ bool setup_rank(const ProblemDev& P, const EdgeWork& w, int d, long long rk, bool fresh,
                                            GroupState& S, const long long* binom, TestSpec& spec, unsigned* status)
 {
@@ -51,7 +52,6 @@ __device__ __forceinline__ bool setup_rank(const ProblemDev& P, const EdgeWork& 
         }
         spec.nrows = d + 2;
         spec.N = P.N;
-        if (BITS) spec.pstride = P.plane_ld >> 2;
     }
     Grp<G>::sync();
     if (r < d + 2) {
@@ -65,7 +65,6 @@ __device__ __forceinline__ bool setup_rank(const ProblemDev& P, const EdgeWork& 
         }
         spec.rows[r] = P.data + (long long)v * P.ld;
         spec.rad[r] = P.ar[v];
-        if (BITS && r < kBitsMaxD + 2) spec.prow[r] = reinterpret_cast<const uint4*>(P.planes + (long long)v * 2 * P.plane_ld);
     }
     Grp<G>::sync();
     long long cells = 1;
@@ -116,25 +115,23 @@ __device__ __forceinline__ int decide_test(const PoolArgs& a, const TestSpec& sp
 }
 
 // Run one rank: 1 = accepts independence, 0 = rejects, -1 = could not run.
-// Counting work of one table (rank 0): C popcounts per 32-sample word from
-// bit planes, or one shared-memory update per sample by histogram.
-template <int G, bool BITS>
+// Counting work of one table (rank 0): one shared-memory update per sample.
+template <int G>
 __device__ __forceinline__ void note_work(GroupState& S, const TestSpec& spec)
 {
     if (Grp<G>::rank() != 0) return;
-    if (BITS) S.popc_work += (unsigned long long)spec.cells * (unsigned long long)((spec.N + 31) >> 5);
-    else S.smem_updates += (unsigned long long)spec.N;
+    S.smem_updates += (unsigned long long)spec.N;
 }
 
-template <int G, bool BITS>
+template <int G>
 __device__ __forceinline__ int run_rank(const PoolArgs& a, int d, const ProblemDev& P, const EdgeWork& w, long long rk,
                                         bool fresh, GroupState& S, TestSpec& spec, int* slice, long long slice_ints,
                                         int* gtab, double* red)
 {
     unsigned* status = &a.ctr->status;
-    if (!setup_rank<G, BITS>(P, w, d, rk, fresh, S, a.binom, spec, status)) return -1;
+    if (!setup_rank<G>(P, w, d, rk, fresh, S, a.binom, spec, status)) return -1;
     int* M = nullptr;
-    const int* T = grp_table<G, BITS>(spec, slice, slice_ints, gtab, a.gscratch_ints, &M);
+    const int* T = grp_table<G>(spec, slice, slice_ints, gtab, a.gscratch_ints, &M);
     if (!T) {   // the global scratch is too small: the host grows it and starts over
         if (Grp<G>::rank() == 0) {
             atomicOr(status, kStatusScratch);
@@ -142,125 +139,16 @@ __device__ __forceinline__ int run_rank(const PoolArgs& a, int d, const ProblemD
         }
         return -1;
     }
-    note_work<G, BITS>(S, spec);
+    note_work<G>(S, spec);
     grp_marginals<G>(spec, T, M);
     return decide_test<G>(a, spec, T, M, S, red, status);
-}
-
-// One rank of a bit-plane test on a warp group, finished in registers.  After
-// the count, row k of the slice holds counter word k of every lane (the
-// bits_word_of layout: cells (z, x, y) and (z, x, y + 1) with z = k / 8,
-// x = (k / 2) mod 4, y = 2 (k mod 2)), so lane l folds row l with 128-bit
-// loads (rotated by the lane: each quarter-warp phase touches all 32 banks
-// once) and ends with the two cells of word l.  Lanes that share z and x, or
-// z and y, differ only in the bits of the other coordinate: the marginals are
-// shuffles, and every cell's coordinates are the lane's bits (no division).
-// Cells outside the table hold zero (values >= an arity never occur; strata
-// >= r_z are not counted).  The FP32 terms and the bound are those of
-// grp_decide_bound with two terms per thread; without the float bracket of
-// crit, with the observed-table df, or when the band straddles crit, the
-// table and marginals go to shared memory in the layout of the other paths
-// and decide_test decides.
-//
-// The edge's lowest accepting rank is read before the set-up and checked
-// after it (the load's latency hides behind the set-up): returns 2, nothing
-// counted, when rk is above it.
-__device__ __forceinline__ int run_rank_bits(const PoolArgs& a, int d, const ProblemDev& P, const EdgeWork& w,
-                                             long long rk, bool fresh, GroupState& S, TestSpec& spec, int* slice,
-                                             double* red, const unsigned long long* min_accept_e)
-{
-    unsigned* status = &a.ctr->status;
-    unsigned long long ma = 0ULL;
-    if ((threadIdx.x & 31) == 0) ma = *((volatile const unsigned long long*)min_accept_e);
-    __syncwarp();   // the previous rank's readers of spec and S are done
-    if (!setup_rank<32, true>(P, w, d, rk, fresh, S, a.binom, spec, status)) return -1;
-    if ((unsigned long long)rk > __shfl_sync(0xffffffffu, ma, 0)) return 2;
-    count_bits<32>(spec, slice + (threadIdx.x & 31));
-    __syncwarp();
-    // the shape is read back from shared memory: nothing of it stays live
-    // across the call
-    const int lane = threadIdx.x & 31;
-    const int rx = spec.rx, ry = spec.ry, N = spec.N;
-    const int rz = d ? spec.rad[0] : 1;
-    const int df = (rx - 1) * (ry - 1) * rz;   // declared arities: >= 1
-    const bool fast = a.df_mode == 0 && df < a.crit.dense_n;
-    // the bracket is read by lane 0 and broadcast: another warp may be
-    // storing it right now, and every lane must take the same branch below
-    // (the branches end in full-warp shuffles)
-    float2 f = make_float2(0.0f, 0.0f);
-    if (fast && lane == 0) f = a.crit.dense_f[df];   // in flight during the fold
-    const int z = lane >> 3, x = (lane >> 1) & 3, y = (lane & 1) * 2;
-    unsigned lo = 0u, hi = 0u;
-    if (z < rz) {
-        const uint4* row = reinterpret_cast<const uint4*>(slice + lane * 32);   // 32 lane columns, 8 uint4
-        if (N < 65536) {   // each half of the sum counts one cell (<= N): packed adds cannot carry
-            unsigned s2 = 0u;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const uint4 v = row[(q + lane) & 7];
-                s2 += v.x + v.y + v.z + v.w;
-            }
-            lo = s2 & 0xFFFFu;
-            hi = s2 >> 16;
-        } else {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const uint4 v = row[(q + lane) & 7];
-                lo += (v.x & 0xFFFFu) + (v.y & 0xFFFFu) + (v.z & 0xFFFFu) + (v.w & 0xFFFFu);
-                hi += (v.x >> 16) + (v.y >> 16) + (v.z >> 16) + (v.w >> 16);
-            }
-        }
-    }
-    // N_x+z over y (lane bit 0), N_+yz over x (bits 1, 2), N_++z over x
-    const unsigned nxz = lo + hi + __shfl_xor_sync(0xffffffffu, lo + hi, 1);
-    unsigned nylo = lo + __shfl_xor_sync(0xffffffffu, lo, 2);
-    unsigned nyhi = hi + __shfl_xor_sync(0xffffffffu, hi, 2);
-    unsigned nzz = nxz + __shfl_xor_sync(0xffffffffu, nxz, 2);
-    nylo += __shfl_xor_sync(0xffffffffu, nylo, 4);
-    nyhi += __shfl_xor_sync(0xffffffffu, nyhi, 4);
-    nzz += __shfl_xor_sync(0xffffffffu, nzz, 4);
-    if (lane == 0) S.popc_work += (unsigned long long)spec.cells * (unsigned long long)((N + 31) >> 5);
-    f.x = __shfl_sync(0xffffffffu, f.x, 0);
-    f.y = __shfl_sync(0xffffffffu, f.y, 0);
-    if (fast && f.y > 0.0f) {
-        float acc = 0.0f, mag = 0.0f;
-        if (a.stat == kStatX2) {
-            x2_term((int)lo, (int)nzz, (int)nxz, (int)nylo, acc);
-            x2_term((int)hi, (int)nzz, (int)nxz, (int)nyhi, acc);
-            mag = acc;
-        } else {
-            if (lo) g2_term((int)lo, (int)nzz, (int)nxz, (int)nylo, acc, mag);
-            if (hi) g2_term((int)hi, (int)nzz, (int)nxz, (int)nyhi, acc, mag);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            mag += __shfl_xor_sync(0xffffffffu, mag, o);
-        }
-        const int dec = __shfl_sync(0xffffffffu, decide_from_sums(acc, mag, 2.0f, 5.0f, a.stat, f.x, f.y), 0);
-        if (dec >= 0) {
-            if (lane == 0) S.tests += 1;   // flushed to the depth counter when the group leaves the pool
-            return dec;
-        }
-    }
-    // shared-memory layout of the other paths: T[(z r_x + x) r_y + y], marginals after it
-    int* T = slice + kBitsWords * 32;
-    if (z < rz && x < rx) {
-        const int c = (z * rx + x) * ry + y;
-        if (y < ry) T[c] = (int)lo;
-        if (y + 1 < ry) T[c + 1] = (int)hi;
-    }
-    __syncwarp();
-    int* M = T + spec.cells;
-    grp_marginals<32>(spec, T, M);
-    return decide_test<32>(a, spec, T, M, S, red, status);
 }
 
 // One part of a split test: count samples [N p / S, N (p + 1) / S) (16-aligned
 // bounds) of rank rk into the test's global table; the part that finishes last
 // copies the table into shared memory (L2 reads), zeroes it, decides and
 // lowers the edge's rank.  Returns 1 when this group decided an acceptance.
-template <int G, bool BITS>
+template <int G>
 __device__ __noinline__ int run_split_part(const PoolArgs& a, int d, const ProblemDev& P, const EdgeWork& w,
                                               long long rk, int split, GroupState& S, TestSpec& spec, int* slice,
                                               long long slice_ints, int* gtab, double* red,
@@ -272,29 +160,25 @@ __device__ __noinline__ int run_split_part(const PoolArgs& a, int d, const Probl
     if (r == 0) S.go = (unsigned long long)rk <= *((volatile const unsigned long long*)min_accept_e);
     Grp<G>::sync();
     bool ready = false;   // spec holds this rank's table shape (uniform over the group)
-    if (S.go && setup_rank<G, BITS>(P, w, d, rk, true, S, a.binom, spec, status)) {
+    if (S.go && setup_rank<G>(P, w, d, rk, true, S, a.binom, spec, status)) {
         ready = true;
         const long long N = P.N;
-        // part bounds on 128-sample boundaries: whole 16-byte vectors of the
-        // byte rows and whole uint4 groups of the bit planes
+        // part bounds on 128-sample boundaries: whole 16-byte vectors
         const long long lo = (N * S.part / split) & ~127LL;
         const long long hi = S.part == split - 1 ? N : ((N * (S.part + 1) / split) & ~127LL);
-        if (r < d + 2) {
-            spec.rows[r] += lo;
-            if (BITS && r < kBitsMaxD + 2) spec.prow[r] += lo >> 7;
-        }
+        if (r < d + 2) spec.rows[r] += lo;
         Grp<G>::sync();
         if (r == 0) spec.N = (int)(hi - lo);
         Grp<G>::sync();
         int* M = nullptr;
-        const int* T = grp_table<G, BITS>(spec, slice, slice_ints, gtab, a.gscratch_ints, &M);
+        const int* T = grp_table<G>(spec, slice, slice_ints, gtab, a.gscratch_ints, &M);
         if (!T) {
             if (r == 0) {
                 atomicOr(status, kStatusScratch);
                 atomicMax(&a.ctr->need_cells, (int)spec.cells);
             }
         } else {
-            note_work<G, BITS>(S, spec);
+            note_work<G>(S, spec);
             for (long long c = r; c < spec.cells; c += G)
                 if (T[c]) atomicAdd(Tg + c, T[c]);
         }
@@ -308,7 +192,7 @@ __device__ __noinline__ int run_split_part(const PoolArgs& a, int d, const Probl
     // the table's shape only (cells, radices), which this part's own setup
     // left in spec when it counted
     __threadfence();
-    if (!ready && !setup_rank<G, BITS>(P, w, d, rk, true, S, a.binom, spec, status)) return 0;
+    if (!ready && !setup_rank<G>(P, w, d, rk, true, S, a.binom, spec, status)) return 0;
     const long long C = spec.cells;
     int* Tl = slice;
     for (long long c = r; c < C; c += G) {
@@ -334,7 +218,7 @@ struct PoolShared {
     unsigned long long base[kBaseSmem];
 };
 
-template <int G, bool BITS = false>
+template <int G>
 __device__ __forceinline__ void pool_body(const PoolArgs& a, int* smem, PoolShared& sh)
 {
     constexpr int NG = kTestThreads / G;   // groups per CTA
@@ -360,7 +244,7 @@ __device__ __forceinline__ void pool_body(const PoolArgs& a, int* smem, PoolShar
     const unsigned long long* base = base_in_smem ? sh.base : a.base;
     GroupState& S = sh.st[g];
     TestSpec& spec = sh.spec[g];
-    if (r == 0) S.tests = S.popc_work = S.smem_updates = 0;
+    if (r == 0) S.tests = S.smem_updates = 0;
     const int split = ctr->split[a.cls] > 1 ? ctr->split[a.cls] : 1;
 
     for (;;) {
@@ -392,30 +276,23 @@ __device__ __forceinline__ void pool_body(const PoolArgs& a, int* smem, PoolShar
         const ProblemDev& P = a.probs[w.prob];
         const long long r0 = S.r0, r1 = S.r1;
         if (split > 1) {   // single-rank items (gs = 1, no edge above kMaxPasses ranks)
-            const int res = run_split_part<G, BITS>(a, d, P, w, r0, split, S, spec, slice, slice_ints, gtab, sh.red,
+            const int res = run_split_part<G>(a, d, P, w, r0, split, S, spec, slice, slice_ints, gtab, sh.red,
                                                     &min_accept[e]);
             if (res == 1 && r == 0) atomicMin(&min_accept[e], (unsigned long long)r0);
             Grp<G>::sync();
             continue;
         }
         for (long long rk = r0; rk < r1; ++rk) {
-            int res;
-            if constexpr (BITS) {   // checks the edge's rank itself (res = 2: above it)
-                static_assert(G == 32, "the bit-plane pool runs warp groups");
-                res = run_rank_bits(a, d, P, w, rk, rk == r0, S, spec, slice, sh.red, &min_accept[e]);
-            } else {
-                if (r == 0) S.go = (unsigned long long)rk <= *((volatile unsigned long long*)&min_accept[e]);
-                Grp<G>::sync();
-                if (!S.go) break;
-                res = run_rank<G, BITS>(a, d, P, w, rk, rk == r0, S, spec, slice, slice_ints, gtab, sh.red);
-            }
+            if (r == 0) S.go = (unsigned long long)rk <= *((volatile unsigned long long*)&min_accept[e]);
+            Grp<G>::sync();
+            if (!S.go) break;
+            const int res = run_rank<G>(a, d, P, w, rk, rk == r0, S, spec, slice, slice_ints, gtab, sh.red);
             if (res == 1 && r == 0) atomicMin(&min_accept[e], (unsigned long long)rk);
             if (res != 0) break;
         }
         Grp<G>::sync();
     }
     if (r == 0 && S.tests) atomicAdd(&a.ctr->tests, S.tests);
-    if (r == 0 && S.popc_work) atomicAdd(&a.ctr->popc_work, S.popc_work);
     if (r == 0 && S.smem_updates) atomicAdd(&a.ctr->smem_updates, S.smem_updates);
 }
 
