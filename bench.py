@@ -537,10 +537,10 @@ def main():
     roofline_gram = None
     if gram_used:
         if w["kind"] == "single":
-            M = int(w["ar"].astype("int64").sum())
+            M = int((w["ar"].astype("int64") - 1).sum())   # one-hot rows: the values >= 1
             flops = float(M) * M * w["data"].shape[1]          # 2 M^2 N / 2
         else:
-            flops = float(sum(int(a.astype("int64").sum()) ** 2 * d.shape[1] for d, a in w["probs"]))
+            flops = float(sum(int((a.astype("int64") - 1).sum()) ** 2 * d.shape[1] for d, a in w["probs"]))
         gms = st["gram_ms"]
         tf = flops / (gms / 1e3) / 1e12
         gtraffic, _ = profiled_traffic("k_gram", name)

@@ -101,7 +101,7 @@ typedef struct fbn_stats {
     double  ms[FBN_MAX_DEPTHS];             /* device time of depth d (device clock, ms) */
     double  test_ms[FBN_MAX_DEPTHS];        /* device time of depth d's CI-test kernels (ms) */
     double  gram_ms;                        /* device time of the one-hot Gram (0 if not used) */
-    int64_t gram_rows;                      /* M = sum of arities, when the Gram ran */
+    int64_t gram_rows;                      /* one-hot rows of the Gram (sum of arities - 1), when it ran */
     int64_t gram_samples;                   /* padded samples of the Gram */
     int64_t test_samples[FBN_MAX_DEPTHS];   /* sum over the tests_oracle[d] tests of their data set's N
                                                (in a batch each test counts its own problem's samples) */

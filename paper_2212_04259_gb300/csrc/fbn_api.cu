@@ -133,8 +133,10 @@ struct Workspace {
     // one-hot Gram of a whole batch
     uint8_t* gram_E = nullptr;                      // one-hot matrices, problem after problem
     long long gram_E_cap = 0;
-    int32_t* gram_G = nullptr;                      // Grams, problem after problem
+    int32_t* gram_G = nullptr;                      // pair tables, problem after problem
     long long gram_G_cap = 0;
+    int32_t* gram_R = nullptr;                      // Grams over the values >= 1, problem after problem
+    long long gram_R_cap = 0, gram_R_used = 0;
     uint8_t* gram_maps = nullptr;                   // tensor maps, one per problem
     long long gram_maps_cap = 0;
     int4* gram_units = nullptr;
@@ -168,7 +170,7 @@ struct Workspace {
     size_t h_tot_cap = 0;
     uint8_t* h_stage = nullptr;
     size_t h_stage_cap = 0;
-    int gram_n_units = 0;
+    int gram_n_units = 0, gram_unit_slices = 0;
     std::vector<uint8_t> h_maps;
     // one-hot layout of the last prepare_gram and the last one whose pad rows
     // were zeroed (k_onehot writes only the rows below M)
@@ -188,7 +190,7 @@ struct Workspace {
         dfree(binom); dfree(vtx_prob); dfree(vtx_first); dfree(probs);
         dfree(sep_pool); dfree(gscratch); dfree(crit_keys); dfree(crit_vals); dfree(crit_dense);
         dfree(crit_dense_f);
-        dfree(gram_E); dfree(gram_G); dfree(gram_maps); dfree(gram_units); dfree(pk);
+        dfree(gram_E); dfree(gram_G); dfree(gram_R); dfree(gram_maps); dfree(gram_units); dfree(pk);
         dfree(split_tab); dfree(split_ticket); dfree(d_tune);
         dfree(d_owned); dfree(d_shard); dfree(d_shard_count);
         if (events) {
@@ -202,7 +204,7 @@ struct Workspace {
         if (h_tot) cudaFreeHost(h_tot);
         if (h_stage) cudaFreeHost(h_stage);
         h_maps.clear();
-        gram_E = nullptr; gram_G = nullptr; gram_maps = nullptr; gram_units = nullptr; pk = nullptr;
+        gram_E = nullptr; gram_G = nullptr; gram_R = nullptr; gram_maps = nullptr; gram_units = nullptr; pk = nullptr;
         split_tab = nullptr; split_ticket = nullptr;
         *this = Workspace();
     }
@@ -258,8 +260,9 @@ struct fbn_handle {
     // one-hot Gram (depth 0 on tensor cores)
     int M = 0;                          // sum of arities
     int Mp = 0;                         // M padded to the tile
+    int Mr = 0;                         // M - n (values >= 1) padded to the tile
     long long K = 0;                    // samples padded to the stage width
-    int32_t* d_off = nullptr;           // [n] first one-hot row of each variable
+    int32_t* d_off = nullptr;           // [n] sum of the arities before each variable; [n] the same of arities - 1
     // results of the last skeleton
     bool learnt = false;
     bool sep_pending = false;           // separating sets still only on the device
@@ -551,10 +554,24 @@ int prepare_gram(fbn_handle* const* hs, int k, Workspace& ws, ProblemDev* P)
 {
     fbn_handle* h = hs[0];
     cudaStream_t st = h->stream;
-    const int prc = prepare_pairs(hs, k, ws, P);
-    if (prc) return prc;
-    long long e_total = 0;
-    for (int p = 0; p < k; ++p) e_total += (long long)hs[p]->Mp * hs[p]->K;
+    long long e_total = 0, r_total = 0, tile_stages = 0;
+    for (int p = 0; p < k; ++p) {
+        const long long T = hs[p]->Mr / 128;
+        e_total += (long long)hs[p]->Mr * hs[p]->K;
+        r_total += (long long)hs[p]->Mr * hs[p]->Mr;
+        tile_stages += (T * (T + 2) / 4 + 1) * (hs[p]->K / 128);
+    }
+    if (r_total > ws.gram_R_cap) {
+        dfree(ws.gram_R);
+        ws.gram_R = nullptr;
+        ws.gram_R_cap = 0;
+        CK(dalloc(&ws.gram_R, r_total));
+        ws.gram_R_cap = r_total;
+    }
+    ws.gram_R_used = r_total;
+    int sms = 0;
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+    ws.gram_unit_slices = gram_unit_slices(tile_stages, sms);
     if (e_total > ws.gram_E_cap) {
         dfree(ws.gram_E);
         ws.gram_E = nullptr;
@@ -572,23 +589,28 @@ int prepare_gram(fbn_handle* const* hs, int k, Workspace& ws, ProblemDev* P)
     }
     ws.h_maps.assign(k * mb, 0);
     std::vector<int4> units;
-    long long eo = 0;
+    long long eo = 0, ro = 0;
     ws.gram_layout.assign(1, (long long)(uintptr_t)ws.gram_E);
     for (int p = 0; p < k; ++p) {
         const fbn_handle* q = hs[p];
         P[p].onehot = ws.gram_E + eo;
         P[p].onehot_ld = q->K;
-        CK(encode_onehot_map(ws.h_maps.data() + p * mb, P[p].onehot, q->Mp, q->K));
+        P[p].off = q->d_off;
+        P[p].roff = q->d_off + q->n;
+        P[p].rgram = ws.gram_R + ro;
+        P[p].rgram_ld = q->Mr;
+        CK(encode_onehot_map(ws.h_maps.data() + p * mb, P[p].onehot, q->Mr, q->K));
         // 128-row tiles a against 256-row tiles b that reach the upper triangle
-        const int T = q->Mp / 128, T2 = (T + 1) / 2, C = gram_chunks(q->K);
+        const int T = q->Mr / 128, T2 = (T + 1) / 2, C = gram_chunks(q->K, ws.gram_unit_slices);
         for (int c = 0; c < C; ++c)
             for (int a = 0; a < T; ++a)
                 for (int b = a / 2; b < T2; ++b) units.push_back(make_int4(p, a, b, c));
         ws.gram_layout.push_back(eo);
         ws.gram_layout.push_back(q->M);
-        ws.gram_layout.push_back(q->Mp);
+        ws.gram_layout.push_back(q->Mr);
         ws.gram_layout.push_back(q->K);
-        eo += (long long)q->Mp * q->K;
+        eo += (long long)q->Mr * q->K;
+        ro += (long long)q->Mr * q->Mr;
     }
     if ((long long)units.size() > ws.gram_units_cap) {
         dfree(ws.gram_units);
@@ -616,9 +638,9 @@ int run_gram(fbn_handle* h, Workspace& ws, int k, int total_vtx, unsigned* d_sta
         ws.gram_zeroed = ws.gram_layout;
     }
     CK(launch_onehot(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx, ctr, st));
-    CK(cudaMemsetAsync(ws.gram_G, 0, ws.gram_G_cap * sizeof(int32_t), st));
+    CK(cudaMemsetAsync(ws.gram_R, 0, ws.gram_R_used * sizeof(int32_t), st));
     if (ev0) CK(cudaEventRecord(ev0, st));
-    CK(launch_gram(ws.gram_maps, ws.gram_units, ws.gram_n_units, ws.probs, sms, d_status, h->opt.wait_limit, st));
+    CK(launch_gram(ws.gram_maps, ws.gram_units, ws.gram_n_units, ws.gram_unit_slices, ws.probs, sms, d_status, h->opt.wait_limit, st));
     if (ev1) CK(cudaEventRecord(ev1, st));
     return FBN_OK;
 }
@@ -831,7 +853,8 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     if (gram) {
         rc = prepare_gram(hs, k, ws, P.data());
         if (rc) return rc;
-    } else if (popc0) {
+    }
+    if (popc0 || (gram && marg1)) {
         rc = prepare_pairs(hs, k, ws, P.data());
         if (rc) return rc;
     }
@@ -865,9 +888,12 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
             ws.up_last.swap(blob);
         }
     }
-    k_init_graph<<<total_vtx, 256, 0, st>>>(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx);
-    CK(cudaGetLastError());
-    long long launches = 1;
+    long long launches = 0;
+    if (!gram) {   // the complete graph (the Gram's decisions write every pair themselves)
+        k_init_graph<<<total_vtx, 256, 0, st>>>(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx);
+        CK(cudaGetLastError());
+        launches = 1;
+    }
     if (nbr1) {
         CK(launch_pack4(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx, st));
         launches += 1;
@@ -1110,14 +1136,20 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     if (shard) {
         // depth by depth below
     } else if (gram) {
-        enqueue_head();
         rc = run_gram(h, ws, k, total_vtx, &ws.d_ctr->status, ws.d_ctr, ws.kev[2 * FBN_MAX_DEPTHS],
                       ws.kev[2 * FBN_MAX_DEPTHS + 1]);
         if (rc) return rc;
-        CK(launch_pairs_decide(ws.edges, ws.edge_cap, ws.probs, ws.min_accept, ct, alpha, ws.d_ctr,
-                               h->opt.statistic, h->opt.df_mode, grid_aux, st));
-        enqueue_tail();
-        launches += 6;
+        PairsGramArgs pa;
+        pa.emit = marg1;
+        pa.total_pairs = edge_cap;
+        pa.crit = ct;
+        pa.alpha = alpha;
+        pa.ctr = ws.d_ctr;
+        pa.stat = h->opt.statistic;
+        pa.df_mode = h->opt.df_mode;
+        CK(launch_pairs_gram(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx, max_n, pa, dev_sms, st));
+        launch_depth_end(ws.d_ctr, ws.d_rec, max_depth, ws.hist, ws.cursor, st);
+        launches += 4;
         d_loop = 1;
     } else if (popc0) {
         enqueue_head();
@@ -1300,7 +1332,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         CK(cudaEventElapsedTime(&gms, ws.kev[2 * FBN_MAX_DEPTHS], ws.kev[2 * FBN_MAX_DEPTHS + 1]));
         stats.gram_ms = gms;
         for (int p = 0; p < k; ++p) {
-            stats.gram_rows += hs[p]->M;
+            stats.gram_rows += hs[p]->M - hs[p]->n;
             stats.gram_samples = std::max<int64_t>(stats.gram_samples, hs[p]->K);
         }
     }
@@ -1741,17 +1773,19 @@ int fbn_create(const uint8_t* data, int32_t n_vars, int64_t n_samples, const uin
         return bail(FBN_EDATA);
     }
     {
-        std::vector<int32_t> off(n_vars);
+        std::vector<int32_t> off(2 * (size_t)n_vars);
         int M = 0;
         for (int v = 0; v < n_vars; ++v) {
             off[v] = M;
+            off[n_vars + v] = M - v;
             M += arities[v];
         }
         h->M = M;
         h->Mp = gram_rows_padded(M);
+        h->Mr = gram_rows_padded(M - n_vars);
         h->K = gram_samples_padded(n_samples);
-        CKC(dalloc(&h->d_off, n_vars));
-        CKC(cudaMemcpy(h->d_off, off.data(), n_vars * sizeof(int32_t), cudaMemcpyHostToDevice));
+        CKC(dalloc(&h->d_off, off.size()));
+        CKC(cudaMemcpy(h->d_off, off.data(), off.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
     }
 #undef CKC
     *out = h;
@@ -1934,6 +1968,16 @@ int fbn_pairwise_counts(fbn_handle* h, int32_t* counts, int64_t cap)
     P.max_arity = h->max_arity;
     rc = prepare_gram(hs, 1, ws, &P);
     if (rc) return rc;
+    // straight into a device buffer of the caller's; else through the workspace
+    cudaPointerAttributes attr{};
+    const bool device_out = ((uintptr_t)counts & 3) == 0 &&
+                            cudaPointerGetAttributes(&attr, counts) == cudaSuccess &&
+                            attr.type == cudaMemoryTypeDevice && attr.device == h->device;
+    cudaGetLastError();
+    if (!device_out) {
+        rc = prepare_pairs(hs, 1, ws, &P);
+        if (rc) return rc;
+    }
     std::vector<int32_t> vp(h->n, 0), vf(1, 0);
     ws.up_last.clear();   // the skeleton's next call uploads its own descriptors again
     CK(cudaMemcpyAsync(ws.probs, &P, sizeof P, cudaMemcpyHostToDevice, h->stream));
@@ -1942,9 +1986,15 @@ int fbn_pairwise_counts(fbn_handle* h, int32_t* counts, int64_t cap)
     CK(cudaMemsetAsync(h->d_status, 0, sizeof(unsigned), h->stream));
     rc = run_gram(h, ws, 1, h->n, h->d_status);
     if (rc) return rc;
-    CK(launch_symmetrize(P.gram, h->Mp, h->M, h->stream));
-    CK(cudaMemcpy2DAsync(counts, (size_t)h->M * sizeof(int32_t), P.gram, (size_t)h->Mp * sizeof(int32_t),
-                         (size_t)h->M * sizeof(int32_t), (size_t)h->M, cudaMemcpyDefault, h->stream));
+    PairsGramArgs pa;
+    pa.emit = pa.sym = 1;
+    pa.out = device_out ? counts : ws.gram_G;
+    pa.ldo = h->M;
+    int sms = 0;
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+    CK(launch_pairs_gram(ws.probs, ws.vtx_prob, ws.vtx_first, h->n, h->n, pa, sms, h->stream));
+    if (!device_out)
+        CK(cudaMemcpyAsync(counts, ws.gram_G, (size_t)MM * sizeof(int32_t), cudaMemcpyDefault, h->stream));
     CK(cudaMemcpyAsync(h->h_status, h->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     return check_status(h, *h->h_status);

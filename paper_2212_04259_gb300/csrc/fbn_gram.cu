@@ -4,8 +4,11 @@
 // For every variable v and value x let e_{v,x} in {0,1}^N mark the samples
 // with V_v = x.  The depth-0 contingency table of the pair (i, j) is
 // N_ij(x, y) = <e_{i,x}, e_{j,y}>, so all n(n-1)/2 tables (Section IV-B: depth
-// zero tests every pair of the complete graph once) are blocks of the Gram
-// matrix E E^T of the one-hot matrix E [sum_v r_v][N].
+// zero tests every pair of the complete graph once) are blocks of a Gram matrix
+// E E^T of one-hot rows.  Only the rows of the values >= 1 are multiplied: the
+// diagonal holds the counts of single values, and every cell of value 0 follows
+// from them.  For arities 2 to 5 that halves the products (rows 3,500 -> 2,500
+// for 1,000 variables) and cuts the operand by 0.71.
 //
 // E is built in HBM as FP8 E4M3 (0 and 1 are exact).  The product runs on
 // tcgen05.mma.kind::f8f6f4 with FP32 accumulators in tensor memory; every
@@ -60,6 +63,7 @@ struct GramArgs {
     const int4* units;          // [n_units] (problem, ti, tj, chunk)
     const ProblemDev* probs;
     int n_units;
+    int unit_slices;            // stages per work unit, at most kSlicesPerChunk (exact accumulation)
     unsigned* status;
     unsigned limit;             // attempts of each role's bounded wait
 };
@@ -121,8 +125,8 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram(GramArgs g)
                     fenced = t.x;
                 }
                 const int slices = (int)(g.probs[t.x].onehot_ld / kKSlice);
-                const int kb0 = t.w * kSlicesPerChunk;
-                const int kb1 = min(kb0 + kSlicesPerChunk, slices);
+                const int kb0 = t.w * g.unit_slices;
+                const int kb1 = min(kb0 + g.unit_slices, slices);
                 for (int kb = kb0; kb < kb1; ++kb) {
                     if (!mbar_wait(smem_u32(&empty[stage]), phase ^ 1u, abort_flag, g.status, g.limit)) break;
                     const uint32_t fb = smem_u32(&full[stage]);
@@ -151,8 +155,8 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram(GramArgs g)
             for (int u = blockIdx.x; u < U && ok; u += gridDim.x) {
                 const int4 t = g.units[u];
                 const int slices = (int)(g.probs[t.x].onehot_ld / kKSlice);
-                const int kb0 = t.w * kSlicesPerChunk;
-                const int kb1 = min(kb0 + kSlicesPerChunk, slices);
+                const int kb0 = t.w * g.unit_slices;
+                const int kb1 = min(kb0 + g.unit_slices, slices);
                 if (!mbar_wait(smem_u32(&acc_empty[acc]), acc_phase ^ 1u, abort_flag, g.status, g.limit)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem + (uint32_t)(acc * kTileN);
@@ -191,8 +195,8 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram(GramArgs g)
         uint32_t acc_phase = 0;
         for (int u = blockIdx.x; u < U; u += gridDim.x) {
             const int4 t = g.units[u];
-            int32_t* G = g.probs[t.x].gram;
-            const long long ldg = g.probs[t.x].gram_ld;
+            int32_t* G = g.probs[t.x].rgram;
+            const long long ldg = g.probs[t.x].rgram_ld;
             if (!mbar_wait(smem_u32(&acc_full[acc]), acc_phase, abort_flag, g.status, g.limit)) break;
             tc_fence_after();
             const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * kTileN);
@@ -238,8 +242,8 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram(GramArgs g)
     }
 }
 
-// One-hot matrix E of every problem: row off_v + x holds 0x38 (E4M3 1.0)
-// where V_v = x, else 0; samples at or beyond N (the padding of the store)
+// One-hot matrix E of every problem: row roff_v + x - 1, x >= 1, holds 0x38
+// (E4M3 1.0) where V_v = x, else 0; samples at or beyond N (the padding of the store)
 // are 0 for every row.  One CTA per variable of the batch.
 // ctr: nullable; the depth whose tests start here.
 __global__ void k_onehot(const ProblemDev* __restrict__ probs, const int32_t* __restrict__ vtx_prob,
@@ -248,240 +252,261 @@ __global__ void k_onehot(const ProblemDev* __restrict__ probs, const int32_t* __
     const int g = blockIdx.x;
     if (g >= total_vertices) return;
     if (ctr && g == 0 && threadIdx.x == 0)
-        if (DepthRecord* r = depth_rec(ctr, ctr->d)) r->t_tests = gtime();
+        if (DepthRecord* r = depth_rec(ctr, ctr->d)) r->t_begin = r->t_tests = gtime();
     const int p = vtx_prob[g];
     const ProblemDev& P = probs[p];
     const int v = g - vtx_first[p];
     const int r = P.ar[v];
     const long long K = P.onehot_ld;
-    const int N = P.N;
     const uint4* row = reinterpret_cast<const uint4*>(P.data + (long long)v * P.ld);
-    uint8_t* E = P.onehot + (long long)P.off[v] * K;
+    uint8_t* E = P.onehot + (long long)P.roff[v] * K;
     const long long nvec = K / 16;
     for (long long q = threadIdx.x; q < nvec; q += blockDim.x) {
-        uint4 w = row[q];
-        const long long s0 = q * 16;
-        uint32_t keep[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {   // byte mask of samples below N
-            uint32_t m = 0;
-#pragma unroll
-            for (int b = 0; b < 4; ++b)
-                if (s0 + 4 * k + b < N) m |= 0xFFu << (8 * b);
-            keep[k] = m;
-        }
-        for (int x = 0; x < r; ++x) {
+        const uint4 w = row[q];   // padding past the samples is value 0: no row
+        for (int x = 1; x < r; ++x) {
             const uint32_t rep = 0x01010101u * (uint32_t)x;
             uint4 o;
-            o.x = __vcmpeq4(w.x, rep) & 0x38383838u & keep[0];
-            o.y = __vcmpeq4(w.y, rep) & 0x38383838u & keep[1];
-            o.z = __vcmpeq4(w.z, rep) & 0x38383838u & keep[2];
-            o.w = __vcmpeq4(w.w, rep) & 0x38383838u & keep[3];
-            reinterpret_cast<uint4*>(E + (long long)x * K)[q] = o;
+            o.x = __vcmpeq4(w.x, rep) & 0x38383838u;
+            o.y = __vcmpeq4(w.y, rep) & 0x38383838u;
+            o.z = __vcmpeq4(w.z, rep) & 0x38383838u;
+            o.w = __vcmpeq4(w.w, rep) & 0x38383838u;
+            reinterpret_cast<uint4*>(E + (long long)(x - 1) * K)[q] = o;
         }
     }
 }
 
-// Critical values of df <= kCritLocal, cached per CTA in shared memory (NaN
-// until first asked): the pairs of a depth share a handful of df, and the
-// global cache's acquire loads would serialise on those few slots.
-constexpr int kCritLocal = 64;
+// --------------------------------------------------------------------------
+// From the Gram over the values >= 1 to every pair's table and decision.
+//
+// A warp takes one variable i and 32 consecutive j, one pair per lane: the
+// lanes read neighbouring columns of i's Gram rows.  The cells of value 0
+// follow from the single counts (the Gram's diagonal): N(x, 0) = N_i(x) - sum_y
+// N(x, y), and so on.  At depth 0 the graph is complete, so the pairs need no
+// edge list: the kernel writes the adjacency, the empty separating sets and the
+// depth's counters itself, and (emit) the full tables that depth 1 reads its
+// margins from.
+struct PairGram {
+    const ProblemDev* P;
+    const int32_t* R;      // Gram rows of i, columns of j
+    const int32_t *si, *sj;   // single counts of value 1 of i and j (diagonal), strides ldr + 1
+    long long ldr;
+    int ri, rj, N;
 
-__device__ __forceinline__ double crit_local(double* local, const CritTableDev& crit, long long df, double alpha,
-                                             unsigned* status)
-{
-    if (df > kCritLocal) return crit_get(crit, df, alpha, status);
-    double c = *((volatile double*)&local[df]);
-    if (c != c) {   // not cached yet: every thread that misses stores the same value
-        c = crit_get(crit, df, alpha, status);
-        *((volatile double*)&local[df]) = c;
+    __device__ __forceinline__ PairGram(const ProblemDev& p, int i, int j) : P(&p)
+    {
+        ldr = p.rgram_ld;
+        const long long oi = p.roff[i], oj = p.roff[j];
+        R = p.rgram + oi * ldr + oj;
+        si = p.rgram + oi * (ldr + 1);
+        sj = p.rgram + oj * (ldr + 1);
+        ri = p.ar[i];
+        rj = p.ar[j];
+        N = p.N;
     }
-    return c;
+    __device__ __forceinline__ int both(int x, int y) const { return R[(x - 1) * ldr + y - 1]; }   // x, y >= 1
+    __device__ __forceinline__ int single_i(int x) const { return si[(x - 1) * (ldr + 1)]; }
+    __device__ __forceinline__ int single_j(int y) const { return sj[(y - 1) * (ldr + 1)]; }
+    // one cell on its own (the exact decision)
+    __device__ int cell(int x, int y) const
+    {
+        if (x > 0 && y > 0) return both(x, y);
+        if (x > 0) {
+            int s = single_i(x);
+            for (int b = 1; b < rj; ++b) s -= both(x, b);
+            return s;
+        }
+        if (y > 0) {
+            int s = single_j(y);
+            for (int a = 1; a < ri; ++a) s -= both(a, y);
+            return s;
+        }
+        int s = N;
+        for (int b = 1; b < rj; ++b) s -= single_j(b);
+        for (int a = 1; a < ri; ++a) {
+            s -= single_i(a);
+            for (int b = 1; b < rj; ++b) s += both(a, b);
+        }
+        return s;
+    }
+    __device__ int margin_i(int x) const
+    {
+        if (x > 0) return single_i(x);
+        int s = N;
+        for (int a = 1; a < ri; ++a) s -= single_i(a);
+        return s;
+    }
+    __device__ int margin_j(int y) const
+    {
+        if (y > 0) return single_j(y);
+        int s = N;
+        for (int b = 1; b < rj; ++b) s -= single_j(b);
+        return s;
+    }
+};
+
+// The exact FP64 statistic of one pair by the whole warp (the pair of the lane
+// whose FP32 band straddled crit).
+__device__ __noinline__ double pair_stat_exact(const ProblemDev& P, int i, int j, int stat)
+{
+    const PairGram g(P, i, j);
+    double st = 0.0;
+    for (int c = threadIdx.x & 31; c < g.ri * g.rj; c += 32) {
+        const int x = c / g.rj, y = c - x * g.rj;
+        const int n = g.cell(x, y);
+        const long long nx = g.margin_i(x), ny = g.margin_j(y);
+        const long long p = (long long)n * g.N, q = nx * ny;
+        if (stat == kStatX2) {
+            if (q > 0) {
+                const double dd = (double)(p - q);
+                st += dd * dd / ((double)g.N * (double)nx * (double)ny);
+            }
+        } else if (n > 0) {
+            st += 2.0 * (double)n * log1p((double)(p - q) / (double)q);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) st += __shfl_xor_sync(0xffffffffu, st, o);
+    return st;
 }
 
-// Decision of one depth-0 pair from its block of the Gram (row sums, column
-// sums and the total from the block itself).  R bounds the arities so that
-// the sums live in registers.  stat: G^2 or Pearson X^2; df_mode: declared
-// arities or the observed table (no degree of freedom left: accept).
-template <int R>
-__device__ __forceinline__ void pair_decide_r(const int32_t* T, long long Mp, int rx, int ry, long long e,
-                                              unsigned long long* __restrict__ min_accept, const CritTableDev& crit,
-                                              double alpha, DepthCounters* ctr, int stat, int df_mode, double* local)
+// DECIDE: the depth-0 decisions into adj, sep_len, sep_off and the counters.
+// emit: full tables into G with row stride ldg (0: the problem's gram), the
+// transposed blocks too when sym.
+template <bool DECIDE>
+__global__ void __launch_bounds__(256) k_pairs_gram(const ProblemDev* __restrict__ probs,
+                                                    const int32_t* __restrict__ vtx_prob,
+                                                    const int32_t* __restrict__ vtx_first, int total_vertices,
+                                                    int blocks_n, int emit, int sym, int32_t* G_out, long long ldg,
+                                                    long long total_pairs, CritTableDev crit, double alpha,
+                                                    DepthCounters* ctr, int stat, int df_mode)
 {
-    int rs[R], cs[R];
-    int tot = 0;
-#pragma unroll
-    for (int q = 0; q < R; ++q) rs[q] = cs[q] = 0;
-#pragma unroll
-    for (int x = 0; x < R; ++x)
-#pragma unroll
-        for (int y = 0; y < R; ++y)
-            if (x < rx && y < ry) {
-                const int nxy = T[(long long)x * Mp + y];
-                rs[x] += nxy;
-                cs[y] += nxy;
-                tot += nxy;
-            }
-    long long df = (long long)(rx - 1) * (ry - 1);
-    if (df_mode) {
-        int ax = 0, ay = 0;
-#pragma unroll
-        for (int q = 0; q < R; ++q) {
-            ax += rs[q] > 0;
-            ay += cs[q] > 0;
+    const int lane = threadIdx.x & 31;
+    if (DECIDE && !ctr->active) return;
+    const long long tasks = (long long)total_vertices * blocks_n;
+    const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
+    unsigned long long removed = 0, samples = 0, tests = 0;
+    for (long long t = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < tasks; t += warps) {
+        const int g = (int)(t / blocks_n), j0 = (int)(t - (long long)g * blocks_n) * 32;
+        const int p = vtx_prob[g];
+        const ProblemDev& P = probs[p];
+        const int i = g - vtx_first[p], n = P.n;
+        if (j0 >= n || j0 + 31 < i) continue;
+        const int j = j0 + lane;
+        int32_t* G = emit ? (G_out ? G_out : P.gram) : nullptr;
+        const long long ld = G_out ? ldg : P.gram_ld;
+        const int oi = P.off[i];
+        if (j == i) {   // the diagonal block
+            const PairGram d(P, i, i);
+            if (G)
+                for (int x = 0; x < d.ri; ++x) {
+                    if (sym)
+                        for (int y = 0; y < d.ri; ++y) G[(oi + x) * ld + oi + y] = 0;
+                    G[(oi + x) * (ld + 1)] = d.margin_i(x);
+                }
+            if (DECIDE) P.adj[(long long)i * n + i] = 0;
         }
-        df = ax > 0 && ay > 0 ? (long long)(ax - 1) * (ay - 1) : 0;
-    }
-    if (df <= 0) {   // p = 1 > alpha
-        min_accept[e] = 0;
-        return;
-    }
-    // terms in FP32 (G^2: within 3.2e-7 of their magnitude; X^2: within 6e-7),
-    // summed in FP32 by this thread (at most R*R additions, each within 6e-8 of
-    // the running sum of magnitudes); exact FP64 only when crit lies inside the
-    // error band
-    const double c = crit_local(local, crit, df, alpha, &ctr->status);
-    float acc = 0.0f, mag = 0.0f;
-#pragma unroll
-    for (int x = 0; x < R; ++x)
-#pragma unroll
-        for (int y = 0; y < R; ++y) {
-            if (x >= rx || y >= ry) continue;
-            const int n = T[(long long)x * Mp + y];
-            if (stat == kStatX2) {
-                if (rs[x] == 0 || cs[y] == 0) continue;
-                const float fd = (float)((long long)n * tot - (long long)rs[x] * cs[y]);
-                const float t = fd * fd / ((float)tot * (float)rs[x] * (float)cs[y]);
-                acc += t;
-                mag += t;
-            } else {
-                if (n == 0) continue;
-                const long long a = (long long)n * tot, b = (long long)rs[x] * cs[y];
-                const float fb = (float)b;
-                const float delta = (float)(a - b) / fb;
-                const float L = fabsf(delta) < 0.5f ? log1pf(delta) : logf((float)a / fb);
-                const float t = (float)n * L;
-                acc += t;
-                mag += fabsf(t);
+        const bool pair = j > i && j < n;
+        int dec = 0;
+        long long df = 0;
+        if (pair) {
+            const PairGram q(P, i, j);
+            const int ri = q.ri, rj = q.rj, N = q.N, oj = P.off[j];
+            const bool narrow = N < 65536;
+            float acc = 0.0f, mag = 0.0f;
+            int ni0 = N, nj0 = N, ax = 0, ay = 0;
+            for (int y = 1; y < rj; ++y) {
+                const int ny = q.single_j(y);
+                nj0 -= ny;
+                ay += ny > 0;
             }
-        }
-    const double scale = stat == kStatX2 ? 1.0 : 2.0;
-    const double st = scale * (double)acc;
-    const double rel = 2.0 * ((stat == kStatX2 ? 6e-7 : 3.2e-7) + (double)(rx * ry) * 6e-8);
-    const double err = scale * rel * (double)mag * 1.0001 + 1e-9;
-    bool accept;
-    if (st + err < c) {
-        accept = true;
-    } else if (st - err >= c) {
-        accept = false;
-    } else {
-        double ex = 0.0;
-#pragma unroll
-        for (int x = 0; x < R; ++x)
-#pragma unroll
-            for (int y = 0; y < R; ++y) {
-                if (x >= rx || y >= ry) continue;
-                const int n = T[(long long)x * Mp + y];
-                if (stat == kStatX2) {
-                    if (rs[x] == 0 || cs[y] == 0) continue;
-                    const double dd = (double)((long long)n * tot - (long long)rs[x] * cs[y]);
-                    ex += dd * dd / ((double)tot * (double)rs[x] * (double)cs[y]);
+            ay += nj0 > 0;
+            auto put = [&](int x, int y, int v) {
+                if (!G) return;
+                G[(oi + x) * ld + oj + y] = v;
+                if (sym) G[(oj + y) * ld + oi + x] = v;
+            };
+            auto term = [&](int v, int nx, int ny) {
+                if (DECIDE && nx > 0 && ny > 0) marg_term(v, N, nx, ny, narrow, stat, acc, mag);
+            };
+            int n00 = nj0;
+            for (int x = 1; x < ri; ++x) {
+                const int nx = q.single_i(x);
+                ni0 -= nx;
+                ax += nx > 0;
+                int rest = nx;
+                for (int y = 1; y < rj; ++y) {
+                    const int v = q.both(x, y);
+                    rest -= v;
+                    put(x, y, v);
+                    term(v, nx, q.single_j(y));
+                }
+                n00 -= rest;
+                put(x, 0, rest);
+                term(rest, nx, nj0);
+            }
+            ax += ni0 > 0;
+            for (int y = 1; y < rj; ++y) {
+                int v = q.single_j(y);
+                for (int x = 1; x < ri; ++x) v -= q.both(x, y);
+                put(0, y, v);
+                term(v, ni0, q.single_j(y));
+            }
+            put(0, 0, n00);
+            term(n00, ni0, nj0);
+            if (DECIDE) {
+                df = df_mode ? (long long)(ax - 1) * (ay - 1) : (long long)(ri - 1) * (rj - 1);
+                if (df <= 0) {
+                    dec = 1;   // p = 1 > alpha
                 } else {
-                    if (n == 0) continue;
-                    const long long a = (long long)n * tot, b = (long long)rs[x] * cs[y];
-                    ex += (double)n * log1p((double)(a - b) / (double)b);
+                    float2 f = make_float2(0.0f, 0.0f);
+                    if (df < crit.dense_n) f = crit.dense_f[df];
+                    if (!(f.y > 0.0f)) {
+                        const double c = crit_get(crit, df, alpha, &ctr->status);
+                        f = make_float2(__double2float_rd(c), __double2float_ru(c));
+                    }
+                    dec = decide_from_sums(acc, mag, (float)(ri * rj), 0.0f, stat, f.x, f.y, kMargTermRel);
                 }
             }
-        accept = scale * ex < c;
-    }
-    if (accept) min_accept[e] = 0;
-}
-
-// Arities above 8: the sums are recomputed from the block (no local arrays),
-// the statistic in FP64.
-__device__ __forceinline__ void pair_decide_wide(const int32_t* T, long long Mp, int rx, int ry, long long e,
-                                                 unsigned long long* __restrict__ min_accept, const CritTableDev& crit,
-                                                 double alpha, DepthCounters* ctr, int stat, int df_mode, double* local)
-{
-    long long tot = 0;
-    for (int x = 0; x < rx; ++x)
-        for (int y = 0; y < ry; ++y) tot += T[(long long)x * Mp + y];
-    long long df = (long long)(rx - 1) * (ry - 1);
-    if (df_mode) {
-        int ax = 0, ay = 0;
-        for (int x = 0; x < rx; ++x) {
-            long long s = 0;
-            for (int y = 0; y < ry; ++y) s += T[(long long)x * Mp + y];
-            ax += s > 0;
         }
-        for (int y = 0; y < ry; ++y) {
-            long long s = 0;
-            for (int x = 0; x < rx; ++x) s += T[(long long)x * Mp + y];
-            ay += s > 0;
-        }
-        df = ax > 0 && ay > 0 ? (long long)(ax - 1) * (ay - 1) : 0;
-    }
-    if (df <= 0) {
-        min_accept[e] = 0;
-        return;
-    }
-    const double c = crit_local(local, crit, df, alpha, &ctr->status);
-    double ex = 0.0;
-    for (int x = 0; x < rx; ++x) {
-        long long rsx = 0;
-        for (int y = 0; y < ry; ++y) rsx += T[(long long)x * Mp + y];
-        for (int y = 0; y < ry; ++y) {
-            const int n = T[(long long)x * Mp + y];
-            long long csy = 0;
-            for (int xx = 0; xx < rx; ++xx) csy += T[(long long)xx * Mp + y];
-            if (stat == kStatX2) {
-                if (rsx == 0 || csy == 0) continue;
-                const double dd = (double)(n * tot - rsx * csy);
-                ex += dd * dd / ((double)tot * (double)rsx * (double)csy);
-            } else {
-                if (n == 0) continue;
-                const long long a = (long long)n * tot, b = rsx * csy;
-                ex += (double)n * log1p((double)(a - b) / (double)b);
+        if constexpr (DECIDE) {
+            unsigned open = __ballot_sync(0xffffffffu, dec < 0);
+            while (open) {   // the band straddles crit: exactly, one such pair at a time
+                const int l = __ffs(open) - 1;
+                open &= open - 1;
+                const double st = pair_stat_exact(P, i, j0 + l, stat);
+                if (lane == l) dec = st < crit_get(crit, df, alpha, &ctr->status);
+                __syncwarp();
+            }
+            if (pair) {
+                P.adj[(long long)i * n + j] = (uint8_t)(dec ? 0 : 1);
+                P.adj[(long long)j * n + i] = (uint8_t)(dec ? 0 : 1);
+                P.sep_len[(long long)i * n + j] = dec ? 0 : -1;
+                P.sep_off[(long long)i * n + j] = 0;
+                removed += dec != 0;
+                tests += 1;
+                samples += (unsigned long long)P.N;
             }
         }
     }
-    if ((stat == kStatX2 ? 1.0 : 2.0) * ex < c) min_accept[e] = 0;
-}
-
-__device__ __forceinline__ void pair_decide(const EdgeWork* __restrict__ edges, long long e,
-                                            const ProblemDev* __restrict__ probs,
-                                            unsigned long long* __restrict__ min_accept, const CritTableDev& crit,
-                                            double alpha, DepthCounters* ctr, int stat, int df_mode, double* local)
-{
-    const EdgeWork w = edges[e];
-    const ProblemDev& P = probs[w.prob];
-    const int rx = P.ar[w.i], ry = P.ar[w.j];
-    const long long Mp = P.gram_ld;
-    const int32_t* T = P.gram + (long long)P.off[w.i] * Mp + P.off[w.j];
-    if (rx <= 4 && ry <= 4) pair_decide_r<4>(T, Mp, rx, ry, e, min_accept, crit, alpha, ctr, stat, df_mode, local);
-    else if (rx <= 8 && ry <= 8) pair_decide_r<8>(T, Mp, rx, ry, e, min_accept, crit, alpha, ctr, stat, df_mode, local);
-    else pair_decide_wide(T, Mp, rx, ry, e, min_accept, crit, alpha, ctr, stat, df_mode, local);
-}
-
-// Depth-0 decisions from the Gram: one thread per edge (i<j) of both classes
-// of the edge list (class 0 at the front of the array, class 1 at the back).
-__global__ void k_pairs_decide(const EdgeWork* __restrict__ edges, long long edge_cap,
-                               const ProblemDev* __restrict__ probs, unsigned long long* __restrict__ min_accept,
-                               CritTableDev crit, double alpha, DepthCounters* ctr, int stat, int df_mode)
-{
-    __shared__ double local[kCritLocal + 1];
-    if (!ctr->active) return;
-    for (int k = threadIdx.x; k <= kCritLocal; k += blockDim.x) local[k] = __longlong_as_double(0x7ff8000000000000LL);
-    __syncthreads();
-    const long long n0 = (long long)ctr->n_edges[0], n1 = (long long)ctr->n_edges[1];
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n0 + n1;
-         k += (long long)gridDim.x * blockDim.x)
-        pair_decide(edges, k < n0 ? k : edge_cap - n1 + (k - n0), probs, min_accept, crit, alpha, ctr, stat,
-                    df_mode, local);
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&ctr->tests, (unsigned long long)(n0 + n1));   // one test per pair
-    __syncthreads();
-    if (threadIdx.x == 0)
-        if (DepthRecord* r = depth_rec(ctr, ctr->d)) atomicMax(&r->t_tests_end, gtime());
+    if constexpr (DECIDE) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            removed += __shfl_xor_sync(0xffffffffu, removed, o);
+            tests += __shfl_xor_sync(0xffffffffu, tests, o);
+            samples += __shfl_xor_sync(0xffffffffu, samples, o);
+        }
+        if (lane == 0 && tests) {   // one test per pair
+            atomicAdd(&ctr->removed, removed);
+            atomicAdd(&ctr->tests, tests);
+            atomicAdd(&ctr->tests_oracle, tests);
+            atomicAdd(&ctr->test_samples, samples);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            if (blockIdx.x == 0) ctr->n_edges[0] = (unsigned long long)total_pairs;   // the depth's edges: every pair
+            if (DepthRecord* r = depth_rec(ctr, ctr->d)) atomicMax(&r->t_tests_end, gtime());
+        }
+    }
 }
 
 // Zero the pad rows M..Mp of every problem's one-hot matrix (one CTA per
@@ -489,19 +514,10 @@ __global__ void k_pairs_decide(const EdgeWork* __restrict__ edges, long long edg
 __global__ void k_zero_pad(const ProblemDev* __restrict__ probs)
 {
     const ProblemDev& P = probs[blockIdx.x];
-    const long long M = (long long)P.off[P.n - 1] + P.ar[P.n - 1];
+    const long long M = (long long)P.roff[P.n - 1] + P.ar[P.n - 1] - 1;
     uint4* E = reinterpret_cast<uint4*>(P.onehot + M * P.onehot_ld);
-    const long long n = (P.gram_ld - M) * P.onehot_ld / 16;
+    const long long n = (P.rgram_ld - M) * P.onehot_ld / 16;
     for (long long q = threadIdx.x; q < n; q += blockDim.x) E[q] = make_uint4(0, 0, 0, 0);
-}
-
-// Mirror the upper block triangle into the lower one (row < col -> col, row).
-__global__ void k_symmetrize(int32_t* G, int Mp, int M)
-{
-    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (long long)M * M) return;
-    const int r = (int)(k / M), c = (int)(k - (long long)r * M);
-    if (r > c) G[(long long)r * Mp + c] = G[(long long)c * Mp + r];
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
@@ -555,19 +571,31 @@ cudaError_t encode_onehot_map(void* map, const uint8_t* E, int Mp, long long K)
 
 size_t tensor_map_bytes() { return sizeof(CUtensorMap); }
 
-int gram_chunks(long long K) { return (int)((K / kKSlice + kSlicesPerChunk - 1) / kSlicesPerChunk); }
+// Stages (128 samples each) per work unit: the whole exact accumulation, or
+// less while the units leave SMs idle.  tiles: output tiles of every problem
+// times its share of the samples' stages, i.e. sum over problems of tiles x
+// stages.  A unit keeps at least 8 stages: its epilogue adds a 128 x 256 tile.
+int gram_unit_slices(long long tile_stages, int num_sms)
+{
+    int s = kSlicesPerChunk;
+    while (s > 8 && tile_stages / s < 2LL * num_sms) s /= 2;
+    return s;
+}
+
+int gram_chunks(long long K, int unit_slices) { return (int)((K / kKSlice + unit_slices - 1) / unit_slices); }
 
 // Gram of every problem's one-hot matrix over the given work units; each
 // problem's Gram must be zero.  maps: device array of tensor maps (one per
 // problem, 64-byte aligned).
-cudaError_t launch_gram(const void* maps, const int4* units, int n_units, const ProblemDev* probs, int num_sms,
-                        unsigned* status, int wait_limit, cudaStream_t st)
+cudaError_t launch_gram(const void* maps, const int4* units, int n_units, int unit_slices, const ProblemDev* probs,
+                        int num_sms, unsigned* status, int wait_limit, cudaStream_t st)
 {
     GramArgs g;
     g.maps = reinterpret_cast<const CUtensorMap*>(maps);
     g.units = units;
     g.probs = probs;
     g.n_units = n_units;
+    g.unit_slices = unit_slices;
     g.status = status;
     g.limit = wait_limit < 0 ? 0u : wait_limit == 0 ? kSpinLimit : (unsigned)wait_limit;
     cudaError_t e = cudaFuncSetAttribute(k_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramSmem);
@@ -578,18 +606,15 @@ cudaError_t launch_gram(const void* maps, const int4* units, int n_units, const 
     return cudaGetLastError();
 }
 
-cudaError_t launch_pairs_decide(const EdgeWork* edges, long long edge_cap, const ProblemDev* probs,
-                                unsigned long long* min_accept, const CritTableDev& crit, double alpha,
-                                DepthCounters* ctr, int stat, int df_mode, int grid, cudaStream_t st)
+cudaError_t launch_pairs_gram(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first,
+                              int total_vertices, int max_n, const PairsGramArgs& a, int num_sms, cudaStream_t st)
 {
-    k_pairs_decide<<<grid, 256, 0, st>>>(edges, edge_cap, probs, min_accept, crit, alpha, ctr, stat, df_mode);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_symmetrize(int32_t* G, int Mp, int M, cudaStream_t st)
-{
-    const long long n = (long long)M * M;
-    k_symmetrize<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(G, Mp, M);
+    const int blocks_n = (max_n + 31) / 32;
+    const long long warps = (long long)total_vertices * blocks_n;
+    const int grid = (int)std::max<long long>(1, std::min<long long>((warps + 7) / 8, (long long)num_sms * 8));
+    auto kern = a.ctr ? k_pairs_gram<true> : k_pairs_gram<false>;
+    kern<<<grid, 256, 0, st>>>(probs, vtx_prob, vtx_first, total_vertices, blocks_n, a.emit, a.sym, a.out, a.ldo,
+                               a.total_pairs, a.crit, a.alpha, a.ctr, a.stat, a.df_mode);
     return cudaGetLastError();
 }
 

@@ -43,12 +43,17 @@ struct ProblemDev {
     int32_t N;
     int32_t max_arity;
     int32_t nplanes;       // one-hot planes per variable: max_arity - 1, or 0 without planes
-    // one-hot Gram of depth 0 (unused when depth 0 runs on the histogram path)
-    const int32_t* off;    // [n] first one-hot row of each variable
-    uint8_t* onehot;       // [gram_ld][onehot_ld] E4M3 one-hot rows
-    int32_t* gram;         // [gram_ld][gram_ld] INT32 Gram (upper tile triangle)
+    // the pair tables of depth 0: table (i, j), i < j, at rows off[i].. and
+    // columns off[j].. of gram; on the diagonal, the counts of single values
+    const int32_t* off;    // [n] sum of the arities before each variable
+    int32_t* gram;         // [gram_ld][gram_ld]
+    int64_t gram_ld;
+    // one-hot Gram over the values >= 1 (the cells of value 0 follow from it)
+    const int32_t* roff;   // [n] first one-hot row of each variable: off[v] - v
+    uint8_t* onehot;       // [rgram_ld][onehot_ld] E4M3 one-hot rows
+    int32_t* rgram;        // [rgram_ld][rgram_ld] INT32 Gram (upper tile triangle)
     int64_t onehot_ld;     // padded samples (multiple of 128)
-    int64_t gram_ld;       // padded rows Mp (multiple of 128)
+    int64_t rgram_ld;      // padded rows (multiple of 128)
     int32_t* eid;          // [n][n] edge of the current depth at each snapshot slot nbr[v][t]
     int32_t* npos;         // [n][n] npos[v][u] = index of u in nbr[v] (u adjacent to v in the snapshot)
     uint8_t* pk;           // [n][pk_ld] samples 4 bits each (depth-1 tensor-core path; arities <= 8)

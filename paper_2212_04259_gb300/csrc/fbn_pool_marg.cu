@@ -142,53 +142,6 @@ __device__ __forceinline__ int2 count_shape(int A, int B, int C, const uint2* x,
     }
 }
 
-// One FP32 term of the bounded decision from a cell and its margins.  Below
-// 65,536 samples both products of the ratio fit 32 bits.  G^2: n ln(N / E) with
-// the exact difference D = n N_z - N_xz N_yz; ln as 2 atanh(D / (sum of the two
-// products)) by its series while the ratio is within [1/2, 2] (|s| <= 1/3: the
-// terms left out are below 2e-9 of the sum), else as lg2 of the ratio (error
-// 2^-22 of a result of at least 1).  Conversions, sums and the approximate
-// quotient (2 ulp) leave each term within 8e-7 of itself.  X^2: D^2 / (N_z N_xz
-// N_yz), within the same bound.
-__device__ __forceinline__ void marg_term(int n, int nz, int nx, int ny, bool narrow, int stat, float& acc, float& mag)
-{
-    float fd, fa, fb;
-    if (narrow) {
-        const unsigned p = (unsigned)n * (unsigned)nz, q = (unsigned)nx * (unsigned)ny;
-        fd = p >= q ? (float)(p - q) : -(float)(q - p);
-        fa = (float)p;
-        fb = (float)q;
-    } else {
-        const long long p = (long long)n * nz, q = (long long)nx * ny;
-        fd = (float)(p - q);
-        fa = (float)p;
-        fb = (float)q;
-    }
-    if (stat == kStatX2) {
-        if (fb > 0.0f) {
-            const float t = __fdividef(fd * fd, fb) / (float)nz;
-            acc += t;
-            mag += t;
-        }
-        return;
-    }
-    const float s = __fdividef(fd, fa + fb);
-    const float s2 = s * s;
-    float p = 1.0f / 15.0f;
-    p = fmaf(p, s2, 1.0f / 13.0f);
-    p = fmaf(p, s2, 1.0f / 11.0f);
-    p = fmaf(p, s2, 1.0f / 9.0f);
-    p = fmaf(p, s2, 1.0f / 7.0f);
-    p = fmaf(p, s2, 1.0f / 5.0f);
-    p = fmaf(p, s2, 1.0f / 3.0f);
-    const float near = 2.0f * fmaf(s * s2, p, s);
-    const float far = __log2f(__fdividef(fa, fb)) * 0.693147181f;
-    const float t = n > 0 ? (float)n * (fabsf(s) <= 0.33333333f ? near : far) : 0.0f;
-    acc += t;
-    mag += fabsf(t);
-}
-constexpr float kMargTermRel = 8.0e-7f;
-
 // What a warp knows of its edge and of one conditioning variable.
 struct MargEdge {
     const uint2 *xp, *yp;   // planes of x and y
