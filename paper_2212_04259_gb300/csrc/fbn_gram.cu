@@ -369,6 +369,8 @@ __device__ __noinline__ double pair_stat_exact(const ProblemDev& P, int i, int j
     return st;
 }
 
+constexpr int kPairArity = 5;   // blocks of at most this many values a side are held in registers
+
 // DECIDE: the depth-0 decisions into adj, sep_len, sep_off and the counters.
 // emit: full tables into G with row stride ldg (0: the problem's gram), the
 // transposed blocks too when sym.
@@ -380,6 +382,7 @@ __global__ void __launch_bounds__(256) k_pairs_gram(const ProblemDev* __restrict
                                                     long long total_pairs, CritTableDev crit, double alpha,
                                                     DepthCounters* ctr, int stat, int df_mode)
 {
+    __shared__ int s_cell[8][kPairArity * kPairArity][32], s_nj[8][kPairArity][32];   // 8 warps: a column per lane
     const int lane = threadIdx.x & 31;
     if (DECIDE && !ctr->active) return;
     const long long tasks = (long long)total_vertices * blocks_n;
@@ -414,12 +417,6 @@ __global__ void __launch_bounds__(256) k_pairs_gram(const ProblemDev* __restrict
             const bool narrow = N < 65536;
             float acc = 0.0f, mag = 0.0f;
             int ni0 = N, nj0 = N, ax = 0, ay = 0;
-            for (int y = 1; y < rj; ++y) {
-                const int ny = q.single_j(y);
-                nj0 -= ny;
-                ay += ny > 0;
-            }
-            ay += nj0 > 0;
             auto put = [&](int x, int y, int v) {
                 if (!G) return;
                 G[(oi + x) * ld + oj + y] = v;
@@ -428,31 +425,90 @@ __global__ void __launch_bounds__(256) k_pairs_gram(const ProblemDev* __restrict
             auto term = [&](int v, int nx, int ny) {
                 if (DECIDE && nx > 0 && ny > 0) marg_term(v, N, nx, ny, narrow, stat, acc, mag);
             };
-            int n00 = nj0;
-            for (int x = 1; x < ri; ++x) {
-                const int nx = q.single_i(x);
-                ni0 -= nx;
-                ax += nx > 0;
-                int rest = nx;
-                for (int y = 1; y < rj; ++y) {
-                    const int v = q.both(x, y);
-                    rest -= v;
-                    put(x, y, v);
-                    term(v, nx, q.single_j(y));
+            if (P.max_arity <= kPairArity) {
+                // the block's loads in flight together, its cells through this
+                // lane's column of shared memory, so that the terms are one
+                // small loop (25 inlined terms spilled)
+                int (*cv)[32] = s_cell[threadIdx.x >> 5];
+                int (*cj)[32] = s_nj[threadIdx.x >> 5];
+                int v[kPairArity - 1][kPairArity - 1], nj[kPairArity - 1], ni[kPairArity - 1];
+#pragma unroll
+                for (int b = 0; b < kPairArity - 1; ++b) nj[b] = b + 1 < rj ? q.single_j(b + 1) : 0;
+#pragma unroll
+                for (int a = 0; a < kPairArity - 1; ++a) {
+                    ni[a] = a + 1 < ri ? q.single_i(a + 1) : 0;
+#pragma unroll
+                    for (int b = 0; b < kPairArity - 1; ++b) v[a][b] = a + 1 < ri && b + 1 < rj ? q.both(a + 1, b + 1) : 0;
                 }
-                n00 -= rest;
-                put(x, 0, rest);
-                term(rest, nx, nj0);
+#pragma unroll
+                for (int b = 0; b < kPairArity - 1; ++b) {
+                    nj0 -= nj[b];
+                    ay += nj[b] > 0;
+                    cj[b + 1][lane] = nj[b];
+                }
+                cj[0][lane] = nj0;
+#pragma unroll
+                for (int a = 0; a < kPairArity - 1; ++a) {
+                    ni0 -= ni[a];
+                    ax += ni[a] > 0;
+                }
+                int n00 = nj0;
+#pragma unroll
+                for (int a = 0; a < kPairArity - 1; ++a) {
+                    int rest = ni[a];
+#pragma unroll
+                    for (int b = 0; b < kPairArity - 1; ++b) {
+                        rest -= v[a][b];
+                        nj[b] -= v[a][b];
+                        cv[(a + 1) * kPairArity + b + 1][lane] = v[a][b];
+                    }
+                    n00 -= rest;
+                    cv[(a + 1) * kPairArity][lane] = rest;
+                }
+#pragma unroll
+                for (int b = 0; b < kPairArity - 1; ++b) cv[b + 1][lane] = nj[b];
+                cv[0][lane] = n00;
+                for (int x = 0; x < ri; ++x) {
+                    const int nx = x ? q.single_i(x) : ni0;
+                    for (int y = 0; y < rj; ++y) {
+                        const int c = cv[x * kPairArity + y][lane];
+                        put(x, y, c);
+                        term(c, nx, cj[y][lane]);
+                    }
+                }
+            } else {   // any arity: the block read twice
+                for (int y = 1; y < rj; ++y) {
+                    const int ny = q.single_j(y);
+                    nj0 -= ny;
+                    ay += ny > 0;
+                }
+                int n00 = nj0;
+                for (int x = 1; x < ri; ++x) {
+                    const int nx = q.single_i(x);
+                    ni0 -= nx;
+                    ax += nx > 0;
+                    int rest = nx;
+                    for (int y = 1; y < rj; ++y) {
+                        const int v = q.both(x, y);
+                        rest -= v;
+                        put(x, y, v);
+                        term(v, nx, q.single_j(y));
+                    }
+                    n00 -= rest;
+                    put(x, 0, rest);
+                    term(rest, nx, nj0);
+                }
+                for (int y = 1; y < rj; ++y) {
+                    int v = q.single_j(y);
+                    for (int x = 1; x < ri; ++x) v -= q.both(x, y);
+                    put(0, y, v);
+                    term(v, ni0, q.single_j(y));
+                }
+                put(0, 0, n00);
+                term(n00, ni0, nj0);
             }
             ax += ni0 > 0;
-            for (int y = 1; y < rj; ++y) {
-                int v = q.single_j(y);
-                for (int x = 1; x < ri; ++x) v -= q.both(x, y);
-                put(0, y, v);
-                term(v, ni0, q.single_j(y));
-            }
-            put(0, 0, n00);
-            term(n00, ni0, nj0);
+            ay += nj0 > 0;
             if (DECIDE) {
                 df = df_mode ? (long long)(ax - 1) * (ay - 1) : (long long)(ri - 1) * (rj - 1);
                 if (df <= 0) {
