@@ -2,6 +2,7 @@
 // skeleton library.  The depth loop of Algorithm 1 runs here; every step of a
 // depth (snapshot, edge list, CI tests, removal) is a kernel in fbn_kernels.cu.
 #include <algorithm>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
@@ -29,7 +30,8 @@ thread_local std::string g_create_error;
 
 constexpr size_t kSmemBytes = 100 * 1024;     // dynamic shared memory of a CTA test group: 2 CTAs / SM with the ~9 KB static
 constexpr long long kSplitStride = 4096;        // cells of a split test's global table at most
-constexpr size_t kWarpSmemBytes = 56 * 1024;  // dynamic shared memory of a CTA of 8 warp groups (3 CTAs / SM)
+constexpr size_t kWarpSmemBytes = 64 * 1024;  // dynamic shared memory of a CTA of the small-table pool (2 CTAs / SM)
+constexpr size_t kBigSmemBytes = 200 * 1024;  // the same of the big-table pool (one CTA of 1,024 threads / SM)
 constexpr int kCritCap = 8192;                // critical-value cache slots (power of two)
 constexpr int kCritDense = 8192;              // critical values kept in a dense table: df < kCritDense
 
@@ -85,6 +87,13 @@ __global__ void k_ingest(const uint8_t* __restrict__ data, int64_t ld, int64_t N
     }
 }
 
+// n ln n for n < count, in units of 2^-kLutBits (see grp_g2_lut).
+__global__ void k_lut(long long* lut, int count)
+{
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n < count) lut[n] = n < 2 ? 0 : __double2ll_rn((double)n * log((double)n) * 68719476736.0);
+}
+
 __global__ void k_init_graph(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first,
                              int total_vertices)
 {
@@ -125,6 +134,9 @@ struct Workspace {
     double* crit_vals = nullptr;
     double* crit_dense = nullptr;
     float2* crit_dense_f = nullptr;
+    long long* crit_dense_q = nullptr;
+    long long* lut = nullptr;                       // n ln n up to the largest N seen (kLutMaxN at most)
+    long long lut_n = 0;
     double crit_alpha = -1.0;
     cudaEvent_t kev[2 * FBN_MAX_DEPTHS + 2] = {};   // the Gram's window at the end
     DepthRecord* d_rec = nullptr;
@@ -189,7 +201,7 @@ struct Workspace {
         if (h_ctr) cudaFreeHost(h_ctr);
         dfree(binom); dfree(vtx_prob); dfree(vtx_first); dfree(probs);
         dfree(sep_pool); dfree(gscratch); dfree(crit_keys); dfree(crit_vals); dfree(crit_dense);
-        dfree(crit_dense_f);
+        dfree(crit_dense_f); dfree(crit_dense_q); dfree(lut);
         dfree(gram_E); dfree(gram_G); dfree(gram_R); dfree(gram_maps); dfree(gram_units); dfree(pk);
         dfree(split_tab); dfree(split_ticket); dfree(d_tune);
         dfree(d_owned); dfree(d_shard); dfree(d_shard_count);
@@ -326,6 +338,7 @@ int grow_workspace(fbn_handle* h, Workspace& ws, long long edge_cap, int max_n, 
         CK(dalloc(&ws.crit_vals, kCritCap));
         CK(dalloc(&ws.crit_dense, kCritDense));
         CK(dalloc(&ws.crit_dense_f, kCritDense));
+        CK(dalloc(&ws.crit_dense_q, kCritDense));
         CK(dalloc(&ws.split_tab, kSplitItems * kSplitStride));
         CK(dalloc(&ws.split_ticket, kSplitItems));
         ws.split_dirty = true;
@@ -414,13 +427,6 @@ int ensure_gscratch(fbn_handle* h, Workspace& ws, long long total_ints)
     CK(dalloc(&ws.gscratch, total_ints));
     ws.gscratch_total = total_ints;
     return FBN_OK;
-}
-
-// Largest table a warp group takes: its eighth of the CTA's shared memory.
-long long warp_cells_cap()
-{
-    const long long slice = (long long)(kWarpSmemBytes / 4) / (kTestThreads / 32);
-    return (slice - 8) * 4 / 9;   // C + 1.25 C <= slice - 8
 }
 
 int check_status(fbn_handle* h, unsigned status)
@@ -902,33 +908,51 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     if (!ws.dev_sms) {
         int sms = 0;
         CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
-        CK(set_kernel_smem(kSmemBytes));
+        CK(set_kernel_smem(kWarpSmemBytes, kBigSmemBytes, kSmemBytes));
         // CTAs of the small-table pool (any group size) and of the big-table pool
         ws.grid_small = sms * std::max(1, pool_blocks_per_sm(kClassWarp, kWarpSmemBytes));
-        ws.grid_big = sms * std::max(1, pool_blocks_per_sm(kClassCta, kSmemBytes));
+        ws.grid_big = sms * std::max(1, pool_blocks_per_sm(kClassCta, kBigSmemBytes));
         ws.grid_marg = sms * std::max(1, pool_blocks_per_sm(kClassMarg, 0));
         ws.dev_sms = sms;
     }
     const int dev_sms = ws.dev_sms, grid_small = ws.grid_small, grid_big = ws.grid_big, grid_marg = ws.grid_marg;
     const long long groups[4] = {(long long)grid_small * 8, (long long)grid_small * 4, (long long)grid_small * 2,
                                  (long long)grid_small};
-    const long long groups_big[4] = {(long long)grid_big * 8, (long long)grid_big * 4, (long long)grid_big * 2,
-                                     (long long)grid_big};
+    const long long groups_big[4] = {grid_big, grid_big, grid_big, grid_big};   // whole CTAs
+    const int grid_plain = 2 * dev_sms;
     double mean_n = 0;
     for (int p = 0; p < k; ++p) mean_n += (double)hs[p]->N / k;
     const int grid_aux = dev_sms * 4;   // grid-stride helpers (ordering, removal)
     // ranks per chunk: fixed by the option, else chosen on the device per depth
     const int gs_forced = plain ? 1 : h->opt.group_size;
     const long long gs_edges = 8LL * grid_small * 8;   // live edges from which 4 ranks per claim pay
-    const long long wcap = plain ? 0 : warp_cells_cap();   // the plain form runs every edge on a CTA
+    // G^2 with the declared df is decided from the n ln n table (pool form)
+    long long max_N = 0;
+    for (int p = 0; p < k; ++p) max_N = std::max<long long>(max_N, hs[p]->N);
+    const bool use_lut = !plain && h->opt.statistic == FBN_STAT_G2 && h->opt.df_mode == FBN_DF_FIXED && max_N < kLutMaxN;
+    if (use_lut && max_N + 1 > ws.lut_n) {
+        dfree(ws.lut);
+        ws.lut = nullptr;
+        ws.lut_n = 0;
+        CK(dalloc(&ws.lut, max_N + 1));
+        ws.lut_n = max_N + 1;
+        k_lut<<<(unsigned)((ws.lut_n + 255) / 256), 256, 0, st>>>(ws.lut, (int)ws.lut_n);
+        CK(cudaGetLastError());
+    }
+    // an entry's error: two roundings of n ln n in FP64, one to the unit
+    const double lut_top = (double)std::max<long long>(max_N, 2) * std::log((double)std::max<long long>(max_N, 2));
+    const long long lut_err = (long long)(lut_top * 5e-16 * 68719476736.0) + 2;
+    // largest table of the small class; the plain form runs every edge on a CTA
+    const long long wcap = plain ? 0 : slice_cells((long long)(kWarpSmemBytes / 4), !use_lut);
     const int forced = h->opt.group_threads;
     if (ws.crit_alpha != alpha) {
         CK(cudaMemsetAsync(ws.crit_keys, 0, kCritCap * sizeof(long long), st));
         CK(cudaMemsetAsync(ws.crit_dense, 0, kCritDense * sizeof(double), st));
         CK(cudaMemsetAsync(ws.crit_dense_f, 0, kCritDense * sizeof(float2), st));
+        CK(cudaMemsetAsync(ws.crit_dense_q, 0, kCritDense * sizeof(long long), st));
         ws.crit_alpha = alpha;
     }
-    CritTableDev ct{ws.crit_keys, ws.crit_vals, kCritCap, kCritDense, ws.crit_dense, ws.crit_dense_f};
+    CritTableDev ct{ws.crit_keys, ws.crit_vals, kCritCap, kCritDense, ws.crit_dense, ws.crit_dense_f, ws.crit_dense_q};
 
     CK(cudaMemsetAsync(ws.d_rec, 0, kMaxDepthRecords * sizeof(DepthRecord), st));
     CK(cudaMemsetAsync(ws.hist, 0, 2 * ws.ord_cap * sizeof(unsigned long long), st));
@@ -962,6 +986,8 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     base.split_tab = ws.split_tab;
     base.split_ticket = ws.split_ticket;
     base.split_stride = kSplitStride;
+    base.lut = use_lut ? ws.lut : nullptr;
+    base.lut_err = lut_err;
 
     if (ws.split_dirty) {
         CK(cudaMemsetAsync(ws.split_tab, 0, kSplitItems * kSplitStride * sizeof(int), st));
@@ -978,10 +1004,10 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
             sc[cls].alive = ws.alive + cls * ws.ord_cap;
             sc[cls].base = ws.base + cls * ws.ord_cap;
             for (int k = 0; k < 4; ++k) sc[cls].groups[k] = cls == 0 ? groups[k] : groups_big[k];
-            sc[cls].smem_ints = (long long)((cls == 0 ? kWarpSmemBytes : kSmemBytes) / 4);
+            sc[cls].smem_ints = (long long)((cls == 0 ? kWarpSmemBytes : kBigSmemBytes) / 4);
         }
         launch_order(ws.probs, ws.edges, ws.edge_cap, marg ? 1 : 2, ws.d_ctr, sc, ws.cursor, ws.cursor + ws.ord_cap,
-                     ws.sorted, mean_n, forced, kSplitStride, 1, marg, grid_aux, st);
+                     ws.sorted, mean_n, forced, kSplitStride, 1, marg, !use_lut, grid_aux, st);
     };
     auto enqueue_tests = [&]() {
         const int nclass = 2;
@@ -990,14 +1016,14 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
             PoolArgs a = base;
             a.cls = cls;
             const bool small = cls == kClassWarp && !plain;
-            const size_t smem = small ? kWarpSmemBytes : kSmemBytes;
+            const size_t smem = small ? kWarpSmemBytes : plain ? kSmemBytes : kBigSmemBytes;
             a.smem_ints = (int)(smem / 4);
             if (!small && ws.gs_cells > 0) {
                 a.gscratch = ws.gscratch;
                 a.gscratch_ints = 3 * ws.gs_cells + 64;
             }
             if (plain) {
-                launch_plain(a, grid_big, kSmemBytes, st);
+                launch_plain(a, grid_plain, kSmemBytes, st);
                 continue;
             }
             a.base = ws.base + cls * ws.ord_cap;
@@ -1103,12 +1129,12 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         };
         const void* ptrs[] = {ws.probs, ws.vtx_prob, ws.vtx_first, ws.binom, ws.edges, ws.min_accept, ws.d_ctr,
                               ws.hist, ws.alive, ws.base, ws.cursor, ws.sorted, ws.gscratch, ws.sep_pool, ws.d_rec,
-                              ws.crit_keys, ws.crit_vals, ws.crit_dense, ws.crit_dense_f, ws.split_tab,
-                              ws.split_ticket};
+                              ws.crit_keys, ws.crit_vals, ws.crit_dense, ws.crit_dense_f, ws.crit_dense_q, ws.lut,
+                              ws.split_tab, ws.split_ticket};
         put(ptrs, sizeof ptrs);
         const long long ints[] = {total_vtx, gs_forced, gs_edges, ws.brows, wcap, ws.edge_cap, ws.ord_cap, forced,
                                   grid_aux, grid_small, grid_big, ws.gs_cells, ws.sep_cap, max_depth, plain,
-                                  h->opt.statistic, h->opt.df_mode,
+                                  h->opt.statistic, h->opt.df_mode, use_lut, lut_err,
                                   groups[0], groups[1], groups[2], groups[3]};
         put(ints, sizeof ints);
         put(&mean_n, sizeof mean_n);
@@ -1300,7 +1326,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         if (c.status & kStatusScratch) {
             if (c.need_cells <= 0 || c.need_cells > kMaxCells) return check_status(h, kStatusTooBig);
             ws.gs_cells = std::max<long long>(2 * ws.gs_cells, c.need_cells);
-            rc = ensure_gscratch(h, ws, (3 * ws.gs_cells + 64) * grid_big);
+            rc = ensure_gscratch(h, ws, (3 * ws.gs_cells + 64) * std::max(grid_big, grid_plain));
             if (rc) return rc;
         }
         *retry = true;

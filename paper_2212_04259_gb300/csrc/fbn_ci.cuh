@@ -119,11 +119,12 @@ __device__ __forceinline__ bool rows_out_of_range(const TestSpec& s)
     return __syncthreads_or(bad) != 0;
 }
 
-// Shared-memory ints a CTA's share of the strata takes: cells and marginals.
+// Shared-memory ints a CTA's share of the strata takes: cells and marginals,
+// rounded to 16 bytes (the CTA's own table follows).
 __host__ __device__ __forceinline__ long long ci_share_ints(long long cells, int rx, int ry, int k)
 {
     const long long nz = cells / (rx * ry);
-    return (nz + k - 1) / k * (rx * ry + rx + ry + 1);
+    return ((nz + k - 1) / k * (rx * ry + rx + ry + 1) + 3) / 4 * 4;
 }
 
 // Whether the test's table runs in shared memory on k CTAs.
@@ -141,7 +142,7 @@ __device__ __forceinline__ void ci_cluster_test(const CiArgs& q)
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     const int k = (int)cl.num_blocks(), r = (int)cl.block_rank();
-    extern __shared__ int smem[];
+    extern __shared__ __align__(16) int smem[];
     __shared__ TestSpec spec;
     __shared__ double red[32];
     __shared__ double part[kCiMaxCluster], part_df[kCiMaxCluster];   // CTA 0: every CTA's share
@@ -188,7 +189,7 @@ __device__ __forceinline__ void ci_cluster_test(const CiArgs& q)
     int* M;          // their marginals
     if (ci_fits_smem(q.cells, q.rx, q.ry, k, q.smem_ints)) {
         const long long share = k > 1 ? ci_share_ints(q.cells, q.rx, q.ry, k) : 0;
-        int* own = grp_table<kTestThreads>(spec, smem + share, q.smem_ints - share, nullptr, 0, &M);
+        int* own = grp_table<kTestThreads>(spec, smem + share, q.smem_ints - share, nullptr, 0, true, &M);
         T = own;
         if (k > 1) {
             if (tid == 0) t_off = (int)(own - smem);
@@ -211,7 +212,7 @@ __device__ __forceinline__ void ci_cluster_test(const CiArgs& q)
         for (int c = c0 + tid; c < c1; c += kTestThreads) q.gtab[c] = 0;
         __threadfence();
         if (k > 1) cl.sync(); else __syncthreads();
-        count_dispatch<kTestThreads, kGlobal>(spec, q.gtab);
+        count_global(spec, q.gtab, tid, kTestThreads);
         __threadfence();
         if (k > 1) cl.sync(); else __syncthreads();
         __threadfence();

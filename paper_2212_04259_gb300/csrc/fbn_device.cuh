@@ -128,6 +128,7 @@ __device__ __forceinline__ double crit_get(const CritTable& t, long long df, dou
         if (!capped) {
             t.dense[df] = c;
             if (t.dense_f) t.dense_f[df] = make_float2(__double2float_rd(c), __double2float_ru(c));
+            if (t.dense_q) t.dense_q[df] = (long long)floor(c * 0.5 * 68719476736.0);   // 2^kLutBits
         }
         return c;
     }
@@ -201,7 +202,7 @@ struct TestSpec {
 
 template <int G>
 struct Grp {
-    static_assert(G == 32 || G == 64 || G == 128 || G == kTestThreads, "group size");
+    static_assert(G == 32 || G == 64 || G == 128 || G == kTestThreads || G == kBigThreads, "group size");
     static constexpr int kWarps = G / 32;
     static __device__ __forceinline__ int rank() { return (int)(threadIdx.x % G); }
     static __device__ __forceinline__ int gid() { return (int)(threadIdx.x / G); }
@@ -209,7 +210,7 @@ struct Grp {
     {
         if (G == 32) {
             __syncwarp();
-        } else if (G == kTestThreads) {
+        } else if (G >= kTestThreads) {   // the whole CTA
             __syncthreads();
         } else {   // named barrier 1 + group index, G threads
             asm volatile("bar.sync %0, %1;" ::"r"(1 + gid()), "r"(G) : "memory");
@@ -235,187 +236,40 @@ __device__ __forceinline__ T grp_sum(T v, T* red)
     return t;
 }
 
-// Two sums in one pass (red: the CTA's scratch of 32 doubles).
-template <int G>
-__device__ __forceinline__ void grp_sum2(double& a, double& b, double* red)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-    }
-    if (G == 32) return;
-    double* r = red + Grp<G>::gid() * 2 * Grp<G>::kWarps;
-    Grp<G>::sync();
-    if ((threadIdx.x & 31) == 0) {
-        r[2 * (Grp<G>::rank() >> 5)] = a;
-        r[2 * (Grp<G>::rank() >> 5) + 1] = b;
-    }
-    Grp<G>::sync();
-    a = 0.0;
-    b = 0.0;
-#pragma unroll
-    for (int w = 0; w < Grp<G>::kWarps; ++w) {
-        a += r[2 * w];
-        b += r[2 * w + 1];
-    }
-}
-
-enum CountMode { kLane = 0, kWarp = 1, kShared = 2, kGlobal = 3, kLane16 = 4 };
-
-template <int MODE>
-__device__ __forceinline__ void bump(int* base, unsigned idx)
-{
-    // kLane: this lane's private column, so no other thread touches the word;
-    // the update is still a shared-memory reduction (red.shared.add) rather
-    // than load-add-store, so consecutive samples do not wait on each other
-    if (MODE == kLane) atomicAdd(base + idx * 32u, 1);
-    else if (MODE == kLane16) atomicAdd(base + (idx >> 1) * 32u, 1 << ((idx & 1u) << 4));   // two 16-bit counters
-    else atomicAdd(base + idx, 1);
-}
-
-// Count 16-sample vectors (one 16-byte load per row) plus the ragged tail.
-// The cell index of two samples is carried in the two 16-bit halves of one
-// 32-bit register (every partial index is below cells <= 65536), so one IMAD
-// advances two samples.  NR > 0: rows known at compile time; NR == 0: runtime.
-template <int NR>
-__device__ __forceinline__ void pack_vector(const TestSpec& s, const uint4* w, unsigned* acc)
-{
+// --------------------------------------------------------------------------
+// Counting: one loop for every table in shared memory.  A table of C cells is
+// kept in K interleaved copies (K a power of two, at most the group's threads):
+// copy k of cell c is word c K + k, and thread t counts into copy t mod K.  K is
+// the largest that fits, so small tables get a copy per thread (no two threads
+// of a warp meet in a word or a bank) and large ones at least a few: a warp's
+// 32 updates of one shared copy met 3.9 deep in a cell (depth 2, arities 2-4),
+// in 4 copies 2.2, in 8 copies 1.8.  The update is a shared-memory reduction,
+// so consecutive samples do not wait on each other.  One loop with a runtime
+// copy count instead of one per strategy keeps the pool's code small: every
+// test runs through all of it, and instruction fetch was a third of the
+// histogram pools' stalls.
+struct SharedCounter {
+    unsigned base;   // shared address of this thread's copy of cell 0
+    unsigned step;   // bytes from a cell to the next: 4 K
+    __device__ __forceinline__ void bump(unsigned idx) const
     {
-        const unsigned ws[4] = {w[0].x, w[0].y, w[0].z, w[0].w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            acc[2 * q] = __byte_perm(ws[q], 0u, 0x4140);      // bytes 0,1 -> halves
-            acc[2 * q + 1] = __byte_perm(ws[q], 0u, 0x4342);  // bytes 2,3 -> halves
-        }
+        asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(base + idx * step) : "memory");
     }
-#pragma unroll
-    for (int k = 1; k < NR; ++k) {
-        const unsigned rk = (unsigned)s.rad[k];
-        const unsigned ws[4] = {w[k].x, w[k].y, w[k].z, w[k].w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            acc[2 * q] = acc[2 * q] * rk + __byte_perm(ws[q], 0u, 0x4140);
-            acc[2 * q + 1] = acc[2 * q + 1] * rk + __byte_perm(ws[q], 0u, 0x4342);
-        }
-    }
-}
+};
 
-template <int MODE>
-__device__ __forceinline__ void bump_packed(int* base, const unsigned* acc)
-{
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        bump<MODE>(base, acc[q] & 0xFFFFu);
-        bump<MODE>(base, acc[q] >> 16);
-    }
-}
+struct GlobalCounter {
+    int* base;
+    __device__ __forceinline__ void bump(unsigned idx) const { atomicAdd(base + idx, 1); }
+};
 
-// Count 16-sample vectors (one 16-byte load per row) plus the ragged tail.
-// The cell index of two samples is carried in the two 16-bit halves of one
-// 32-bit register (every partial index is below cells <= 65536), so one IMAD
-// advances two samples.  Two vectors are loaded before either is counted, to
-// keep 2 (d + 2) loads in flight per thread.  NR > 0: rows known at compile
-// time; NR == 0: runtime.
-template <int G, int NR, int MODE>
-__device__ __forceinline__ void count_packed(const TestSpec& s, int* base)
+// The ragged tail: samples past the last whole 16-sample vector.
+template <class Counter>
+__device__ __forceinline__ void count_tail(const TestSpec& s, const Counter& cnt, int rank, int G)
 {
-    const int nvec = s.N >> 4;
-    const int t0 = Grp<G>::rank();
-    const int nr = NR > 0 ? NR : s.nrows;
-    if (NR > 0) {
-        const uint4* r[NR > 0 ? NR : 1];
-#pragma unroll
-        for (int k = 0; k < NR; ++k) r[k] = reinterpret_cast<const uint4*>(s.rows[k]);
-        int v = t0;
-        for (; v + G < nvec; v += 2 * G) {
-            uint4 w0[NR > 0 ? NR : 1], w1[NR > 0 ? NR : 1];
-#pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                w0[k] = __ldg(r[k] + v);
-                w1[k] = __ldg(r[k] + v + G);
-            }
-            if (v + 3 * G < nvec) {   // the next iteration's lines into L1 while these are counted
-#pragma unroll
-                for (int k = 0; k < NR; ++k) {
-                    asm volatile("prefetch.global.L1 [%0];" ::"l"(r[k] + v + 2 * G));
-                    asm volatile("prefetch.global.L1 [%0];" ::"l"(r[k] + v + 3 * G));
-                }
-            }
-            unsigned acc[8];
-            pack_vector<NR>(s, w0, acc);
-            bump_packed<MODE>(base, acc);
-            pack_vector<NR>(s, w1, acc);
-            bump_packed<MODE>(base, acc);
-        }
-        if (v < nvec) {
-            uint4 w0[NR > 0 ? NR : 1];
-#pragma unroll
-            for (int k = 0; k < NR; ++k) w0[k] = __ldg(r[k] + v);
-            unsigned acc[8];
-            pack_vector<NR>(s, w0, acc);
-            bump_packed<MODE>(base, acc);
-        }
-    } else {
-        for (int v = t0; v < nvec; v += G) {
-            unsigned acc[8];
-            {
-                const uint4 w = __ldg(reinterpret_cast<const uint4*>(s.rows[0]) + v);
-                const unsigned ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    acc[2 * q] = __byte_perm(ws[q], 0u, 0x4140);
-                    acc[2 * q + 1] = __byte_perm(ws[q], 0u, 0x4342);
-                }
-            }
-            for (int k = 1; k < nr; ++k) {
-                const uint4 w = __ldg(reinterpret_cast<const uint4*>(s.rows[k]) + v);
-                const unsigned rk = (unsigned)s.rad[k];
-                const unsigned ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    acc[2 * q] = acc[2 * q] * rk + __byte_perm(ws[q], 0u, 0x4140);
-                    acc[2 * q + 1] = acc[2 * q + 1] * rk + __byte_perm(ws[q], 0u, 0x4342);
-                }
-            }
-            bump_packed<MODE>(base, acc);
-        }
-    }
-    for (int t = (nvec << 4) + t0; t < s.N; t += G) {
-        unsigned idx = s.rows[0][t];
-        for (int k = 1; k < nr; ++k) idx = idx * (unsigned)s.rad[k] + s.rows[k][t];
-        bump<MODE>(base, idx);
-    }
-}
-
-// Same, one sample per 32-bit index (tables above 65536 cells).
-template <int G, int MODE>
-__device__ __forceinline__ void count_wide(const TestSpec& s, int* base)
-{
-    const int nvec = s.N >> 4;
-    const int t0 = Grp<G>::rank();
-    for (int v = t0; v < nvec; v += G) {
-        unsigned idx[16];
-        {
-            const uint4 w = __ldg(reinterpret_cast<const uint4*>(s.rows[0]) + v);
-            const unsigned ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-            for (int b = 0; b < 16; ++b) idx[b] = (ws[b >> 2] >> ((b & 3) * 8)) & 0xFFu;
-        }
-        for (int k = 1; k < s.nrows; ++k) {
-            const uint4 w = __ldg(reinterpret_cast<const uint4*>(s.rows[k]) + v);
-            const unsigned rk = (unsigned)s.rad[k];
-            const unsigned ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-            for (int b = 0; b < 16; ++b) idx[b] = idx[b] * rk + ((ws[b >> 2] >> ((b & 3) * 8)) & 0xFFu);
-        }
-#pragma unroll
-        for (int b = 0; b < 16; ++b) bump<MODE>(base, idx[b]);
-    }
-    for (int t = (nvec << 4) + t0; t < s.N; t += G) {
+    for (int t = (s.N & ~15) + rank; t < s.N; t += G) {
         unsigned idx = s.rows[0][t];
         for (int k = 1; k < s.nrows; ++k) idx = idx * (unsigned)s.rad[k] + s.rows[k][t];
-        bump<MODE>(base, idx);
+        cnt.bump(idx);
     }
 }
 
@@ -423,21 +277,16 @@ __device__ __forceinline__ void count_wide(const TestSpec& s, int* base)
 // so the four samples of a 32-bit word advance together in its four bytes --
 // acc * r_k + row_k never carries out of a byte because the result stays below
 // the cells counted so far.  One IMAD per row and 4 samples, then one byte
-// extraction per sample.
-template <int MODE>
-__device__ __forceinline__ void bump_bytes(int* base, unsigned acc)
-{
-    bump<MODE>(base, __byte_perm(acc, 0u, 0x4440));
-    bump<MODE>(base, __byte_perm(acc, 0u, 0x4441));
-    bump<MODE>(base, __byte_perm(acc, 0u, 0x4442));
-    bump<MODE>(base, __byte_perm(acc, 0u, 0x4443));
-}
-
-template <int G, int NR, int MODE>
-__device__ __forceinline__ void count_bytes(const TestSpec& s, int* base)
+// extraction per sample.  The next kCountDepth vectors of each row are in
+// flight while one is counted.
+// (measured at depth 2 of 256 problems: 1 vector ahead 2.9 ms at three CTAs per
+// SM and 3.1 at two; 2 ahead at two CTAs 2.3; 3 ahead 2.1 there, the others
+// unchanged, for 32 more registers)
+constexpr int kCountDepth = 2;
+template <int NR>
+__device__ __forceinline__ void count_bytes(const TestSpec& s, const SharedCounter& cnt, int rank, int G)
 {
     const int nvec = s.N >> 4;
-    const int t0 = Grp<G>::rank();
     const uint4* r[NR];
     unsigned rad[NR];
 #pragma unroll
@@ -445,177 +294,213 @@ __device__ __forceinline__ void count_bytes(const TestSpec& s, int* base)
         r[k] = reinterpret_cast<const uint4*>(s.rows[k]);
         rad[k] = (unsigned)s.rad[k];
     }
-    int v = t0;
-    for (; v + G < nvec; v += 2 * G) {
-        uint4 w0[NR], w1[NR];
+    uint4 w[kCountDepth][NR];
+    const int last = nvec - 1;
+    if (rank > last) return;
 #pragma unroll
-        for (int k = 0; k < NR; ++k) {
-            w0[k] = __ldg(r[k] + v);
-            w1[k] = __ldg(r[k] + v + G);
-        }
-        if (v + 3 * G < nvec) {   // the next iteration's lines into L1 while these are counted
+    for (int i = 0; i < kCountDepth; ++i)
 #pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                asm volatile("prefetch.global.L1 [%0];" ::"l"(r[k] + v + 2 * G));
-                asm volatile("prefetch.global.L1 [%0];" ::"l"(r[k] + v + 3 * G));
+        for (int k = 0; k < NR; ++k) w[i][k] = __ldg(r[k] + min(rank + i * G, last));
+#pragma unroll 1
+    for (int v = rank; v <= last; v += kCountDepth * G) {
+#pragma unroll
+        for (int i = 0; i < kCountDepth; ++i) {
+            if (i && v + i * G > last) break;
+            uint4 a = w[i][0];
+#pragma unroll
+            for (int k = 1; k < NR; ++k) {
+                a.x = a.x * rad[k] + w[i][k].x; a.y = a.y * rad[k] + w[i][k].y;
+                a.z = a.z * rad[k] + w[i][k].z; a.w = a.w * rad[k] + w[i][k].w;
+            }
+            const int vn = min(v + (kCountDepth + i) * G, last);
+#pragma unroll
+            for (int k = 0; k < NR; ++k) w[i][k] = __ldg(r[k] + vn);
+            const unsigned q[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                cnt.bump(__byte_perm(q[t], 0u, 0x4440));
+                cnt.bump(__byte_perm(q[t], 0u, 0x4441));
+                cnt.bump(__byte_perm(q[t], 0u, 0x4442));
+                cnt.bump(__byte_perm(q[t], 0u, 0x4443));
             }
         }
-        uint4 a0 = w0[0], a1 = w1[0];
-#pragma unroll
-        for (int k = 1; k < NR; ++k) {
-            a0.x = a0.x * rad[k] + w0[k].x; a0.y = a0.y * rad[k] + w0[k].y;
-            a0.z = a0.z * rad[k] + w0[k].z; a0.w = a0.w * rad[k] + w0[k].w;
-            a1.x = a1.x * rad[k] + w1[k].x; a1.y = a1.y * rad[k] + w1[k].y;
-            a1.z = a1.z * rad[k] + w1[k].z; a1.w = a1.w * rad[k] + w1[k].w;
-        }
-        bump_bytes<MODE>(base, a0.x); bump_bytes<MODE>(base, a0.y);
-        bump_bytes<MODE>(base, a0.z); bump_bytes<MODE>(base, a0.w);
-        bump_bytes<MODE>(base, a1.x); bump_bytes<MODE>(base, a1.y);
-        bump_bytes<MODE>(base, a1.z); bump_bytes<MODE>(base, a1.w);
-    }
-    if (v < nvec) {
-        uint4 a = __ldg(r[0] + v);
-#pragma unroll
-        for (int k = 1; k < NR; ++k) {
-            const uint4 w = __ldg(r[k] + v);
-            a.x = a.x * rad[k] + w.x; a.y = a.y * rad[k] + w.y;
-            a.z = a.z * rad[k] + w.z; a.w = a.w * rad[k] + w.w;
-        }
-        bump_bytes<MODE>(base, a.x); bump_bytes<MODE>(base, a.y);
-        bump_bytes<MODE>(base, a.z); bump_bytes<MODE>(base, a.w);
-    }
-    for (int t = (nvec << 4) + t0; t < s.N; t += G) {
-        unsigned idx = s.rows[0][t];
-#pragma unroll
-        for (int k = 1; k < NR; ++k) idx = idx * rad[k] + s.rows[k][t];
-        bump<MODE>(base, idx);
     }
 }
 
-template <int G, int MODE>
-__device__ __forceinline__ void count_dispatch(const TestSpec& s, int* base)
+// At most 65,536 cells: the indices of two samples ride in the 16-bit halves of
+// one register (every partial index is below the cells), one IMAD for both.
+// NR = 0: any number of rows.
+template <int NR, class Counter>
+__device__ __forceinline__ void count_packed(const TestSpec& s, const Counter& cnt, int rank, int G)
 {
-    if (s.cells > 65536) {
-        count_wide<G, MODE>(s, base);
-        return;
+    const int nvec = s.N >> 4;
+    const int nr = NR > 0 ? NR : s.nrows;
+    constexpr int kBuf = NR > 0 ? NR : 1;
+    uint4 w[kBuf];
+    const int last = nvec - 1;
+    if (NR > 0 && rank <= last) {
+#pragma unroll
+        for (int k = 0; k < kBuf; ++k) w[k] = __ldg(reinterpret_cast<const uint4*>(s.rows[k]) + rank);
     }
+#pragma unroll 1
+    for (int v = rank; v <= last; v += G) {
+        unsigned acc[8];
+        if (NR > 0) {
+#pragma unroll
+            for (int k = 0; k < kBuf; ++k) {
+                const unsigned ws[4] = {w[k].x, w[k].y, w[k].z, w[k].w};
+                const unsigned rk = (unsigned)s.rad[k];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const unsigned lo = __byte_perm(ws[q], 0u, 0x4140), hi = __byte_perm(ws[q], 0u, 0x4342);
+                    acc[2 * q] = k ? acc[2 * q] * rk + lo : lo;          // bytes 0, 1 -> halves
+                    acc[2 * q + 1] = k ? acc[2 * q + 1] * rk + hi : hi;  // bytes 2, 3 -> halves
+                }
+            }
+            const int vn = min(v + G, last);
+#pragma unroll
+            for (int k = 0; k < kBuf; ++k) w[k] = __ldg(reinterpret_cast<const uint4*>(s.rows[k]) + vn);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) acc[q] = 0u;
+            for (int k = 0; k < nr; ++k) {
+                const uint4 x = __ldg(reinterpret_cast<const uint4*>(s.rows[k]) + v);
+                const unsigned ws[4] = {x.x, x.y, x.z, x.w};
+                const unsigned rk = (unsigned)s.rad[k];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    acc[2 * q] = acc[2 * q] * rk + __byte_perm(ws[q], 0u, 0x4140);
+                    acc[2 * q + 1] = acc[2 * q + 1] * rk + __byte_perm(ws[q], 0u, 0x4342);
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            cnt.bump(acc[q] & 0xFFFFu);
+            cnt.bump(acc[q] >> 16);
+        }
+    }
+}
+
+// Above: one sample per 32-bit index.
+template <class Counter>
+__device__ __forceinline__ void count_wide(const TestSpec& s, const Counter& cnt, int rank, int G)
+{
+    const int nvec = s.N >> 4;
+#pragma unroll 1
+    for (int v = rank; v < nvec; v += G) {
+        unsigned idx[16];
+#pragma unroll
+        for (int b = 0; b < 16; ++b) idx[b] = 0u;
+        for (int k = 0; k < s.nrows; ++k) {
+            const uint4 w = __ldg(reinterpret_cast<const uint4*>(s.rows[k]) + v);
+            const unsigned rk = (unsigned)s.rad[k];
+            const unsigned ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int b = 0; b < 16; ++b) idx[b] = idx[b] * rk + ((ws[b >> 2] >> ((b & 3) * 8)) & 0xFFu);
+        }
+#pragma unroll
+        for (int b = 0; b < 16; ++b) cnt.bump(idx[b]);
+    }
+}
+
+// The samples of the test into shared copies, by thread `rank` of G.
+static __device__ __noinline__ void count_shared(const TestSpec& s, SharedCounter cnt, int rank, int G)
+{
     if (s.cells <= 256) {
         switch (s.nrows) {
-            case 2: count_bytes<G, 2, MODE>(s, base); return;
-            case 3: count_bytes<G, 3, MODE>(s, base); return;
-            case 4: count_bytes<G, 4, MODE>(s, base); return;
-            case 5: count_bytes<G, 5, MODE>(s, base); return;
-            default: break;
+            case 2: count_bytes<2>(s, cnt, rank, G); break;
+            case 3: count_bytes<3>(s, cnt, rank, G); break;
+            case 4: count_bytes<4>(s, cnt, rank, G); break;
+            case 5: count_bytes<5>(s, cnt, rank, G); break;
+            default: count_packed<0>(s, cnt, rank, G); break;
+        }
+    } else {
+        switch (s.nrows) {
+            case 4: count_packed<4>(s, cnt, rank, G); break;
+            case 5: count_packed<5>(s, cnt, rank, G); break;
+            default: count_packed<0>(s, cnt, rank, G); break;
         }
     }
-    switch (s.nrows) {
-        case 2: count_packed<G, 2, MODE>(s, base); break;
-        case 3: count_packed<G, 3, MODE>(s, base); break;
-        case 4: count_packed<G, 4, MODE>(s, base); break;
-        case 5: count_packed<G, 5, MODE>(s, base); break;
-        case 6: count_packed<G, 6, MODE>(s, base); break;
-        default: count_packed<G, 0, MODE>(s, base); break;
-    }
+    count_tail(s, cnt, rank, G);
 }
 
-// Shared-memory ints needed by each counting strategy for a table of C cells
-// (marg = marginal entries); kGlobal when none fits.  kLane16 (warp groups)
-// packs two lane-private counters per word: a lane counts at most
-// N / 32 + 16 samples, which must stay below 2^16.  Its extra zeroing and
-// merge only pay off when the sample loop is long (measured: a gain at
-// N = 100,000, a loss for the batched problems of 1,000-50,000 samples),
-// hence N >= 65536.
-template <int G>
-__device__ __forceinline__ int pick_mode(long long C, long long marg, long long slice_ints, int N)
+// The same into one global table.
+static __device__ __noinline__ void count_global(const TestSpec& s, int* table, int rank, int G)
 {
-    // private copies cost their zeroing and folding (C words per copy); they
-    // pay only while that stays below the samples counted (short sample
-    // ranges: split tests, small problems, take fewer copies)
-    if (C * G + C + marg <= slice_ints && C * G <= N) return kLane;
-    if (G == 32 && N >= 65536 && N / 32 + 32 < 65536 && (C + 1) / 2 * 32 + C + marg <= slice_ints) return kLane16;
-    if (Grp<G>::kWarps > 1 && C * Grp<G>::kWarps + marg <= slice_ints && 2 * C * Grp<G>::kWarps <= N) return kWarp;
-    if (C + marg <= slice_ints) return kShared;
-    return kGlobal;
+    const GlobalCounter cnt{table};
+    if (s.cells > 65536) count_wide(s, cnt, rank, G);
+    else count_packed<0>(s, cnt, rank, G);
+    count_tail(s, cnt, rank, G);
 }
 
-// Count the table of the test and merge private copies.  Returns the merged
-// table T and sets *M to the space for the marginals; returns nullptr when the
-// table fits neither the slice nor the global scratch.
+// Copies of a table of C cells: the most that fit, while zeroing and folding
+// them (C K words each) stays below the samples counted.
 template <int G>
-__device__ int* grp_table(const TestSpec& s, int* slice, long long slice_ints, int* gtab, long long gtab_ints,
-                          int** M)
+__device__ __forceinline__ int table_copies(long long C, long long slice_ints, int N)
 {
-    const long long C = s.cells;
-    const long long nz = C / (s.rx * s.ry);
-    const long long marg = nz * (s.rx + s.ry + 1);
-    const int mode = pick_mode<G>(C, marg, slice_ints, s.N);
-    if (mode == kGlobal && (gtab == nullptr || C + marg > gtab_ints)) return nullptr;
-    const int r = Grp<G>::rank();
-    const int lane = threadIdx.x & 31;
-    const int warp = r >> 5;                     // warp within the group
-    constexpr int W = Grp<G>::kWarps;
-    int* cnt = mode == kGlobal ? gtab : slice;
-    const long long zero_n = mode == kLane ? C * G : mode == kLane16 ? (C + 1) / 2 * 32
-                                    : mode == kWarp ? C * W : C;
-    for (int k = r; k < (int)zero_n; k += G) cnt[k] = 0;   // zero_n <= 2^27
-    Grp<G>::sync();
-    switch (mode) {
-        case kLane: count_dispatch<G, kLane>(s, cnt + (long long)warp * C * 32 + lane); break;
-        case kLane16: count_dispatch<G, kLane16>(s, cnt + lane); break;
-        case kWarp: count_dispatch<G, kWarp>(s, cnt + (long long)warp * C); break;
-        default: count_dispatch<G, kShared>(s, cnt); break;
+    int K = G;
+    while (K > 1 && (C * K > slice_ints || 2 * C * K > N)) K >>= 1;
+    return K;
+}
+
+// Count the table of the test.  Returns the table T -- in the slice, or in the
+// global scratch when the slice cannot hold it (with its marginals when the
+// caller needs them: need_marg) -- and sets *M to the space for the marginals;
+// nullptr when the table fits neither.
+template <int G>
+__device__ __forceinline__ int* grp_table(const TestSpec& s, int* slice, long long slice_ints, int* gtab,
+                                          long long gtab_ints, bool need_marg, int** M)
+{
+    const int C = (int)s.cells;   // <= kMaxCells
+    const long long marg = need_marg ? (long long)(C / (s.rx * s.ry)) * (s.rx + s.ry + 1) : 0;
+    const int r = Grp<G>::rank(), lane = threadIdx.x & 31;
+    if (C + marg > slice_ints) {
+        if (gtab == nullptr || C + marg > gtab_ints) return nullptr;
+        for (int k = r; k < C; k += G) gtab[k] = 0;
+        Grp<G>::sync();
+        count_global(s, gtab, r, G);
+        Grp<G>::sync();
+        *M = marg <= slice_ints ? slice : gtab + C;
+        return gtab;
     }
+    const int K = table_copies<G>(C, slice_ints, s.N);
+    uint4* z = reinterpret_cast<uint4*>(slice);   // slices are whole 16-byte words
+    for (int k = r; k < (C * K + 3) / 4; k += G) z[k] = make_uint4(0u, 0u, 0u, 0u);
     Grp<G>::sync();
-    int* T;
-    if (mode == kLane16) {   // one warp: lane l folds the 32 columns of cells l, l + 32, ...
-        T = slice + (C + 1) / 2 * 32;
-        for (int c = lane; c < (int)C; c += 32) {
-            const int* row = cnt + (c >> 1) * 32;
-            const int sh = (int)(c & 1) * 16;
+    SharedCounter cnt;
+    cnt.base = (unsigned)__cvta_generic_to_shared(slice) + 4u * (unsigned)(r & (K - 1));
+    cnt.step = 4u * (unsigned)K;
+    count_shared(s, cnt, r, G);
+    Grp<G>::sync();
+    if (K > 1) {
+        // fold in place: cell c's sum goes to word c, which lies in copies read
+        // in this round or before (words past them are not written); lanes
+        // start at rotated words of their cells (no bank conflicts)
+        const int rot = K >= 32 ? lane : (lane * K) >> 5;
+        for (int c0 = 0; c0 < C; c0 += G) {
+            const int c = c0 + r;
             int sum = 0;
-#pragma unroll 8
-            for (int l = 0; l < 32; ++l) sum += (row[(l + (int)c) & 31] >> sh) & 0xFFFF;
-            T[c] = sum;
-        }
-        *M = T + C;
-    } else if (mode == kLane) {
-        // stage 1: each warp folds its 32 lane columns, lane l taking cells
-        // c = l, l + 32, ...; the sum goes to column (c mod 32) of cell c's
-        // row, which only that lane touches (and which keeps stage 2 free of
-        // bank conflicts).  stage 2: fold the warps' partial sums.
-        int* own = cnt + (long long)warp * C * 32;
-        for (int c = lane; c < (int)C; c += 32) {
-            const int* col = own + c * 32;
-            int sum = 0;
-#pragma unroll 8
-            for (int l = 0; l < 32; ++l) sum += col[(l + (int)c) & 31];
-            own[c * 32 + (c & 31)] = sum;
+            if (c < C) {
+                if (K == 2) {
+                    const int2 v = reinterpret_cast<const int2*>(slice)[c];
+                    sum = v.x + v.y;
+                } else {
+                    const int4* row = reinterpret_cast<const int4*>(slice + (long long)c * K);
+#pragma unroll 2
+                    for (int q = 0; q < K / 4; ++q) {
+                        const int4 v = row[(q + rot) & (K / 4 - 1)];
+                        sum += v.x + v.y + v.z + v.w;
+                    }
+                }
+            }
+            Grp<G>::sync();
+            if (c < C) slice[c] = sum;
         }
         Grp<G>::sync();
-        T = slice + C * G;
-        for (int c = r; c < (int)C; c += G) {
-            int sum = 0;
-            for (int w = 0; w < W; ++w) sum += cnt[(w * (int)C + c) * 32 + (c & 31)];
-            T[c] = sum;
-        }
-        *M = T + C;
-    } else if (mode == kWarp) {
-        T = cnt;
-        for (int c = r; c < (int)C; c += G) {
-            int sum = 0;
-            for (int w = 0; w < W; ++w) sum += cnt[w * (int)C + c];
-            T[c] = sum;
-        }
-        *M = slice + C * W;
-    } else if (mode == kShared) {
-        T = cnt;
-        *M = slice + C;
-    } else {
-        T = cnt;
-        *M = marg <= slice_ints ? slice : gtab + C;
     }
-    Grp<G>::sync();
-    return T;
+    *M = slice + C;
+    return slice;
 }
 
 // Marginals N_x+z [nz*rx], N_+yz [nz*ry], N_++z [nz] into M.
@@ -893,8 +778,81 @@ __device__ __forceinline__ int grp_decide_bound(const TestSpec& s, const int* T,
         }
     }
     const float per_thread = (float)((C + G - 1) / G);   // exact: C < 2^24
-    const float levels = (G == 32 ? 5.0f : G == 64 ? 6.0f : G == 128 ? 7.0f : 8.0f);
+    const float levels = (G == 32 ? 5.0f : G == 64 ? 6.0f : G == 128 ? 7.0f : G == 256 ? 8.0f : 10.0f);
     return decide_from_sums(v.x, v.y, per_thread, levels, stat, crit_lo, crit_hi, stat == kStatX2 ? 6.0e-7f : 3.2e-7f);
+}
+
+// --------------------------------------------------------------------------
+// G^2 from a table of n ln n.  G^2 / 2 = sum n_xyz ln n_xyz - sum N_x+z ln N_x+z -
+// sum N_+yz ln N_+yz + sum N_++z ln N_++z, with n ln n as 64-bit fixed point
+// (2^-kLutBits) from a table indexed by the count: the sums are exact, each
+// entry within lut_err units of its value, so the comparison with crit needs no
+// cell coordinates, logarithms, divisions or marginals per cell, and its error
+// (about 1e-7 for 1,000 cells of 50,000 samples) leaves almost no test for the
+// FP64 recomputation, where FP32 terms leave about one in 1,000.
+constexpr int kLutBits = 36;
+constexpr long long kLutMaxN = 1LL << 20;   // 2^20 ln 2^20 < 2^24: 60 bits
+
+// Exact G^2 in FP64 from the table alone (no stored marginals).  Rare.
+template <int G>
+__device__ __noinline__ double grp_g2_cells(const TestSpec& s, const int* T, double* red)
+{
+    const int rx = s.rx, ry = s.ry, rxy = rx * ry, C = (int)s.cells;
+    double acc = 0.0;
+    for (int c = Grp<G>::rank(); c < C; c += G) {
+        const int n = T[c];
+        if (n == 0) continue;
+        const int z = c / rxy, rem = c - z * rxy, x = rem / ry, y = rem - x * ry;
+        const int* S = T + z * rxy;
+        long long nx = 0, ny = 0, nz = 0;
+        for (int q = 0; q < ry; ++q) nx += S[x * ry + q];
+        for (int q = 0; q < rx; ++q) ny += S[q * ry + y];
+        for (int q = 0; q < rxy; ++q) nz += S[q];
+        const long long a = (long long)n * nz, b = nx * ny;
+        acc += (double)n * log1p((double)(a - b) / (double)b);
+    }
+    return 2.0 * grp_sum<G>(acc, red);
+}
+
+// Twice this is G^2, in units of 2^-kLutBits (every thread of the group).
+template <int G>
+__device__ __forceinline__ long long grp_g2_lut(const TestSpec& s, const int* T, const long long* __restrict__ lut,
+                                                double* red)
+{
+    const int rx = s.rx, ry = s.ry, rxy = rx * ry, C = (int)s.cells, r = Grp<G>::rank();
+    const int nz = C / rxy;
+    long long acc = 0;
+#pragma unroll 1
+    for (int k = r; k < nz * rx; k += G) {   // rows (x, z): their cells and N_x+z
+        int n = 0;
+        const int* t = T + k * ry;
+#pragma unroll 4
+        for (int y = 0; y < ry; ++y) {
+            const int v = t[y];
+            n += v;
+            acc += __ldg(lut + v);
+        }
+        acc -= __ldg(lut + n);
+    }
+    const unsigned m = 0xFFFFFFFFu / (unsigned)ry + 1u;   // k / ry = umulhi(k, m) while k ry < 2^32
+#pragma unroll 1
+    for (int k = r; k < nz * ry; k += G) {   // columns (y, z): N_+yz
+        const int z = ry == 1 ? k : (int)__umulhi((unsigned)k, m);
+        const int* t = T + z * rxy + (k - z * ry);
+        int n = 0;
+#pragma unroll 4
+        for (int x = 0; x < rx; ++x) n += t[x * ry];
+        acc -= __ldg(lut + n);
+    }
+#pragma unroll 1
+    for (int z = r; z < nz; z += G) {        // strata: N_++z
+        int n = 0;
+        const int* t = T + z * rxy;
+#pragma unroll 4
+        for (int q = 0; q < rxy; ++q) n += t[q];
+        acc += __ldg(lut + n);
+    }
+    return grp_sum<G>(acc, reinterpret_cast<long long*>(red));
 }
 
 }  // namespace fbn

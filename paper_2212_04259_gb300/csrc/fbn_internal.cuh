@@ -14,6 +14,7 @@ constexpr long long kBinomSat = 1LL << 62;
 constexpr long long kMaxCells = 1LL << 24;  // largest contingency table (cells)
 constexpr int kMaxVars = 32767;           // neighbour positions are stored in 16 bits
 constexpr int kTestThreads = 256;         // threads of a test CTA
+constexpr int kBigThreads = 1024;         // threads of a CTA of the big-table class
 constexpr int kBaseSmem = 512;            // pass bases cached in shared memory
 
 // device status bits
@@ -190,6 +191,7 @@ struct CritTableDev {
     int dense_n;           // df < dense_n: dense[df], 0 until a test computes it
     double* dense;
     float2* dense_f;       // df < dense_n: the float bracket (largest float <= crit, smallest >= crit), 0 until set
+    long long* dense_q;    // df < dense_n: floor(crit / 2) in units of 2^-kLutBits, 0 until set
 };
 
 // Work pool of one depth and one edge class.  Sizes, the depth and the class
@@ -216,6 +218,16 @@ struct PoolArgs {
     long long split_stride;           // ints per split table
     int32_t stat;                     // CI statistic: 0 = G^2, 1 = Pearson X^2
     int32_t df_mode;                  // degrees of freedom: 0 = declared arities, 1 = observed table
+    const long long* lut;             // n ln n in units of 2^-kLutBits up to the largest N, or nullptr: FP32 terms
+    long long lut_err;                // bound of an entry's error, in its units
 };
+
+// Shared ints -> largest table a group's slice takes: the cells alone with the
+// n ln n table, else the cells and their marginals (at most 1.25 C as r_x, r_y
+// >= 2).
+__host__ __device__ __forceinline__ long long slice_cells(long long slice_ints, bool need_marg)
+{
+    return need_marg ? (slice_ints - 8) * 4 / 9 : slice_ints;
+}
 
 }  // namespace fbn

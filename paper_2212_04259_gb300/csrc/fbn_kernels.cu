@@ -253,7 +253,7 @@ constexpr double kTestOverhead = 10000.0;
 constexpr double kCyclesPerSample = 8.0;
 
 __global__ void k_scan(ScanClass c0, ScanClass c1, DepthCounters* ctr, double mean_n, int forced_group,
-                       long long split_stride, int allow_split, int marg)
+                       long long split_stride, int allow_split, int marg, int need_marg)
 {
     pdl_enter();
     __shared__ unsigned long long sh[32];
@@ -308,8 +308,12 @@ __global__ void k_scan(ScanClass c0, ScanClass c1, DepthCounters* ctr, double me
             const long long groups[4] = {g32, g64, g128, g256};
             int best = kTestThreads;
             double best_t = 1e300;
+            // group sizes whose slice holds the class's largest table (the whole CTA's does)
+            const long long mcells = (long long)ctr->max_cells[cls];
+            auto fits = [&](int G) { return G >= kTestThreads || mcells <= slice_cells(smem_ints * G / kTestThreads, need_marg); };
             for (int k = 0; k < 4; ++k) {
                 const int G = 32 << k;
+                if (!fits(G)) continue;
                 const double rounds = (double)((W + groups[k] - 1) / groups[k]);
                 const double t = rounds * (kTestOverhead + kCyclesPerSample * mean_n / G);
                 if (t < best_t) {
@@ -319,7 +323,9 @@ __global__ void k_scan(ScanClass c0, ScanClass c1, DepthCounters* ctr, double me
             }
             // the caller's choice, the autotuner's for this depth, or the cost model's
             const int tuned = tune_code(ctr->tune, ctr->d) & kTuneGroupMask;
-            ctr->gsel = forced_group ? forced_group : tuned ? tuned : best;
+            int G = forced_group ? forced_group : tuned ? tuned : best;
+            while (!fits(G)) G *= 2;
+            ctr->gsel = G;
         }
         // sample split: few single-rank tests against the groups of the class
         const int G = cls == 0 ? ctr->gsel : kTestThreads;
@@ -627,11 +633,11 @@ void launch_edges(const ProblemDev* probs, const int32_t* vtx_prob, const int32_
 
 void launch_order(const ProblemDev* probs, const EdgeWork* edges, long long edge_cap, int nclass, DepthCounters* ctr,
                   const ScanClass* sc, unsigned long long* cursor0, unsigned long long* cursor1, int32_t* sorted,
-                  double mean_n, int forced_group, long long split_stride, int allow_split, int marg, int grid,
-                  cudaStream_t st)
+                  double mean_n, int forced_group, long long split_stride, int allow_split, int marg, int need_marg,
+                  int grid, cudaStream_t st)
 {
     launch_pdl(k_scan, dim3(nclass), dim3(256), 0, st, sc[0], sc[nclass > 1 ? 1 : 0], ctr, mean_n, forced_group,
-               split_stride, allow_split, marg);
+               split_stride, allow_split, marg, need_marg);
     launch_pdl(k_place, dim3(grid), dim3(256), 0, st, probs, edges, edge_cap, nclass, ctr, (const unsigned long long*)sc[0].alive,
                cursor0, (const unsigned long long*)sc[nclass > 1 ? 1 : 0].alive, cursor1, sorted);
 }
@@ -639,7 +645,7 @@ void launch_order(const ProblemDev* probs, const EdgeWork* edges, long long edge
 void launch_pool(const PoolArgs& a, int cls, int grid, size_t smem_bytes, cudaStream_t st)
 {
     if (cls == kClassWarp) launch_pdl(k_pool_small, dim3(grid), dim3(kTestThreads), smem_bytes, st, a);
-    else launch_pdl(k_pool_big, dim3(grid), dim3(kTestThreads), smem_bytes, st, a);
+    else launch_pdl(k_pool_big, dim3(grid), dim3(kBigThreads), smem_bytes, st, a);
 }
 
 void launch_pool_marg(const PoolArgs& a, int grid, cudaStream_t st)
@@ -701,12 +707,12 @@ void set_pdl(bool on)
     g_pdl = on;
 }
 
-cudaError_t set_kernel_smem(size_t max_smem)
+cudaError_t set_kernel_smem(size_t small_smem, size_t big_smem, size_t plain_smem)
 {
     cudaError_t e;
-    const int b = (int)max_smem;
-    if ((e = cudaFuncSetAttribute(k_pool_small, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
-    if ((e = cudaFuncSetAttribute(k_pool_big, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
+    const int b = (int)plain_smem;
+    if ((e = cudaFuncSetAttribute(k_pool_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)small_smem))) return e;
+    if ((e = cudaFuncSetAttribute(k_pool_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)big_smem))) return e;
     if ((e = cudaFuncSetAttribute(k_plain, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
     return cudaSuccess;
 }
@@ -719,7 +725,7 @@ int pool_blocks_per_sm(int cls, size_t smem_bytes)
     else if (cls == kClassWarp)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pool_small, kTestThreads, smem_bytes);
     else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pool_big, kTestThreads, smem_bytes);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pool_big, kBigThreads, smem_bytes);
     return nb;
 }
 

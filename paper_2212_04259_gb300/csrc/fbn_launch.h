@@ -20,11 +20,12 @@ void launch_edges(const ProblemDev* probs, const int32_t* vtx_prob, const int32_
                   unsigned long long* hist, cudaStream_t st);
 // Ordering of the depth's edges, one CTA per class (nclass = 1: the small-
 // table class only), then the placement of both classes.
-// marg: the depth's pool is k_pool_marg.
+// marg: the depth's pool is k_pool_marg.  need_marg: the pools keep a table's
+// marginals beside it (no n ln n table).
 void launch_order(const ProblemDev* probs, const EdgeWork* edges, long long edge_cap, int nclass, DepthCounters* ctr,
                   const ScanClass* sc, unsigned long long* cursor0, unsigned long long* cursor1, int32_t* sorted,
-                  double mean_n, int forced_group, long long split_stride, int allow_split, int marg, int grid,
-                  cudaStream_t st);
+                  double mean_n, int forced_group, long long split_stride, int allow_split, int marg, int need_marg,
+                  int grid, cudaStream_t st);
 void launch_pool(const PoolArgs& a, int cls, int grid, size_t smem_bytes, cudaStream_t st);
 void launch_pool_marg(const PoolArgs& a, int grid, cudaStream_t st);
 void launch_pairs_popc(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first, int total_vertices,
@@ -50,7 +51,7 @@ void set_pdl(bool on);
 // Explicit tests: the kernel's limits and its largest cluster, then one test.
 cudaError_t prepare_ci(size_t smem_bytes, int* max_cluster);
 cudaError_t launch_ci(const CiArgs& q, int cluster, size_t smem_bytes, cudaStream_t st);
-cudaError_t set_kernel_smem(size_t max_smem);
+cudaError_t set_kernel_smem(size_t small_smem, size_t big_smem, size_t plain_smem);
 // Sets the message fbn_last_error(NULL) returns.
 void fbn_internal_set_error(const char* msg);
 int pool_blocks_per_sm(int cls, size_t smem_bytes);

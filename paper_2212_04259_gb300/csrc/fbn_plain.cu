@@ -6,7 +6,7 @@ namespace fbn {
 __global__ void __launch_bounds__(kTestThreads, 2) k_plain(PoolArgs a)
 {
     pdl_enter();
-    extern __shared__ int smem[];
+    extern __shared__ __align__(16) int smem[];
     __shared__ TestSpec spec;
     __shared__ GroupState S;
     __shared__ double red[32];

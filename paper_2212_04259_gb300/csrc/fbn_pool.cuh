@@ -27,6 +27,7 @@ struct GroupState {
     int go;
     double crit;       // exact critical value, 0 until the exact decision needs it
     float crit_lo, crit_hi;
+    long long crit_q;  // floor(crit / 2) of the n ln n decision
     int pos[kMaxD];
 };
 
@@ -82,9 +83,10 @@ __device__ __forceinline__ bool setup_rank(const ProblemDev& P, const EdgeWork& 
 // declared arities or from the observed table (no degree of freedom left:
 // the test cannot reject), crit from the cache, then the bounded statistic.
 template <int G>
-__device__ __forceinline__ int decide_test(const PoolArgs& a, const TestSpec& spec, const int* T, const int* M,
-                                           GroupState& S, double* red, unsigned* status)
+__device__ __noinline__ int decide_test(const PoolArgs& a, const TestSpec& spec, const int* T, int* M,
+                                        GroupState& S, double* red, unsigned* status)
 {
+    grp_marginals<G>(spec, T, M);
     const int nz = (int)spec.cells / (spec.rx * spec.ry);   // cells <= kMaxCells < 2^31: 32-bit
     const long long df = a.df_mode ? grp_df_adjusted<G>(spec, M, red)
                                    : (long long)((spec.rx - 1) * (spec.ry - 1)) * nz;
@@ -114,6 +116,32 @@ __device__ __forceinline__ int decide_test(const PoolArgs& a, const TestSpec& sp
     return ex < S.crit ? 1 : 0;
 }
 
+// G^2 with the declared df from the n ln n table; FP64 when the error bound
+// straddles crit.
+template <int G>
+__device__ __forceinline__ int decide_lut(const PoolArgs& a, const TestSpec& spec, const int* T, GroupState& S,
+                                          double* red, unsigned* status)
+{
+    const int nz = (int)spec.cells / (spec.rx * spec.ry);
+    const long long df = (long long)((spec.rx - 1) * (spec.ry - 1)) * nz;
+    if (Grp<G>::rank() == 0) {
+        long long q = df < a.crit.dense_n ? a.crit.dense_q[df] : 0;
+        if (q == 0) q = (long long)floor(crit_get(a.crit, df, a.alpha, status) * 0.5 * 68719476736.0);   // 2^kLutBits
+        S.crit_q = q;
+        S.tests += 1;   // flushed to the depth counter when the group leaves the pool
+    }
+    const long long g = grp_g2_lut<G>(spec, T, a.lut, red);
+    Grp<G>::sync();
+    const long long q = S.crit_q;
+    const long long err = a.lut_err * ((long long)spec.cells + (long long)nz * (spec.rx + spec.ry + 1));
+    if (g + err < q) return 1;
+    if (g - err > q) return 0;   // q + 1 bounds crit from above
+    const double ex = grp_g2_cells<G>(spec, T, red);
+    if (Grp<G>::rank() == 0) S.crit = crit_get(a.crit, df, a.alpha, status);
+    Grp<G>::sync();
+    return ex < S.crit ? 1 : 0;
+}
+
 // Run one rank: 1 = accepts independence, 0 = rejects, -1 = could not run.
 // Counting work of one table (rank 0): one shared-memory update per sample.
 template <int G>
@@ -131,7 +159,7 @@ __device__ __forceinline__ int run_rank(const PoolArgs& a, int d, const ProblemD
     unsigned* status = &a.ctr->status;
     if (!setup_rank<G>(P, w, d, rk, fresh, S, a.binom, spec, status)) return -1;
     int* M = nullptr;
-    const int* T = grp_table<G>(spec, slice, slice_ints, gtab, a.gscratch_ints, &M);
+    const int* T = grp_table<G>(spec, slice, slice_ints, gtab, a.gscratch_ints, a.lut == nullptr, &M);
     if (!T) {   // the global scratch is too small: the host grows it and starts over
         if (Grp<G>::rank() == 0) {
             atomicOr(status, kStatusScratch);
@@ -140,8 +168,7 @@ __device__ __forceinline__ int run_rank(const PoolArgs& a, int d, const ProblemD
         return -1;
     }
     note_work<G>(S, spec);
-    grp_marginals<G>(spec, T, M);
-    return decide_test<G>(a, spec, T, M, S, red, status);
+    return a.lut ? decide_lut<G>(a, spec, T, S, red, status) : decide_test<G>(a, spec, T, M, S, red, status);
 }
 
 // One part of a split test: count samples [N p / S, N (p + 1) / S) (16-aligned
@@ -171,7 +198,7 @@ __device__ __noinline__ int run_split_part(const PoolArgs& a, int d, const Probl
         if (r == 0) spec.N = (int)(hi - lo);
         Grp<G>::sync();
         int* M = nullptr;
-        const int* T = grp_table<G>(spec, slice, slice_ints, gtab, a.gscratch_ints, &M);
+        const int* T = grp_table<G>(spec, slice, slice_ints, gtab, a.gscratch_ints, a.lut == nullptr, &M);
         if (!T) {
             if (r == 0) {
                 atomicOr(status, kStatusScratch);
@@ -205,9 +232,8 @@ __device__ __noinline__ int run_split_part(const PoolArgs& a, int d, const Probl
     }
     Grp<G>::sync();
     if (!S.go) return 0;
-    int* M = Tl + C;
-    grp_marginals<G>(spec, Tl, M);
-    return decide_test<G>(a, spec, Tl, M, S, red, status);
+    return a.lut ? decide_lut<G>(a, spec, Tl, S, red, status)
+                 : decide_test<G>(a, spec, Tl, Tl + C, S, red, status);
 }
 
 // Shared state of a pool CTA, sized for the most groups per CTA (8 warps).
@@ -221,7 +247,7 @@ struct PoolShared {
 template <int G>
 __device__ __forceinline__ void pool_body(const PoolArgs& a, int* smem, PoolShared& sh)
 {
-    constexpr int NG = kTestThreads / G;   // groups per CTA
+    constexpr int NG = G >= kTestThreads ? 1 : kTestThreads / G;   // groups per CTA
     const DepthCounters* ctr = a.ctr;
     const int d = ctr->d;
     const long long maxc = (long long)ctr->maxc[a.cls];
