@@ -18,6 +18,7 @@
 #include "../../include/fbn.h"
 #include "fbn_ci.cuh"
 #include "fbn_gram.h"
+#include "fbn_loop.h"
 #include "fbn_nbr.h"
 #include "fbn_sepsets.h"
 #include "fbn_launch.h"
@@ -32,6 +33,15 @@ constexpr size_t kSmemBytes = 100 * 1024;     // dynamic shared memory of a CTA 
 constexpr long long kSplitStride = 4096;        // cells of a split test's global table at most
 constexpr size_t kWarpSmemBytes = 64 * 1024;  // dynamic shared memory of a CTA of the small-table pool (2 CTAs / SM)
 constexpr size_t kBigSmemBytes = 200 * 1024;  // the same of the big-table pool (one CTA of 1,024 threads / SM)
+// Variables of a call whose skeleton runs as one persistent kernel; above, the
+// kernels of a depth as a graph: with more variables the phases fill the chip
+// and a depth's fixed cost (37-41 us as kernels, 25-30 in the loop) no longer
+// shows.  Learning and reading 20 variables x 5,000 samples 282 -> 182 us, 40 x
+// 50,000 405 -> 310 us, 101 x 9,973 460 -> 385 us.  Up to kLoopOneCta variables
+// one CTA per SM instead of two (20 variables: 157 us against 170 to learn; 101:
+// 359 both, with depth 1 at 64 against 49 us).
+constexpr int kLoopVertices = 512;
+constexpr int kLoopOneCta = 32;
 constexpr int kCritCap = 8192;                // critical-value cache slots (power of two)
 constexpr int kCritDense = 8192;              // critical values kept in a dense table: df < kCritDense
 
@@ -171,7 +181,7 @@ struct Workspace {
     long long shard_cap = 0;
     unsigned long long* d_shard_count = nullptr;
     // launch geometry of the device, fixed once (kernel attributes set)
-    int dev_sms = 0, grid_small = 0, grid_big = 0, grid_marg = 0;
+    int dev_sms = 0, grid_small = 0, grid_big = 0, grid_marg = 0, grid_loop = 0;
     // the problem descriptors and vertex maps as last uploaded (skipped when
     // unchanged), staged through pinned memory
     std::vector<uint8_t> up_last;
@@ -182,6 +192,10 @@ struct Workspace {
     size_t h_tot_cap = 0;
     uint8_t* h_stage = nullptr;
     size_t h_stage_cap = 0;
+    unsigned* d_bar = nullptr;                      // barrier of the persistent loop
+    unsigned* d_bits = nullptr;                     // its adjacency bit matrix
+    uint8_t* h_adj = nullptr;                       // pinned: the adjacency it leaves
+    size_t h_adj_cap = 0;
     int gram_n_units = 0, gram_unit_slices = 0;
     std::vector<uint8_t> h_maps;
     // one-hot layout of the last prepare_gram and the last one whose pad rows
@@ -215,6 +229,8 @@ struct Workspace {
         if (h_up) cudaFreeHost(h_up);
         if (h_tot) cudaFreeHost(h_tot);
         if (h_stage) cudaFreeHost(h_stage);
+        if (h_adj) cudaFreeHost(h_adj);
+        dfree(d_bar); dfree(d_bits);
         h_maps.clear();
         gram_E = nullptr; gram_G = nullptr; gram_R = nullptr; gram_maps = nullptr; gram_units = nullptr; pk = nullptr;
         split_tab = nullptr; split_ticket = nullptr;
@@ -277,7 +293,9 @@ struct fbn_handle {
     int32_t* d_off = nullptr;           // [n] sum of the arities before each variable; [n] the same of arities - 1
     // results of the last skeleton
     bool learnt = false;
-    bool sep_pending = false;           // separating sets still only on the device
+    bool sep_pending = false;           // separating sets not in the csr vectors yet
+    bool sep_staged = false;            // ... but already in the pinned staging (sep_R pairs, sep_M members)
+    long long sep_R = 0, sep_M = 0;
     unsigned long long sep_pool_used = 0;
     // members of a batch's separating sets: a device copy of the batch's
     // shared pool, held by every handle of that batch until it learns again
@@ -739,6 +757,11 @@ int materialize_sepsets(fbn_handle* h, Workspace& ws)
         q->sep_pending = false;
     };
     int rc = FBN_OK;
+    if (h->sep_staged) {   // the skeleton's own kernel left them in the staging
+        unpack(h, ws.h_stage, (long long)h->n * (h->n - 1) / 2, h->sep_R, h->sep_M);
+        h->sep_staged = false;
+        return FBN_OK;
+    }
     if (k == 1) {
         fbn_handle* q = todo[0];
         const long long Rmax = (long long)q->n * (q->n - 1) / 2;
@@ -895,7 +918,9 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         }
     }
     long long launches = 0;
-    if (!gram) {   // the complete graph (the Gram's decisions write every pair themselves)
+    const bool persistent = !shard && !plain && !gram && !nbr1 && h->opt.loop == FBN_LOOP_DEVICE &&
+                            total_vtx <= kLoopVertices;
+    if (!gram && !persistent) {   // the complete graph (the Gram's decisions write every pair themselves)
         k_init_graph<<<total_vtx, 256, 0, st>>>(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx);
         CK(cudaGetLastError());
         launches = 1;
@@ -913,6 +938,9 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         ws.grid_small = sms * std::max(1, pool_blocks_per_sm(kClassWarp, kWarpSmemBytes));
         ws.grid_big = sms * std::max(1, pool_blocks_per_sm(kClassCta, kBigSmemBytes));
         ws.grid_marg = sms * std::max(1, pool_blocks_per_sm(kClassMarg, 0));
+        int per_sm = 0;
+        CK(prepare_loop(kWarpSmemBytes, &per_sm));
+        ws.grid_loop = sms * std::min(2, per_sm);
         ws.dev_sms = sms;
     }
     const int dev_sms = ws.dev_sms, grid_small = ws.grid_small, grid_big = ws.grid_big, grid_marg = ws.grid_marg;
@@ -954,9 +982,11 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     }
     CritTableDev ct{ws.crit_keys, ws.crit_vals, kCritCap, kCritDense, ws.crit_dense, ws.crit_dense_f, ws.crit_dense_q};
 
-    CK(cudaMemsetAsync(ws.d_rec, 0, kMaxDepthRecords * sizeof(DepthRecord), st));
-    CK(cudaMemsetAsync(ws.hist, 0, 2 * ws.ord_cap * sizeof(unsigned long long), st));
-    CK(cudaMemsetAsync(ws.cursor, 0, 2 * ws.ord_cap * sizeof(unsigned long long), st));
+    if (!persistent) {
+        CK(cudaMemsetAsync(ws.d_rec, 0, kMaxDepthRecords * sizeof(DepthRecord), st));
+        CK(cudaMemsetAsync(ws.hist, 0, 2 * ws.ord_cap * sizeof(unsigned long long), st));
+        CK(cudaMemsetAsync(ws.cursor, 0, 2 * ws.ord_cap * sizeof(unsigned long long), st));
+    }
     if (h->tune != ws.tune_loaded) {   // the autotuner's per-depth choices
         std::vector<int> t(kMaxDepthRecords, 0);
         for (size_t d = 0; d < h->tune.size() && d < t.size(); ++d) t[d] = h->tune[d];
@@ -968,7 +998,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     c0.tune = h->tune.empty() ? nullptr : ws.d_tune;
     c0.rec = ws.d_rec;
     *ws.h_ctr = c0;
-    CK(cudaMemcpyAsync(ws.d_ctr, ws.h_ctr, sizeof(DepthCounters), cudaMemcpyHostToDevice, st));
+    if (!persistent) CK(cudaMemcpyAsync(ws.d_ctr, ws.h_ctr, sizeof(DepthCounters), cudaMemcpyHostToDevice, st));
 
     PoolArgs base{};
     base.probs = ws.probs;
@@ -1121,7 +1151,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     // device-driven while loop whose body tests a depth, removes its edges,
     // ends it and lists the next depth's edges (k_gate: go on or stop).
     // Captured once per configuration: every argument it holds is in the key.
-    if (!shard) {
+    if (!shard && !persistent) {
         std::vector<uint8_t> key;
         auto put = [&](const void* p, size_t n) {
             const uint8_t* b = (const uint8_t*)p;
@@ -1158,9 +1188,93 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
 
     fbn_stats stats{};
     int d_loop = 0;   // first depth of the graph loop
+    const bool direct_out = persistent && k == 1;
+    const long long* h_tot = nullptr;
+    if (persistent) {
+        LoopArgs la{};
+        la.probs = ws.probs;
+        la.vtx_prob = ws.vtx_prob;
+        la.vtx_first = ws.vtx_first;
+        la.total_vertices = total_vtx;
+        la.max_n = max_n;
+        la.gs_forced = gs_forced;
+        la.gs_edges = gs_edges;
+        la.binom = ws.binom;
+        la.brows = ws.brows;
+        la.warp_cells_cap = wcap;
+        la.edges = ws.edges;
+        la.min_accept = ws.min_accept;
+        la.edge_cap = ws.edge_cap;
+        la.ctr = ws.d_ctr;
+        la.hist = ws.hist;
+        la.cursor = ws.cursor;
+        la.ord_cap = ws.ord_cap;
+        const int grid = total_vtx <= kLoopOneCta ? dev_sms : ws.grid_loop;
+        for (int cls = 0; cls < 2; ++cls) {
+            la.sc[cls].hist = ws.hist + cls * ws.ord_cap;
+            la.sc[cls].alive = ws.alive + cls * ws.ord_cap;
+            la.sc[cls].base = ws.base + cls * ws.ord_cap;
+            for (int q = 0; q < 4; ++q) la.sc[cls].groups[q] = cls == 0 ? ((long long)grid * 8) >> q : grid;
+            la.sc[cls].smem_ints = (long long)(kWarpSmemBytes / 4);
+        }
+        la.sorted = ws.sorted;
+        la.mean_n = mean_n;
+        la.forced_group = forced;
+        la.split_stride = kSplitStride;
+        la.need_marg = !use_lut;
+        la.sep_pool = ws.sep_pool;
+        la.sep_cap = ws.sep_cap;
+        la.rec = ws.d_rec;
+        la.max_depth = max_depth;
+        la.popc0 = popc0;
+        la.marg1 = marg1;
+        la.small = base;
+        la.small.cls = kClassWarp;
+        la.small.smem_ints = (int)(kWarpSmemBytes / 4);
+        la.small.base = ws.base;
+        la.big = la.small;
+        la.big.cls = kClassCta;
+        la.big.base = ws.base + ws.ord_cap;
+        if (ws.gs_cells > 0) {
+            la.big.gscratch = ws.gscratch;
+            la.big.gscratch_ints = 3 * ws.gs_cells + 64;
+        }
+        la.spin_limit = 1u << 23;   // seconds
+        if (!ws.d_bar) {
+            CK(dalloc(&ws.d_bar, 2));
+            CK(cudaMemsetAsync(ws.d_bar, 0, 2 * sizeof(unsigned), st));
+        }
+        la.bar = ws.d_bar;
+        if (k == 1 && h->n <= kTurnVertices) {
+            if (!ws.d_bits) CK(dalloc(&ws.d_bits, kTurnVertices * (kTurnVertices / 32)));
+            la.bits = ws.d_bits;
+        }
+        la.init = c0;
+        if (direct_out) {   // one problem: every result straight to the host
+            const long long R = edge_cap;
+            CK(grow_pinned(&ws.h_adj, &ws.h_adj_cap, ((size_t)h->n * h->n + 15) / 16 * 16));
+            const size_t csr = (size_t)R * (2 * sizeof(int32_t) + sizeof(int64_t)) + (size_t)ws.sep_cap * sizeof(int32_t);
+            CK(grow_pinned(&ws.h_stage, &ws.h_stage_cap, (csr + 15) / 16 * 16 + 16));
+            if (!h->d_sep_cnt) CK(dalloc(&h->d_sep_cnt, 4 * (size_t)h->n + 4));
+            uint8_t* stage = nullptr;
+            CK(cudaHostGetDevicePointer((void**)&la.h_ctr, ws.h_ctr, 0));
+            CK(cudaHostGetDevicePointer((void**)&la.h_rec, ws.h_rec, 0));
+            CK(cudaHostGetDevicePointer((void**)&stage, ws.h_stage, 0));
+            if (adj_out && adj_out[0]) CK(cudaHostGetDevicePointer((void**)&la.h_adj, ws.h_adj, 0));
+            la.h_pairs = reinterpret_cast<int32_t*>(stage);   // as materialize_sepsets lays it out
+            la.h_offs = reinterpret_cast<int64_t*>(stage + 2 * (size_t)R * sizeof(int32_t));
+            la.h_members = reinterpret_cast<int32_t*>(stage + (size_t)R * (2 * sizeof(int32_t) + sizeof(int64_t)));
+            la.h_tot = reinterpret_cast<long long*>(stage + (csr + 15) / 16 * 16);
+            h_tot = reinterpret_cast<const long long*>(ws.h_stage + (csr + 15) / 16 * 16);
+            la.sep_cnt = h->d_sep_cnt;
+        }
+        if (direct_out) ws.h_ctr->status = kStatusTimeout;   // overwritten by the loop's last phase
+        CK(launch_loop(la, grid, kWarpSmemBytes, st));
+        launches += 1;
+    }
     bool direct1 = false;   // depth 1 as the neighbourhood product (timed by events)
-    if (shard) {
-        // depth by depth below
+    if (shard || persistent) {
+        // depth by depth below; one kernel above
     } else if (gram) {
         rc = run_gram(h, ws, k, total_vtx, &ws.d_ctr->status, ws.d_ctr, ws.kev[2 * FBN_MAX_DEPTHS],
                       ws.kev[2 * FBN_MAX_DEPTHS + 1]);
@@ -1184,7 +1298,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         launches += 5;
         d_loop = 1;
     }
-    if (marg1 && !shard) {
+    if (marg1 && !shard && !persistent) {
         enqueue_head(true);
         enqueue_marg();
         enqueue_tail();
@@ -1208,7 +1322,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         direct1 = true;
         d_loop = 2;
     }
-    const bool loop = max_depth < 0 || d_loop <= max_depth;
+    const bool loop = !persistent && (max_depth < 0 || d_loop <= max_depth);
     const bool host_loop = h->opt.loop == FBN_LOOP_HOST || shard;
     if (shard) {
         // Several processes learn this skeleton together (Section IV-A's
@@ -1303,13 +1417,26 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         launches += 3;
     }
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(ws.h_ctr, ws.d_ctr, sizeof(DepthCounters), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(ws.h_rec, ws.d_rec, kMaxDepthRecords * sizeof(DepthRecord), cudaMemcpyDeviceToHost, st));
-    if (adj_out)   // the adjacency goes out with the counters (dropped if the call is retried)
+    bool adj_staged = false;   // the adjacency comes from the pinned staging after the synchronisation
+    if (direct_out) {
+        if (adj_out && adj_out[0]) {
+            cudaPointerAttributes attr{};
+            const cudaError_t pe = cudaPointerGetAttributes(&attr, adj_out[0]);
+            cudaGetLastError();
+            adj_staged = pe != cudaSuccess || attr.type == cudaMemoryTypeUnregistered || attr.type == cudaMemoryTypeHost;
+        }
+    } else {
+        CK(cudaMemcpyAsync(ws.h_ctr, ws.d_ctr, sizeof(DepthCounters), cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(ws.h_rec, ws.d_rec, kMaxDepthRecords * sizeof(DepthRecord), cudaMemcpyDeviceToHost, st));
+    }
+    if (adj_out && !adj_staged)   // the adjacency goes out with the counters (dropped if the call is retried)
         for (int p = 0; p < k; ++p)
             if (adj_out[p])
                 CK(cudaMemcpyAsync(adj_out[p], hs[p]->d_adj, (size_t)hs[p]->n * hs[p]->n, cudaMemcpyDefault, st));
     CK(cudaStreamSynchronize(st));
+    if (adj_staged) std::memcpy(adj_out[0], ws.h_adj, (size_t)h->n * h->n);
+    if (persistent && (ws.h_ctr->status & kStatusTimeout))   // a barrier gave up: its counters are not whole
+        CK(cudaMemset(ws.d_bar, 0, 2 * sizeof(unsigned)));
     if (loop && !shard) launches += (long long)(body_launches - (host_loop ? 1 : 0)) * std::max(0, ws.h_ctr->d - d_loop);
     if (direct1) {
         float kms = 0.f;
@@ -1326,7 +1453,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         if (c.status & kStatusScratch) {
             if (c.need_cells <= 0 || c.need_cells > kMaxCells) return check_status(h, kStatusTooBig);
             ws.gs_cells = std::max<long long>(2 * ws.gs_cells, c.need_cells);
-            rc = ensure_gscratch(h, ws, (3 * ws.gs_cells + 64) * std::max(grid_big, grid_plain));
+            rc = ensure_gscratch(h, ws, (3 * ws.gs_cells + 64) * std::max({grid_big, grid_plain, ws.grid_loop}));
             if (rc) return rc;
         }
         *retry = true;
@@ -1378,6 +1505,11 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         hs[p]->stats = stats;
         hs[p]->learnt = true;
         hs[p]->sep_pending = true;
+        hs[p]->sep_staged = direct_out;
+        if (direct_out) {
+            hs[p]->sep_R = h_tot[0];
+            hs[p]->sep_M = h_tot[1];
+        }
         hs[p]->sep_pool_used = c.sep_used;
         set_snapshot(hs[p], snap);
     }
@@ -1768,7 +1900,7 @@ int fbn_create(const uint8_t* data, int32_t n_vars, int64_t n_samples, const uin
     h->nplanes = max_ar <= kMargMaxArity ? max_ar - 1 : 0;
     CKC(dalloc(&h->d_planes, (size_t)n_vars * h->nplanes * h->plane_ld));
     CKC(dalloc(&h->d_ar, n_vars));
-    CKC(dalloc(&h->d_adj, nn));
+    CKC(dalloc(&h->d_adj, (nn + 15) / 16 * 16));   // read in whole 16-byte words
     CKC(dalloc(&h->d_nbr, nn));
     CKC(dalloc(&h->d_eid, nn));
     CKC(dalloc(&h->d_npos, nn));

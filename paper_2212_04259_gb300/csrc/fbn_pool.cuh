@@ -258,12 +258,13 @@ __device__ __forceinline__ void pool_body(const PoolArgs& a, int* smem, PoolShar
     unsigned long long* min_accept = a.min_accept + cb;
     unsigned long long* next_item = &a.ctr->next_item[a.cls];
     const int gs = ctr->gs;
+    const bool direct = ctr->direct != 0;
     const int g = Grp<G>::gid();
     const int r = Grp<G>::rank();
     const long long slice_ints = a.smem_ints / NG;
     int* slice = smem + g * slice_ints;
     int* gtab = a.gscratch ? a.gscratch + ((long long)blockIdx.x * NG + g) * a.gscratch_ints : nullptr;
-    const bool base_in_smem = maxc + 1 <= kBaseSmem;
+    const bool base_in_smem = !direct && maxc + 1 <= kBaseSmem;
     if (base_in_smem)
         for (long long k = threadIdx.x; k <= maxc; k += blockDim.x) sh.base[k] = a.base[k];
     __syncthreads();
@@ -272,21 +273,35 @@ __device__ __forceinline__ void pool_body(const PoolArgs& a, int* smem, PoolShar
     TestSpec& spec = sh.spec[g];
     if (r == 0) S.tests = S.smem_updates = 0;
     const int split = ctr->split[a.cls] > 1 ? ctr->split[a.cls] : 1;
+    // a group's first item is its own index, the later ones come from the
+    // counter (no claim at all when there are fewer items than groups)
+    const unsigned long long all_groups = (unsigned long long)gridDim.x * NG;
+    unsigned long long own = (unsigned long long)blockIdx.x * NG + g;
 
     for (;;) {
         if (r == 0) {
-            const unsigned long long wi = atomicAdd(next_item, 1ULL);
+            unsigned long long wi = own;
+            if (wi == ~0ULL) wi = total > all_groups ? all_groups + atomicAdd(next_item, 1ULL) : total;
+            own = ~0ULL;
             const unsigned long long w = split == 1 ? wi : wi / (unsigned long long)split;
             S.item = w;
             S.part = (int)(wi - w * (unsigned long long)split);
             S.e = -1;
             if (wi < total) {
-                long long lo = 0, hi = maxc - 1;   // pass k: largest k with base[k] <= w
-                while (lo < hi) {
-                    const long long mid = (lo + hi + 1) >> 1;
-                    if (base[mid] <= w) lo = mid; else hi = mid - 1;
+                long long lo = 0;
+                int e;
+                if (direct) {
+                    const unsigned E = (unsigned)ctr->n_edges[a.cls];   // w < 2^31
+                    lo = (unsigned)w / E;
+                    e = (int)((unsigned)w - (unsigned)lo * E);
+                } else {
+                    long long hi = maxc - 1;   // pass k: largest k with base[k] <= w
+                    while (lo < hi) {
+                        const long long mid = (lo + hi + 1) >> 1;
+                        if (base[mid] <= w) lo = mid; else hi = mid - 1;
+                    }
+                    e = a.sorted[cb + (long long)(w - base[lo])];
                 }
-                const int e = a.sorted[cb + (long long)(w - base[lo])];
                 const long long tot = edges[e].total;
                 const long long cr = chunk_ranks(tot, gs);
                 const long long r0 = lo * cr;
@@ -301,6 +316,10 @@ __device__ __forceinline__ void pool_body(const PoolArgs& a, int* smem, PoolShar
         const EdgeWork w = edges[e];
         const ProblemDev& P = a.probs[w.prob];
         const long long r0 = S.r0, r1 = S.r1;
+        if (r0 >= r1) {   // past the edge's last chunk
+            Grp<G>::sync();
+            continue;
+        }
         if (split > 1) {   // single-rank items (gs = 1, no edge above kMaxPasses ranks)
             const int res = run_split_part<G>(a, d, P, w, r0, split, S, spec, slice, slice_ints, gtab, sh.red,
                                                     &min_accept[e]);

@@ -1,0 +1,90 @@
+"""Small problems as one persistent kernel against the oracle.
+
+Covered: variable counts around the bounds of the one-CTA turn (128) and of the
+persistent loop (512), small batches, a depth with more items than the turn
+lays out (the general phases take over and give back), every kind of output
+buffer, separating sets read late, twice, or never between calls, and a changing
+maximum depth on one handle.
+"""
+import numpy as np
+import pytest
+
+import bnsynth
+import oracle
+from _compare import compare
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def F():
+    from paper_2212_04259_gb300 import build
+    build.build()
+    import paper_2212_04259_gb300 as f
+    return f
+
+
+def _same(F, h, adj, ref):
+    hard, _, _ = compare(np.asarray(adj), F.fbn_export_sepsets(h), ref)
+    assert not hard, hard[:3]
+    st = F.fbn_get_stats(h)
+    if not ref.near:
+        assert st["tests_oracle"] == ref.tests and st["removed"] == ref.removed
+    return st
+
+
+@pytest.mark.parametrize("n,N,md", [(2, 100, -1), (3, 33, -1), (31, 500, -1), (33, 500, -1), (127, 300, 2), (128, 300, 2),
+                                    (129, 300, 2), (511, 150, 1), (512, 150, 1), (513, 150, 1)])
+@pytest.mark.parametrize("arities", [(2, 3, 4), (2, 6)])
+def test_sizes(F, n, N, md, arities):
+    data, ar, _ = bnsynth.make_dataset(n + N, n, max(1, int(1.2 * n) if n > 3 else 1), 3, arities, 1.0, N)
+    ref = oracle.pc_stable(data, ar, 0.05, md)
+    h = F.fbn_create(data, ar)
+    st = _same(F, h, F.fbn_learn_skeleton(h, 0.05, md), ref)
+    assert (st["launches"] == 1) == (n <= 512)
+
+
+def test_too_many_items_for_the_turn(F):
+    # nearly complete graph: depths 2 and 3 have far more conditioning sets than the turn lays out
+    rng = np.random.default_rng(4)
+    base = rng.integers(0, 8, 4000)
+    ar = np.full(40, 2, dtype=np.uint8)
+    data = np.stack([np.where(rng.random(4000) < 0.75, (base >> (k % 3)) & 1, rng.integers(0, 2, 4000)) for k in range(40)]
+                    ).astype(np.uint8)
+    ref = oracle.pc_stable(data, ar, 0.01, 3)
+    h = F.fbn_create(data, ar)
+    _same(F, h, F.fbn_learn_skeleton(h, 0.01, 3), ref)
+    assert max(ref.tests) > 40000
+
+
+def test_outputs_and_late_reads(F):
+    import torch
+    data, ar, alpha, md, _ = bnsynth.workload("small")
+    n = len(ar)
+    refs = {m: oracle.pc_stable(data, ar, alpha, m) for m in (-1, 0, 1, 2)}
+    h = F.fbn_create(data, ar)
+    for m in (-1, 1, 0, 2, -1):
+        for out in (None, np.zeros((n, n), np.uint8), torch.zeros((n, n), dtype=torch.uint8).pin_memory(),
+                    torch.zeros((n, n), dtype=torch.uint8, device="cuda")):
+            adj = F.fbn_learn_skeleton(h, alpha, m, out)
+            adj = adj.cpu().numpy() if isinstance(adj, torch.Tensor) else adj
+            assert np.array_equal(adj, refs[m].adj)
+        assert F.fbn_export_sepsets(h) == refs[m].sepsets == F.fbn_export_sepsets(h)
+    F.fbn_learn_skeleton(h, alpha, -1)          # not read before new samples arrive
+    F.fbn_update_data(h, data)
+    with pytest.raises(F.FbnError):
+        F.fbn_export_sepsets(h)
+
+
+def test_small_batch_and_members(F):
+    probs = bnsynth.batched_workload(4, first=3, n_range=(20, 60), samples_range=(500, 3000))
+    hs = [F.fbn_create(d, a) for d, a, _ in probs]
+    alone = F.fbn_learn_skeleton(hs[0], 0.05, -1)
+    adjs = F.fbn_learn_skeleton_batch(hs, 0.05, -1)
+    assert np.array_equal(alone, adjs[0])
+    for (d, a, _), h, adj in zip(probs, hs, adjs):
+        hard, _, _ = compare(adj, F.fbn_export_sepsets(h), oracle.pc_stable(d, a, 0.05, -1))
+        assert not hard
+    d, a, _ = probs[0]
+    hard, _, _ = compare(F.fbn_learn_skeleton(hs[0], 0.01, -1), F.fbn_export_sepsets(hs[0]), oracle.pc_stable(d, a, 0.01, -1))
+    assert not hard
