@@ -226,16 +226,16 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_loop(const __grid_constant_
         if (popc) {
             pairs_popc_body(a.probs, a.vtx_prob, a.vtx_first, a.total_vertices, a.max_n, nullptr, a.small);
         } else if (marg) {
-            marg_body(a.small);
+            marg_body<true>(a.small);
         } else {
             switch (ctr->gsel) {
-                case 32: pool_body<32>(a.small, smem, sh); break;
-                case 64: pool_body<64>(a.small, smem, sh); break;
-                case 128: pool_body<128>(a.small, smem, sh); break;
-                default: pool_body<kTestThreads>(a.small, smem, sh); break;
+                case 32: pool_body<32, true>(a.small, smem, sh); break;
+                case 64: pool_body<64, true>(a.small, smem, sh); break;
+                case 128: pool_body<128, true>(a.small, smem, sh); break;
+                default: pool_body<kTestThreads, true>(a.small, smem, sh); break;
             }
             __syncthreads();
-            pool_body<kTestThreads>(a.big, smem, sh);
+            pool_body<kTestThreads, true>(a.big, smem, sh);
         }
         tests_done(ctr);
         const auto next = [&] { if (a.bits) turn(a, turn_sh, direct, warps); };

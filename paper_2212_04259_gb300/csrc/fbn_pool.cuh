@@ -236,103 +236,112 @@ __device__ __noinline__ int run_split_part(const PoolArgs& a, int d, const Probl
                  : decide_test<G>(a, spec, Tl, Tl + C, S, red, status);
 }
 
-// Shared state of a pool CTA, sized for the most groups per CTA (8 warps).
+// Shared state of a pool CTA, sized for the most groups per CTA (8 warps), and
+// what a claim needs of the depth (kept here, not in every thread's registers:
+// the counting loops use all of them).
 struct PoolShared {
     TestSpec spec[kTestThreads / 32];
     GroupState st[kTestThreads / 32];
     double red[32];
-    unsigned long long base[kBaseSmem];
+    unsigned long long total, groups;   // items of the class; items taken without a claim
+    long long cb, maxc;                 // the class's first edge, its passes
+    const unsigned long long* base;     // first item of each pass
+    unsigned edges;                     // edges of the class when the items are laid out directly, else 0
+    int gs, split;
+    unsigned long long pass_base[kBaseSmem];
 };
 
-template <int G>
+// One thread of a group: item wi, or for ~0 the next one of the counter, into S
+// (e = -1: none left).
+static __device__ __noinline__ void claim_item(const PoolArgs& a, const PoolShared& sh, GroupState& S,
+                                               unsigned long long wi)
+{
+    if (wi == ~0ULL)
+        wi = sh.total > sh.groups ? sh.groups + atomicAdd(&a.ctr->next_item[a.cls], 1ULL) : sh.total;
+    S.e = -1;
+    if (wi >= sh.total) return;
+    const unsigned long long w = sh.split == 1 ? wi : wi / (unsigned long long)sh.split;
+    S.item = w;
+    S.part = (int)(wi - w * (unsigned long long)sh.split);
+    long long pass;
+    int e;
+    if (sh.edges) {   // w < 2^31
+        pass = (unsigned)w / sh.edges;
+        e = (int)((unsigned)w - (unsigned)pass * sh.edges);
+    } else {
+        long long lo = 0, hi = sh.maxc - 1;   // largest pass with base[pass] <= w
+        while (lo < hi) {
+            const long long mid = (lo + hi + 1) >> 1;
+            if (sh.base[mid] <= w) lo = mid; else hi = mid - 1;
+        }
+        pass = lo;
+        e = a.sorted[sh.cb + (long long)(w - sh.base[lo])];
+    }
+    const long long tot = a.edges[sh.cb + e].total;
+    const long long cr = chunk_ranks(tot, sh.gs);
+    const long long r0 = pass * cr;
+    S.e = e;
+    S.r0 = r0;
+    S.r1 = r0 + cr < tot ? r0 + cr : tot;
+}
+
+// LOOP: in the persistent loop a group's first item is its own index and the
+// later ones come from the counter (no claim at all with fewer items than
+// groups: one round trip less on a small problem's critical path).
+template <int G, bool LOOP = false>
 __device__ __forceinline__ void pool_body(const PoolArgs& a, int* smem, PoolShared& sh)
 {
     constexpr int NG = G >= kTestThreads ? 1 : kTestThreads / G;   // groups per CTA
-    const DepthCounters* ctr = a.ctr;
-    const int d = ctr->d;
-    const long long maxc = (long long)ctr->maxc[a.cls];
-    const unsigned long long total = ctr->total_items[a.cls];
-    if (total == 0) return;
-    const long long cb = class_base(ctr, a.cls, a.edge_cap);
-    const EdgeWork* edges = a.edges + cb;
-    unsigned long long* min_accept = a.min_accept + cb;
-    unsigned long long* next_item = &a.ctr->next_item[a.cls];
-    const int gs = ctr->gs;
-    const bool direct = ctr->direct != 0;
+    const int d = a.ctr->d;
+    if (a.ctr->total_items[a.cls] == 0) return;
     const int g = Grp<G>::gid();
     const int r = Grp<G>::rank();
+    if (threadIdx.x == 0) {
+        const DepthCounters* ctr = a.ctr;
+        sh.total = ctr->total_items[a.cls];
+        sh.groups = LOOP ? (unsigned long long)gridDim.x * NG : 0;
+        sh.cb = class_base(ctr, a.cls, a.edge_cap);
+        sh.maxc = (long long)ctr->maxc[a.cls];
+        sh.edges = ctr->direct ? (unsigned)ctr->n_edges[a.cls] : 0u;
+        sh.base = !sh.edges && sh.maxc + 1 <= kBaseSmem ? sh.pass_base : a.base;
+        sh.gs = ctr->gs;
+        sh.split = ctr->split[a.cls] > 1 ? ctr->split[a.cls] : 1;
+    }
+    __syncthreads();
+    if (sh.base == sh.pass_base)
+        for (long long k = threadIdx.x; k <= sh.maxc; k += blockDim.x) sh.pass_base[k] = a.base[k];
     const long long slice_ints = a.smem_ints / NG;
     int* slice = smem + g * slice_ints;
     int* gtab = a.gscratch ? a.gscratch + ((long long)blockIdx.x * NG + g) * a.gscratch_ints : nullptr;
-    const bool base_in_smem = !direct && maxc + 1 <= kBaseSmem;
-    if (base_in_smem)
-        for (long long k = threadIdx.x; k <= maxc; k += blockDim.x) sh.base[k] = a.base[k];
-    __syncthreads();
-    const unsigned long long* base = base_in_smem ? sh.base : a.base;
     GroupState& S = sh.st[g];
     TestSpec& spec = sh.spec[g];
     if (r == 0) S.tests = S.smem_updates = 0;
-    const int split = ctr->split[a.cls] > 1 ? ctr->split[a.cls] : 1;
-    // a group's first item is its own index, the later ones come from the
-    // counter (no claim at all when there are fewer items than groups)
-    const unsigned long long all_groups = (unsigned long long)gridDim.x * NG;
-    unsigned long long own = (unsigned long long)blockIdx.x * NG + g;
+    __syncthreads();
 
-    for (;;) {
-        if (r == 0) {
-            unsigned long long wi = own;
-            if (wi == ~0ULL) wi = total > all_groups ? all_groups + atomicAdd(next_item, 1ULL) : total;
-            own = ~0ULL;
-            const unsigned long long w = split == 1 ? wi : wi / (unsigned long long)split;
-            S.item = w;
-            S.part = (int)(wi - w * (unsigned long long)split);
-            S.e = -1;
-            if (wi < total) {
-                long long lo = 0;
-                int e;
-                if (direct) {
-                    const unsigned E = (unsigned)ctr->n_edges[a.cls];   // w < 2^31
-                    lo = (unsigned)w / E;
-                    e = (int)((unsigned)w - (unsigned)lo * E);
-                } else {
-                    long long hi = maxc - 1;   // pass k: largest k with base[k] <= w
-                    while (lo < hi) {
-                        const long long mid = (lo + hi + 1) >> 1;
-                        if (base[mid] <= w) lo = mid; else hi = mid - 1;
-                    }
-                    e = a.sorted[cb + (long long)(w - base[lo])];
-                }
-                const long long tot = edges[e].total;
-                const long long cr = chunk_ranks(tot, gs);
-                const long long r0 = lo * cr;
-                S.e = e;
-                S.r0 = r0;
-                S.r1 = r0 + cr < tot ? r0 + cr : tot;
-            }
-        }
+    for (bool first = LOOP;; first = false) {
+        if (r == 0) claim_item(a, sh, S, first ? (unsigned long long)g * gridDim.x + blockIdx.x : ~0ULL);
         Grp<G>::sync();
-        const int e = S.e;
-        if (e < 0) break;
-        const EdgeWork w = edges[e];
+        if (S.e < 0) break;
+        const EdgeWork w = a.edges[sh.cb + S.e];
         const ProblemDev& P = a.probs[w.prob];
+        unsigned long long* min_accept = a.min_accept + sh.cb + S.e;
         const long long r0 = S.r0, r1 = S.r1;
         if (r0 >= r1) {   // past the edge's last chunk
             Grp<G>::sync();
             continue;
         }
-        if (split > 1) {   // single-rank items (gs = 1, no edge above kMaxPasses ranks)
-            const int res = run_split_part<G>(a, d, P, w, r0, split, S, spec, slice, slice_ints, gtab, sh.red,
-                                                    &min_accept[e]);
-            if (res == 1 && r == 0) atomicMin(&min_accept[e], (unsigned long long)r0);
+        if (sh.split > 1) {   // single-rank items (gs = 1, no edge above kMaxPasses ranks)
+            const int res = run_split_part<G>(a, d, P, w, r0, sh.split, S, spec, slice, slice_ints, gtab, sh.red, min_accept);
+            if (res == 1 && r == 0) atomicMin(min_accept, (unsigned long long)r0);
             Grp<G>::sync();
             continue;
         }
         for (long long rk = r0; rk < r1; ++rk) {
-            if (r == 0) S.go = (unsigned long long)rk <= *((volatile unsigned long long*)&min_accept[e]);
+            if (r == 0) S.go = (unsigned long long)rk <= *((volatile unsigned long long*)min_accept);
             Grp<G>::sync();
             if (!S.go) break;
             const int res = run_rank<G>(a, d, P, w, rk, rk == r0, S, spec, slice, slice_ints, gtab, sh.red);
-            if (res == 1 && r == 0) atomicMin(&min_accept[e], (unsigned long long)rk);
+            if (res == 1 && r == 0) atomicMin(min_accept, (unsigned long long)rk);
             if (res != 0) break;
         }
         Grp<G>::sync();

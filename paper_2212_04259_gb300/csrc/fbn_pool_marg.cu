@@ -7,7 +7,7 @@ __global__ void __launch_bounds__(kMargThreads, 2) k_pool_marg(PoolArgs a)
 {
     pdl_enter();
     if (!a.ctr->active) return;
-    marg_body(a);
+    marg_body<false>(a);
     tests_done(a.ctr);
 }
 

@@ -292,6 +292,11 @@ __device__ __forceinline__ int marg_test(const PoolArgs& a, const ProblemDev& P,
 // without an instruction, 8.0 ms; the loops of one shape together: 6.0 ms), then
 // the loads of a pass (the next word's planes in flight: 5.4 ms).  Two CTAs of
 // 128 registers: three (80 registers, spills) 6.7 ms, five of 128 threads 6.2 ms.
+// LOOP: in the persistent loop, where the items may be laid out directly and a
+// warp's first item is its own index (a claim less on the critical path; with
+// many items the counter's order is the better one: depth 1 of 20 problems 0.64
+// against 0.68 ms).
+template <bool LOOP>
 __device__ __forceinline__ void marg_body(const PoolArgs& a)
 {
     __shared__ unsigned long long s_base[kBaseSmem];
@@ -300,7 +305,7 @@ __device__ __forceinline__ void marg_body(const PoolArgs& a)
     const unsigned long long total = ctr->total_items[kClassWarp];
     if (total == 0) return;
     const int lane = threadIdx.x & 31, lx = lane / kMA, ly = lane - lx * kMA;
-    const bool whole = ctr->whole != 0, direct = ctr->direct != 0;
+    const bool whole = ctr->whole != 0, direct = LOOP && ctr->direct != 0;
     const int gs = ctr->gs;
     const long long maxc = (long long)ctr->maxc[kClassWarp];
     const bool base_in_smem = !whole && !direct && maxc + 1 <= kBaseSmem;
@@ -309,13 +314,12 @@ __device__ __forceinline__ void marg_body(const PoolArgs& a)
     __syncthreads();
     const unsigned long long* base = base_in_smem ? s_base : a.base;
     unsigned long long tests = 0, work = 0;
-    // a warp's first item is its own index, the later ones come from the counter
-    const unsigned long long all_warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-    bool first = true;
+    const unsigned long long all_warps = LOOP ? (unsigned long long)gridDim.x * (blockDim.x >> 5) : 0;
+    bool first = LOOP;
     for (;;) {
-        unsigned long long wi = (unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+        unsigned long long wi = (unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
         if (!first) {
-            if (total <= all_warps) break;
+            if (LOOP && total <= all_warps) break;
             if (lane == 0) wi = all_warps + atomicAdd(&a.ctr->next_item[kClassWarp], 1ULL);
             wi = __shfl_sync(0xffffffffu, wi, 0);
         }
