@@ -59,41 +59,84 @@ void dfree(void* p)
 }
 
 // ---- small kernels of the host engine ------------------------------------
-// One pass over new samples: the first value at or above its arity (row-major
-// index over n x N), and the one-hot planes (nplanes > 0).  One thread per
-// 32-sample word: two 16-byte loads, four comparisons per 32-bit word and
-// value; a multiply gathers a word's four comparison bits.  The rows' zero
-// padding covers the words past the samples.  (Checking and planes took two
-// passes before, the check one byte per thread and load.)
-__global__ void k_ingest(const uint8_t* __restrict__ data, int64_t ld, int64_t N, const uint8_t* __restrict__ ar,
-                         int nplanes, int64_t wp, uint32_t* __restrict__ planes, unsigned long long* first_bad)
+// One pass over new samples (a row per grid.y): into the padded store (data;
+// nullptr: they are there already), the first value at or above its arity
+// (row-major index over n x N), and the one-hot planes (nplanes > 0).  The
+// samples come from any device-addressable memory, pinned host memory included,
+// at any alignment: a CTA reads its 8,192 samples as whole aligned 16-byte words
+// into shared memory and every thread shifts its 32 samples out of it.  Bounded
+// by the host link (206 GB/s measured): one pass per data set, where a strided
+// copy, a check and the planes took 40 us for 2.4 MB, three times its transfer.
+constexpr int kIngestSamples = 8192;   // per CTA and step: 32 a thread
+
+__global__ void __launch_bounds__(256) k_ingest(const uint8_t* src, int64_t stride, const uint8_t* src_end, int64_t N,
+                                                int64_t ld, const uint8_t* __restrict__ ar, int nplanes, int64_t wp,
+                                                uint8_t* data, uint32_t* __restrict__ planes,
+                                                unsigned long long* first_bad)
 {
-    const int v = blockIdx.y;
+    constexpr int kWords = kIngestSamples / 4 + 4;
+    __shared__ unsigned s_w[kWords + kWords / 32 + 1];   // word i at i + i / 32: no bank conflicts at 8 words a thread
+    const int v = blockIdx.y, tid = threadIdx.x;
     const int r = ar[v];
     const unsigned rr = 0x01010101u * (unsigned)r;
-    const uint8_t* row = data + (long long)v * ld;
     const int values = nplanes > 0 ? r - 1 : 0;
-    for (long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x; w < wp; w += (long long)gridDim.x * blockDim.x) {
-        const uint4* p = reinterpret_cast<const uint4*>(row + w * 32);
-        const uint4 a = p[0], b = p[1];
-        const unsigned q[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-        unsigned bad = 0;
+    const long long words = data ? ld / 32 : wp;
+    for (long long s0 = (long long)blockIdx.x * kIngestSamples; s0 < words * 32; s0 += (long long)gridDim.x * kIngestSamples) {
+        const long long left = N - s0;
+        const int cnt = left <= 0 ? 0 : left < kIngestSamples ? (int)left : kIngestSamples;
+        const uint8_t* at = src + v * stride + s0;
+        const int skip = (int)((uintptr_t)at & 15);
+        const uint8_t* at0 = at - skip;
+        for (int c = tid; c < (cnt ? (skip + cnt + 15) / 16 : 0); c += 256) {
+            const uint8_t* p = at0 + 16 * c;
+            unsigned q[4] = {0u, 0u, 0u, 0u};
+            if (p >= src && p + 16 <= src_end) {
+                const uint4 t = *reinterpret_cast<const uint4*>(p);
+                q[0] = t.x; q[1] = t.y; q[2] = t.z; q[3] = t.w;
+            } else {   // the buffer's first or last word
+                for (int b = 0; b < 16; ++b)
+                    if (p + b >= src && p + b < src_end) q[b >> 2] |= (unsigned)p[b] << ((b & 3) * 8);
+            }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) bad |= __vcmpgeu4(q[k], rr);
-        if (bad) {
-            for (int k = 0; k < 32; ++k)
-                if (((q[k >> 2] >> ((k & 3) * 8)) & 0xFFu) >= (unsigned)r && w * 32 + k < N) {
-                    atomicMin(first_bad, (unsigned long long)v * (unsigned long long)N + (unsigned long long)(w * 32 + k));
-                    break;
+            for (int k = 0; k < 4; ++k) s_w[4 * c + k + (4 * c + k) / 32] = q[k];
+        }
+        __syncthreads();
+        const long long w = s0 / 32 + tid;
+        if (w < words) {
+            const int i0 = (skip + 32 * tid) >> 2, sh = (skip & 3) * 8;
+            const long long have = N - w * 32;
+            unsigned x[9], q[8];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) x[k] = s_w[i0 + k + (i0 + k) / 32];
+            unsigned bad = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const long long m = have - 4 * k;   // samples of this word below N
+                q[k] = __funnelshift_r(x[k], x[k + 1], sh) & (m >= 4 ? ~0u : m <= 0 ? 0u : (1u << (8 * (int)m)) - 1u);
+                bad |= __vcmpgeu4(q[k], rr);
+            }
+            if (data) {
+                uint4* d = reinterpret_cast<uint4*>(data + v * ld + w * 32);
+                d[0] = make_uint4(q[0], q[1], q[2], q[3]);
+                d[1] = make_uint4(q[4], q[5], q[6], q[7]);
+            }
+            if (bad) {
+                for (int k = 0; k < 32; ++k)
+                    if (((q[k >> 2] >> ((k & 3) * 8)) & 0xFFu) >= (unsigned)r) {
+                        atomicMin(first_bad, (unsigned long long)v * (unsigned long long)N + (unsigned long long)(w * 32 + k));
+                        break;
+                    }
+            }
+            if (w < wp)
+                for (int y = 1; y <= values; ++y) {
+                    unsigned m = 0;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        m |= (((__vcmpeq4(q[k], 0x01010101u * (unsigned)y) & 0x08040201u) * 0x01010101u) >> 24) << (4 * k);
+                    planes[((long long)v * nplanes + y - 1) * wp + w] = m;
                 }
         }
-        for (int x = 1; x <= values; ++x) {
-            unsigned m = 0;
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                m |= (((__vcmpeq4(q[k], 0x01010101u * (unsigned)x) & 0x08040201u) * 0x01010101u) >> 24) << (4 * k);
-            planes[((long long)v * nplanes + x - 1) * wp + w] = m;
-        }
+        __syncthreads();
     }
 }
 
@@ -192,6 +235,8 @@ struct Workspace {
     size_t h_tot_cap = 0;
     uint8_t* h_stage = nullptr;
     size_t h_stage_cap = 0;
+    unsigned long long *d_bads = nullptr, *h_bads = nullptr;   // first bad values of a batch of uploads
+    size_t bad_cap = 0;
     unsigned* d_bar = nullptr;                      // barrier of the persistent loop
     unsigned* d_bits = nullptr;                     // its adjacency bit matrix
     uint8_t* h_adj = nullptr;                       // pinned: the adjacency it leaves
@@ -230,6 +275,8 @@ struct Workspace {
         if (h_tot) cudaFreeHost(h_tot);
         if (h_stage) cudaFreeHost(h_stage);
         if (h_adj) cudaFreeHost(h_adj);
+        if (h_bads) cudaFreeHost(h_bads);
+        dfree(d_bads);
         dfree(d_bar); dfree(d_bits);
         h_maps.clear();
         gram_E = nullptr; gram_G = nullptr; gram_R = nullptr; gram_maps = nullptr; gram_units = nullptr; pk = nullptr;
@@ -458,13 +505,30 @@ int check_status(fbn_handle* h, unsigned status)
     return FBN_OK;
 }
 
-// Check and planes of the samples now in d_data; h->d_bad receives the first
-// bad value (all ones: none).
-int launch_ingest(fbn_handle* h, cudaStream_t st)
+// New samples into the handle's store, with their check and planes; *bad (device,
+// all ones before) receives the first bad value.  Pinned host memory and memory
+// of the handle's device are read by the kernel itself; pageable memory (and
+// any other) is copied first.
+int ingest(fbn_handle* h, const uint8_t* data, unsigned long long* bad, cudaStream_t st)
 {
-    CK(cudaMemsetAsync(h->d_bad, 0xff, sizeof(unsigned long long), st));
-    dim3 grid((unsigned)std::min<long long>((h->plane_ld + 255) / 256, 64), h->n);
-    k_ingest<<<grid, 256, 0, st>>>(h->d_data, h->ld, h->N, h->d_ar, h->nplanes, h->plane_ld, h->d_planes, h->d_bad);
+    const uint8_t* src = nullptr;
+    cudaPointerAttributes attr{};
+    if (cudaPointerGetAttributes(&attr, data) == cudaSuccess && attr.devicePointer &&
+        (attr.type == cudaMemoryTypeHost || (attr.type == cudaMemoryTypeDevice && attr.device == h->device)))
+        src = (const uint8_t*)attr.devicePointer;
+    cudaGetLastError();
+    int64_t stride = h->N;
+    uint8_t* store = h->d_data;
+    if (!src) {
+        CK(cudaMemcpy2DAsync(h->d_data, h->ld, data, h->N, h->N, h->n, cudaMemcpyDefault, st));
+        src = h->d_data;
+        stride = h->ld;
+        store = nullptr;
+    }
+    // grid.y is limited to 65,535: kMaxVars rows fit
+    dim3 grid((unsigned)std::min<long long>((h->ld + kIngestSamples - 1) / kIngestSamples, 1024), h->n);
+    k_ingest<<<grid, 256, 0, st>>>(src, stride, src + (h->n - 1) * stride + h->N, h->N, h->ld, h->d_ar, h->nplanes,
+                                   h->plane_ld, store, h->d_planes, bad);
     CK(cudaGetLastError());
     return FBN_OK;
 }
@@ -1916,10 +1980,10 @@ int fbn_create(const uint8_t* data, int32_t n_vars, int64_t n_samples, const uin
     cudaStream_t st = h->stream;
     CKC(cudaMemsetAsync(h->d_data, 0, (size_t)n_vars * h->ld, st));
     CKC(cudaMemsetAsync(h->d_eid, 0, nn * sizeof(int32_t), st));
-    CKC(cudaMemcpy2DAsync(h->d_data, h->ld, data, n_samples, n_samples, n_vars, cudaMemcpyDefault, st));
+    CKC(cudaMemsetAsync(h->d_bad, 0xff, sizeof(unsigned long long), st));
     CKC(cudaMemcpyAsync(h->d_ar, arities, n_vars, cudaMemcpyHostToDevice, st));
     // values must lie below their arity: checked on the device
-    if (launch_ingest(h, st)) return bail(FBN_ECUDA);
+    if (const int irc = ingest(h, data, h->d_bad, st)) return bail(irc);
     unsigned long long first_bad = 0;
     CKC(cudaMemcpyAsync(h->h_status, h->d_bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
     CKC(cudaStreamSynchronize(st));
@@ -1958,14 +2022,14 @@ int fbn_update_data(fbn_handle* h, const uint8_t* data)
     cudaStream_t st = h->stream;
     h->learnt = false;
     h->sep_pending = false;
-    CK(cudaMemcpy2DAsync(h->d_data, h->ld, data, h->N, h->N, h->n, cudaMemcpyDefault, st));
-    const int prc = launch_ingest(h, st);
+    const int prc = ingest(h, data, h->d_bad, st);
     if (prc) return prc;
     CK(cudaMemcpyAsync(h->h_status, h->d_bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     unsigned long long first_bad;
     std::memcpy(&first_bad, h->h_status, sizeof first_bad);
     if (first_bad != ~0ULL) {
+        CK(cudaMemset(h->d_bad, 0xff, sizeof(unsigned long long)));   // all ones between calls
         const long long v = (long long)(first_bad / (unsigned long long)h->N);
         const long long smp = (long long)(first_bad % (unsigned long long)h->N);
         return fail(h, FBN_EDATA, "value of variable %lld at sample %lld is >= its arity %d", v, smp,
@@ -1985,20 +2049,29 @@ int fbn_update_data_batch(fbn_handle* const* hs, int32_t k, const uint8_t* const
     }
     CK(cudaSetDevice(h->device));
     cudaStream_t st = h->stream;
-    for (int p = 0; p < k; ++p) {   // every copy, check and bit-plane build queued on one stream
+    Workspace& ws = h->ws;
+    if ((size_t)k > ws.bad_cap) {   // one flag per data set
+        dfree(ws.d_bads);
+        if (ws.h_bads) cudaFreeHost(ws.h_bads);
+        ws.d_bads = ws.h_bads = nullptr;
+        ws.bad_cap = 0;
+        CK(dalloc(&ws.d_bads, k));
+        CK(cudaMallocHost((void**)&ws.h_bads, k * sizeof(unsigned long long)));
+        ws.bad_cap = (size_t)k;
+    }
+    CK(cudaMemsetAsync(ws.d_bads, 0xff, k * sizeof(unsigned long long), st));
+    for (int p = 0; p < k; ++p) {   // every data set queued on one stream
         fbn_handle* q = hs[p];
         q->learnt = false;
         q->sep_pending = false;
-        CK(cudaMemcpy2DAsync(q->d_data, q->ld, data[p], q->N, q->N, q->n, cudaMemcpyDefault, st));
-        const int prc = launch_ingest(q, st);
+        const int prc = ingest(q, data[p], ws.d_bads + p, st);
         if (prc) return fail(h, prc, "%s", q->err.c_str());
-        CK(cudaMemcpyAsync(q->h_status, q->d_bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
     }
+    CK(cudaMemcpyAsync(ws.h_bads, ws.d_bads, k * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     for (int p = 0; p < k; ++p) {
         const fbn_handle* q = hs[p];
-        unsigned long long first_bad;
-        std::memcpy(&first_bad, q->h_status, sizeof first_bad);
+        const unsigned long long first_bad = ws.h_bads[p];
         if (first_bad != ~0ULL) {
             const long long v = (long long)(first_bad / (unsigned long long)q->N);
             const long long smp = (long long)(first_bad % (unsigned long long)q->N);

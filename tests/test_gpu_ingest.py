@@ -1,0 +1,65 @@
+"""New samples from every kind of memory, at every alignment.
+
+The store, its check and the one-hot planes come from one pass over the
+caller's rows: pinned host memory and device memory read in place (rows of any
+length and buffers starting at any byte), pageable memory through a copy.
+Tables and skeletons must be the oracle's, and a bad value is found in the
+first, last and ragged words.
+"""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def F():
+    from paper_2212_04259_gb300 import build
+    build.build()
+    import paper_2212_04259_gb300 as f
+    return f
+
+
+def _place(data, where, shift):
+    """The samples in `where` memory, starting `shift` bytes into a buffer of
+    values that would be refused."""
+    import torch
+    n, N = data.shape
+    buf = torch.full((n * N + shift,), 255, dtype=torch.uint8)
+    if where == "pinned":
+        buf = buf.pin_memory()
+    elif where == "device":
+        buf = buf.cuda()
+    out = buf[shift:].view(n, N)
+    out.copy_(torch.from_numpy(data))
+    return out
+
+
+@pytest.mark.parametrize("where", ["pinned", "device", "pageable"])
+@pytest.mark.parametrize("N", [1, 15, 31, 33, 255, 257, 8191, 8192, 8193, 16400])
+def test_every_memory_and_alignment(F, where, N):
+    rng = np.random.default_rng(N)
+    ar = np.array([5, 2, 4, 3, 5], dtype=np.uint8)
+    first = np.stack([rng.integers(0, r, N) for r in ar]).astype(np.uint8)
+    h = F.fbn_create(_place(first, where, 3), ar)
+    for shift in (0, 1, 2, 7, 13):
+        data = np.stack([rng.integers(0, r, N) for r in ar]).astype(np.uint8)
+        F.fbn_update_data_batch([h], [_place(data, where, shift)]) if shift & 1 else F.fbn_update_data(h, _place(data, where, shift))
+        for x, y, S in ((0, 1, []), (2, 4, [3]), (4, 0, [2, 1])):
+            assert np.array_equal(F.fbn_ci_table(h, x, y, S), oracle.ci_table(data, ar, x, y, S))
+        ref = oracle.pc_stable(data, ar, 0.4, 1)   # depths 0 and 1 from the planes
+        if not ref.near:
+            assert np.array_equal(F.fbn_learn_skeleton(h, 0.4, 1), ref.adj)
+    for v, smp in ((0, 0), (4, N - 1), (2, N // 2)):
+        bad = first.copy()
+        bad[v, smp] = ar[v]
+        for call in (lambda: F.fbn_update_data(h, _place(bad, where, 5)),
+                     lambda: F.fbn_update_data_batch([h], [_place(bad, where, 6)]),
+                     lambda: F.fbn_create(_place(bad, where, 9), ar)):
+            with pytest.raises(F.FbnError) as e:
+                call()
+            assert e.value.code == -2 and f"variable {v} at sample {smp} " in str(e.value)
+        F.fbn_update_data(h, _place(first, where, 0))   # usable again
+        assert np.array_equal(F.fbn_ci_table(h, 0, 1), oracle.ci_table(first, ar, 0, 1))
