@@ -164,6 +164,18 @@ __global__ void k_init_graph(const ProblemDev* probs, const int32_t* vtx_prob, c
 
 }  // namespace
 
+// Pinned host memory that holds exported separating sets: the workspace's until
+// it exports again, and every handle's whose sets lie in it.
+struct HostStage {
+    uint8_t* p = nullptr;
+    uint8_t* dev = nullptr;   // as the device addresses it
+    size_t cap = 0;
+    ~HostStage()
+    {
+        if (p) cudaFreeHost(p);
+    }
+};
+
 // ---- workspace shared by the depth loop ----------------------------------
 struct Workspace {
     long long edge_cap = 0;
@@ -233,8 +245,7 @@ struct Workspace {
     // pinned staging of the separating-set export: totals, then the arrays
     long long* h_tot = nullptr;
     size_t h_tot_cap = 0;
-    uint8_t* h_stage = nullptr;
-    size_t h_stage_cap = 0;
+    std::shared_ptr<HostStage> stage;
     unsigned long long *d_bads = nullptr, *h_bads = nullptr;   // first bad values of a batch of uploads
     size_t bad_cap = 0;
     unsigned* d_bar = nullptr;                      // barrier of the persistent loop
@@ -273,7 +284,6 @@ struct Workspace {
         if (h_rec) cudaFreeHost(h_rec);
         if (h_up) cudaFreeHost(h_up);
         if (h_tot) cudaFreeHost(h_tot);
-        if (h_stage) cudaFreeHost(h_stage);
         if (h_adj) cudaFreeHost(h_adj);
         if (h_bads) cudaFreeHost(h_bads);
         dfree(d_bads);
@@ -340,19 +350,19 @@ struct fbn_handle {
     int32_t* d_off = nullptr;           // [n] sum of the arities before each variable; [n] the same of arities - 1
     // results of the last skeleton
     bool learnt = false;
-    bool sep_pending = false;           // separating sets not in the csr vectors yet
-    bool sep_staged = false;            // ... but already in the pinned staging (sep_R pairs, sep_M members)
-    long long sep_R = 0, sep_M = 0;
+    bool sep_pending = false;           // separating sets still only on the device
     unsigned long long sep_pool_used = 0;
     // members of a batch's separating sets: a device copy of the batch's
     // shared pool, held by every handle of that batch until it learns again
     std::shared_ptr<DeviceInts> sep_snap;
-    // separating sets on the host, CSR: removed pairs (i < j) ascending, their
-    // member offsets (one more than pairs), the members
-    std::vector<int32_t> csr_pairs;
-    std::vector<int64_t> csr_offs;
-    std::vector<int32_t> csr_members;
-    // row counts of the compaction on the device: [2n] counts, then [2][n + 1] row offsets
+    // separating sets on the host, CSR in pinned memory: removed pairs (i < j)
+    // ascending, their member offsets, the members
+    std::shared_ptr<HostStage> csr_hold;
+    const int32_t* csr_pairs = nullptr;
+    const int64_t* csr_offs = nullptr;
+    const int32_t* csr_members = nullptr;
+    long long csr_R = 0, csr_M = 0;
+    // row counts of the compaction on the device, [2n]
     long long* d_sep_cnt = nullptr;
     fbn_stats stats{};
     // the autotuner's choices (empty: the fixed rules): a per-depth code
@@ -759,13 +769,63 @@ cudaError_t grow_pinned(T** p, size_t* cap, size_t n)
     return e;
 }
 
+// Pinned memory of at least `bytes` for an export; a new block when a handle
+// still reads from the old one.
+cudaError_t acquire_stage(Workspace& ws, size_t bytes)
+{
+    if (ws.stage && ws.stage.use_count() == 1 && ws.stage->cap >= bytes) return cudaSuccess;
+    auto fresh = std::make_shared<HostStage>();
+    cudaError_t e = cudaMallocHost((void**)&fresh->p, std::max<size_t>(bytes, 16));
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&fresh->dev, fresh->p, 0);
+    if (e != cudaSuccess) return e;
+    fresh->cap = bytes;
+    ws.stage = std::move(fresh);
+    return cudaSuccess;
+}
+
+// A skeleton's CSR laid out for L pairs from an offset of the stage: pairs int32
+// [2L], offsets int64 [L], members int32.
+struct CsrPlace {
+    size_t pairs, offs, members;
+    CsrPlace(size_t at, long long L)
+        : pairs(at), offs(at + 2 * (size_t)L * sizeof(int32_t)),
+          members(at + (size_t)L * (2 * sizeof(int32_t) + sizeof(int64_t)))
+    {
+    }
+    static size_t bytes(long long L, long long M)   // rounded to 16
+    {
+        return ((size_t)L * (2 * sizeof(int32_t) + sizeof(int64_t)) + (size_t)M * sizeof(int32_t) + 15) & ~(size_t)15;
+    }
+};
+
+// The handle's sets are R pairs and M members at a place of the stage.
+void take_csr(fbn_handle* q, const std::shared_ptr<HostStage>& stage, const CsrPlace& at, long long R, long long M)
+{
+    q->csr_hold = stage;
+    q->csr_pairs = reinterpret_cast<const int32_t*>(stage->p + at.pairs);
+    q->csr_offs = reinterpret_cast<const int64_t*>(stage->p + at.offs);
+    q->csr_members = reinterpret_cast<const int32_t*>(stage->p + at.members);
+    q->csr_R = R;
+    q->csr_M = M;
+    q->sep_pending = false;
+}
+
+// Results of the last skeleton are dropped.
+void drop_sepsets(fbn_handle* q)
+{
+    q->sep_pending = false;
+    q->csr_hold.reset();
+    q->csr_pairs = q->csr_members = nullptr;
+    q->csr_offs = nullptr;
+    q->csr_R = q->csr_M = 0;
+}
+
 // The handle's separating sets as host CSR, compacted on the device by a
-// kernel that writes the compact arrays straight into pinned host staging
-// (device-addressable). One handle: staging sized by bounds known on the
-// host (every pair removed; every pool entry its own), one synchronisation.
-// A handle of a batch: every member whose sets are still on the device, in
-// two passes (row counts and totals; then the arrays), one synchronisation
-// each.
+// kernel that writes the compact arrays straight into pinned host memory, where
+// they stay.  One handle: sized by bounds known on the host (every pair removed;
+// every pool entry its own), one synchronisation.  A handle of a batch: every
+// member whose sets are still on the device, in two passes (row counts and
+// totals; then the arrays), one synchronisation each.
 int materialize_sepsets(fbn_handle* h, Workspace& ws)
 {
     if (!h->sep_pending) return FBN_OK;
@@ -779,100 +839,65 @@ int materialize_sepsets(fbn_handle* h, Workspace& ws)
         todo.push_back(h);
     }
     const size_t k = todo.size();
-    auto align16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
-    // staging of one handle laid out for L pairs: pairs int32 [2L], offsets
-    // int64 [L], members int32
-    auto place = [](uint8_t* base, long long L, int32_t** pr, int64_t** of, int32_t** mb) {
-        *pr = reinterpret_cast<int32_t*>(base);
-        *of = reinterpret_cast<int64_t*>(base + 2 * (size_t)L * sizeof(int32_t));
-        *mb = reinterpret_cast<int32_t*>(base + (size_t)L * (2 * sizeof(int32_t) + sizeof(int64_t)));
-    };
-    auto count = [&](fbn_handle* q, long long* tot) -> int {
-        const int n = q->n;
-        if (!q->d_sep_cnt) CK(dalloc(&q->d_sep_cnt, 4 * (size_t)n + 4));
-        long long* roff_p = q->d_sep_cnt + 2 * (size_t)n;
-        long long* roff_m = roff_p + n + 1;
-        CK(launch_sep_count(q->d_sep_len, n, q->d_sep_cnt, roff_p, roff_m, st));
-        CK(cudaMemcpyAsync(tot, roff_p + n, sizeof(long long), cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(tot + 1, roff_m + n, sizeof(long long), cudaMemcpyDeviceToHost, st));
-        return FBN_OK;
-    };
-    auto write = [&](fbn_handle* q, uint8_t* base, long long L) -> int {
-        const int n = q->n;
-        const int32_t* pool = q->sep_snap ? q->sep_snap->d : q->ws.sep_pool;
-        long long* roff_p = q->d_sep_cnt + 2 * (size_t)n;
-        long long* roff_m = roff_p + n + 1;
-        int32_t* pr = nullptr;
-        int64_t* of = nullptr;
-        int32_t* mb = nullptr;
-        place(base, L, &pr, &of, &mb);
-        CK(launch_sep_write(q->d_sep_len, q->d_sep_off, pool, n, roff_p, roff_m, pr, of, mb, st));
-        return FBN_OK;
-    };
-    auto unpack = [&](fbn_handle* q, uint8_t* base, long long L, long long R, long long Mtot) {
-        int32_t* pr = nullptr;
-        int64_t* of = nullptr;
-        int32_t* mb = nullptr;
-        place(base, L, &pr, &of, &mb);
-        q->csr_pairs.assign(pr, pr + 2 * (size_t)R);
-        q->csr_offs.assign(of, of + (size_t)R);
-        q->csr_offs.push_back(Mtot);
-        q->csr_members.assign(mb, mb + (size_t)Mtot);
-        q->sep_pending = false;
-    };
-    int rc = FBN_OK;
-    if (h->sep_staged) {   // the skeleton's own kernel left them in the staging
-        unpack(h, ws.h_stage, (long long)h->n * (h->n - 1) / 2, h->sep_R, h->sep_M);
-        h->sep_staged = false;
-        return FBN_OK;
+    CK(grow_pinned(&ws.h_tot, &ws.h_tot_cap, 2 * k));
+    long long* tot = nullptr;
+    CK(cudaHostGetDevicePointer((void**)&tot, ws.h_tot, 0));
+    std::vector<SepJob> jobs(k);
+    for (size_t i = 0; i < k; ++i) {
+        fbn_handle* q = todo[i];
+        if (!q->d_sep_cnt) CK(dalloc(&q->d_sep_cnt, 2 * (size_t)q->n));
+        SepJob& j = jobs[i];
+        j = SepJob{};
+        j.sep_len = q->d_sep_len;
+        j.sep_off = q->d_sep_off;
+        j.pool = q->sep_snap ? q->sep_snap->d : q->ws.sep_pool;
+        j.n = q->n;
+        j.cnt = q->d_sep_cnt;
+        j.tot = tot + 2 * i;
     }
+    auto place = [&](size_t i, const CsrPlace& at) {
+        jobs[i].pairs = reinterpret_cast<int32_t*>(ws.stage->dev + at.pairs);
+        jobs[i].offs = reinterpret_cast<int64_t*>(ws.stage->dev + at.offs);
+        jobs[i].members = reinterpret_cast<int32_t*>(ws.stage->dev + at.members);
+    };
+    CK(launch_sep_count(jobs.data(), (int)k, st));
     if (k == 1) {
         fbn_handle* q = todo[0];
-        const long long Rmax = (long long)q->n * (q->n - 1) / 2;
-        const long long Mmax = (long long)q->sep_pool_used;
-        const size_t bytes = align16((size_t)Rmax * (2 * sizeof(int32_t) + sizeof(int64_t)) +
-                                     (size_t)Mmax * sizeof(int32_t));
-        CK(grow_pinned(&ws.h_stage, &ws.h_stage_cap, bytes + 16));
-        uint8_t* dstage = nullptr;   // the staging as the device addresses it
-        CK(cudaHostGetDevicePointer((void**)&dstage, ws.h_stage, 0));
-        long long* tot = reinterpret_cast<long long*>(ws.h_stage + bytes);
-        if ((rc = count(q, tot)) || (rc = write(q, dstage, Rmax))) return rc;
+        const long long Rmax = (long long)q->n * (q->n - 1) / 2, Mmax = (long long)q->sep_pool_used;
+        CK(acquire_stage(ws, CsrPlace::bytes(Rmax, Mmax)));
+        const CsrPlace at(0, Rmax);
+        place(0, at);
+        CK(launch_sep_write(jobs.data(), 1, st));
         CK(cudaStreamSynchronize(st));
-        if (tot[0] > Rmax || tot[1] > Mmax) return fail(h, FBN_ECUDA, "separating-set export over its bounds");
-        unpack(q, ws.h_stage, Rmax, tot[0], tot[1]);
+        if (ws.h_tot[0] > Rmax || ws.h_tot[1] > Mmax) return fail(h, FBN_ECUDA, "separating-set export over its bounds");
+        take_csr(q, ws.stage, at, ws.h_tot[0], ws.h_tot[1]);
         return FBN_OK;
     }
-    CK(grow_pinned(&ws.h_tot, &ws.h_tot_cap, 2 * k));
-    for (size_t i = 0; i < k; ++i)   // pass 1: row counts and offsets, totals to the host
-        if ((rc = count(todo[i], ws.h_tot + 2 * i))) return rc;
     CK(cudaStreamSynchronize(st));
-    std::vector<size_t> at(k + 1, 0);   // staging offsets (bytes, 16-aligned)
-    for (size_t i = 0; i < k; ++i) {
-        const long long R = ws.h_tot[2 * i], Mtot = ws.h_tot[2 * i + 1];
-        at[i + 1] = at[i] + align16((size_t)R * (2 * sizeof(int32_t) + sizeof(int64_t)) +
-                                    (size_t)Mtot * sizeof(int32_t));
-    }
-    CK(grow_pinned(&ws.h_stage, &ws.h_stage_cap, std::max<size_t>(at[k], 16)));
-    uint8_t* dstage = nullptr;
-    CK(cudaHostGetDevicePointer((void**)&dstage, ws.h_stage, 0));
-    for (size_t i = 0; i < k; ++i)   // pass 2: the compact arrays into the staging
-        if (ws.h_tot[2 * i] > 0 && (rc = write(todo[i], dstage + at[i], ws.h_tot[2 * i]))) return rc;
+    std::vector<size_t> begin(k + 1, 0);
+    for (size_t i = 0; i < k; ++i) begin[i + 1] = begin[i] + CsrPlace::bytes(ws.h_tot[2 * i], ws.h_tot[2 * i + 1]);
+    CK(acquire_stage(ws, begin[k]));
+    for (size_t i = 0; i < k; ++i) place(i, CsrPlace(begin[i], ws.h_tot[2 * i]));
+    CK(launch_sep_write(jobs.data(), (int)k, st));
     CK(cudaStreamSynchronize(st));
     for (size_t i = 0; i < k; ++i)
-        unpack(todo[i], ws.h_stage + at[i], ws.h_tot[2 * i], ws.h_tot[2 * i], ws.h_tot[2 * i + 1]);
+        take_csr(todo[i], ws.stage, CsrPlace(begin[i], ws.h_tot[2 * i]), ws.h_tot[2 * i], ws.h_tot[2 * i + 1]);
     return FBN_OK;
 }
+
+// End of pair k's members.
+int64_t csr_end(const fbn_handle* h, long long k) { return k + 1 < h->csr_R ? h->csr_offs[k + 1] : h->csr_M; }
 
 // Index of the removed pair (i < j) in the handle's CSR, or -1.
 long long find_sepset(const fbn_handle* h, int i, int j)
 {
-    long long lo = 0, hi = (long long)h->csr_offs.size() - 1;   // pairs [0, R)
+    long long lo = 0, hi = h->csr_R;   // pairs [0, R)
     while (lo < hi) {
         const long long mid = (lo + hi) >> 1;
         const int a = h->csr_pairs[2 * mid], b = h->csr_pairs[2 * mid + 1];
         if (a < i || (a == i && b < j)) lo = mid + 1; else hi = mid;
     }
-    if (lo < (long long)h->csr_offs.size() - 1 && h->csr_pairs[2 * lo] == i && h->csr_pairs[2 * lo + 1] == j) return lo;
+    if (lo < h->csr_R && h->csr_pairs[2 * lo] == i && h->csr_pairs[2 * lo + 1] == j) return lo;
     return -1;
 }
 
@@ -1317,19 +1342,18 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         if (direct_out) {   // one problem: every result straight to the host
             const long long R = edge_cap;
             CK(grow_pinned(&ws.h_adj, &ws.h_adj_cap, ((size_t)h->n * h->n + 15) / 16 * 16));
-            const size_t csr = (size_t)R * (2 * sizeof(int32_t) + sizeof(int64_t)) + (size_t)ws.sep_cap * sizeof(int32_t);
-            CK(grow_pinned(&ws.h_stage, &ws.h_stage_cap, (csr + 15) / 16 * 16 + 16));
-            if (!h->d_sep_cnt) CK(dalloc(&h->d_sep_cnt, 4 * (size_t)h->n + 4));
-            uint8_t* stage = nullptr;
+            const size_t csr = CsrPlace::bytes(R, ws.sep_cap);
+            CK(acquire_stage(ws, csr + 16));
+            if (!h->d_sep_cnt) CK(dalloc(&h->d_sep_cnt, 2 * (size_t)h->n));
             CK(cudaHostGetDevicePointer((void**)&la.h_ctr, ws.h_ctr, 0));
             CK(cudaHostGetDevicePointer((void**)&la.h_rec, ws.h_rec, 0));
-            CK(cudaHostGetDevicePointer((void**)&stage, ws.h_stage, 0));
             if (adj_out && adj_out[0]) CK(cudaHostGetDevicePointer((void**)&la.h_adj, ws.h_adj, 0));
-            la.h_pairs = reinterpret_cast<int32_t*>(stage);   // as materialize_sepsets lays it out
-            la.h_offs = reinterpret_cast<int64_t*>(stage + 2 * (size_t)R * sizeof(int32_t));
-            la.h_members = reinterpret_cast<int32_t*>(stage + (size_t)R * (2 * sizeof(int32_t) + sizeof(int64_t)));
-            la.h_tot = reinterpret_cast<long long*>(stage + (csr + 15) / 16 * 16);
-            h_tot = reinterpret_cast<const long long*>(ws.h_stage + (csr + 15) / 16 * 16);
+            const CsrPlace at(0, R);
+            la.h_pairs = reinterpret_cast<int32_t*>(ws.stage->dev + at.pairs);
+            la.h_offs = reinterpret_cast<int64_t*>(ws.stage->dev + at.offs);
+            la.h_members = reinterpret_cast<int32_t*>(ws.stage->dev + at.members);
+            la.h_tot = reinterpret_cast<long long*>(ws.stage->dev + csr);
+            h_tot = reinterpret_cast<const long long*>(ws.stage->p + csr);
             la.sep_cnt = h->d_sep_cnt;
         }
         if (direct_out) ws.h_ctr->status = kStatusTimeout;   // overwritten by the loop's last phase
@@ -1569,20 +1593,17 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         hs[p]->stats = stats;
         hs[p]->learnt = true;
         hs[p]->sep_pending = true;
-        hs[p]->sep_staged = direct_out;
-        if (direct_out) {
-            hs[p]->sep_R = h_tot[0];
-            hs[p]->sep_M = h_tot[1];
-        }
         hs[p]->sep_pool_used = c.sep_used;
         set_snapshot(hs[p], snap);
     }
+    if (direct_out) take_csr(h, ws.stage, CsrPlace(0, edge_cap), h_tot[0], h_tot[1]);   // already on the host
     return FBN_OK;
 }
 
 int run_skeleton(fbn_handle* const* hs, int k, double alpha, int32_t max_depth, uint8_t* const* adj_out = nullptr,
                  const ShardHooks* shard = nullptr)
 {
+    for (int p = 0; p < k; ++p) drop_sepsets(hs[p]);   // their pinned memory is written again
     for (int attempt = 0; attempt < 6; ++attempt) {
         bool retry = false;
         const int rc = run_skeleton_once(hs, k, alpha, max_depth, &retry, adj_out, shard);
@@ -2021,7 +2042,7 @@ int fbn_update_data(fbn_handle* h, const uint8_t* data)
     CK(cudaSetDevice(h->device));
     cudaStream_t st = h->stream;
     h->learnt = false;
-    h->sep_pending = false;
+    drop_sepsets(h);
     const int prc = ingest(h, data, h->d_bad, st);
     if (prc) return prc;
     CK(cudaMemcpyAsync(h->h_status, h->d_bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
@@ -2063,7 +2084,7 @@ int fbn_update_data_batch(fbn_handle* const* hs, int32_t k, const uint8_t* const
     for (int p = 0; p < k; ++p) {   // every data set queued on one stream
         fbn_handle* q = hs[p];
         q->learnt = false;
-        q->sep_pending = false;
+        drop_sepsets(q);
         const int prc = ingest(q, data[p], ws.d_bads + p, st);
         if (prc) return fail(h, prc, "%s", q->err.c_str());
     }
@@ -2123,7 +2144,7 @@ int fbn_ci_table(fbn_handle* h, int32_t x, int32_t y, const int32_t* z, int32_t 
 int fbn_learn_skeleton(fbn_handle* h, double alpha, int32_t max_depth, uint8_t* adj_out)
 {
     if (!h) return FBN_EINVAL;
-    h->sep_pending = false;
+    drop_sepsets(h);
     if (!(alpha > 0.0 && alpha < 1.0)) return fail(h, FBN_EINVAL, "alpha=%g outside (0, 1)", alpha);
     if (max_depth < -1) return fail(h, FBN_EINVAL, "max_depth=%d < -1", max_depth);
     h->learnt = false;
@@ -2143,7 +2164,7 @@ int fbn_learn_skeleton_batch(fbn_handle* const* hs, int32_t k, double alpha, int
         if (!hs[p]) return fail(h, FBN_EINVAL, "handle %d is NULL", p);
         if (hs[p]->device != h->device) return fail(h, FBN_EINVAL, "handle %d is on another device", p);
         hs[p]->learnt = false;
-        hs[p]->sep_pending = false;
+        drop_sepsets(hs[p]);
     }
     if (!(alpha > 0.0 && alpha < 1.0)) return fail(h, FBN_EINVAL, "alpha=%g outside (0, 1)", alpha);
     if (max_depth < -1) return fail(h, FBN_EINVAL, "max_depth=%d < -1", max_depth);
@@ -2156,7 +2177,7 @@ int fbn_learn_skeleton_sharded(fbn_handle* h, double alpha, int32_t max_depth, f
                                fbn_shard_exchange_fn exchange, void* ctx, uint8_t* adj_out)
 {
     if (!h) return FBN_EINVAL;
-    h->sep_pending = false;
+    drop_sepsets(h);
     h->learnt = false;
     if (!own || !exchange) return fail(h, FBN_EINVAL, "own and exchange callbacks are required");
     if (!(alpha > 0.0 && alpha < 1.0)) return fail(h, FBN_EINVAL, "alpha=%g outside (0, 1)", alpha);
@@ -2175,7 +2196,7 @@ int fbn_autotune(fbn_handle* const* hs, int32_t k, double alpha, int32_t max_dep
         if (!hs[p]) return fail(h, FBN_EINVAL, "handle %d is NULL", p);
         if (hs[p]->device != h->device) return fail(h, FBN_EINVAL, "handle %d is on another device", p);
         hs[p]->learnt = false;
-        hs[p]->sep_pending = false;
+        drop_sepsets(hs[p]);
     }
     if (!(alpha > 0.0 && alpha < 1.0)) return fail(h, FBN_EINVAL, "alpha=%g outside (0, 1)", alpha);
     if (max_depth < -1) return fail(h, FBN_EINVAL, "max_depth=%d < -1", max_depth);
@@ -2243,7 +2264,7 @@ int32_t fbn_get_sepset(const fbn_handle* hc, int32_t i, int32_t j, int32_t* buf,
     if (i > j) std::swap(i, j);
     const long long k = find_sepset(h, i, j);
     if (k < 0) return -1;
-    const int32_t L = (int32_t)(h->csr_offs[k + 1] - h->csr_offs[k]);
+    const int32_t L = (int32_t)(csr_end(h, k) - h->csr_offs[k]);
     if (L > 0 && cap > 0 && !buf) return FBN_EINVAL;
     for (int t = 0; t < L && t < cap; ++t) buf[t] = h->csr_members[(size_t)h->csr_offs[k] + t];
     return L;
@@ -2258,10 +2279,10 @@ int fbn_export_sepsets(const fbn_handle* hc, int64_t* n_removed, int64_t* n_memb
         const int rc = materialize_sepsets(h, h->ws);
         if (rc) return rc;
     }
-    const int64_t nr = (int64_t)h->csr_offs.size() - 1, nm = h->csr_offs.back();
-    if (pairs && nr > 0) std::memcpy(pairs, h->csr_pairs.data(), 2 * (size_t)nr * sizeof(int32_t));
-    if (offsets && nr > 0) std::memcpy(offsets, h->csr_offs.data(), (size_t)nr * sizeof(int64_t));
-    if (members && nm > 0) std::memcpy(members, h->csr_members.data(), (size_t)nm * sizeof(int32_t));
+    const int64_t nr = h->csr_R, nm = h->csr_M;
+    if (pairs && nr > 0) std::memcpy(pairs, h->csr_pairs, 2 * (size_t)nr * sizeof(int32_t));
+    if (offsets && nr > 0) std::memcpy(offsets, h->csr_offs, (size_t)nr * sizeof(int64_t));
+    if (members && nm > 0) std::memcpy(members, h->csr_members, (size_t)nm * sizeof(int32_t));
     if (offsets) offsets[nr] = nm;
     *n_removed = nr;
     *n_members = nm;
@@ -2290,7 +2311,7 @@ int fbn_orient_cpdag(const fbn_handle* hc, uint8_t* cpdag_out)
     auto in_sepset = [&](int a, int b, int k) {   // a < b, not adjacent
         const long long r = find_sepset(h, a, b);
         if (r < 0) return false;
-        for (int64_t t = h->csr_offs[r]; t < h->csr_offs[r + 1]; ++t)
+        for (int64_t t = h->csr_offs[r]; t < csr_end(h, r); ++t)
             if (h->csr_members[(size_t)t] == k) return true;
         return false;
     };

@@ -2,7 +2,9 @@
 // SepSet) compacted on the device into CSR form: the removed pairs i < j in
 // ascending (i, j), one offset per pair, the members in pair order.  The
 // writer's outputs may be pinned host memory (device-addressable): only the
-// compact arrays cross to the host.
+// compact arrays cross to the host.  Every kernel takes a batch of skeletons
+// (grid.y), whose descriptors go by value: the export of 20 problems was 100
+// launches and copies.
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -11,15 +13,22 @@
 namespace fbn {
 namespace {
 
+constexpr int kSepJobs = 32;   // skeletons per launch
+struct SepJobs {
+    SepJob j[kSepJobs];
+};
+
 // Per row i (one warp): removed pairs (i, j > i) and their member total.
-__global__ void k_sep_count(const int32_t* __restrict__ sep_len, int n, long long* __restrict__ cnt)
+__global__ void k_sep_count(const __grid_constant__ SepJobs jobs)
 {
+    const SepJob& q = jobs.j[blockIdx.y];
+    const int n = q.n;
     const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (i >= n) return;
     long long pairs = 0, members = 0;
     for (int j = i + 1 + lane; j < n; j += 32) {
-        const int32_t L = sep_len[(long long)i * n + j];
+        const int32_t L = q.sep_len[(long long)i * n + j];
         if (L >= 0) {
             pairs += 1;
             members += L;
@@ -31,15 +40,18 @@ __global__ void k_sep_count(const int32_t* __restrict__ sep_len, int n, long lon
         members += __shfl_xor_sync(0xffffffffu, members, o);
     }
     if (lane == 0) {
-        cnt[i] = pairs;
-        cnt[n + i] = members;
+        q.cnt[i] = pairs;
+        q.cnt[n + i] = members;
     }
 }
 
-// One CTA: exclusive row offsets of pairs and members; totals at index n.
-__global__ void k_sep_scan(const long long* __restrict__ cnt, int n, long long* __restrict__ roff_p,
-                           long long* __restrict__ roff_m)
+// One CTA per skeleton: exclusive row offsets of pairs and members, in place;
+// the totals.
+__global__ void k_sep_scan(const __grid_constant__ SepJobs jobs)
 {
+    const SepJob& q = jobs.j[blockIdx.x];
+    const int n = q.n;
+    long long* cnt = q.cnt;
     __shared__ long long sp[1024], sm[1024];
     const int t = threadIdx.x, T = blockDim.x;
     const int per = (n + T - 1) / T;
@@ -61,30 +73,30 @@ __global__ void k_sep_scan(const long long* __restrict__ cnt, int n, long long* 
     }
     long long bp = sp[t] - p, bm = sm[t] - m;
     for (int i = lo; i < hi; ++i) {
-        roff_p[i] = bp;
-        roff_m[i] = bm;
-        bp += cnt[i];
-        bm += cnt[n + i];
+        const long long cp = cnt[i], cm = cnt[n + i];
+        cnt[i] = bp;
+        cnt[n + i] = bm;
+        bp += cp;
+        bm += cm;
     }
     if (t == T - 1) {
-        roff_p[n] = sp[T - 1];
-        roff_m[n] = sm[T - 1];
+        q.tot[0] = sp[T - 1];
+        q.tot[1] = sm[T - 1];
     }
 }
 
 // Per row i (one warp): the row's pairs, offsets and members at its offsets.
-__global__ void k_sep_write(const int32_t* __restrict__ sep_len, const int64_t* __restrict__ sep_off,
-                            const int32_t* __restrict__ pool, int n, const long long* __restrict__ roff_p,
-                            const long long* __restrict__ roff_m, int32_t* __restrict__ pairs,
-                            int64_t* __restrict__ offs, int32_t* __restrict__ members)
+__global__ void k_sep_write(const __grid_constant__ SepJobs jobs)
 {
+    const SepJob& q = jobs.j[blockIdx.y];
+    const int n = q.n;
     const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (i >= n) return;
-    long long p = roff_p[i], m = roff_m[i];
+    long long p = q.cnt[i], m = q.cnt[n + i];
     for (int j0 = i + 1; j0 < n; j0 += 32) {
         const int j = j0 + lane;
-        const int32_t L = j < n ? sep_len[(long long)i * n + j] : -1;
+        const int32_t L = j < n ? q.sep_len[(long long)i * n + j] : -1;
         const bool take = L >= 0;
         const unsigned ballot = __ballot_sync(0xffffffffu, take);
         long long inc = take ? L : 0;   // inclusive scan of the lengths
@@ -96,11 +108,12 @@ __global__ void k_sep_write(const int32_t* __restrict__ sep_len, const int64_t* 
         if (take) {
             const long long k = p + __popc(ballot & ((1u << lane) - 1u));
             const long long mo = m + inc - L;
-            pairs[2 * k] = i;
-            pairs[2 * k + 1] = j;
-            offs[k] = mo;
-            const int64_t src = sep_off[(long long)i * n + j];
-            for (int t = 0; t < L; ++t) members[mo + t] = pool[src + t];
+            reinterpret_cast<int2*>(q.pairs)[k] = make_int2(i, j);
+            q.offs[k] = mo;
+            if (L > 0) {
+                const int32_t* src = q.pool + q.sep_off[(long long)i * n + j];
+                for (int t = 0; t < L; ++t) q.members[mo + t] = src[t];
+            }
         }
         p += __popc(ballot);
         m += __shfl_sync(0xffffffffu, inc, 31);
@@ -109,23 +122,35 @@ __global__ void k_sep_write(const int32_t* __restrict__ sep_len, const int64_t* 
 
 }  // namespace
 
-cudaError_t launch_sep_count(const int32_t* sep_len, int n, long long* cnt, long long* roff_p, long long* roff_m,
-                             cudaStream_t st)
+// Launches kern over the jobs, rows of up to 8 per CTA on grid.x.
+template <class K>
+cudaError_t each_batch(K kern, const SepJob* jobs, int k, bool rows, int threads, cudaStream_t st)
 {
-    const int warps = 8;
-    k_sep_count<<<(n + warps - 1) / warps, warps * 32, 0, st>>>(sep_len, n, cnt);
-    k_sep_scan<<<1, 1024, 0, st>>>(cnt, n, roff_p, roff_m);
-    return cudaGetLastError();
+    for (int at = 0; at < k; at += kSepJobs) {
+        SepJobs a{};
+        const int m = k - at < kSepJobs ? k - at : kSepJobs;
+        int max_n = 1;
+        for (int t = 0; t < m; ++t) {
+            a.j[t] = jobs[at + t];
+            max_n = jobs[at + t].n > max_n ? jobs[at + t].n : max_n;
+        }
+        const dim3 grid = rows ? dim3((max_n + 7) / 8, m) : dim3(m);
+        kern<<<grid, threads, 0, st>>>(a);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
-cudaError_t launch_sep_write(const int32_t* sep_len, const int64_t* sep_off, const int32_t* pool, int n,
-                             const long long* roff_p, const long long* roff_m, int32_t* pairs, int64_t* offs,
-                             int32_t* members, cudaStream_t st)
+cudaError_t launch_sep_count(const SepJob* jobs, int k, cudaStream_t st)
 {
-    const int warps = 8;
-    k_sep_write<<<(n + warps - 1) / warps, warps * 32, 0, st>>>(sep_len, sep_off, pool, n, roff_p, roff_m, pairs,
-                                                               offs, members);
-    return cudaGetLastError();
+    const cudaError_t e = each_batch(k_sep_count, jobs, k, true, 256, st);
+    return e != cudaSuccess ? e : each_batch(k_sep_scan, jobs, k, false, 1024, st);
+}
+
+cudaError_t launch_sep_write(const SepJob* jobs, int k, cudaStream_t st)
+{
+    return each_batch(k_sep_write, jobs, k, true, 256, st);
 }
 
 }  // namespace fbn
