@@ -652,12 +652,14 @@ int prepare_gram(fbn_handle* const* hs, int k, Workspace& ws, ProblemDev* P)
 {
     fbn_handle* h = hs[0];
     cudaStream_t st = h->stream;
-    long long e_total = 0, r_total = 0, tile_stages = 0;
+    long long e_total = 0, r_total = 0;
+    std::vector<long long> tiles(k), stages(k);
     for (int p = 0; p < k; ++p) {
-        const long long T = hs[p]->Mr / 128;
         e_total += (long long)hs[p]->Mr * hs[p]->K;
         r_total += (long long)hs[p]->Mr * hs[p]->Mr;
-        tile_stages += (T * (T + 2) / 4 + 1) * (hs[p]->K / 128);
+        const int T = hs[p]->Mr / 128, T2 = (T + 1) / 2;
+        for (int a = 0; a < T; ++a) tiles[p] += T2 - a / 2;
+        stages[p] = hs[p]->K / 128;
     }
     if (r_total > ws.gram_R_cap) {
         dfree(ws.gram_R);
@@ -669,7 +671,7 @@ int prepare_gram(fbn_handle* const* hs, int k, Workspace& ws, ProblemDev* P)
     ws.gram_R_used = r_total;
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
-    ws.gram_unit_slices = gram_unit_slices(tile_stages, sms);
+    ws.gram_unit_slices = gram_unit_slices(tiles.data(), stages.data(), k, sms);
     if (e_total > ws.gram_E_cap) {
         dfree(ws.gram_E);
         ws.gram_E = nullptr;

@@ -47,6 +47,7 @@ constexpr int kKSlice = 128;                         // samples (bytes) per pipe
 constexpr int kChunk = 8192;                         // samples per exact accumulation
 constexpr int kSlicesPerChunk = kChunk / kKSlice;
 constexpr int kStages = 4;
+constexpr int kEpilogueStages = 48;                  // a unit's epilogue in stages (gram_unit_slices)
 constexpr int kTileBytes = kTile * kKSlice;          // 16 KB
 constexpr int kStageBytes = 3 * kTileBytes;          // A + the two 128-row halves of B
 constexpr int kGramThreads = 192;
@@ -627,15 +628,35 @@ cudaError_t encode_onehot_map(void* map, const uint8_t* E, int Mp, long long K)
 
 size_t tensor_map_bytes() { return sizeof(CUtensorMap); }
 
-// Stages (128 samples each) per work unit: the whole exact accumulation, or
-// less while the units leave SMs idle.  tiles: output tiles of every problem
-// times its share of the samples' stages, i.e. sum over problems of tiles x
-// stages.  A unit keeps at least 8 stages: its epilogue adds a 128 x 256 tile.
-int gram_unit_slices(long long tile_stages, int num_sms)
+// Stages (128 samples each) per work unit for problems of tiles[p] output tiles
+// over stages[p] stages: the count up to the exact accumulation's for which the
+// CTA with the most work ends first.  Its rounds over the units cost a unit's
+// stages, or the epilogue of the unit before where that takes longer, and one
+// epilogue stays at the end.  An epilogue is 32,768 atomic additions, and with every
+// SM busy the chip takes some 370 per ns: 13.5 us, 45 stages (thousand variables at
+// 200,000 samples with units of 8 stages: 2,140 us instead of 730).  300 variables at
+// 20,011 samples, 9 tiles of 157 stages: 144 units of 10 stages in one round, 95 us
+// with the transfers, where powers of two had given 180 of 8 in two, 109 us; units of
+// 32 stages take 104 us.
+int gram_unit_slices(const long long* tiles, const long long* stages, int k, int num_sms)
 {
-    int s = kSlicesPerChunk;
-    while (s > 8 && tile_stages / s < 2LL * num_sms) s /= 2;
-    return s;
+    long long best = -1;
+    int unit = kSlicesPerChunk;
+    for (int s = kSlicesPerChunk; s >= 8; --s) {
+        long long units = 0, whole = 0;
+        for (int p = 0; p < k; ++p) {
+            units += tiles[p] * ((stages[p] + s - 1) / s);
+            whole += tiles[p] * (stages[p] / s);
+        }
+        const long long before = (units + num_sms - 1) / num_sms - 1;   // rounds before the last
+        const long long last = k == 1 && before * num_sms >= whole ? stages[0] % s : s;
+        const long long cost = before * std::max(s, kEpilogueStages) + last + kEpilogueStages;
+        if (best < 0 || cost < best) {
+            best = cost;
+            unit = s;
+        }
+    }
+    return unit;
 }
 
 int gram_chunks(long long K, int unit_slices) { return (int)((K / kKSlice + unit_slices - 1) / unit_slices); }

@@ -17,7 +17,7 @@ cudaError_t launch_onehot(const ProblemDev* probs, const int32_t* vtx_prob, cons
 cudaError_t launch_zero_pad(const ProblemDev* probs, int nprob, cudaStream_t st);
 cudaError_t encode_onehot_map(void* map, const uint8_t* E, int Mp, long long K);
 size_t tensor_map_bytes();
-int gram_unit_slices(long long tile_stages, int num_sms);
+int gram_unit_slices(const long long* tiles, const long long* stages, int k, int num_sms);
 int gram_chunks(long long K, int unit_slices);
 cudaError_t launch_gram(const void* maps, const int4* units, int n_units, int unit_slices, const ProblemDev* probs,
                         int num_sms, unsigned* status, int wait_limit, cudaStream_t st);

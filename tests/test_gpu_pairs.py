@@ -34,7 +34,8 @@ def _data(n, N, hi, seed):
     return np.stack(rows).astype(np.uint8), ar
 
 
-@pytest.mark.parametrize("n,N,hi", [(3, 1, 2), (31, 130, 5), (33, 8193, 24), (65, 300, 4), (130, 1000, 2)])
+@pytest.mark.parametrize("n,N,hi", [(3, 1, 2), (31, 130, 5), (33, 8193, 24), (65, 300, 4), (130, 1000, 2),
+                                    (24, 40000, 3), (200, 20011, 4)])   # few tiles of many samples: units of 8 stages and up
 def test_pair_tables(F, n, N, hi):
     import torch
     data, ar = _data(n, N, hi, n + N)
