@@ -68,7 +68,7 @@ inline int ci_cluster(long long N, long long cells, int max_cluster)
 // prefix product, where one thread's recurrence would wait for 32 dependent
 // divisions.  Warp 1 evaluates the factor and erfc meanwhile: a dependent FP64
 // operation takes some 100 cycles here, and the two chains are equally long
-// (16 tests of 100,003 samples, one after the other: 260 us with both on one
+// (8 tests of 100,003 samples, one after the other: 260 us with both on one
 // warp, 247 us so).
 __device__ __forceinline__ double chisq_q_warps(double df, double g2, double lgamma_a, unsigned* status, double* share)
 {
