@@ -86,8 +86,7 @@ def parse():
                     help="autotune the counting per depth before the warm-up (fbn_autotune; untimed), or keep the "
                          "fixed rules")
     ap.add_argument("--count", choices=["auto", "hist", "bits"], default="auto",
-                    help="table counting: bit planes for small tables (auto), byte histograms only, bit planes "
-                         "wherever they fit")
+                    help="table counting of depth 1: one-hot planes where they apply (auto, bits) or byte histograms only")
     ap.add_argument("--ablation", action="store_true",
                     help="instead of the bench line: the group-size, granularity, sample-size and network-size "
                          "studies, one JSON line per configuration")
@@ -324,7 +323,10 @@ def run_ablation(args):
     import paper_2212_04259_gb300 as F
     from paper_2212_04259_gb300 import build
     build.build()
-    stream = torch.cuda.current_stream()
+    # a stream of its own: the default stream's handle is 0, which leaves the library on its own
+    # non-blocking stream, unordered with the flush and the events
+    stream = torch.cuda.Stream()
+    torch.cuda.set_stream(stream)
     flush = torch.empty(64 * 1024 * 1024, dtype=torch.int32, device="cuda")
 
     def measure(data, ar, alpha, md, **opt):
@@ -403,7 +405,10 @@ def main():
         if dist is not None:
             dist.barrier()
 
-    stream = torch.cuda.current_stream()
+    # a stream of its own: the default stream's handle is 0, which leaves the library on its own
+    # non-blocking stream, unordered with the flush and the events
+    stream = torch.cuda.Stream()
+    torch.cuda.set_stream(stream)
     gs = args.gs
     if w["kind"] == "single":
         data_dev = torch.from_numpy(w["data"]).cuda()
@@ -501,8 +506,8 @@ def main():
 
     # the unit that binds the counting: measured on this device by the
     # library (fbn_measure_unit_rates).  The dominant pool depth's kernel is
-    # reported against it: POPC for tables counted from bit planes (cells x
-    # 32-sample words of work), shared-memory reductions for byte histograms
+    # reported against it: POPC for tables counted from one-hot planes (counted
+    # cells x 32-sample words), shared-memory reductions for byte histograms
     # (one per sample); the work counters are the executed tests' (redundant
     # tests included), the time the depth's test window.
     rates = F.fbn_measure_unit_rates(local)

@@ -1,6 +1,7 @@
 // fbn_api.cu -- host engine and C ABI (include/fbn.h) of the GB300 PC-stable
-// skeleton library.  The depth loop of Algorithm 1 runs here; every step of a
-// depth (snapshot, edge list, CI tests, removal) is a kernel in fbn_kernels.cu.
+// skeleton library.  The depth loop of Algorithm 1 is set up here; the steps of a depth
+// (snapshot, edge list, CI tests, removal) are kernels in fbn_kernels.cu, the
+// Gram and pools' files, or for small calls phases of one kernel (fbn_loop.cu).
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>

@@ -5,8 +5,8 @@
 //   * shared-memory reductions: red.shared.add on 32-bit words, every thread
 //     on its own column (no bank conflicts, no contention) -- the operation the
 //     byte histograms of the work pool issue once per sample;
-//   * POPC: independent population counts -- the operation the bit-plane
-//     count issues once per cell and 32 samples.
+//   * POPC: independent population counts -- the operation the count
+//     from one-hot planes issues once per counted cell and 32 samples.
 //
 // Each kernel runs a few milliseconds over every SM (8 CTAs of 256 threads per
 // SM), timed with CUDA events after a warm-up launch; the reductions are

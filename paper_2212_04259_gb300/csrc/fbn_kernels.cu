@@ -11,12 +11,13 @@
 //   k_scan / k_place
 //                order each class by chunk count (counted by k_edges), so that
 //                pass k of the work pool is a prefix of that order
-//   k_pool<G>    persistent CI-level work pool (Section IV-B): each group (a
+//   k_pool_*     persistent CI-level work pool (Section IV-B): each group (a
 //                warp or a CTA) claims work items -- one chunk of gs
 //                consecutive conditioning sets of one edge -- from one atomic
 //                counter; items are laid out pass by pass, so every live edge
 //                gets its k-th chunk before any edge gets its (k+1)-th; chunks
 //                above an edge's lowest accepting rank are skipped
+//   k_pool_marg  the pool of depth 1 from one-hot planes (fbn_pool_marg.cuh)
 //   k_plain      edge-level form (Section IV-A): one CTA per edge, sequential
 //                conditioning sets with early exit
 //   k_apply      end-of-depth removal over the snapshot; the separating set is
@@ -27,7 +28,7 @@
 // Every kernel reads the depth and the sizes from the device counters, so one
 // captured sequence serves every depth (the body of the depth loop's while
 // node); a kernel that runs after the loop ended finds active == 0 and does
-// nothing.
+// nothing.  Small calls run the same phases inside one kernel (fbn_loop.cu).
 #include <cstdint>
 #include <cuda_runtime.h>
 
