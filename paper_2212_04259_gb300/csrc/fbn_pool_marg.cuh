@@ -345,7 +345,11 @@ __device__ __forceinline__ void marg_body(const PoolArgs& a)
         unsigned long long* min_accept = a.min_accept + e;
         const long long cr = whole ? w.total : chunk_ranks(w.total, gs);
         const int r0 = (int)(pass * cr), r1 = (int)(r0 + cr < w.total ? r0 + cr : w.total);
-        if (!whole && (unsigned long long)r0 > *((volatile unsigned long long*)min_accept)) continue;
+        if (!whole) {   // read by lane 0 and broadcast: other warps lower it, and the warp must stay together
+            unsigned long long ma = 0;
+            if (lane == 0) ma = *((volatile unsigned long long*)min_accept);
+            if ((unsigned long long)r0 > __shfl_sync(0xffffffffu, ma, 0)) continue;
+        }
         MargEdge E;
         const int ri = P.ar[w.i], rj = P.ar[w.j];
         E.vx = ri >= rj ? w.i : w.j;

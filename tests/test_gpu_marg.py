@@ -6,7 +6,8 @@ ranks.  Covered: every pair of arities 2..5 (the counting shapes, with two
 strata per pass or one), samples around the 64-sample word and across 65,536
 (two counts per reduction below it), both statistics and both degrees of
 freedom, values that never occur, pair tables from the Gram and from the
-planes, an arity above 5 (histograms), and enough edges for whole-edge items.
+planes, an arity above 5 (histograms), enough edges for whole-edge items, and
+edges whose lowest accepting rank many warps lower and read at once.
 """
 import numpy as np
 import pytest
@@ -92,3 +93,23 @@ def test_many_edges(F, opt):
         d, a = probs[p]
         hard, _, _ = compare(adjs[p], F.fbn_export_sepsets(hs[p]), oracle.pc_stable(d, a, 1e-4, 1))
         assert not hard, hard[:3]
+
+
+# 1,965 edges, each conditioning set an item of its own, and two edges in three have a set that
+# accepts: warps read an edge's rank, and skip their item, while others lower it.
+@pytest.mark.parametrize("opt", [dict(), dict(loop="host"), dict(group_size=1)])
+def test_ranks_lowered_while_read(F, opt):
+    rng = np.random.default_rng(11)
+    N = 700
+    base = rng.integers(0, 3, N)
+    ar = np.array([2 + k % 3 for k in range(64)], dtype=np.uint8)
+    data = np.stack([np.where(rng.random(N) < 0.45, base % r, rng.integers(0, r, N)) for r in ar]).astype(np.uint8)
+    ref = oracle.pc_stable(data, ar, 1e-3, 1)
+    h = F.fbn_create(data, ar, **opt)
+    for _ in range(50):
+        adj = F.fbn_learn_skeleton(h, 1e-3, 1)
+        hard, _, _ = compare(adj, F.fbn_export_sepsets(h), ref)
+        assert not hard, hard[:3]
+        st = F.fbn_get_stats(h)
+        assert st["tests_oracle"] == ref.tests and st["removed"] == ref.removed
+    assert st["edges"][1] > 1000 and st["removed"][1] > 0
