@@ -247,7 +247,10 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_loop(const __grid_constant_
                         a.bits);
             if (!loop_barrier(a.bar, &ctr->status, gen, a.spin_limit, next)) return;
         }
-        if (!ctr->active) break;   // the same for every CTA
+        // turn() set it before the barrier opened.  Without the bit matrix the last
+        // CTA may be ending the depth already (depth_end above): every CTA then
+        // reads it behind the snapshot's barrier
+        if (a.bits && !ctr->active) break;
     }
     if (a.h_ctr) loop_results(a, gen, warp0, warps, t0, threads);
 }

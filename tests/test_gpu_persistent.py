@@ -3,8 +3,9 @@
 Covered: variable counts around the bounds of the one-CTA turn (128) and of the
 persistent loop (512), small batches, a depth with more items than the turn
 lays out (the general phases take over and give back), every kind of output
-buffer, separating sets read late, twice, or never between calls, and a changing
-maximum depth on one handle.
+buffer, separating sets read late, twice, or never between calls, a changing
+maximum depth on one handle, and many repeats of calls that stop at their maximum
+depth in the general phases (no bit matrix: above 128 variables, or a batch).
 """
 import numpy as np
 import pytest
@@ -88,3 +89,30 @@ def test_small_batch_and_members(F):
     d, a, _ = probs[0]
     hard, _, _ = compare(F.fbn_learn_skeleton(hs[0], 0.01, -1), F.fbn_export_sepsets(hs[0]), oracle.pc_stable(d, a, 0.01, -1))
     assert not hard
+
+
+# Above 128 variables and in batches the last CTA ends a depth while the others
+# list the next one's neighbours: a CTA that read the loop's flag between the two
+# left a phase early.  Repeats of calls that stop there, separating sets included.
+@pytest.mark.parametrize("n,md", [(129, 0), (129, 1), (300, 0), (300, 2), (512, 0), (512, 1)])
+def test_stop_at_maximum_depth_repeatedly(F, n, md):
+    data, ar, _ = bnsynth.make_dataset(n, n, int(1.2 * n), 3, (2, 3), 1.0, 150)
+    ref = oracle.pc_stable(data, ar, 0.05, md)
+    h = F.fbn_create(data, ar)
+    first = np.array(F.fbn_learn_skeleton(h, 0.05, md))
+    _same(F, h, first, ref)
+    sets = F.fbn_export_sepsets(h, as_dict=False)
+    for _ in range(300):
+        assert np.array_equal(np.asarray(F.fbn_learn_skeleton(h, 0.05, md)), first)
+        assert all(np.array_equal(a, b) for a, b in zip(F.fbn_export_sepsets(h, as_dict=False), sets))
+
+
+def test_batch_stops_at_maximum_depth_repeatedly(F):
+    probs = bnsynth.batched_workload(4, first=3, n_range=(20, 60), samples_range=(500, 3000))
+    refs = [oracle.pc_stable(d, a, 0.05, 1) for d, a, _ in probs]
+    hs = [F.fbn_create(d, a) for d, a, _ in probs]
+    for _ in range(200):
+        adjs = F.fbn_learn_skeleton_batch(hs, 0.05, 1)
+    for h, adj, ref in zip(hs, adjs, refs):
+        hard, _, _ = compare(adj, F.fbn_export_sepsets(h), ref)
+        assert not hard, hard[:3]
