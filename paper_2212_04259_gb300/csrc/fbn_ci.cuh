@@ -163,6 +163,7 @@ __device__ __forceinline__ void ci_cluster_test(const CiArgs& q)
     extern __shared__ __align__(16) int smem[];
     __shared__ TestSpec spec;
     __shared__ double red[32];
+    __shared__ double share[2];   // warp 1's half of the p-value (not red: warp 0 may still be adding up the statistic there)
     __shared__ double part[kCiMaxCluster], part_df[kCiMaxCluster];   // CTA 0: every CTA's share
     __shared__ int t_off, s_bad;
     __shared__ unsigned s_status;
@@ -272,7 +273,7 @@ __device__ __forceinline__ void ci_cluster_test(const CiArgs& q)
     double lg = q.lgamma_a;
     if (q.df_mode) lg = df > 0.0 ? lgamma(0.5 * df) : 0.0;
     else df = (double)(q.rx - 1) * (double)(q.ry - 1) * (double)nz;
-    const double p = df > 0.0 ? chisq_q_warps(df, st, lg, &s_status, red) : 1.0;
+    const double p = df > 0.0 ? chisq_q_warps(df, st, lg, &s_status, share) : 1.0;
     __syncwarp();
     if (tid == 0) {
         q.out[0] = st;

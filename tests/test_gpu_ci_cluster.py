@@ -56,3 +56,17 @@ def test_cluster_tests_match_oracle(F, arities, S, N, dep):
     rg2, rdf, rp = oracle.ci_test(data, ar, 0, 1, S)
     assert out[1].item() == rdf and out[0].item() == pytest.approx(rg2, rel=1e-6, abs=1e-12)
     assert abs(out[2].item() - rp) <= 1e-9 and np.array_equal(table.cpu().numpy(), ref)
+
+
+# One CTA (few samples, few cells): the warp that adds up the statistic and the one that
+# prepares the p-value run side by side, so every repeat has to give the same bits.
+@pytest.mark.parametrize("stat,df_mode", [("g2", "fixed"), ("g2", "adjusted"), ("x2", "fixed"), ("x2", "adjusted")])
+def test_one_cta_repeats_bit_for_bit(F, stat, df_mode):
+    data, ar = _data(3001, [2, 3, 2, 4], 0.05)
+    h = F.fbn_create(data, ar, statistic=stat, df=df_mode)
+    for S in ([], [2], [3, 2]):
+        ref = oracle.ci_test(data, ar, 0, 1, S, stat=stat, df_mode=df_mode)
+        first = F.fbn_ci_test(h, 0, 1, S)
+        assert first[1] == ref[1] and first[0] == pytest.approx(ref[0], rel=1e-6) and abs(first[2] - ref[2]) <= 1e-9
+        for _ in range(1000):
+            assert F.fbn_ci_test(h, 0, 1, S) == first
