@@ -466,7 +466,9 @@ int grow_workspace(fbn_handle* h, Workspace& ws, long long edge_cap, int max_n, 
             }
         }
         CK(dalloc(&ws.binom, B.size()));
-        CK(cudaMemcpy(ws.binom, B.data(), B.size() * sizeof(long long), cudaMemcpyHostToDevice));
+        // on the handle's stream: it does not wait for the legacy one (as below)
+        CK(cudaMemcpyAsync(ws.binom, B.data(), B.size() * sizeof(long long), cudaMemcpyHostToDevice, h->stream));
+        CK(cudaStreamSynchronize(h->stream));
         ws.brows = rows;
     }
     if (total_vtx > ws.vtx_cap) {
@@ -1103,7 +1105,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     if (h->tune != ws.tune_loaded) {   // the autotuner's per-depth choices
         std::vector<int> t(kMaxDepthRecords, 0);
         for (size_t d = 0; d < h->tune.size() && d < t.size(); ++d) t[d] = h->tune[d];
-        CK(cudaMemcpy(ws.d_tune, t.data(), t.size() * sizeof(int), cudaMemcpyHostToDevice));
+        CK(cudaMemcpyAsync(ws.d_tune, t.data(), t.size() * sizeof(int), cudaMemcpyHostToDevice, st));
         ws.tune_loaded = h->tune;
     }
     DepthCounters c0{};
@@ -1588,8 +1590,10 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     if (adj_staged) std::memcpy(adj_out[0], ws.h_adj, (size_t)h->n * h->n);
     for (size_t s = 0; s < staged.size(); ++s)
         std::memcpy(adj_out[staged[s]], ws.h_adj + staged_at[s], (size_t)hs[staged[s]]->n * hs[staged[s]]->n);
-    if (persistent && (ws.h_ctr->status & kStatusTimeout))   // a barrier gave up: its counters are not whole
-        CK(cudaMemset(ws.d_bar, 0, 2 * sizeof(unsigned)));
+    if (persistent && (ws.h_ctr->status & kStatusTimeout)) {   // a barrier gave up: its counters are not whole
+        CK(cudaMemsetAsync(ws.d_bar, 0, 2 * sizeof(unsigned), st));
+        CK(cudaStreamSynchronize(st));
+    }
     if (loop && !shard) launches += (long long)(body_launches - (host_loop ? 1 : 0)) * std::max(0, ws.h_ctr->d - d_loop);
     if (direct1) {
         float kms = 0.f;
@@ -2068,6 +2072,19 @@ int fbn_create(const uint8_t* data, int32_t n_vars, int64_t n_samples, const uin
     CKC(cudaMemsetAsync(h->d_eid, 0, nn * sizeof(int32_t), st));
     CKC(cudaMemsetAsync(h->d_bad, 0xff, sizeof(unsigned long long), st));
     CKC(cudaMemcpyAsync(h->d_ar, arities, n_vars, cudaMemcpyHostToDevice, st));
+    std::vector<int32_t> off(2 * (size_t)n_vars);
+    int M = 0;
+    for (int v = 0; v < n_vars; ++v) {
+        off[v] = M;
+        off[n_vars + v] = M - v;
+        M += arities[v];
+    }
+    h->M = M;
+    h->Mp = gram_rows_padded(M);
+    h->Mr = gram_rows_padded(M - n_vars);
+    h->K = gram_samples_padded(n_samples);
+    CKC(dalloc(&h->d_off, off.size()));
+    CKC(cudaMemcpyAsync(h->d_off, off.data(), off.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     // values must lie below their arity: checked on the device
     if (const int irc = ingest(h, data, h->d_bad, st)) return bail(irc);
     unsigned long long first_bad = 0;
@@ -2079,21 +2096,6 @@ int fbn_create(const uint8_t* data, int32_t n_vars, int64_t n_samples, const uin
         const long long s = (long long)(first_bad % (unsigned long long)n_samples);
         fail(h, FBN_EDATA, "value of variable %lld at sample %lld is >= its arity %d", v, s, (int)arities[v]);
         return bail(FBN_EDATA);
-    }
-    {
-        std::vector<int32_t> off(2 * (size_t)n_vars);
-        int M = 0;
-        for (int v = 0; v < n_vars; ++v) {
-            off[v] = M;
-            off[n_vars + v] = M - v;
-            M += arities[v];
-        }
-        h->M = M;
-        h->Mp = gram_rows_padded(M);
-        h->Mr = gram_rows_padded(M - n_vars);
-        h->K = gram_samples_padded(n_samples);
-        CKC(dalloc(&h->d_off, off.size()));
-        CKC(cudaMemcpy(h->d_off, off.data(), off.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
     }
 #undef CKC
     *out = h;
@@ -2115,7 +2117,8 @@ int fbn_update_data(fbn_handle* h, const uint8_t* data)
     unsigned long long first_bad;
     std::memcpy(&first_bad, h->h_status, sizeof first_bad);
     if (first_bad != ~0ULL) {
-        CK(cudaMemset(h->d_bad, 0xff, sizeof(unsigned long long)));   // all ones between calls
+        CK(cudaMemsetAsync(h->d_bad, 0xff, sizeof(unsigned long long), st));   // all ones between calls
+        CK(cudaStreamSynchronize(st));                                         // whatever the next call's stream
         const long long v = (long long)(first_bad / (unsigned long long)h->N);
         const long long smp = (long long)(first_bad % (unsigned long long)h->N);
         return fail(h, FBN_EDATA, "value of variable %lld at sample %lld is >= its arity %d", v, smp,

@@ -63,3 +63,25 @@ def test_every_memory_and_alignment(F, where, N):
             assert e.value.code == -2 and f"variable {v} at sample {smp} " in str(e.value)
         F.fbn_update_data(h, _place(first, where, 0))   # usable again
         assert np.array_equal(F.fbn_ci_table(h, 0, 1), oracle.ci_table(first, ar, 0, 1))
+
+
+# The first bad value of a refused upload must not reach the next call, whatever its stream.
+@pytest.mark.parametrize("where", ["pinned", "device"])
+def test_refused_then_valid_repeatedly(F, where):
+    import torch
+    rng = np.random.default_rng(7)
+    ar = np.array([3, 2, 4], dtype=np.uint8)
+    good = np.stack([rng.integers(0, r, 4001) for r in ar]).astype(np.uint8)
+    bad = good.copy()
+    bad[1, 17] = 2
+    good_m, bad_m = _place(good, where, 3), _place(bad, where, 3)
+    h = F.fbn_create(good_m, ar)
+    streams = [torch.cuda.Stream().cuda_stream, 0]
+    for t in range(400):
+        with pytest.raises(F.FbnError) as e:
+            F.fbn_update_data(h, bad_m)
+        assert "variable 1 at sample 17 " in str(e.value)
+        if t % 3 == 0:
+            F.fbn_set_stream(h, streams[t // 3 % 2])
+        F.fbn_update_data(h, good_m)
+    assert np.array_equal(F.fbn_ci_table(h, 2, 1, [0]), oracle.ci_table(good, ar, 2, 1, [0]))
