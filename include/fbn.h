@@ -63,8 +63,9 @@ extern "C" {
 #define FBN_TUNE_AUTO 1    /* the first skeleton call on a workload shape runs fbn_autotune (or reuses its result
                               for this device and shape from earlier in the process) and applies its choices */
 
-#define FBN_LOOP_DEVICE 0  /* the depths after any launched directly run as one CUDA graph whose while node the
-                              device drives (no host round trip between depths) */
+#define FBN_LOOP_DEVICE 0  /* no host round trip between depths: calls of up to 512 variables without a tensor-core
+                              depth run as one persistent kernel, the others launch the first depths directly and
+                              the rest as one CUDA graph whose while node the device drives */
 #define FBN_LOOP_HOST   1  /* the same kernels, one depth at a time from the host, which reads the loop flag
                               between depths (for tools that profile kernel by kernel) */
 
@@ -74,9 +75,10 @@ typedef struct fbn_options {
     int32_t depth0;      /* FBN_DEPTH0_* */
     int32_t device;      /* CUDA device ordinal; -1 = the current device */
     int32_t group_threads; /* threads per CI test in the pool: 32, 64, 128 or 256; 0 = chosen per depth */
-    int32_t wait_limit;  /* attempts of each bounded device wait of the depth-0 Gram pipeline; 0 = default
-                            (2^22); -1 = give up at once, which exercises the FBN_ETIMEOUT path (also the depth-1
-                            tensor-core pipeline) */
+    int32_t wait_limit;  /* attempts of each bounded device wait; 0 = default, -1 = give up at once.  The depth-0
+                            Gram and the depth-1 tensor-core pipelines (default 2^22) then end with FBN_ETIMEOUT;
+                            the persistent kernel (default 2^23 polls without progress) gives way to the
+                            graph, with the same results */
     int32_t depth1;      /* FBN_DEPTH1_*: how depth 1 counts its tables (pool form only); every test of a
                             vertex's neighbourhood at once on the tensor cores, or the work pool */
     int32_t statistic;   /* FBN_STAT_G2 (default) or FBN_STAT_X2: the statistic of every CI test */

@@ -271,6 +271,7 @@ struct Workspace {
     unsigned long long *d_bads = nullptr, *h_bads = nullptr;   // first bad values of a batch of uploads
     size_t bad_cap = 0;
     unsigned* d_bar = nullptr;                      // barrier of the persistent loop
+    unsigned* h_gave_up = nullptr;                  // pinned: 1 when a wait of the loop ran out
     unsigned* d_bits = nullptr;                     // its adjacency bit matrix
     uint8_t* h_adj = nullptr;                       // pinned: the adjacency it leaves
     size_t h_adj_cap = 0;
@@ -310,6 +311,7 @@ struct Workspace {
         if (h_bads) cudaFreeHost(h_bads);
         dfree(d_bads);
         dfree(d_bar); dfree(d_bits);
+        if (h_gave_up) cudaFreeHost(h_gave_up);
         h_maps.clear();
         gram_E = nullptr; gram_G = nullptr; gram_R = nullptr; gram_maps = nullptr; gram_units = nullptr; pk = nullptr;
         split_tab = nullptr; split_ticket = nullptr;
@@ -936,11 +938,11 @@ struct ShardHooks {
 
 // The depth loop of Algorithm 1 over one or more problems sharing a stream,
 // one attempt.  Every kernel of a depth takes the depth and the sizes from the
-// device counters, so the host queues depth d+1 before depth d has finished
-// and only waits for the loop flag of depth d-1.  *retry is set when a
-// separating-set pool or global-table scratch turned out too small (both are
-// grown before returning).
-int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_depth, bool* retry,
+// device counters.  *retry is set when a separating-set pool or global-table
+// scratch turned out too small (both are grown before returning), or when a
+// wait of the persistent loop ran out (*allow_loop is cleared: the depths then
+// run as a graph, whose kernels wait for nothing).
+int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_depth, bool* retry, bool* allow_loop,
                       uint8_t* const* adj_out, const ShardHooks* shard = nullptr)
 {
     fbn_handle* h = hs[0];
@@ -1033,7 +1035,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         }
     }
     long long launches = 0;
-    const bool persistent = !shard && !plain && !gram && !nbr1 && h->opt.loop == FBN_LOOP_DEVICE &&
+    const bool persistent = *allow_loop && !shard && !plain && !gram && !nbr1 && h->opt.loop == FBN_LOOP_DEVICE &&
                             total_vtx <= kLoopVertices;
     if (!gram && !persistent) {   // the complete graph (the Gram's decisions write every pair themselves)
         k_init_graph<<<total_vtx, 256, 0, st>>>(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx);
@@ -1354,11 +1356,15 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
             la.big.gscratch = ws.gscratch;
             la.big.gscratch_ints = 3 * ws.gs_cells + 64;
         }
-        la.spin_limit = 1u << 23;   // seconds
+        // 2^23 polls are seconds
+        la.spin_limit = h->opt.wait_limit < 0 ? 0u : h->opt.wait_limit > 0 ? (unsigned)h->opt.wait_limit : 1u << 23;
         if (!ws.d_bar) {
             CK(dalloc(&ws.d_bar, 2));
             CK(cudaMemsetAsync(ws.d_bar, 0, 2 * sizeof(unsigned), st));
         }
+        if (!ws.h_gave_up) CK(cudaMallocHost((void**)&ws.h_gave_up, sizeof(unsigned)));
+        CK(cudaHostGetDevicePointer((void**)&la.gave_up, ws.h_gave_up, 0));
+        *ws.h_gave_up = 0;
         la.bar = ws.d_bar;
         if (k == 1 && h->n <= kTurnVertices) {
             if (!ws.d_bits) CK(dalloc(&ws.d_bits, kTurnVertices * (kTurnVertices / 32)));
@@ -1382,7 +1388,6 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
             h_tot = reinterpret_cast<const long long*>(ws.stage->p + csr);
             la.sep_cnt = h->d_sep_cnt;
         }
-        if (direct_out) ws.h_ctr->status = kStatusTimeout;   // overwritten by the loop's last phase
         CK(launch_loop(la, grid, kWarpSmemBytes, st));
         launches += 1;
     }
@@ -1587,13 +1592,16 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         }
     }
     CK(cudaStreamSynchronize(st));
+    if (persistent && *ws.h_gave_up) {   // the barrier's words and the counters are not whole
+        CK(cudaMemsetAsync(ws.d_bar, 0, 2 * sizeof(unsigned), st));
+        CK(cudaStreamSynchronize(st));
+        *allow_loop = false;
+        *retry = true;
+        return FBN_OK;
+    }
     if (adj_staged) std::memcpy(adj_out[0], ws.h_adj, (size_t)h->n * h->n);
     for (size_t s = 0; s < staged.size(); ++s)
         std::memcpy(adj_out[staged[s]], ws.h_adj + staged_at[s], (size_t)hs[staged[s]]->n * hs[staged[s]]->n);
-    if (persistent && (ws.h_ctr->status & kStatusTimeout)) {   // a barrier gave up: its counters are not whole
-        CK(cudaMemsetAsync(ws.d_bar, 0, 2 * sizeof(unsigned), st));
-        CK(cudaStreamSynchronize(st));
-    }
     if (loop && !shard) launches += (long long)(body_launches - (host_loop ? 1 : 0)) * std::max(0, ws.h_ctr->d - d_loop);
     if (direct1) {
         float kms = 0.f;
@@ -1673,9 +1681,10 @@ int run_skeleton(fbn_handle* const* hs, int k, double alpha, int32_t max_depth, 
                  const ShardHooks* shard = nullptr)
 {
     for (int p = 0; p < k; ++p) drop_sepsets(hs[p]);   // their pinned memory is written again
-    for (int attempt = 0; attempt < 6; ++attempt) {
+    bool allow_loop = true;
+    for (int attempt = 0; attempt < 7; ++attempt) {
         bool retry = false;
-        const int rc = run_skeleton_once(hs, k, alpha, max_depth, &retry, adj_out, shard);
+        const int rc = run_skeleton_once(hs, k, alpha, max_depth, &retry, &allow_loop, adj_out, shard);
         if (rc || !retry) return rc;
     }
     return fail(hs[0], FBN_ENOMEM, "scratch or separating-set pool kept overflowing");

@@ -130,6 +130,8 @@ struct DepthCounters {
     unsigned long long max_total[2];    // largest rank count of an edge per class
     int split[2];                       // sample parts per test per class (1 = whole tests)
     int whole;                          // depth 1 from one-hot planes: an item is a whole edge (set by k_edges)
+    unsigned int beat;                  // persistent loop: ranks begun after an item's first (its barriers wait on while
+                                        // this or next_item moves)
     int direct;                         // 1: item w is chunk w / E of the class's edge w mod E (empty past its last)
     DepthRecord* rec;                   // per-depth records (persists)
     const int* tune;                    // per-depth choices of the autotuner, or nullptr (persists):

@@ -24,17 +24,52 @@ namespace {
 
 constexpr long long kPlaceSerial = 2048;   // edges the last CTA of the edge list orders by itself
 
+constexpr unsigned kGaveUp = 1u << 31;   // bar[0]: the phase will not open
+
+__device__ __forceinline__ unsigned phases_open(const unsigned* bar)
+{
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&bar[1]) : "memory");
+    return v;
+}
+
+// A CTA that has waited too long marks the phase as given up, unless it is open
+// or about to be; true when it is given up.  The mark goes on a count that still
+// lacks a CTA, and the CTA that completes a marked count does not open the phase:
+// so every CTA passes a barrier, or none.  (A count read or marked may belong to
+// the next phase when this one has opened meanwhile; the open word, read after a
+// fence, tells, and the next phase is then given up by all.)
+__device__ __noinline__ bool give_up(unsigned* bar, unsigned gen)
+{
+    unsigned w = *((volatile unsigned*)&bar[0]);
+    for (;;) {
+        __threadfence();
+        if (phases_open(bar) == gen + 1) return false;
+        if (w & kGaveUp) return true;
+        if (w == 0 || w == gridDim.x) return false;   // everyone is here: the last one is opening it
+        const unsigned old = atomicCAS(&bar[0], w, w | kGaveUp);
+        if (old == w) {
+            __threadfence();
+            return phases_open(bar) != gen + 1;
+        }
+        w = old;
+    }
+}
+
 // All CTAs of the (cooperative) grid; the one that arrives last runs `last`
-// first.  The wait is bounded: false when it gave up (the status bit is set,
-// every CTA then leaves).
+// first.  The wait is bounded: after a.spin_limit polls during which no CTA claimed
+// an item or finished a test within one, the waiting CTA gives the phase up; every
+// CTA then leaves (false), and the host runs the call as a graph.
 template <class Last>
-__device__ __forceinline__ bool loop_barrier(unsigned* bar, unsigned* status, unsigned& gen, unsigned limit, Last last)
+__device__ __forceinline__ bool loop_barrier(const LoopArgs& a, unsigned& gen, Last last)
 {
     __shared__ int s_role;   // 1: the last to arrive; 0: waited; -1: gave up
+    unsigned* bar = a.bar;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        s_role = atomicAdd(&bar[0], 1u) == gridDim.x - 1 ? 1 : 0;
+        const unsigned before = atomicAdd(&bar[0], 1u);
+        s_role = before == gridDim.x - 1 ? 1 : before & kGaveUp ? -1 : 0;
     }
     __syncthreads();
     if (s_role == 1) {
@@ -46,20 +81,25 @@ __device__ __forceinline__ bool loop_barrier(unsigned* bar, unsigned* status, un
             __threadfence();
             asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&bar[1]), "r"(gen + 1) : "memory");
         }
-    } else if (threadIdx.x == 0) {
-        unsigned it = 0, open = 0;
-        for (; it < limit; ++it) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(open) : "l"(&bar[1]) : "memory");
-            if (open == gen + 1) break;
-        }
-        if (it == limit) {
-            if (status) atomicOr(status, kStatusTimeout);
-            s_role = -1;
+    } else if (s_role == 0 && threadIdx.x == 0) {
+        unsigned long long seen = ~0ULL;
+        unsigned it = 0;
+        while (phases_open(bar) != gen + 1) {
+            if (it++ < a.spin_limit) continue;
+            const volatile DepthCounters* c = a.ctr;
+            const unsigned long long now = c->next_item[0] + c->next_item[1] + c->beat;   // items claimed, tests within them
+            if ((now == seen || a.spin_limit == 0) && give_up(bar, gen)) {
+                s_role = -1;
+                break;
+            }
+            seen = now;
+            it = 0;
         }
         __threadfence();
     }
     __syncthreads();
     ++gen;
+    if (s_role < 0 && threadIdx.x == 0) *((volatile unsigned*)a.gave_up) = 1u;
     return s_role >= 0;
 }
 
@@ -101,10 +141,7 @@ __device__ __forceinline__ void loop_results(const LoopArgs& a, unsigned& gen, i
         for (int k = threadIdx.x; k < (int)(kMaxDepthRecords * sizeof(DepthRecord) / 4); k += kTestThreads) dst[k] = src[k];
     }
     if (status != 0) return;   // the same for every CTA: nothing changes it any more
-    if (!loop_barrier(a.bar, nullptr, gen, a.spin_limit, [] {})) {
-        if (threadIdx.x == 0) *((volatile unsigned*)&a.h_ctr->status) = kStatusTimeout;
-        return;
-    }
+    if (!loop_barrier(a, gen, [] {})) return;
     for (int i = warp0; i < n; i += warps) {
         int p = 0, m = 0;   // pairs and members of the rows before i
         for (int r = lane; r < i; r += 32) {
@@ -178,7 +215,7 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_loop(const __grid_constant_
             P.sep_off[(long long)i * n + j] = 0;
         }
     }
-    if (!loop_barrier(a.bar, &ctr->status, gen, a.spin_limit, none)) return;
+    if (!loop_barrier(a, gen, none)) return;
 
     for (int d = 0;; ++d) {
         const bool popc = d == 0 && a.popc0, marg = d == 1 && a.marg1;
@@ -190,7 +227,7 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_loop(const __grid_constant_
             DepthRecord* begin = d < kMaxDepthRecords ? a.rec + d : nullptr;
             for (int g = warp0; g < a.total_vertices; g += warps)
                 snapshot_vertex(a.probs, a.vtx_prob, a.vtx_first, g, ctr, begin);
-            if (!loop_barrier(a.bar, &ctr->status, gen, a.spin_limit, none)) return;
+            if (!loop_barrier(a, gen, none)) return;
             if (!ctr->active) break;   // the same for every CTA
             for (int g = warp0; g < a.total_vertices; g += warps)
                 edges_vertex(a.probs, a.vtx_prob, a.vtx_first, g, a.gs_forced, a.gs_edges, a.binom, a.brows,
@@ -216,15 +253,15 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_loop(const __grid_constant_
                 }
                 if (E <= kPlaceSerial) place(threadIdx.x, kTestThreads);
             };
-            if (!loop_barrier(a.bar, &ctr->status, gen, a.spin_limit, order)) return;
+            if (!loop_barrier(a, gen, order)) return;
             if (!ctr->active) break;   // the same for every CTA
             if (!popc && (long long)(ctr->n_edges[0] + ctr->n_edges[1]) > kPlaceSerial) {
                 place(t0, threads);
-                if (!loop_barrier(a.bar, &ctr->status, gen, a.spin_limit, none)) return;
+                if (!loop_barrier(a, gen, none)) return;
             }
         }
         if (popc) {
-            pairs_popc_body(a.probs, a.vtx_prob, a.vtx_first, a.total_vertices, a.max_n, nullptr, a.small);
+            pairs_popc_body<true>(a.probs, a.vtx_prob, a.vtx_first, a.total_vertices, a.max_n, nullptr, a.small);
         } else if (marg) {
             marg_body<true>(a.small);
         } else {
@@ -240,12 +277,12 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_loop(const __grid_constant_
         tests_done(ctr);
         const auto next = [&] { if (a.bits) turn(a, turn_sh, direct, warps); };
         if (direct) {   // removal, end of depth and the next depth's items
-            if (!loop_barrier(a.bar, &ctr->status, gen, a.spin_limit, next)) return;
+            if (!loop_barrier(a, gen, next)) return;
         } else {
-            if (!loop_barrier(a.bar, &ctr->status, gen, a.spin_limit, none)) return;
+            if (!loop_barrier(a, gen, none)) return;
             apply_edges(a.probs, a.edges, a.min_accept, a.edge_cap, a.binom, a.sep_pool, a.sep_cap, ctr, t0, threads,
                         a.bits);
-            if (!loop_barrier(a.bar, &ctr->status, gen, a.spin_limit, next)) return;
+            if (!loop_barrier(a, gen, next)) return;
         }
         // turn() set it before the barrier opened.  Without the bit matrix the last
         // CTA may be ending the depth already (depth_end above): every CTA then

@@ -40,10 +40,11 @@ struct LoopArgs {
     int max_depth;
     int popc0, marg1;                    // depths 0 and 1 from one-hot planes
     PoolArgs small, big;                 // the two classes
-    unsigned spin_limit;                 // polls of a phase barrier before the loop gives up
+    unsigned spin_limit;                 // polls of a phase barrier without progress before the loop gives up
+    unsigned* gave_up;                   // pinned host memory: 1 when it did
     unsigned* bits;                      // one problem of <= kTurnVertices variables: its adjacency as a bit
                                          // matrix [kTurnVertices][kTurnVertices / 32] (nullptr: general phases only)
-    unsigned* bar;                       // [2] arrivals of the current phase, phases opened so far
+    unsigned* bar;                       // [2] arrivals of the current phase (and kGaveUp), phases opened so far
     DepthCounters init;                  // the counters' first state
     // one problem: results straight to pinned host memory (nullptr: left on
     // the device): counters, records, adjacency, and the separating sets as

@@ -338,6 +338,7 @@ __device__ __forceinline__ void pool_body(const PoolArgs& a, int* smem, PoolShar
         }
         for (long long rk = r0; rk < r1; ++rk) {
             if (r == 0) S.go = (unsigned long long)rk <= *((volatile unsigned long long*)min_accept);
+            if (LOOP && r == 0 && rk > r0) atomicAdd(&a.ctr->beat, 1u);
             Grp<G>::sync();
             if (!S.go) break;
             const int res = run_rank<G>(a, d, P, w, rk, rk == r0, S, spec, slice, slice_ints, gtab, sh.red);

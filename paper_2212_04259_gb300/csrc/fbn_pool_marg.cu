@@ -17,7 +17,7 @@ __global__ void __launch_bounds__(kTestThreads) k_pairs_popc(const ProblemDev* p
 {
     pdl_enter();
     if (!a.ctr->active) return;
-    pairs_popc_body(probs, vtx_prob, vtx_first, total_vertices, max_n, owned, a);
+    pairs_popc_body<false>(probs, vtx_prob, vtx_first, total_vertices, max_n, owned, a);
     tests_done(a.ctr);
 }
 

@@ -384,6 +384,7 @@ __device__ __forceinline__ void marg_body(const PoolArgs& a)
                 if (!whole && q > 0) {
                     unsigned long long ma = 0;
                     if (lane == 0) ma = *((volatile unsigned long long*)min_accept);
+                    if (LOOP && lane == 0) atomicAdd(&a.ctr->beat, 1u);
                     if ((unsigned long long)(rb + q) > __shfl_sync(0xffffffffu, ma, 0)) {
                         done = true;
                         break;
@@ -486,6 +487,7 @@ __device__ __noinline__ int pair_exact(const PoolArgs& a, bool cell, int n, int 
 
 }  // namespace
 
+template <bool LOOP>
 __device__ __forceinline__ void pairs_popc_body(const ProblemDev* probs, const int32_t* vtx_prob,
                                                 const int32_t* vtx_first, int total_vertices, int max_n,
                                                 const uint8_t* owned, const PoolArgs& a)
@@ -535,6 +537,7 @@ __device__ __forceinline__ void pairs_popc_body(const ProblemDev* probs, const i
         }
         if (owned && !owned[(long long)i * P.n + j]) continue;   // another process tests the pair
         tests += 1;
+        if (LOOP && lane == 0 && t >= warps) atomicAdd(&ctr->beat, 1u);
         work += (unsigned long long)((rx - 1) * (ry - 1)) * (unsigned)((P.N + 31) >> 5);
         // the decision: one stratum holding every sample
         float acc = 0.0f, mag = 0.0f;

@@ -116,3 +116,24 @@ def test_batch_stops_at_maximum_depth_repeatedly(F):
     for h, adj, ref in zip(hs, adjs, refs):
         hard, _, _ = compare(adj, F.fbn_export_sepsets(h), ref)
         assert not hard, hard[:3]
+
+
+# A phase's wait that runs out ends the kernel on every CTA; the call goes on as a graph.
+@pytest.mark.parametrize("limit", [-1, 1, 30, 300, 3000])
+def test_waits_that_run_out(F, limit):
+    for n, N, ar_set, md in ((20, 2000, (2, 3, 4), -1), (101, 1000, (2, 6), 2), (300, 200, (2, 3), 2)):
+        data, ar, _ = bnsynth.make_dataset(n + N, n, int(1.2 * n), 3, ar_set, 1.0, N)
+        ref = oracle.pc_stable(data, ar, 0.05, md)
+        h = F.fbn_create(data, ar, wait_limit=limit)
+        for _ in range(20):
+            st = _same(F, h, F.fbn_learn_skeleton(h, 0.05, md), ref)
+            assert limit >= 0 or st["launches"] > 1
+        h = F.fbn_create(data, ar)
+        assert _same(F, h, F.fbn_learn_skeleton(h, 0.05, md), ref)["launches"] == 1
+    probs = bnsynth.batched_workload(4, first=3, n_range=(20, 60), samples_range=(500, 3000))
+    hs = [F.fbn_create(d, a, wait_limit=limit) for d, a, _ in probs]
+    for _ in range(5):
+        adjs = F.fbn_learn_skeleton_batch(hs, 0.05, -1)
+    for (d, a, _), h, adj in zip(probs, hs, adjs):
+        hard, _, _ = compare(adj, F.fbn_export_sepsets(h), oracle.pc_stable(d, a, 0.05, -1))
+        assert not hard, hard[:3]
