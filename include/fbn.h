@@ -5,8 +5,9 @@
  *
  * Every entry point returns an int status: FBN_OK (0) on success, a negative
  * FBN_E* code otherwise; fbn_last_error() then gives a one-line reason.  A
- * handle is not thread-safe: calls on one handle must not overlap.  Outputs go
- * to caller-provided buffers.  Pointers documented as "host or device" are
+ * handle is not thread-safe: calls on one handle must not overlap; calls on
+ * different handles may, and share the device (small skeletons of several
+ * threads take a share of the SMs each).  Outputs go to caller-provided buffers.  Pointers documented as "host or device" are
  * classified with cudaPointerGetAttributes; device pointers must belong to the
  * handle's device.  No function falls back to the CPU: without a usable CUDA
  * device, fbn_create returns FBN_ECUDA.

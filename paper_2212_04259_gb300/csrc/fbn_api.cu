@@ -3,6 +3,7 @@
 // (snapshot, edge list, CI tests, removal) are kernels in fbn_kernels.cu, the
 // Gram and pools' files, or for small calls phases of one kernel (fbn_loop.cu).
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -43,6 +44,42 @@ constexpr size_t kBigSmemBytes = 200 * 1024;  // the same of the big-table pool 
 // 359 both, with depth 1 at 64 against 49 us).
 constexpr int kLoopVertices = 512;
 constexpr int kLoopOneCta = 32;
+
+// Persistent calls of this process under way per device, those of other threads
+// included.  All CTAs of such a call are resident at once, so a grid that fills the
+// chip makes the calls of several threads wait for one another; each takes its share
+// of the CTAs instead (the results do not depend on the grid), at least a quarter of
+// the SMs: below, a call lasts as many times longer as there are fewer CTAs.  Calls
+// per second of 1 / 2 / 4 / 8 threads, 101 variables x 9,973 samples: grids that fill
+// the chip 3,215 3,403 3,402 3,394, one CTA on every second SM 2,460 4,839 8,556
+// 8,842, on every fourth 1,910 3,784 7,386 12,858; the kernels of a depth as a graph
+// 2,480 3,770 4,980 6,150.
+constexpr int kLoopDevices = 64;
+std::atomic<int> g_loops[kLoopDevices];
+
+class LoopShare {
+public:
+    LoopShare(int device, bool take) : n_(take && device < kLoopDevices ? &g_loops[device] : nullptr)
+    {
+        if (n_) calls_ = n_->fetch_add(1) + 1;
+    }
+    ~LoopShare()
+    {
+        if (n_) n_->fetch_sub(1);
+    }
+    LoopShare(const LoopShare&) = delete;
+    LoopShare& operator=(const LoopShare&) = delete;
+    int grid(int full, int sms) const
+    {
+        int g = full;
+        for (int c = 1; c < calls_ && g / 2 >= sms / 4; c *= 2) g /= 2;
+        return g;
+    }
+
+private:
+    std::atomic<int>* n_;
+    int calls_ = 1;
+};
 constexpr size_t kAdjStageBytes = (size_t)16 << 20;   // pinned bytes a call's graphs pass through at most
 constexpr int kCritCap = 8192;                // critical-value cache slots (power of two)
 constexpr int kCritDense = 8192;              // critical values kept in a dense table: df < kCritDense
@@ -1037,6 +1074,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     long long launches = 0;
     const bool persistent = *allow_loop && !shard && !plain && !gram && !nbr1 && h->opt.loop == FBN_LOOP_DEVICE &&
                             total_vtx <= kLoopVertices;
+    const LoopShare share(h->device, persistent);   // until this call's work is done
     if (!gram && !persistent) {   // the complete graph (the Gram's decisions write every pair themselves)
         k_init_graph<<<total_vtx, 256, 0, st>>>(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx);
         CK(cudaGetLastError());
@@ -1326,7 +1364,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         la.hist = ws.hist;
         la.cursor = ws.cursor;
         la.ord_cap = ws.ord_cap;
-        const int grid = total_vtx <= kLoopOneCta ? dev_sms : ws.grid_loop;
+        const int grid = share.grid(total_vtx <= kLoopOneCta ? dev_sms : ws.grid_loop, dev_sms);
         for (int cls = 0; cls < 2; ++cls) {
             la.sc[cls].hist = ws.hist + cls * ws.ord_cap;
             la.sc[cls].alive = ws.alive + cls * ws.ord_cap;
