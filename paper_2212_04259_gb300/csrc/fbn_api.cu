@@ -1190,6 +1190,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
             sc[cls].base = ws.base + cls * ws.ord_cap;
             for (int k = 0; k < 4; ++k) sc[cls].groups[k] = cls == 0 ? groups[k] : groups_big[k];
             sc[cls].smem_ints = (long long)((cls == 0 ? kWarpSmemBytes : kBigSmemBytes) / 4);
+            sc[cls].mid_ints = (long long)(kSmemBytes / 4);
         }
         launch_order(ws.probs, ws.edges, ws.edge_cap, marg ? 1 : 2, ws.d_ctr, sc, ws.cursor, ws.cursor + ws.ord_cap,
                      ws.sorted, mean_n, forced, kSplitStride, 1, marg, !use_lut, grid_aux, st);
@@ -1214,6 +1215,10 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
             a.base = ws.base + cls * ws.ord_cap;
             a.sorted = ws.sorted;
             launch_pool(a, cls, small ? grid_small : grid_big, smem, st);
+            if (!small && !use_lut) {   // one of the two runs (choose_pool)
+                a.smem_ints = (int)(kSmemBytes / 4);
+                launch_pool_mid(a, grid_plain, kSmemBytes, st);
+            }
         }
     };
     // depth 1 from one-hot planes: every edge is in the small-table class
@@ -1241,7 +1246,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
                      grid_aux, st);
         launch_depth_end(ws.d_ctr, ws.d_rec, max_depth, ws.hist, ws.cursor, st);
     };
-    const int body_launches = plain ? 7 : 9;
+    const int body_launches = plain ? 7 : use_lut ? 9 : 10;
     auto capture_loop = [&]() -> cudaError_t {
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaGraphCreate(&g, 0);

@@ -264,6 +264,10 @@ __device__ __forceinline__ void choose_pool(const ScanClass& sc, int cls, unsign
         sp = sp < kMaxSplit ? sp : kMaxSplit;
         sp = sp > 1 ? sp : 1;
     }
+    // the big-table class where the decision needs marginals: CTAs of 256 threads when
+    // its tests are more than one round of CTAs of 1,024 and fit their shared memory
+    // (a round takes them 44 us against 30, on half as many tests)
+    if (cls == 1) ctr->wide = !need_marg || (long long)W <= g256 || mcell > sc.mid_ints;
     ctr->split[cls] = (int)sp;
     ctr->total_items[cls] = W * (unsigned long long)sp;
 }

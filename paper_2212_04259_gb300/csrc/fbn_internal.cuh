@@ -129,6 +129,7 @@ struct DepthCounters {
     unsigned long long nbr_claim;       // vertex claims of the depth-1 tensor-core kernel
     unsigned long long max_total[2];    // largest rank count of an edge per class
     int split[2];                       // sample parts per test per class (1 = whole tests)
+    int wide;                           // the big-table class runs on k_pool_big (0: k_pool_mid)
     int whole;                          // depth 1 from one-hot planes: an item is a whole edge (set by k_edges)
     unsigned int beat;                  // persistent loop: ranks begun after an item's first (its barriers wait on while
                                         // this or next_item moves)
@@ -183,6 +184,7 @@ struct ScanClass {
     unsigned long long* base;         // [maxc + 1] first item of pass k
     long long groups[4];              // groups of 32, 64, 128, 256 threads the class's pool runs
     long long smem_ints;              // shared ints of one pool CTA of the class
+    long long mid_ints;               // big-table class: the same of a k_pool_mid CTA (0: no such kernel)
 };
 
 // Cache of critical values, see fbn_device.cuh.

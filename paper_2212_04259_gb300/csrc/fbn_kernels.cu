@@ -1,6 +1,6 @@
 // fbn_kernels.cu -- per-depth kernels of the PC-stable skeleton (Algorithm 1)
 // and their host launchers, for sm_103a.  The work-pool kernels live in
-// fbn_pool_small.cu, fbn_pool_big.cu, fbn_plain.cu (device code in
+// fbn_pool_small.cu, fbn_pool_big.cu, fbn_pool_mid.cu, fbn_plain.cu (device code in
 // fbn_pool.cuh) and fbn_pool_marg.cu; the explicit-test kernel in fbn_ci.cu.
 //
 // Depth pipeline (every kernel runs over all problems of a batch at once):
@@ -47,6 +47,7 @@ __global__ void k_pool_marg(PoolArgs a);
 __global__ void k_pairs_popc(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first,
                              int total_vertices, int max_n, const uint8_t* owned, PoolArgs a);
 __global__ void k_pool_big(PoolArgs a);
+__global__ void k_pool_mid(PoolArgs a);
 __global__ void k_plain(PoolArgs a);
 
 // --------------------------------------------------------------------------
@@ -276,6 +277,11 @@ void launch_pool(const PoolArgs& a, int cls, int grid, size_t smem_bytes, cudaSt
     else launch_pdl(k_pool_big, dim3(grid), dim3(kBigThreads), smem_bytes, st, a);
 }
 
+void launch_pool_mid(const PoolArgs& a, int grid, size_t smem_bytes, cudaStream_t st)
+{
+    launch_pdl(k_pool_mid, dim3(grid), dim3(kTestThreads), smem_bytes, st, a);
+}
+
 void launch_pool_marg(const PoolArgs& a, int grid, cudaStream_t st)
 {
     launch_pdl(k_pool_marg, dim3(grid), dim3(kMargThreads), 0, st, a);
@@ -335,12 +341,13 @@ void set_pdl(bool on)
     g_pdl = on;
 }
 
-cudaError_t set_kernel_smem(size_t small_smem, size_t big_smem, size_t plain_smem)
+cudaError_t set_kernel_smem(size_t small_smem, size_t big_smem, size_t cta_smem)
 {
     cudaError_t e;
-    const int b = (int)plain_smem;
+    const int b = (int)cta_smem;
     if ((e = cudaFuncSetAttribute(k_pool_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)small_smem))) return e;
     if ((e = cudaFuncSetAttribute(k_pool_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)big_smem))) return e;
+    if ((e = cudaFuncSetAttribute(k_pool_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
     if ((e = cudaFuncSetAttribute(k_plain, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
     return cudaSuccess;
 }

@@ -27,6 +27,7 @@ void launch_order(const ProblemDev* probs, const EdgeWork* edges, long long edge
                   double mean_n, int forced_group, long long split_stride, int allow_split, int marg, int need_marg,
                   int grid, cudaStream_t st);
 void launch_pool(const PoolArgs& a, int cls, int grid, size_t smem_bytes, cudaStream_t st);
+void launch_pool_mid(const PoolArgs& a, int grid, size_t smem_bytes, cudaStream_t st);
 void launch_pool_marg(const PoolArgs& a, int grid, cudaStream_t st);
 void launch_pairs_popc(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first, int total_vertices,
                        int max_n, const uint8_t* owned, const PoolArgs& a, int grid, cudaStream_t st);
@@ -51,7 +52,7 @@ void set_pdl(bool on);
 // Explicit tests: the kernel's limits and its largest cluster, then one test.
 cudaError_t prepare_ci(size_t smem_bytes, int* max_cluster);
 cudaError_t launch_ci(const CiArgs& q, int cluster, size_t smem_bytes, cudaStream_t st);
-cudaError_t set_kernel_smem(size_t small_smem, size_t big_smem, size_t plain_smem);
+cudaError_t set_kernel_smem(size_t small_smem, size_t big_smem, size_t cta_smem);   // cta: k_plain, k_pool_mid
 // Sets the message fbn_last_error(NULL) returns.
 void fbn_internal_set_error(const char* msg);
 int pool_blocks_per_sm(int cls, size_t smem_bytes);

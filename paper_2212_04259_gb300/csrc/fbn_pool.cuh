@@ -2,7 +2,7 @@
 // IV-B) and of the edge-level form (Section IV-A): per-group state, the set-up
 // of one conditioning set (Section IV-C), counting, the bounded decision,
 // sample-split tests and the pool loop.  Each pool kernel is defined in its
-// own translation unit (fbn_pool_small.cu, fbn_pool_big.cu, fbn_plain.cu;
+// own translation unit (fbn_pool_small.cu, _big.cu, _mid.cu, fbn_plain.cu;
 // depth 1 from one-hot planes in fbn_pool_marg.cu), so that they compile in
 // parallel.
 #pragma once

@@ -12,7 +12,7 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_pool_big(PoolArgs a)
     pdl_enter();
     extern __shared__ __align__(16) int smem[];
     __shared__ PoolShared sh;
-    if (!a.ctr->active) return;
+    if (!a.ctr->active || !a.ctr->wide) return;
     pool_body<kBigThreads>(a, smem, sh);
     tests_done(a.ctr);
 }
