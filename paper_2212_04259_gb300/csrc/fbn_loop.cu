@@ -246,8 +246,8 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_loop(const __grid_constant_
                     if (E == 0) ctr->active = 0;
                 }
                 if (E == 0 || popc) return;
-                for (int cls = 0; cls < 2; ++cls) {
-                    if ((cls ? E1 : E0) == 0) continue;
+                for (int cls = 0; cls < 2; ++cls) {   // class 0, also when empty, notes where the tests begin
+                    if (cls && E1 == 0) continue;
                     scan_class(a.sc[cls], cls, ctr, a.mean_n, a.forced_group, a.split_stride, 1, marg, a.need_marg);
                     __syncthreads();
                 }

@@ -40,5 +40,6 @@ def test_big_tables(F, n, r, md, stat, df, loop):
     hard, _, _ = compare(adj, F.fbn_export_sepsets(h), ref)
     assert not hard, hard[:3]
     st = F.fbn_get_stats(h)
+    assert all(0 < t <= m for t, m in zip(st["test_ms"], st["ms"])), st
     if not ref.near:
         assert st["tests_oracle"] == ref.tests and st["removed"] == ref.removed
