@@ -308,7 +308,7 @@ struct Workspace {
     unsigned long long *d_bads = nullptr, *h_bads = nullptr;   // first bad values of a batch of uploads
     size_t bad_cap = 0;
     unsigned* d_bar = nullptr;                      // barrier of the persistent loop
-    unsigned* h_gave_up = nullptr;                  // pinned: 1 when a wait of the loop ran out
+    unsigned* h_left = nullptr;                     // pinned: how the loop ended early (LoopArgs::left)
     unsigned* d_bits = nullptr;                     // its adjacency bit matrix
     uint8_t* h_adj = nullptr;                       // pinned: the adjacency it leaves
     size_t h_adj_cap = 0;
@@ -348,7 +348,7 @@ struct Workspace {
         if (h_bads) cudaFreeHost(h_bads);
         dfree(d_bads);
         dfree(d_bar); dfree(d_bits);
-        if (h_gave_up) cudaFreeHost(h_gave_up);
+        if (h_left) cudaFreeHost(h_left);
         h_maps.clear();
         gram_E = nullptr; gram_G = nullptr; gram_R = nullptr; gram_maps = nullptr; gram_units = nullptr; pk = nullptr;
         split_tab = nullptr; split_ticket = nullptr;
@@ -1311,7 +1311,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     // device-driven while loop whose body tests a depth, removes its edges,
     // ends it and lists the next depth's edges (k_gate: go on or stop).
     // Captured once per configuration: every argument it holds is in the key.
-    if (!shard && !persistent) {
+    auto ensure_graph = [&]() -> int {
         std::vector<uint8_t> key;
         auto put = [&](const void* p, size_t n) {
             const uint8_t* b = (const uint8_t*)p;
@@ -1344,11 +1344,13 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
             if (!ws.loop) return fail(h, FBN_ECUDA, "depth loop graph: %s", cudaGetErrorString(err));
             ws.graph_key = key;
         }
-    }
+        return FBN_OK;
+    };
+    if (!shard && !persistent && (rc = ensure_graph())) return rc;
 
     fbn_stats stats{};
     int d_loop = 0;   // first depth of the graph loop
-    const bool direct_out = persistent && k == 1;
+    bool direct_out = persistent && k == 1;
     const long long* h_tot = nullptr;
     if (persistent) {
         LoopArgs la{};
@@ -1395,19 +1397,16 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         la.big = la.small;
         la.big.cls = kClassCta;
         la.big.base = ws.base + ws.ord_cap;
-        if (ws.gs_cells > 0) {
-            la.big.gscratch = ws.gscratch;
-            la.big.gscratch_ints = 3 * ws.gs_cells + 64;
-        }
+        la.small.hand_over = la.big.hand_over = 1;
         // 2^23 polls are seconds
         la.spin_limit = h->opt.wait_limit < 0 ? 0u : h->opt.wait_limit > 0 ? (unsigned)h->opt.wait_limit : 1u << 23;
         if (!ws.d_bar) {
             CK(dalloc(&ws.d_bar, 2));
             CK(cudaMemsetAsync(ws.d_bar, 0, 2 * sizeof(unsigned), st));
         }
-        if (!ws.h_gave_up) CK(cudaMallocHost((void**)&ws.h_gave_up, sizeof(unsigned)));
-        CK(cudaHostGetDevicePointer((void**)&la.gave_up, ws.h_gave_up, 0));
-        *ws.h_gave_up = 0;
+        if (!ws.h_left) CK(cudaMallocHost((void**)&ws.h_left, sizeof(unsigned)));
+        CK(cudaHostGetDevicePointer((void**)&la.left, ws.h_left, 0));
+        *ws.h_left = 0;
         la.bar = ws.d_bar;
         if (k == 1 && h->n <= kTurnVertices) {
             if (!ws.d_bits) CK(dalloc(&ws.d_bits, kTurnVertices * (kTurnVertices / 32)));
@@ -1484,7 +1483,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         direct1 = true;
         d_loop = 2;
     }
-    const bool loop = !persistent && (max_depth < 0 || d_loop <= max_depth);
+    bool loop = !persistent && (max_depth < 0 || d_loop <= max_depth);
     const bool host_loop = h->opt.loop == FBN_LOOP_HOST || shard;
     if (shard) {
         // Several processes learn this skeleton together (Section IV-A's
@@ -1579,68 +1578,88 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         launches += 3;
     }
     CK(cudaGetLastError());
+    // The counters and the graphs to the host, with the call's synchronisation.
     bool adj_staged = false;   // the adjacency comes from the pinned staging after the synchronisation
-    if (direct_out) {
-        if (adj_out && adj_out[0]) {
-            cudaPointerAttributes attr{};
-            const cudaError_t pe = cudaPointerGetAttributes(&attr, adj_out[0]);
-            cudaGetLastError();
-            adj_staged = pe != cudaSuccess || attr.type == cudaMemoryTypeUnregistered || attr.type == cudaMemoryTypeHost;
-        }
-    } else {
-        CK(cudaMemcpyAsync(ws.h_ctr, ws.d_ctr, sizeof(DepthCounters), cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(ws.h_rec, ws.d_rec, kMaxDepthRecords * sizeof(DepthRecord), cudaMemcpyDeviceToHost, st));
-    }
-    // The graphs go out with the counters (dropped if the call is retried): a
-    // batch's for pageable memory through one pinned buffer of at most
-    // kAdjStageBytes, the others and what is over that by a copy each.  (One
-    // graph of 1,000 variables takes as long either way.)
     std::vector<int> staged;
     std::vector<size_t> staged_at;
-    if (adj_out && !adj_staged) {
-        size_t total = 0;
-        for (int p = 0; p < k; ++p) {
-            if (!adj_out[p]) continue;
-            const size_t nn = (size_t)hs[p]->n * hs[p]->n, padded = (nn + 15) / 16 * 16;
-            cudaPointerAttributes attr{};
-            const cudaError_t pe = cudaPointerGetAttributes(&attr, adj_out[p]);
-            cudaGetLastError();
-            if (k > 1 && (pe != cudaSuccess || attr.type == cudaMemoryTypeUnregistered) && total + padded <= kAdjStageBytes) {
-                staged.push_back(p);
-                staged_at.push_back(total);
-                total += padded;
-            } else {
-                CK(cudaMemcpyAsync(adj_out[p], hs[p]->d_adj, nn, cudaMemcpyDefault, st));
+    auto fetch = [&]() -> int {
+        adj_staged = false;
+        if (direct_out) {
+            if (adj_out && adj_out[0]) {
+                cudaPointerAttributes attr{};
+                const cudaError_t pe = cudaPointerGetAttributes(&attr, adj_out[0]);
+                cudaGetLastError();
+                adj_staged = pe != cudaSuccess || attr.type == cudaMemoryTypeUnregistered || attr.type == cudaMemoryTypeHost;
             }
+        } else {
+            CK(cudaMemcpyAsync(ws.h_ctr, ws.d_ctr, sizeof(DepthCounters), cudaMemcpyDeviceToHost, st));
+            CK(cudaMemcpyAsync(ws.h_rec, ws.d_rec, kMaxDepthRecords * sizeof(DepthRecord), cudaMemcpyDeviceToHost, st));
         }
-        if (total) {
-            CK(grow_pinned(&ws.h_adj, &ws.h_adj_cap, total));
-            uint4* dst = nullptr;
-            CK(cudaHostGetDevicePointer((void**)&dst, ws.h_adj, 0));
-            for (size_t s0 = 0; s0 < staged.size(); s0 += kAdjJob) {
-                const int m = (int)std::min<size_t>(kAdjJob, staged.size() - s0);
-                AdjJob job{};
-                long long most = 1;
-                for (int q = 0; q < m; ++q) {
-                    const fbn_handle* g = hs[staged[s0 + q]];
-                    job.src[q] = g->d_adj;
-                    job.words[q] = ((long long)g->n * g->n + 15) / 16;
-                    job.off[q] = (long long)(staged_at[s0 + q] / 16);
-                    most = std::max(most, job.words[q]);
+        // The graphs go out with the counters (dropped if the call is retried): a
+        // batch's for pageable memory through one pinned buffer of at most
+        // kAdjStageBytes, the others and what is over that by a copy each.  (One
+        // graph of 1,000 variables takes as long either way.)
+        staged.clear();
+        staged_at.clear();
+        if (adj_out && !adj_staged) {
+            size_t total = 0;
+            for (int p = 0; p < k; ++p) {
+                if (!adj_out[p]) continue;
+                const size_t nn = (size_t)hs[p]->n * hs[p]->n, padded = (nn + 15) / 16 * 16;
+                cudaPointerAttributes attr{};
+                const cudaError_t pe = cudaPointerGetAttributes(&attr, adj_out[p]);
+                cudaGetLastError();
+                if (k > 1 && (pe != cudaSuccess || attr.type == cudaMemoryTypeUnregistered) && total + padded <= kAdjStageBytes) {
+                    staged.push_back(p);
+                    staged_at.push_back(total);
+                    total += padded;
+                } else {
+                    CK(cudaMemcpyAsync(adj_out[p], hs[p]->d_adj, nn, cudaMemcpyDefault, st));
                 }
-                k_adj_out<<<dim3((unsigned)std::min<long long>((most + 1023) / 1024, 1024), m), 256, 0, st>>>(job, dst);
-                CK(cudaGetLastError());
-                launches += 1;
+            }
+            if (total) {
+                CK(grow_pinned(&ws.h_adj, &ws.h_adj_cap, total));
+                uint4* dst = nullptr;
+                CK(cudaHostGetDevicePointer((void**)&dst, ws.h_adj, 0));
+                for (size_t s0 = 0; s0 < staged.size(); s0 += kAdjJob) {
+                    const int m = (int)std::min<size_t>(kAdjJob, staged.size() - s0);
+                    AdjJob job{};
+                    long long most = 1;
+                    for (int q = 0; q < m; ++q) {
+                        const fbn_handle* g = hs[staged[s0 + q]];
+                        job.src[q] = g->d_adj;
+                        job.words[q] = ((long long)g->n * g->n + 15) / 16;
+                        job.off[q] = (long long)(staged_at[s0 + q] / 16);
+                        most = std::max(most, job.words[q]);
+                    }
+                    k_adj_out<<<dim3((unsigned)std::min<long long>((most + 1023) / 1024, 1024), m), 256, 0, st>>>(job, dst);
+                    CK(cudaGetLastError());
+                    launches += 1;
+                }
             }
         }
-    }
-    CK(cudaStreamSynchronize(st));
-    if (persistent && *ws.h_gave_up) {   // the barrier's words and the counters are not whole
+        CK(cudaStreamSynchronize(st));
+        return FBN_OK;
+    };
+    if ((rc = fetch())) return rc;
+    if (persistent && *ws.h_left == kLoopGaveUp) {   // the barrier's words and the counters are not whole
         CK(cudaMemsetAsync(ws.d_bar, 0, 2 * sizeof(unsigned), st));
         CK(cudaStreamSynchronize(st));
         *allow_loop = false;
         *retry = true;
         return FBN_OK;
+    }
+    if (persistent && *ws.h_left >= kLoopHandedOver) {   // the depths from there on as a graph
+        d_loop = (int)(*ws.h_left - kLoopHandedOver);
+        direct_out = false;
+        loop = true;
+        if ((rc = ensure_graph())) return rc;
+        // parts of split tests may not have run
+        CK(cudaMemsetAsync(ws.split_tab, 0, kSplitItems * kSplitStride * sizeof(int), st));
+        CK(cudaMemsetAsync(ws.split_ticket, 0, kSplitItems * sizeof(unsigned), st));
+        CK(cudaGraphLaunch(ws.loop, st));
+        launches += 3;
+        if ((rc = fetch())) return rc;
     }
     if (adj_staged) std::memcpy(adj_out[0], ws.h_adj, (size_t)h->n * h->n);
     for (size_t s = 0; s < staged.size(); ++s)
@@ -1661,7 +1680,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         if (c.status & kStatusScratch) {
             if (c.need_cells <= 0 || c.need_cells > kMaxCells) return check_status(h, kStatusTooBig);
             ws.gs_cells = std::max<long long>(2 * ws.gs_cells, c.need_cells);
-            rc = ensure_gscratch(h, ws, (3 * ws.gs_cells + 64) * std::max({grid_big, grid_plain, ws.grid_loop}));
+            rc = ensure_gscratch(h, ws, (3 * ws.gs_cells + 64) * std::max(grid_big, grid_plain));
             if (rc) return rc;
         }
         *retry = true;

@@ -133,6 +133,7 @@ struct DepthCounters {
     int whole;                          // depth 1 from one-hot planes: an item is a whole edge (set by k_edges)
     unsigned int beat;                  // persistent loop: ranks begun after an item's first (its barriers wait on while
                                         // this or next_item moves)
+    int hand_over;                      // persistent loop: a table of this depth does not fit its shared memory
     int direct;                         // 1: item w is chunk w / E of the class's edge w mod E (empty past its last)
     DepthRecord* rec;                   // per-depth records (persists)
     const int* tune;                    // per-depth choices of the autotuner, or nullptr (persists):
@@ -213,7 +214,7 @@ struct PoolArgs {
     long long gscratch_ints;
     CritTableDev crit;
     int32_t cls;
-    int32_t pad;
+    int32_t hand_over;                // 1: the persistent loop (a table over its shared memory ends the loop)
     int32_t smem_ints;
     int32_t binom_rows;
     double alpha;

@@ -12,8 +12,12 @@
 // host memory.
 // The phases are those of the per-depth kernels (fbn_graph.cuh, fbn_pool.cuh,
 // fbn_pool_marg.cuh), so the results are too.  Larger problems keep the
-// kernels: their phases fill the chip, the big-table pool gets more shared
-// memory, and the fixed cost per depth no longer shows.
+// kernels: their phases fill the chip, and the fixed cost per depth no longer
+// shows.  So does a depth with a table over the loop's shared memory: the loop
+// ends before that depth's removal and the graph goes on there, whose big-table
+// pools have 100 to 200 KB (20 variables of 12 values x 50,000 samples to depth 2,
+// 20,736 cells: 48 ms with these tables in global memory, 9.0 handed over; 14
+// variables of 7 values to depth 3, 16,807 cells: 33 and 5.5 ms).
 #include "fbn_graph.cuh"
 #include "fbn_loop.h"
 #include "fbn_pool_marg.cuh"
@@ -99,8 +103,27 @@ __device__ __forceinline__ bool loop_barrier(const LoopArgs& a, unsigned& gen, L
     }
     __syncthreads();
     ++gen;
-    if (s_role < 0 && threadIdx.x == 0) *((volatile unsigned*)a.gave_up) = 1u;
+    if (s_role < 0 && threadIdx.x == 0) *((volatile unsigned*)a.left) = kLoopGaveUp;
     return s_role >= 0;
+}
+
+// A table of depth ctr->d did not fit (the last CTA, all tests of the depth done):
+// nothing is removed, and the depth's state is as before its edge list, for the
+// kernels of a depth to start there.  Its tests stay counted.
+__device__ __noinline__ void hand_over(const LoopArgs& a, DepthCounters* ctr)
+{
+    const long long used[2] = {(long long)ctr->maxc[0] + 1, (long long)ctr->maxc[1] + 1};
+    __syncthreads();
+    for (int c = 0; c < 2; ++c)
+        for (long long k = threadIdx.x; k < used[c]; k += kTestThreads) a.hist[c * a.ord_cap + k] = a.cursor[c * a.ord_cap + k] = 0;
+    if (threadIdx.x == 0) {
+        for (int c = 0; c < 2; ++c)
+            ctr->n_edges[c] = ctr->maxc[c] = ctr->next_item[c] = ctr->total_items[c] = ctr->max_cells[c] = ctr->max_total[c] = 0;
+        ctr->split[0] = ctr->split[1] = 1;
+        ctr->adj_ends = 0;
+        ctr->gsel = ctr->whole = ctr->direct = 0;
+        *((volatile unsigned*)a.left) = kLoopHandedOver + (unsigned)ctr->d;
+    }
 }
 
 // The results to pinned host memory (one problem), after the last depth.
@@ -220,6 +243,7 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_loop(const __grid_constant_
     for (int d = 0;; ++d) {
         const bool popc = d == 0 && a.popc0, marg = d == 1 && a.marg1;
         const bool direct = ctr->direct != 0;   // listed by the last CTA of the depth before
+        long long big = (long long)ctr->n_edges[kClassCta];   // listed directly, else read below
         if (!direct) {
             // the last CTA ends the depth before, the others list the neighbours
             // (the degree sum, which they add up, was cleared by the phase before)
@@ -254,8 +278,10 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_loop(const __grid_constant_
                 if (E <= kPlaceSerial) place(threadIdx.x, kTestThreads);
             };
             if (!loop_barrier(a, gen, order)) return;
+            const long long all = (long long)(ctr->n_edges[0] + ctr->n_edges[1]);
+            big = (long long)ctr->n_edges[kClassCta];
             if (!ctr->active) break;   // the same for every CTA
-            if (!popc && (long long)(ctr->n_edges[0] + ctr->n_edges[1]) > kPlaceSerial) {
+            if (!popc && all > kPlaceSerial) {
                 place(t0, threads);
                 if (!loop_barrier(a, gen, none)) return;
             }
@@ -265,21 +291,36 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_loop(const __grid_constant_
         } else if (marg) {
             marg_body<true>(a.small);
         } else {
-            switch (ctr->gsel) {
-                case 32: pool_body<32, true>(a.small, smem, sh); break;
-                case 64: pool_body<64, true>(a.small, smem, sh); break;
-                case 128: pool_body<128, true>(a.small, smem, sh); break;
-                default: pool_body<kTestThreads, true>(a.small, smem, sh); break;
+            bool small = true;
+            if (big > 0) {   // first: a table over the shared memory ends the loop
+                __shared__ int s_over;
+                pool_body<kTestThreads, true>(a.big, smem, sh);
+                __syncthreads();
+                if (threadIdx.x == 0) s_over = *((volatile int*)&ctr->hand_over);
+                __syncthreads();
+                small = !s_over;
             }
-            __syncthreads();
-            pool_body<kTestThreads, true>(a.big, smem, sh);
+            if (small) {
+                switch (ctr->gsel) {
+                    case 32: pool_body<32, true>(a.small, smem, sh); break;
+                    case 64: pool_body<64, true>(a.small, smem, sh); break;
+                    case 128: pool_body<128, true>(a.small, smem, sh); break;
+                    default: pool_body<kTestThreads, true>(a.small, smem, sh); break;
+                }
+            }
         }
         tests_done(ctr);
-        const auto next = [&] { if (a.bits) turn(a, turn_sh, direct, warps); };
+        const auto over = [&] { if (big > 0 && ctr->hand_over) hand_over(a, ctr); };
+        const auto next = [&] {
+            if (big > 0 && ctr->hand_over) hand_over(a, ctr);
+            else if (a.bits) turn(a, turn_sh, direct, warps);
+        };
         if (direct) {   // removal, end of depth and the next depth's items
             if (!loop_barrier(a, gen, next)) return;
+            if (big > 0 && ctr->hand_over) return;   // set before the barrier: the same for every CTA
         } else {
-            if (!loop_barrier(a, gen, none)) return;
+            if (!loop_barrier(a, gen, over)) return;
+            if (big > 0 && ctr->hand_over) return;
             apply_edges(a.probs, a.edges, a.min_accept, a.edge_cap, a.binom, a.sep_pool, a.sep_cap, ctr, t0, threads,
                         a.bits);
             if (!loop_barrier(a, gen, next)) return;

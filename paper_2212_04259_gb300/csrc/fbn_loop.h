@@ -11,6 +11,8 @@ namespace fbn {
 
 constexpr int kTurnVertices = 128;   // variables of a problem whose depths one CTA prepares (fbn_turn.cuh)
 constexpr int kTurnItems = 32768;    // items of a class it lays out
+constexpr unsigned kLoopGaveUp = 1;      // a phase's wait ran out: the call starts over without the loop
+constexpr unsigned kLoopHandedOver = 2;  // + d: depth d holds a table that does not fit: the kernels of a depth go on there
 
 // Everything the loop's phases take, by value.
 struct LoopArgs {
@@ -41,7 +43,7 @@ struct LoopArgs {
     int popc0, marg1;                    // depths 0 and 1 from one-hot planes
     PoolArgs small, big;                 // the two classes
     unsigned spin_limit;                 // polls of a phase barrier without progress before the loop gives up
-    unsigned* gave_up;                   // pinned host memory: 1 when it did
+    unsigned* left;                      // pinned host memory: how the loop ended early (below), 0 if it did not
     unsigned* bits;                      // one problem of <= kTurnVertices variables: its adjacency as a bit
                                          // matrix [kTurnVertices][kTurnVertices / 32] (nullptr: general phases only)
     unsigned* bar;                       // [2] arrivals of the current phase (and kGaveUp), phases opened so far

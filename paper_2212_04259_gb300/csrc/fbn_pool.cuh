@@ -160,10 +160,15 @@ __device__ __forceinline__ int run_rank(const PoolArgs& a, int d, const ProblemD
     if (!setup_rank<G>(P, w, d, rk, fresh, S, a.binom, spec, status)) return -1;
     int* M = nullptr;
     const int* T = grp_table<G>(spec, slice, slice_ints, gtab, a.gscratch_ints, a.lut == nullptr, &M);
-    if (!T) {   // the global scratch is too small: the host grows it and starts over
+    if (!T) {
         if (Grp<G>::rank() == 0) {
-            atomicOr(status, kStatusScratch);
-            atomicMax(&a.ctr->need_cells, (int)spec.cells);
+            if (a.hand_over) {   // the kernels of a depth take it from here: no further claims
+                *((volatile int*)&a.ctr->hand_over) = 1;
+                for (int c = 0; c < 2; ++c) atomicAdd(&a.ctr->next_item[c], 1ULL << 40);
+            } else {   // the global scratch is too small: the host grows it and starts over
+                atomicOr(status, kStatusScratch);
+                atomicMax(&a.ctr->need_cells, (int)spec.cells);
+            }
         }
         return -1;
     }

@@ -2,7 +2,8 @@
 
 Covered: both kernels of the class (many tests and few, tables that fit the
 256-thread kernel's shared memory, ones that only fit the 1,024-thread one's, and
-ones that go to global memory), with and without marginals beside the table.
+ones that go to global memory), with and without marginals beside the table, and the
+persistent loop handing a depth over to them.
 """
 import numpy as np
 import pytest
@@ -43,3 +44,28 @@ def test_big_tables(F, n, r, md, stat, df, loop):
     assert all(0 < t <= m for t, m in zip(st["test_ms"], st["ms"])), st
     if not ref.near:
         assert st["tests_oracle"] == ref.tests and st["removed"] == ref.removed
+
+
+# The loop's shared memory holds 16,384 ints: 15,625 cells run in it, 17,576 end it at depth 1, 27,000 at
+# depth 1 of the second problem of a batch, 16,807 at depth 3 (after depths laid out directly).
+@pytest.mark.parametrize("n,r,md,over", [(9, 25, 1, False), (9, 26, 1, True), (8, 7, 3, True), (130, 26, 1, True)])
+def test_loop_hands_over(F, n, r, md, over):
+    import torch
+    data, ar = _linked(r, n, r, 20000 if r == 7 else 2000, 0.6 if n < 100 else 0.3)
+    ref = oracle.pc_stable(data, ar, 0.05, md)
+    h = F.fbn_create(data, ar)
+    for out in (None, np.zeros((n, n), np.uint8), torch.zeros((n, n), dtype=torch.uint8, device="cuda")) * 2:
+        adj = F.fbn_learn_skeleton(h, 0.05, md, out)
+        adj = adj.cpu().numpy() if isinstance(adj, torch.Tensor) else adj
+        hard, _, _ = compare(adj, F.fbn_export_sepsets(h), ref)
+        assert not hard, hard[:3]
+        st = F.fbn_get_stats(h)
+        assert (st["launches"] > 1) == over and st["depths"] == len(ref.tests)
+        assert ref.near or (st["tests_oracle"] == ref.tests and st["removed"] == ref.removed)
+    other, oar = _linked(3, 20, 3, 1500)
+    hs = [F.fbn_create(other, oar), h]
+    for _ in range(3):
+        adjs = F.fbn_learn_skeleton_batch(hs, 0.05, md)
+    for q, adj, w in zip(hs, adjs, (oracle.pc_stable(other, oar, 0.05, md), ref)):
+        hard, _, _ = compare(adj, F.fbn_export_sepsets(q), w)
+        assert not hard, hard[:3]
