@@ -264,10 +264,11 @@ struct Grp {
 };
 
 // Sum over the group; every thread of the group gets the total.  red: the
-// CTA's scratch of 32 entries, of which the group uses kWarps.
+// CTA's scratch of 32 entries of 8 bytes, of which the group uses kWarps.
 template <int G, typename T>
 __device__ __forceinline__ T grp_sum(T v, T* red)
 {
+    static_assert(sizeof(T) == 8, "a smaller type's slots would overlap another group's");
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (G == 32) return v;
@@ -462,6 +463,8 @@ static __device__ __noinline__ void count_shared(const TestSpec& s, SharedCounte
         }
     } else {
         switch (s.nrows) {
+            case 2: count_packed<2>(s, cnt, rank, G); break;
+            case 3: count_packed<3>(s, cnt, rank, G); break;
             case 4: count_packed<4>(s, cnt, rank, G); break;
             case 5: count_packed<5>(s, cnt, rank, G); break;
             default: count_packed<0>(s, cnt, rank, G); break;
@@ -552,6 +555,21 @@ __device__ __forceinline__ int* grp_table(const TestSpec& s, int* slice, long lo
     return slice;
 }
 
+// c / d for c, d < 2^16 as one multiplication (the general division is some 25
+// instructions, of which a cell of a decision took two).
+struct Divider {
+    unsigned m, d;
+    bool small;   // every dividend is below 2^16
+    __device__ __forceinline__ Divider(int divisor, int dividends)
+        : m(divisor == 1 ? 0u : 0xFFFFFFFFu / (unsigned)divisor + 1u), d((unsigned)divisor), small(dividends <= 65536)
+    {
+    }
+    __device__ __forceinline__ int operator()(int c) const   // m = ceil(2^32 / d): exact while c d < 2^32
+    {
+        return m == 0 ? c : small ? (int)__umulhi((unsigned)c, m) : c / (int)d;
+    }
+};
+
 // Marginals N_x+z [nz*rx], N_+yz [nz*ry], N_++z [nz] into M.
 template <int G>
 __device__ __forceinline__ void grp_marginals(const TestSpec& s, const int* T, int* M)
@@ -568,8 +586,9 @@ __device__ __forceinline__ void grp_marginals(const TestSpec& s, const int* T, i
         for (int y = 0; y < ry; ++y) sum += T[k * ry + y];
         Nxz[k] = sum;
     }
+    const Divider by_ry(ry, nz * ry);
     for (int k = r; k < nz * ry; k += G) {
-        const int z = k / ry;
+        const int z = by_ry(k);
         const int y = k - z * ry;
         int sum = 0;
         for (int x = 0; x < rx; ++x) sum += T[(z * rx + x) * ry + y];
@@ -652,14 +671,14 @@ __device__ __forceinline__ long long grp_df_adjusted(const TestSpec& s, const in
     const int nz = (int)s.cells / (rx * ry);
     const int* Nxz = M;
     const int* Nyz = M + nz * rx;
-    double acc = 0.0;
+    long long acc = 0;   // whole numbers: additions in FP64 take a test of 32 cells a ninth longer
     for (int z = Grp<G>::rank(); z < nz; z += G) {
         int ax = 0, ay = 0;
         for (int x = 0; x < rx; ++x) ax += Nxz[z * rx + x] > 0;
         for (int y = 0; y < ry; ++y) ay += Nyz[z * ry + y] > 0;
-        if (ax > 0 && ay > 0) acc += (double)(ax - 1) * (double)(ay - 1);
+        if (ax > 0 && ay > 0) acc += (ax - 1) * (ay - 1);
     }
-    return (long long)(grp_sum<G>(acc, red) + 0.5);
+    return grp_sum<G>(acc, reinterpret_cast<long long*>(red));
 }
 
 // One FP32 term of the bounded decisions.  G^2: n ln(N / E) with the ratio
@@ -667,22 +686,39 @@ __device__ __forceinline__ long long grp_df_adjusted(const TestSpec& s, const in
 // as log1p of the exact difference over the denominator (n > 0).  X^2:
 // (n N_++z - N_x+z N_+yz)^2 / (N_++z N_x+z N_+yz) with the difference exact,
 // skipped when a margin is empty.
-__device__ __forceinline__ void g2_term(int n, int nzz, int nx, int ny, float& acc, float& mag)
+// Below 65,536 samples (narrow) the products fit 32 bits: the same values, without
+// 64-bit conversions, which run at the FP64 rate.
+__device__ __forceinline__ void product_floats(int n, int nzz, int nx, int ny, bool narrow, float& fa, float& fb, float& fd)
 {
-    const long long a = (long long)n * nzz;
-    const long long b = (long long)nx * ny;
-    const float fb = (float)b;
-    const float delta = (float)(a - b) / fb;
-    const float L = fabsf(delta) < 0.5f ? log1pf(delta) : logf((float)a / fb);
+    if (narrow) {
+        const unsigned a = (unsigned)n * (unsigned)nzz, b = (unsigned)nx * (unsigned)ny;
+        fa = (float)a;
+        fb = (float)b;
+        fd = a >= b ? (float)(a - b) : -(float)(b - a);
+    } else {
+        const long long a = (long long)n * nzz, b = (long long)nx * ny;
+        fa = (float)a;
+        fb = (float)b;
+        fd = (float)(a - b);
+    }
+}
+
+__device__ __forceinline__ void g2_term(int n, int nzz, int nx, int ny, bool narrow, float& acc, float& mag)
+{
+    float fa, fb, fd;
+    product_floats(n, nzz, nx, ny, narrow, fa, fb, fd);
+    const float delta = fd / fb;
+    const float L = fabsf(delta) < 0.5f ? log1pf(delta) : logf(fa / fb);
     const float t = (float)n * L;
     acc += t;
     mag += fabsf(t);
 }
 
-__device__ __forceinline__ void x2_term(int n, int nzz, int nx, int ny, float& acc)
+__device__ __forceinline__ void x2_term(int n, int nzz, int nx, int ny, bool narrow, float& acc)
 {
     if (nx == 0 || ny == 0) return;
-    const float fd = (float)((long long)n * nzz - (long long)nx * ny);
+    float fa, fb, fd;
+    product_floats(n, nzz, nx, ny, narrow, fa, fb, fd);
     acc += fd * fd / ((float)nzz * (float)nx * (float)ny);
 }
 
@@ -785,23 +821,25 @@ __device__ __forceinline__ int grp_decide_bound(const TestSpec& s, const int* T,
     const int* Nxz = M;
     const int* Nyz = M + nz * rx;
     const int* Nzz = Nyz + nz * ry;
+    const Divider by_rxy(rxy, C), by_ry(ry, rxy);
+    const bool narrow = s.N < 65536;
     float acc = 0.0f, mag = 0.0f;
     if (stat == kStatX2) {
         for (int c = Grp<G>::rank(); c < C; c += G) {
-            const int z = c / rxy;
+            const int z = by_rxy(c);
             const int rem = c - z * rxy;
-            const int x = rem / ry, y = rem - x * ry;
-            x2_term(T[c], Nzz[z], Nxz[z * rx + x], Nyz[z * ry + y], acc);
+            const int x = by_ry(rem), y = rem - x * ry;
+            x2_term(T[c], Nzz[z], Nxz[z * rx + x], Nyz[z * ry + y], narrow, acc);
         }
         mag = acc;
     } else {
         for (int c = Grp<G>::rank(); c < C; c += G) {
             const int n = T[c];
             if (n == 0) continue;
-            const int z = c / rxy;
+            const int z = by_rxy(c);
             const int rem = c - z * rxy;
-            const int x = rem / ry, y = rem - x * ry;
-            g2_term(n, Nzz[z], Nxz[z * rx + x], Nyz[z * ry + y], acc, mag);
+            const int x = by_ry(rem), y = rem - x * ry;
+            g2_term(n, Nzz[z], Nxz[z * rx + x], Nyz[z * ry + y], narrow, acc, mag);
         }
     }
     float2 v = make_float2(acc, mag);

@@ -82,8 +82,10 @@ __device__ __forceinline__ bool setup_rank(const ProblemDev& P, const EdgeWork& 
 // The decision of a counted test from its table and marginals: df from the
 // declared arities or from the observed table (no degree of freedom left:
 // the test cannot reject), crit from the cache, then the bounded statistic.
+// In line: as a call it kept a fifth of the small tests' time (depth 2 of 40
+// variables of 5 values x 1,000 samples, X^2: 7.2 -> 5.8 ms).
 template <int G>
-__device__ __noinline__ int decide_test(const PoolArgs& a, const TestSpec& spec, const int* T, int* M,
+__device__ __forceinline__ int decide_test(const PoolArgs& a, const TestSpec& spec, const int* T, int* M,
                                         GroupState& S, double* red, unsigned* status)
 {
     grp_marginals<G>(spec, T, M);
@@ -232,6 +234,7 @@ __device__ __noinline__ int run_split_part(const PoolArgs& a, int d, const Probl
         Tg[c] = 0;
     }
     if (r == 0) {
+        spec.N = P.N;   // the table holds every part's samples
         a.split_ticket[S.item] = 0;
         S.go = (unsigned long long)rk <= *((volatile const unsigned long long*)min_accept_e);
     }

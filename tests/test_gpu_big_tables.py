@@ -3,7 +3,8 @@
 Covered: both kernels of the class (many tests and few, tables that fit the
 256-thread kernel's shared memory, ones that only fit the 1,024-thread one's, and
 ones that go to global memory), with and without marginals beside the table, and the
-persistent loop handing a depth over to them.
+persistent loop handing a depth over to them.  Few tests of many samples: split by
+samples, the decision over all of them.
 """
 import numpy as np
 import pytest
@@ -69,3 +70,25 @@ def test_loop_hands_over(F, n, r, md, over):
     for q, adj, w in zip(hs, adjs, (oracle.pc_stable(other, oar, 0.05, md), ref)):
         hard, _, _ = compare(adj, F.fbn_export_sepsets(q), w)
         assert not hard, hard[:3]
+
+
+# 70,001 samples in parts of fewer than 65,536: the counts' products pass 32 bits.
+@pytest.mark.parametrize("stat,df", [("g2", "fixed"), ("x2", "fixed"), ("g2", "adjusted"), ("x2", "adjusted")])
+@pytest.mark.parametrize("loop", ["host", "device"])
+def test_split_by_samples(F, stat, df, loop):
+    for n, ars, N, keep in ((4, [2, 6, 3, 7], 70001, 0.1), (5, [6, 2, 3, 9, 4], 200003, 0.02)):
+        rng = np.random.default_rng(N)
+        base = rng.integers(0, 36, N)
+        data = np.stack([np.where(rng.random(N) < keep, base % r, (rng.random(N) < 0.97) * rng.integers(0, r, N)) for r in ars]).astype(np.uint8)
+        ar = np.array(ars, np.uint8)
+        ref = oracle.pc_stable(data, ar, 0.05, -1, stat=stat, df_mode=df)
+        h = F.fbn_create(data, ar, statistic=stat, df=df, loop=loop)
+        adj = F.fbn_learn_skeleton(h, 0.05, -1)
+        hard, _, _ = compare(adj, F.fbn_export_sepsets(h), ref)
+        assert not hard, hard[:3]
+        st = F.fbn_get_stats(h)
+        assert ref.near or (st["tests_oracle"] == ref.tests and st["removed"] == ref.removed)
+        data[:, 1:] = 0   # one value nearly everywhere: products near N^2
+        ref = oracle.pc_stable(data, ar, 0.05, -1, stat=stat, df_mode=df)
+        F.fbn_update_data(h, data)
+        assert np.array_equal(np.asarray(F.fbn_learn_skeleton(h, 0.05, -1)), ref.adj) or ref.near
