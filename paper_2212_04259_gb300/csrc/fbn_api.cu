@@ -1448,9 +1448,10 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         pa.ctr = ws.d_ctr;
         pa.stat = h->opt.statistic;
         pa.df_mode = h->opt.df_mode;
+        for (int p = 0; p < k; ++p) pa.max_arity = std::max(pa.max_arity, hs[p]->max_arity);
         CK(launch_pairs_gram(ws.probs, ws.vtx_prob, ws.vtx_first, total_vtx, max_n, pa, dev_sms, st));
         launch_depth_end(ws.d_ctr, ws.d_rec, max_depth, ws.hist, ws.cursor, st);
-        launches += 4;
+        launches += pa.max_arity > kWideArity ? 5 : 4;
         d_loop = 1;
     } else if (popc0) {
         enqueue_head();
@@ -2381,6 +2382,7 @@ int fbn_pairwise_counts(fbn_handle* h, int32_t* counts, int64_t cap)
     pa.emit = pa.sym = 1;
     pa.out = device_out ? counts : ws.gram_G;
     pa.ldo = h->M;
+    pa.max_arity = h->max_arity;
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     CK(launch_pairs_gram(ws.probs, ws.vtx_prob, ws.vtx_first, h->n, h->n, pa, sms, h->stream));

@@ -33,7 +33,10 @@ struct PairsGramArgs {
     double alpha = 0.0;
     DepthCounters* ctr = nullptr;
     int stat = 0, df_mode = 0;
+    int max_arity = 0;       // of the call
 };
+// Problems with a variable of more values than this go through k_pairs_wide, a launch of its own.
+constexpr int kWideArity = 8;
 cudaError_t launch_pairs_gram(const ProblemDev* probs, const int32_t* vtx_prob, const int32_t* vtx_first,
                               int total_vertices, int max_n, const PairsGramArgs& a, int num_sms, cudaStream_t st);
 

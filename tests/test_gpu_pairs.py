@@ -1,7 +1,8 @@
 """Pair tables and depth-0 decisions from the Gram over the values >= 1.
 
 The cells of value 0 follow from the single counts.  Covered: arities up to
-24, values that never occur, variable counts around the 32 pairs of a warp and
+255 (a lane per pair up to 8, a warp up to 32, a CTA of 256 threads up to 64 and of 1,024
+above, narrow and wide problems in a batch), values that never occur, variable counts around the 32 pairs of a warp and
 the 128 rows of a tile, output into host and device buffers, depth-0 decisions
 with both statistics and both degrees of freedom, and depth 1 reading the
 tables.  Counts and graphs equal to the oracle's.
@@ -35,7 +36,8 @@ def _data(n, N, hi, seed):
 
 
 @pytest.mark.parametrize("n,N,hi", [(3, 1, 2), (31, 130, 5), (33, 8193, 24), (65, 300, 4), (130, 1000, 2),
-                                    (24, 40000, 3), (200, 20011, 4)])   # few tiles of many samples: units of 8 stages and up
+                                    (24, 40000, 3), (200, 20011, 4), (9, 700, 9), (12, 3000, 32), (7, 5000, 33), (6, 900, 65),
+                                    (5, 2001, 255)])   # few tiles of many samples: units of 8 stages and up
 def test_pair_tables(F, n, N, hi):
     import torch
     data, ar = _data(n, N, hi, n + N)
@@ -49,7 +51,8 @@ def test_pair_tables(F, n, N, hi):
 
 
 @pytest.mark.parametrize("stat,df", [("g2", "fixed"), ("g2", "adjusted"), ("x2", "fixed"), ("x2", "adjusted")])
-@pytest.mark.parametrize("n,N,hi", [(33, 2000, 12), (70, 900, 5), (40, 66001, 5)])
+@pytest.mark.parametrize("n,N,hi", [(33, 2000, 12), (70, 900, 5), (40, 66001, 5), (10, 3000, 8), (10, 3000, 9), (14, 70001, 32),
+                                    (9, 30000, 33), (5, 70001, 255)])
 def test_depth0_decisions(F, n, N, hi, stat, df):
     data, ar = _data(n, N, hi, 7 * n + N)
     ref = oracle.pc_stable(data, ar, 0.05, 1 if n < 50 and N < 5000 else 0, stat=stat, df_mode=df)
@@ -59,3 +62,16 @@ def test_depth0_decisions(F, n, N, hi, stat, df):
     assert not hard, hard[:3]
     st = F.fbn_get_stats(h)
     assert st["edges"][0] == n * (n - 1) // 2 == st["tests"][0] and (ref.near or st["removed"] == ref.removed)
+
+
+@pytest.mark.parametrize("stat,df", [("g2", "fixed"), ("x2", "adjusted")])
+def test_batch_of_narrow_and_wide(F, stat, df):
+    probs = [_data(n, N, hi, 3 * n) for n, N, hi in ((12, 2000, 4), (9, 3000, 20), (8, 4000, 60), (10, 1500, 8))]
+    hs = [F.fbn_create(d, a, statistic=stat, df=df, depth0="gram") for d, a in probs]
+    adjs = F.fbn_learn_skeleton_batch(hs, 0.05, 1)
+    refs = [oracle.pc_stable(d, a, 0.05, 1, stat=stat, df_mode=df) for d, a in probs]
+    for h, adj, ref in zip(hs, adjs, refs):
+        hard, _, _ = compare(adj, F.fbn_export_sepsets(h), ref)
+        assert not hard, hard[:3]
+    st = F.fbn_get_stats(hs[0])
+    assert st["edges"][0] == st["tests"][0] == sum(r.tests[0] for r in refs)
