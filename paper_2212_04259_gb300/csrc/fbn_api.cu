@@ -1651,13 +1651,14 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         return FBN_OK;
     }
     if (persistent && *ws.h_left >= kLoopHandedOver) {   // the depths from there on as a graph
-        d_loop = (int)(*ws.h_left - kLoopHandedOver);
+        d_loop = (int)((*ws.h_left & (kLoopSplit - 1)) - kLoopHandedOver);
         direct_out = false;
         loop = true;
         if ((rc = ensure_graph())) return rc;
-        // parts of split tests may not have run
-        CK(cudaMemsetAsync(ws.split_tab, 0, kSplitItems * kSplitStride * sizeof(int), st));
-        CK(cudaMemsetAsync(ws.split_ticket, 0, kSplitItems * sizeof(unsigned), st));
+        if (*ws.h_left & kLoopSplit) {
+            CK(cudaMemsetAsync(ws.split_tab, 0, kSplitItems * kSplitStride * sizeof(int), st));
+            CK(cudaMemsetAsync(ws.split_ticket, 0, kSplitItems * sizeof(unsigned), st));
+        }
         CK(cudaGraphLaunch(ws.loop, st));
         launches += 3;
         if ((rc = fetch())) return rc;

@@ -217,8 +217,9 @@ constexpr float kTestOverhead = 10000.0f;
 constexpr float kCyclesPerSample = 8.0f;
 
 // One thread, with the depth's maxima and ranks per chunk in ctr: the group
-// size of the small-table class and the sample split of class cls for W items.
-__device__ __forceinline__ void choose_pool(const ScanClass& sc, int cls, unsigned long long W, DepthCounters* ctr,
+// size of the small-table class and the sample split of class cls for W items;
+// returns the estimated cycles of the class's tests.
+__device__ __forceinline__ float choose_pool(const ScanClass& sc, int cls, unsigned long long W, DepthCounters* ctr,
                                             double mean_n, int forced_group, long long split_stride, int allow_split,
                                             int need_marg)
 {
@@ -270,6 +271,9 @@ __device__ __forceinline__ void choose_pool(const ScanClass& sc, int cls, unsign
     if (cls == 1) ctr->wide = !need_marg || (long long)W <= g256 || mcell > sc.mid_ints;
     ctr->split[cls] = (int)sp;
     ctr->total_items[cls] = W * (unsigned long long)sp;
+    // the class's tests in cycles, every rank tested (the ranks of the longest chunk, in FP32: see above)
+    const float most = (float)ctr->max_total[cls], ranks = fminf(most, fmaxf((float)ctr->gs, most * (1.0f / (float)kMaxPasses)));
+    return ceilf((float)W / (float)groups) * ranks * (kTestOverhead + kCyclesPerSample * (float)mean_n / (float)G);
 }
 
 __device__ __forceinline__ void scan_class(const ScanClass& sc, int cls, DepthCounters* ctr, double mean_n,
@@ -319,7 +323,7 @@ __device__ __forceinline__ void scan_class(const ScanClass& sc, int cls, DepthCo
         const unsigned long long W = base[maxc];
         ctr->total_items[cls] = W;
         ctr->next_item[cls] = 0;
-        choose_pool(sc, cls, W, ctr, mean_n, forced_group, split_stride, allow_split, need_marg);
+        ctr->cost[cls] = choose_pool(sc, cls, W, ctr, mean_n, forced_group, split_stride, allow_split, need_marg);
     }
 }
 
@@ -446,6 +450,7 @@ __device__ __forceinline__ void depth_end(DepthCounters* ctr, DepthRecord* rec, 
         ctr->nbr_claim = 0;
         ctr->max_total[0] = ctr->max_total[1] = 0;
         ctr->split[0] = ctr->split[1] = 1;
+        ctr->cost[0] = ctr->cost[1] = 0.0f;
         ctr->whole = 0;
         ctr->direct = 0;
         ctr->d = next;

@@ -121,7 +121,7 @@ struct DepthCounters {
     unsigned long long sep_used;        // separating-set pool entries in use (persists)
     unsigned int status;                // error bits (persists)
     int d;                              // current depth (persists)
-    int active;                         // 1 while Algorithm 1 continues (persists)
+    int active;                         // 1 while Algorithm 1 continues (persists); -1: the persistent loop handed over
     int gsel;                           // group size of the small-table class this depth
     int need_cells;                     // largest table that missed the global scratch (persists)
     int gs;                             // ranks per chunk this depth (set by k_edges)
@@ -133,6 +133,7 @@ struct DepthCounters {
     int whole;                          // depth 1 from one-hot planes: an item is a whole edge (set by k_edges)
     unsigned int beat;                  // persistent loop: ranks begun after an item's first (its barriers wait on while
                                         // this or next_item moves)
+    float cost[2];                      // estimated cycles of the depth's tests per class (choose_pool)
     int hand_over;                      // persistent loop: a table of this depth does not fit its shared memory
     int direct;                         // 1: item w is chunk w / E of the class's edge w mod E (empty past its last)
     DepthRecord* rec;                   // per-depth records (persists)

@@ -107,25 +107,6 @@ __device__ __forceinline__ bool loop_barrier(const LoopArgs& a, unsigned& gen, L
     return s_role >= 0;
 }
 
-// A table of depth ctr->d did not fit (the last CTA, all tests of the depth done):
-// nothing is removed, and the depth's state is as before its edge list, for the
-// kernels of a depth to start there.  Its tests stay counted.
-__device__ __noinline__ void hand_over(const LoopArgs& a, DepthCounters* ctr)
-{
-    const long long used[2] = {(long long)ctr->maxc[0] + 1, (long long)ctr->maxc[1] + 1};
-    __syncthreads();
-    for (int c = 0; c < 2; ++c)
-        for (long long k = threadIdx.x; k < used[c]; k += kTestThreads) a.hist[c * a.ord_cap + k] = a.cursor[c * a.ord_cap + k] = 0;
-    if (threadIdx.x == 0) {
-        for (int c = 0; c < 2; ++c)
-            ctr->n_edges[c] = ctr->maxc[c] = ctr->next_item[c] = ctr->total_items[c] = ctr->max_cells[c] = ctr->max_total[c] = 0;
-        ctr->split[0] = ctr->split[1] = 1;
-        ctr->adj_ends = 0;
-        ctr->gsel = ctr->whole = ctr->direct = 0;
-        *((volatile unsigned*)a.left) = kLoopHandedOver + (unsigned)ctr->d;
-    }
-}
-
 // The results to pinned host memory (one problem), after the last depth.
 __device__ __forceinline__ void loop_results(const LoopArgs& a, unsigned& gen, int warp0, int warps, long long t0,
                                              long long threads)
@@ -275,12 +256,15 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_loop(const __grid_constant_
                     scan_class(a.sc[cls], cls, ctr, a.mean_n, a.forced_group, a.split_stride, 1, marg, a.need_marg);
                     __syncthreads();
                 }
-                if (E <= kPlaceSerial) place(threadIdx.x, kTestThreads);
+                if (depth_is_heavy(ctr->cost[0] + ctr->cost[1], ctr->d, a.rec)) hand_over(a, ctr);
+                else if (E <= kPlaceSerial) place(threadIdx.x, kTestThreads);
             };
             if (!loop_barrier(a, gen, order)) return;
             const long long all = (long long)(ctr->n_edges[0] + ctr->n_edges[1]);
             big = (long long)ctr->n_edges[kClassCta];
-            if (!ctr->active) break;   // the same for every CTA
+            const int active = ctr->active;   // the same for every CTA
+            if (active < 0) return;
+            if (!active) break;
             if (!popc && all > kPlaceSerial) {
                 place(t0, threads);
                 if (!loop_barrier(a, gen, none)) return;
@@ -317,10 +301,10 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_loop(const __grid_constant_
         };
         if (direct) {   // removal, end of depth and the next depth's items
             if (!loop_barrier(a, gen, next)) return;
-            if (big > 0 && ctr->hand_over) return;   // set before the barrier: the same for every CTA
+            if (big > 0 && ctr->active < 0) return;   // set before the barrier: the same for every CTA
         } else {
             if (!loop_barrier(a, gen, over)) return;
-            if (big > 0 && ctr->hand_over) return;
+            if (big > 0 && ctr->active < 0) return;
             apply_edges(a.probs, a.edges, a.min_accept, a.edge_cap, a.binom, a.sep_pool, a.sep_cap, ctr, t0, threads,
                         a.bits);
             if (!loop_barrier(a, gen, next)) return;
@@ -328,7 +312,11 @@ __global__ void __launch_bounds__(kTestThreads, 2) k_loop(const __grid_constant_
         // turn() set it before the barrier opened.  Without the bit matrix the last
         // CTA may be ending the depth already (depth_end above): every CTA then
         // reads it behind the snapshot's barrier
-        if (a.bits && !ctr->active) break;
+        if (a.bits) {
+            const int active = ctr->active;
+            if (active < 0) return;
+            if (!active) break;
+        }
     }
     if (a.h_ctr) loop_results(a, gen, warp0, warps, t0, threads);
 }

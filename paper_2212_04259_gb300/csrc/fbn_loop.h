@@ -12,7 +12,8 @@ namespace fbn {
 constexpr int kTurnVertices = 128;   // variables of a problem whose depths one CTA prepares (fbn_turn.cuh)
 constexpr int kTurnItems = 32768;    // items of a class it lays out
 constexpr unsigned kLoopGaveUp = 1;      // a phase's wait ran out: the call starts over without the loop
-constexpr unsigned kLoopHandedOver = 2;  // + d: depth d holds a table that does not fit: the kernels of a depth go on there
+constexpr unsigned kLoopHandedOver = 2;  // + d: the kernels of a depth go on at depth d ...
+constexpr unsigned kLoopSplit = 1u << 16;   // ... and tests split by samples may not have run to their end
 
 // Everything the loop's phases take, by value.
 struct LoopArgs {

@@ -28,7 +28,7 @@ struct TurnShared {
     unsigned short pair[kTurnPairs];                // the live edges: i << 8 | j
     unsigned long long tests, sep_base;
     unsigned max_cells[2], max_total[2];
-    int removed, live, edges[2], at[2], items[2], chunks[2], too_big;
+    int removed, live, edges[2], at[2], items[2], chunks[2], too_big, heavy;
 };
 
 // The slot-th set bit of a row.
@@ -62,6 +62,44 @@ __device__ __forceinline__ int row_slot(const unsigned* row, int j)
     return c;
 }
 
+// The kernels of a depth take over at depth ctr->d (one CTA, the others waiting): a
+// table did not fit, or the depth is long enough for their speed to show.  Nothing of
+// the depth is removed, and its state is as before its edge list.  Tests made stay
+// counted.
+__device__ __noinline__ void hand_over(const LoopArgs& a, DepthCounters* ctr)
+{
+    const long long used[2] = {(long long)ctr->maxc[0] + 1, (long long)ctr->maxc[1] + 1};
+    __syncthreads();
+    for (int c = 0; c < 2; ++c)
+        for (long long k = threadIdx.x; k < used[c]; k += kTestThreads) a.hist[c * a.ord_cap + k] = a.cursor[c * a.ord_cap + k] = 0;
+    if (threadIdx.x == 0) {
+        for (int c = 0; c < 2; ++c)
+            ctr->n_edges[c] = ctr->maxc[c] = ctr->next_item[c] = ctr->total_items[c] = ctr->max_cells[c] = ctr->max_total[c] = 0;
+        const bool split = ctr->split[0] > 1 || ctr->split[1] > 1;
+        ctr->split[0] = ctr->split[1] = 1;
+        ctr->active = -1;
+        ctr->adj_ends = 0;
+        ctr->gsel = ctr->whole = ctr->direct = 0;
+        *((volatile unsigned*)a.left) = kLoopHandedOver + (unsigned)ctr->d + (split ? kLoopSplit : 0u);
+    }
+}
+
+// From this estimate of a depth's tests on the pools' own kernels win back a hand-over,
+// which costs some 80 us: their rows have more L1, and up to kLoopOneCta variables
+// twice the CTAs.  In the loop and handed over: 60 binary variables x 3,000 samples to
+// depth 3 375 and 318 ms, 30 of them 24.1 and 11.0, depth 1 of 25 variables of 16 values
+// x 100,000 (estimate 6.0e5), X^2, 1.67 and 1.28; depth 0 of 512 variables, 5.4e5, stays.
+// choose_pool counts every rank; the edges that the depth before left say how many are
+// tested (511 variables x 150 samples, 94% removed at depth 0: 20,235 of 579,390).
+constexpr float kLoopHeavy = 5.7e5f;   // cycles
+
+__device__ __forceinline__ bool depth_is_heavy(float cost, int d, const DepthRecord* rec)
+{
+    if (!(cost > kLoopHeavy) || d == 0 || d >= kMaxDepthRecords) return cost > kLoopHeavy;
+    const float edges = (float)rec[d - 1].edges;
+    return cost * (edges - (float)rec[d - 1].removed) > kLoopHeavy * edges;
+}
+
 // After the tests of depth ctr->d (apply: its removals are still to be made,
 // the depth's items having been listed here), the whole CTA.
 __device__ __noinline__ void turn(const LoopArgs& a, TurnShared& T, bool apply, int warps)
@@ -86,7 +124,7 @@ __device__ __noinline__ void turn(const LoopArgs& a, TurnShared& T, bool apply, 
     }
     if (tid == 0) {
         T.tests = 0;
-        T.removed = T.live = T.too_big = 0;
+        T.removed = T.live = T.too_big = T.heavy = 0;
         T.sep_base = ctr->sep_used;
     }
     __syncthreads();
@@ -232,6 +270,7 @@ __device__ __noinline__ void turn(const LoopArgs& a, TurnShared& T, bool apply, 
         a.min_accept[e] = (unsigned long long)total;
     }
     if (tid == 0) {
+        float cost = 0.0f;
         ctr->n_edges[0] = E0;
         ctr->n_edges[1] = E1;
         ctr->gs = gs;
@@ -243,7 +282,7 @@ __device__ __noinline__ void turn(const LoopArgs& a, TurnShared& T, bool apply, 
             ctr->next_item[c] = 0;
             ctr->total_items[c] = (unsigned long long)W[c];
             if (W[c] > 0 && !marg) {   // by the items that hold a test
-                choose_pool(a.sc[c], c, (unsigned long long)T.items[c], ctr, a.mean_n, a.forced_group, a.split_stride,
+                cost += choose_pool(a.sc[c], c, (unsigned long long)T.items[c], ctr, a.mean_n, a.forced_group, a.split_stride,
                             W[c] <= kSplitItems, a.need_marg);
                 ctr->total_items[c] = (unsigned long long)W[c] * (unsigned long long)ctr->split[c];
             }
@@ -252,7 +291,10 @@ __device__ __noinline__ void turn(const LoopArgs& a, TurnShared& T, bool apply, 
             r->t_begin = begin;
             r->t_tests = gtime();
         }
+        T.heavy = depth_is_heavy(cost, nd, a.rec);
     }
+    __syncthreads();
+    if (T.heavy) hand_over(a, ctr);
 }
 
 }  // namespace fbn

@@ -5,7 +5,8 @@ persistent loop (512), small batches, a depth with more items than the turn
 lays out (the general phases take over and give back), every kind of output
 buffer, separating sets read late, twice, or never between calls, a changing
 maximum depth on one handle, and many repeats of calls that stop at their maximum
-depth in the general phases (no bit matrix: above 128 variables, or a batch).
+depth in the general phases (no bit matrix: above 128 variables, or a batch), long
+depths that the graph takes over, waits that run out, and calls of several threads.
 """
 import numpy as np
 import pytest
@@ -56,6 +57,22 @@ def test_too_many_items_for_the_turn(F):
     h = F.fbn_create(data, ar)
     _same(F, h, F.fbn_learn_skeleton(h, 0.01, 3), ref)
     assert max(ref.tests) > 40000
+
+
+@pytest.mark.parametrize("stat", ["g2", "x2"])
+@pytest.mark.parametrize("n,r,md", [(24, 2, 3), (22, 6, 2), (70, 6, 1), (130, 6, 1)])
+def test_long_depths_go_to_the_graph(F, n, r, md, stat):
+    # listed directly (up to 128 variables), by the general phases (too many items, or more variables), and at depth 0
+    rng = np.random.default_rng(n + r)
+    N, keep = (1500, 0.4) if n < 100 else (400, 0.3)
+    base = rng.integers(0, r, N)
+    data = np.stack([np.where(rng.random(N) < keep, base, rng.integers(0, r, N)) for _ in range(n)]).astype(np.uint8)
+    ar = np.full(n, r, dtype=np.uint8)
+    ref = oracle.pc_stable(data, ar, 0.05, md, stat=stat)
+    h = F.fbn_create(data, ar, statistic=stat)
+    for _ in range(3):
+        st = _same(F, h, F.fbn_learn_skeleton(h, 0.05, md), ref)
+        assert st["depths"] == len(ref.tests) and (st["launches"] > 1 or n == 70)
 
 
 def test_outputs_and_late_reads(F):
