@@ -724,7 +724,7 @@ __device__ __forceinline__ void x2_term(int n, int nzz, int nx, int ny, bool nar
 
 // The bounded comparison shared by the FP32 decisions: sum = the group's FP32
 // sum of the terms, mag = the sum of their magnitudes, per_thread = terms a
-// thread added, levels = the depth of the cross-thread addition tree, term_rel
+// thread added, levels = the additions across threads a value goes through, term_rel
 // = a bound of a term's error against its own magnitude.  The
 // error analysis is the one stated for grp_decide_bound below.  Returns 1
 // (accept), 0 (reject) or -1 (the band straddles the bracket of crit).
@@ -744,11 +744,14 @@ __device__ __forceinline__ int decide_from_sums(float sum, float mag, float per_
 // 65,536 samples both products of the ratio fit 32 bits.  G^2: n ln(N / E) with
 // the exact difference D = n N_z - N_xz N_yz; ln as 2 atanh(D / (sum of the two
 // products)) by its series while the ratio is within [1/2, 2] (|s| <= 1/3: the
-// terms left out are below 2e-9 of the sum), else as lg2 of the ratio (error
-// 2^-22 of a result of at least 1).  64-bit integers are converted by halves (the
-// single conversion runs at the FP64 rate).  Conversions, sums and the approximate
-// quotient (2 ulp) leave each term within 8e-7 of itself.  X^2: D^2 / (N_z N_xz
-// N_yz), within the same bound.
+// terms left out are below 2e-9 of the sum), else as lg2 of the ratio.  64-bit
+// integers are converted by halves (the single conversion runs at the FP64 rate).
+// A term's error against itself, at most: in the series D and the sum (1.2e-7 and
+// 1.8e-7) and the quotient (2 ulp: 2.4e-7), 1.08 times as much of the logarithm, the
+// series and the product with n 2.2e-7: 8.1e-7; past a ratio of 2 two conversions and
+// the quotient (4.8e-7 of the ratio, over ln 2), lg2 (2 ulp: 2.4e-7), two products and
+// a conversion (1.8e-7): 1.12e-6.  X^2, D^2 / (N_z N_xz N_yz): 7.8e-7.  The largest of
+// 2e8 terms measured: 3.6e-7, 5.4e-7 and 4.3e-7.
 __device__ __forceinline__ float u64_float(unsigned long long v)   // within 1.2e-7 of itself
 {
     return fmaf((float)(unsigned)(v >> 32), 4294967296.0f, (float)(unsigned)v);
@@ -791,18 +794,19 @@ __device__ __forceinline__ void marg_term(int n, int nz, int nx, int ny, bool na
     acc += t;
     mag += fabsf(t);
 }
-constexpr float kMargTermRel = 8.0e-7f;
+constexpr float kMargTermRel = 1.2e-6f;
 
 // Decision "p > alpha" as "G^2 < crit" from FP32 terms under an error bound,
 // all in FP32 (the FP64 pipe of this part is 1/64 of FP32, and every thread
 // of a group would otherwise run the bound in it).  The terms are evaluated
-// with FP32 logarithms -- each within 3.2e-7 of its own magnitude, CUDA's logf
-// and log1pf being within 1 ulp and the ratio formed from exact 64-bit
-// integers -- and summed in FP32: a thread adds at most ceil(C/G) terms and
-// the group tree adds log2(G) levels, each addition erring by at most 6e-8 of
-// the running sum of magnitudes.  G^2 is thus within 2 (3.2e-7 + (ceil(C/G) +
-// log2 G) 6e-8) sum|term| of its exact value; the bound is doubled for margin,
-// formed with upward rounding, and compared against a float bracket [lo, hi]
+// with FP32 logarithms -- each within 7e-7 of its own magnitude: the ratio of
+// exact integers within 1.8e-7 (two conversions, a quotient), over ln 1.5 at most
+// 4.4e-7 of the logarithm, CUDA's logf and log1pf within 1 ulp (1.2e-7), the product
+// with n 1.2e-7 -- and summed in FP32: a thread adds at most ceil(C/G) terms, a warp
+// its lanes' sums in 5 levels, the group its warps' one after the other, each
+// addition erring by at most 6e-8 of the running sum of magnitudes.  G^2 is thus
+// within 2 (7e-7 + (ceil(C/G) + 4 + G/32) 6e-8) sum|term| of its exact value; the
+// bound is doubled for margin, formed with upward rounding, and compared against a float bracket [lo, hi]
 // of crit (lo <= crit <= hi): accept when G^2 + err < lo, reject when G^2 -
 // err >= hi (both rounded outward).  Returns 1 (accept), 0 (reject) or -1
 // when the band straddles the bracket and the caller decides exactly.
@@ -865,8 +869,8 @@ __device__ __forceinline__ int grp_decide_bound(const TestSpec& s, const int* T,
         }
     }
     const float per_thread = (float)((C + G - 1) / G);   // exact: C < 2^24
-    const float levels = (G == 32 ? 5.0f : G == 64 ? 6.0f : G == 128 ? 7.0f : G == 256 ? 8.0f : 10.0f);
-    return decide_from_sums(v.x, v.y, per_thread, levels, stat, crit_lo, crit_hi, stat == kStatX2 ? 6.0e-7f : 3.2e-7f);
+    constexpr float levels = 4.0f + (float)Grp<G>::kWarps;
+    return decide_from_sums(v.x, v.y, per_thread, levels, stat, crit_lo, crit_hi, stat == kStatX2 ? 6.0e-7f : 7.0e-7f);
 }
 
 // --------------------------------------------------------------------------

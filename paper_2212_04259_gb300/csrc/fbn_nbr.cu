@@ -170,7 +170,7 @@ __device__ __forceinline__ int warp_scan(int v, int lane)
 
 // G^2 decision of the test (x, y | z) from the INT32 sums: rows
 // zrow + c * rx + a, columns ycol + b.  Terms n ln(n n_c / (n_ac n_bc)) with
-// FP32 logarithms (each within 3.2e-7 of its magnitude, the ratio formed from
+// FP32 logarithms (each within 7e-7 of its magnitude, the ratio formed from
 // exact 64-bit integers) summed in FP32 by one thread (cells additions, each
 // within 6e-8 of the running sum of magnitudes); recomputed in FP64 only when
 // crit lies inside the error band.  Returns true when p > alpha.
@@ -212,7 +212,7 @@ __device__ bool test_decide(const int* T0, int rx, int ry, int rz, double crit)
             }
     }
     const double cells = (double)rx * ry * rz;
-    const double rel = 2.0 * (3.2e-7 + cells * 6e-8);
+    const double rel = 2.0 * (7e-7 + cells * 6e-8);
     const double g2 = 2.0 * (double)acc;
     const double err = 2.0 * rel * (double)mag * 1.0001 + 1e-9;
     if (g2 + err < crit) return true;
