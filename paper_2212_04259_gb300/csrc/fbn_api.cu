@@ -360,10 +360,12 @@ struct Workspace {
 struct DeviceInts {
     int32_t* d = nullptr;
     long long n = 0;
+    cudaEvent_t ready = nullptr;        // after the copy that fills d, on the batch's stream
     std::vector<fbn_handle*> members;   // the handles whose sets live here (a batch)
     ~DeviceInts()
     {
         if (d) cudaFree(d);
+        if (ready) cudaEventDestroy(ready);
     }
 };
 
@@ -898,6 +900,7 @@ int materialize_sepsets(fbn_handle* h, Workspace& ws)
     cudaStream_t st = h->stream;
     std::vector<fbn_handle*> todo;
     if (h->sep_snap) {
+        CK(cudaStreamWaitEvent(st, h->sep_snap->ready, 0));   // a member's stream need not be the batch's
         for (fbn_handle* q : h->sep_snap->members)
             if (q->sep_pending && q->device == h->device) todo.push_back(q);
     } else {
@@ -987,6 +990,7 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
     cudaStream_t st = h->stream;
     *retry = false;
     CK(cudaSetDevice(h->device));
+    if (h->sep_snap) CK(cudaStreamWaitEvent(st, h->sep_snap->ready, 0));   // a batch's copy out of this pool, on another stream perhaps
     long long edge_cap = 0;
     int max_n = 0, total_vtx = 0;
     std::vector<ProblemDev> P(k);
@@ -1729,6 +1733,8 @@ int run_skeleton_once(fbn_handle* const* hs, int k, double alpha, int32_t max_de
         CK(dalloc(&snap->d, snap->n));
         if (c.sep_used)
             CK(cudaMemcpyAsync(snap->d, ws.sep_pool, c.sep_used * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
+        CK(cudaEventCreateWithFlags(&snap->ready, cudaEventDisableTiming));
+        CK(cudaEventRecord(snap->ready, st));
     }
     for (int p = 0; p < k; ++p) {
         hs[p]->stats = stats;
