@@ -580,18 +580,28 @@ int check_status(fbn_handle* h, unsigned status)
     return FBN_OK;
 }
 
+// The address at which kernels of `device` reach [p, p + bytes) in place: memory of
+// the device or, with host, pinned host memory, from the first byte to the last;
+// else nullptr (then a copy, which checks the range itself).
+const void* device_range(const void* p, size_t bytes, int device, bool host)
+{
+    cudaPointerAttributes a{}, b{};
+    const char* last = (const char*)p + (bytes ? bytes - 1 : 0);
+    const bool ok = cudaPointerGetAttributes(&a, p) == cudaSuccess && a.devicePointer &&
+                    ((host && a.type == cudaMemoryTypeHost) || (a.type == cudaMemoryTypeDevice && a.device == device)) &&
+                    cudaPointerGetAttributes(&b, last) == cudaSuccess && b.type == a.type &&
+                    (const char*)b.devicePointer - (const char*)a.devicePointer == last - (const char*)p;
+    cudaGetLastError();
+    return ok ? a.devicePointer : nullptr;
+}
+
 // New samples into the handle's store, with their check and planes; *bad (device,
 // all ones before) receives the first bad value.  Pinned host memory and memory
 // of the handle's device are read by the kernel itself; pageable memory (and
 // any other) is copied first.
 int ingest(fbn_handle* h, const uint8_t* data, unsigned long long* bad, cudaStream_t st)
 {
-    const uint8_t* src = nullptr;
-    cudaPointerAttributes attr{};
-    if (cudaPointerGetAttributes(&attr, data) == cudaSuccess && attr.devicePointer &&
-        (attr.type == cudaMemoryTypeHost || (attr.type == cudaMemoryTypeDevice && attr.device == h->device)))
-        src = (const uint8_t*)attr.devicePointer;
-    cudaGetLastError();
+    const uint8_t* src = (const uint8_t*)device_range(data, (size_t)h->n * h->N, h->device, true);
     int64_t stride = h->N;
     uint8_t* store = h->d_data;
     if (!src) {
@@ -2368,11 +2378,7 @@ int fbn_pairwise_counts(fbn_handle* h, int32_t* counts, int64_t cap)
     rc = prepare_gram(hs, 1, ws, &P);
     if (rc) return rc;
     // straight into a device buffer of the caller's; else through the workspace
-    cudaPointerAttributes attr{};
-    const bool device_out = ((uintptr_t)counts & 3) == 0 &&
-                            cudaPointerGetAttributes(&attr, counts) == cudaSuccess &&
-                            attr.type == cudaMemoryTypeDevice && attr.device == h->device;
-    cudaGetLastError();
+    const bool device_out = ((uintptr_t)counts & 3) == 0 && device_range(counts, (size_t)MM * sizeof(int32_t), h->device, false);
     if (!device_out) {
         rc = prepare_pairs(hs, 1, ws, &P);
         if (rc) return rc;

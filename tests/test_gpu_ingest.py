@@ -85,3 +85,31 @@ def test_refused_then_valid_repeatedly(F, where):
             F.fbn_set_stream(h, streams[t // 3 % 2])
         F.fbn_update_data(h, good_m)
     assert np.array_equal(F.fbn_ci_table(h, 2, 1, [0]), oracle.ci_table(good, ar, 2, 1, [0]))
+
+
+# Only a part of the samples' memory is pinned: read through a copy, or refused by it, never in place.
+@pytest.mark.parametrize("part", ["first", "last"])
+def test_partly_pinned_samples(F, part):
+    import torch
+    rng = np.random.default_rng(3)
+    ar = np.array([3, 2, 4, 5], dtype=np.uint8)
+    N = 200_000
+    buf = np.zeros(4 * N + 8192, np.uint8)
+    at = -buf.ctypes.data % 4096
+    data = buf[at:at + 4 * N].reshape(4, N)
+    data[:] = np.stack([rng.integers(0, r, N) for r in ar])
+    good = data.copy()
+    h = F.fbn_create(good, ar)
+    rt = torch.cuda.cudart()
+    p = data.ctypes.data if part == "first" else data.ctypes.data + 4 * N // 4096 // 2 * 4096
+    assert int(rt.cudaHostRegister(p, 2 * N // 4096 * 4096, 0)) == 0
+    try:
+        try:
+            F.fbn_update_data(h, data)
+        except F.FbnError as e:
+            print("refused:", e)
+            F.fbn_update_data(h, good)
+        assert np.array_equal(F.fbn_ci_table(h, 0, 1, [2]), oracle.ci_table(good, ar, 0, 1, [2]))
+        assert np.array_equal(F.fbn_ci_table(h, 3, 2, []), oracle.ci_table(good, ar, 3, 2, []))
+    finally:
+        assert int(rt.cudaHostUnregister(p)) == 0
