@@ -284,10 +284,10 @@ __device__ __forceinline__ T grp_sum(T v, T* red)
 
 // --------------------------------------------------------------------------
 // Counting: one loop for every table in shared memory.  A table of C cells is
-// kept in K interleaved copies (K a power of two, at most the group's threads):
+// kept in K interleaved copies (K a power of two, at most 32):
 // copy k of cell c is word c K + k, and thread t counts into copy t mod K.  K is
-// the largest that fits, so small tables get a copy per thread (no two threads
-// of a warp meet in a word or a bank) and large ones at least a few: a warp's
+// the largest up to 32 that fits, so small tables get a copy per lane (no two
+// threads of a warp meet in a word or a bank) and large ones at least a few: a warp's
 // 32 updates of one shared copy met 3.9 deep in a cell (depth 2, arities 2-4),
 // in 4 copies 2.2, in 8 copies 1.8.  The update is a shared-memory reduction,
 // so consecutive samples do not wait on each other.  One loop with a runtime
@@ -483,7 +483,9 @@ static __device__ __noinline__ void count_global(const TestSpec& s, int* table, 
 }
 
 // Copies of a table of C cells: the most that fit, while zeroing and folding
-// them (C K words each) stays below the samples counted; where the marginals are
+// them (C K words each) stays below the samples counted, and at most one per lane of
+// a warp (with one per thread of a CTA few threads fold many words each: the
+// edge-level form of 300 variables x 30,000 samples 3.72 ms, 3.40 with 32); where the marginals are
 // kept too, one from kOneCopy cells on, where a warp's updates hardly meet (13 M
 // tests of 7,776 cells and 50,000 samples, X^2 with the observed df: 1,357 ms with
 // two copies, 1,230 with one; G^2 from the n ln n table: 637 and 639).
@@ -491,7 +493,7 @@ constexpr long long kOneCopy = 4096;
 template <int G>
 __device__ __forceinline__ int table_copies(long long C, long long slice_ints, int N, bool need_marg)
 {
-    int K = need_marg && C >= kOneCopy ? 1 : G;
+    int K = need_marg && C >= kOneCopy ? 1 : 32;
     while (K > 1 && (C * K > slice_ints || 2 * C * K > N)) K >>= 1;
     return K;
 }

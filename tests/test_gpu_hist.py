@@ -1,6 +1,6 @@
 """The histogram pools and the n ln n decision against the oracle.
 
-Tables in interleaved copies at every group size, from a copy per thread to
+Tables in interleaved copies at every group size, from a copy per lane to
 one; tables around a warp's, a CTA's and the big class's shared memory and in
 global memory; sample counts around the 16-sample vectors and two vectors per
 thread; the same skeletons without the n ln n table (Pearson's statistic,
