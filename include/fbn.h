@@ -66,7 +66,8 @@ extern "C" {
 
 #define FBN_LOOP_DEVICE 0  /* no host round trip between depths: calls of up to 512 variables without a tensor-core
                               depth run as one persistent kernel, the others launch the first depths directly and
-                              the rest as one CUDA graph whose while node the device drives */
+                              the rest as one CUDA graph whose while node the device drives.  The kernel hands
+                              over to the graph, once, at a depth of long tests or of tables above 64 KB */
 #define FBN_LOOP_HOST   1  /* the same kernels, one depth at a time from the host, which reads the loop flag
                               between depths (for tools that profile kernel by kernel) */
 

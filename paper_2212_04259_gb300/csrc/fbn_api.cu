@@ -820,8 +820,6 @@ int run_gram(fbn_handle* h, Workspace& ws, int k, int total_vtx, unsigned* d_sta
     return FBN_OK;
 }
 
-// Copy the separating sets of h (in the pool of workspace ws) to the host,
-// as CSR rows per removed pair.
 // Move a handle to another separating-set snapshot (or to none).
 void set_snapshot(fbn_handle* h, std::shared_ptr<DeviceInts> snap)
 {

@@ -248,8 +248,8 @@ __device__ __forceinline__ void ci_cluster_test(const CiArgs& q)
         __syncthreads();
         if (c1 > c0) {
             grp_marginals<kTestThreads>(spec, T, M);
-            st = q.stat == kStatX2 ? grp_x2_exact<kTestThreads>(spec, T, M, red, nullptr)
-                                   : grp_g2_exact<kTestThreads>(spec, T, M, red, nullptr);
+            st = q.stat == kStatX2 ? grp_x2_exact<kTestThreads>(spec, T, M, red)
+                                   : grp_g2_exact<kTestThreads>(spec, T, M, red);
             if (q.df_mode) {
                 __syncthreads();
                 df = (double)grp_df_adjusted<kTestThreads>(spec, M, red);

@@ -610,8 +610,7 @@ __device__ __forceinline__ void grp_marginals(const TestSpec& s, const int* T, i
 // integers and its log taken as log1p of the exact difference over the
 // denominator.
 template <int G>
-__device__ __forceinline__ double grp_g2_exact(const TestSpec& s, const int* T, const int* M, double* red,
-                                               int32_t* table_out)
+__device__ __forceinline__ double grp_g2_exact(const TestSpec& s, const int* T, const int* M, double* red)
 {
     const int rx = s.rx, ry = s.ry, rxy = rx * ry, C = (int)s.cells;
     const int nz = C / rxy;
@@ -621,7 +620,6 @@ __device__ __forceinline__ double grp_g2_exact(const TestSpec& s, const int* T, 
     double acc = 0.0;
     for (int c = Grp<G>::rank(); c < C; c += G) {
         const int n = T[c];
-        if (table_out) table_out[c] = n;
         if (n == 0) continue;
         const int z = c / rxy;
         const int rem = c - z * rxy;
@@ -641,8 +639,7 @@ constexpr int kStatX2 = 1;
 // cells included), each term (N_xyz N_++z - N_x+z N_+yz)^2 / (N_++z N_x+z
 // N_+yz) with the difference an exact 64-bit integer.
 template <int G>
-__device__ __forceinline__ double grp_x2_exact(const TestSpec& s, const int* T, const int* M, double* red,
-                                               int32_t* table_out)
+__device__ __forceinline__ double grp_x2_exact(const TestSpec& s, const int* T, const int* M, double* red)
 {
     const int rx = s.rx, ry = s.ry, rxy = rx * ry, C = (int)s.cells;
     const int nz = C / rxy;
@@ -652,7 +649,6 @@ __device__ __forceinline__ double grp_x2_exact(const TestSpec& s, const int* T, 
     double acc = 0.0;
     for (int c = Grp<G>::rank(); c < C; c += G) {
         const int n = T[c];
-        if (table_out) table_out[c] = n;
         const int z = c / rxy;
         const int rem = c - z * rxy;
         const int x = rem / ry, y = rem - x * ry;

@@ -430,7 +430,8 @@ __global__ void __launch_bounds__(256) k_pairs_gram(const ProblemDev* __restrict
             if (P.max_arity <= kPairArity) {
                 // the block's loads in flight together, its cells through this
                 // lane's column of shared memory, so that the terms are one
-                // small loop (25 inlined terms spilled)
+                // small loop (the loads still spill some 250 bytes of 128
+                // registers in the deciding kernel)
                 int (*cv)[32] = s_cell[threadIdx.x >> 5];
                 int (*cj)[32] = s_nj[threadIdx.x >> 5];
                 int v[kPairArity - 1][kPairArity - 1], nj[kPairArity - 1], ni[kPairArity - 1];
@@ -573,7 +574,8 @@ __global__ void __launch_bounds__(256) k_pairs_gram(const ProblemDev* __restrict
 // added the terms in FP32: pair counts on the device of 10 variables of 200 values x
 // 3,000 samples 9.19 -> 0.11 ms, of 100 of 30 values x 20,000 0.49 -> 0.22 ms, depth 0
 // of 40 of 255 values x 10,000 45.8 -> 6.2 ms.  FP64 costs where blocks are small:
-// depth 0 of 300 variables of 10 values x 20,000 0.25 -> 0.65 ms.
+// depth 0 of 300 variables of 10 values x 20,000 0.25 -> 0.65 ms.  (With 1,024 threads
+// the deciding kernel spills 408 bytes of stores, in the FP64 logarithm's call.)
 template <int G>
 constexpr int kWideThreads = G > kTestThreads ? G : kTestThreads;
 

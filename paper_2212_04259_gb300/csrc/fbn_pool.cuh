@@ -114,7 +114,7 @@ __device__ __forceinline__ int decide_test(const PoolArgs& a, const TestSpec& sp
     // the band straddles crit: exact FP64 statistic against the exact value
     if (Grp<G>::rank() == 0 && S.crit == 0.0) S.crit = crit_get(a.crit, df, a.alpha, status);
     Grp<G>::sync();
-    const double ex = a.stat == kStatX2 ? grp_x2_exact<G>(spec, T, M, red, nullptr) : grp_g2_exact<G>(spec, T, M, red, nullptr);
+    const double ex = a.stat == kStatX2 ? grp_x2_exact<G>(spec, T, M, red) : grp_g2_exact<G>(spec, T, M, red);
     return ex < S.crit ? 1 : 0;
 }
 
@@ -144,7 +144,6 @@ __device__ __forceinline__ int decide_lut(const PoolArgs& a, const TestSpec& spe
     return ex < S.crit ? 1 : 0;
 }
 
-// Run one rank: 1 = accepts independence, 0 = rejects, -1 = could not run.
 // Counting work of one table (rank 0): one shared-memory update per sample.
 template <int G>
 __device__ __forceinline__ void note_work(GroupState& S, const TestSpec& spec)
@@ -153,6 +152,7 @@ __device__ __forceinline__ void note_work(GroupState& S, const TestSpec& spec)
     S.smem_updates += (unsigned long long)spec.N;
 }
 
+// Run one rank: 1 = accepts independence, 0 = rejects, -1 = could not run.
 template <int G>
 __device__ __forceinline__ int run_rank(const PoolArgs& a, int d, const ProblemDev& P, const EdgeWork& w, long long rk,
                                         bool fresh, GroupState& S, TestSpec& spec, int* slice, long long slice_ints,
