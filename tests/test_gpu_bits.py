@@ -1,16 +1,15 @@
-"""Bit-plane counting against the oracle.
+"""The counting option against the oracle.
 
-Tables of tests whose variables all have arity <= 4 (and at most two
-conditioning variables) can be counted from two bit planes per variable with
-popcounts (count="bits" forces it wherever it fits, count="auto" uses it for
-small tables).  Tables must be bit-exact, G^2 within 1e-6 relative and p
-within 1e-9 absolute of the oracle, and skeletons and separating sets
-identical to the oracle's (the near-alpha rule of tests/_compare.py).
-Covered: every value of every arity (minterms 0-3 and the zero padding),
-sample counts around the 32-sample word and the 128-sample group, tables
-with arities above 4 (counted by the byte histogram instead), explicit tests
-(a CTA group) and the work pool at every group size, with sample-split
-tests, single problems and a batch.
+Skeletons of variables with at most 5 values count depths 0 and 1 from one-hot
+bit planes with popcounts (count="auto" and "bits"); count="hist", the deeper
+depths and explicit tests count byte histograms.  Whatever the option, tables
+must be bit-exact, G^2 within 1e-6 relative and p within 1e-9 absolute of the
+oracle, and skeletons and separating sets identical to the oracle's (the
+near-alpha rule of tests/_compare.py).  Covered: explicit tests of handles with
+planes, at sample counts around the 32-sample word and the 128-sample group and
+with constant rows; skeletons at every group size, with sample-split tests,
+mixed arities, single problems and a batch, and that their first two depths were
+counted from the planes; an update of the samples.
 """
 import numpy as np
 import pytest
@@ -35,7 +34,7 @@ def _rand(seed, arities, N, skew=False):
     rng = np.random.default_rng(seed)
     rows = []
     for r in arities:
-        if skew:   # mostly the top value: the all-ones minterm
+        if skew:   # mostly the top value
             rows.append(np.where(rng.random(N) < 0.7, r - 1, rng.integers(0, r, N)))
         else:
             rows.append(rng.integers(0, r, N))
@@ -70,7 +69,7 @@ def test_bits_tests_match_oracle(F, skew):
 
 
 def test_bits_constant_and_top_values(F):
-    # constant rows (only one minterm occupied), rows at the top value only
+    # constant rows, rows at the top value only
     N = 5003
     data = np.stack([np.zeros(N), np.full(N, 3), np.full(N, 1), np.arange(N) % 4, (np.arange(N) // 7) % 3]
                     ).astype(np.uint8)
@@ -95,10 +94,11 @@ def test_bits_skeletons_match_oracle(F, gt, count):
         assert not hard and not excused and not cascade, (name, gt, count, hard[:3])
         st = F.fbn_get_stats(h)
         assert st["tests_oracle"] == ref.tests and st["removed"] == ref.removed
+        assert st["popc_work"][0] > 0 and st["popc_work"][1] > 0 and st["smem_updates"][:2] == [0, 0]
 
 
 def test_bits_skeleton_mixed_arities(F):
-    # arities up to 5: tests with an arity-5 variable fall back to the histogram
+    # arities up to 5, the most that the planes hold
     data, ar, _ = bnsynth.make_dataset(515, 30, 40, 3, (2, 3, 4, 5), 0.7, 20000)
     ref = oracle.pc_stable(data, ar, 0.05, -1)
     for count in ("auto", "bits"):
@@ -106,6 +106,8 @@ def test_bits_skeleton_mixed_arities(F):
         adj = F.fbn_learn_skeleton(h, 0.05, -1)
         hard, _, _ = compare(adj, F.fbn_export_sepsets(h), ref)
         assert not hard, (count, hard[:3])
+        st = F.fbn_get_stats(h)
+        assert st["popc_work"][1] > 0 and st["smem_updates"][1] == 0
 
 
 def test_bits_batch_matches_oracle(F):
