@@ -38,8 +38,8 @@
 namespace fbn {
 
 // Launches of the depth kernels go through launch_pdl; set_pdl(false)
-// launches them without the attribute.
-static bool g_pdl = true;
+// launches them without the attribute, on this thread (a capture's retry).
+static thread_local bool g_pdl = true;
 
 // The work-pool kernels, each defined in its own translation unit.
 __global__ void k_pool_small(PoolArgs a);

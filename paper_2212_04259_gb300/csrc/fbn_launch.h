@@ -47,7 +47,7 @@ void launch_depth_end(DepthCounters* ctr, DepthRecord* rec, int max_depth, unsig
                       unsigned long long* cursor, cudaStream_t st);
 // The depth loop's condition: 1 while the next depth has an edge to test.
 void launch_gate(DepthCounters* ctr, cudaGraphConditionalHandle loop, cudaStream_t st);
-// Programmatic dependent launch for the depth kernels (on by default).
+// Programmatic dependent launch for this thread's depth kernels (on by default).
 void set_pdl(bool on);
 // Explicit tests: the kernel's limits and its largest cluster, then one test.
 cudaError_t prepare_ci(size_t smem_bytes, int* max_cluster);
